@@ -17,83 +17,79 @@ namespace nk {
 namespace {
 
 // ------------------------------------------------------ tile GEMM engine ---
-// C(m, n) = sum_{k in split} A(m, k) B(n, k): 64 x 64 tile per block, 256
-// threads with 4 x 4 outputs, K staged 16 at a time in shared memory.  The
-// loaders say whether k (kContig = true) or m/n is the contiguous index in
-// memory so that the staging loads coalesce either way.
+// C(m, n) = sum_{k in split} A(m, k) B(n, k) in FP64: 16 x 16 tile per block,
+// one output per thread, K staged 32 at a time in shared memory with the next
+// 32 already in registers.  The loaders say whether k (kContig = true) or m/n
+// is the contiguous index in memory so that the staging loads coalesce either
+// way.
+// The FP64 pipe of this part (2 lanes a clock and SM) bounds every shape, so
+// the tile is as small as the block: nothing is computed for padding beyond
+// 15 rows and columns, and a small product still spreads over many SMs (64 x
+// 64 tiles with 4 x 4 outputs a thread, on one SM: 296 us for a 17 x 17 x 256
+// product, 244 us for 46 x 38 x 1025).  Products large enough for the tensor
+// cores do not come here (f64_on_tensor).
+
+constexpr int kGT = 16, kGK = 32;
 
 template <class LA, class LB, class EP>
-__global__ void __launch_bounds__(256) k_gemm64(int64_t Md, int64_t Nd, int64_t Kd, int64_t kchunk,
+__global__ void __launch_bounds__(256) k_gemm16(int64_t Md, int64_t Nd, int64_t Kd, int64_t kchunk,
                                                 LA la, LB lb, EP ep) {
-    __shared__ double As[16][64 + 1];
-    __shared__ double Bs[16][64 + 1];
+    __shared__ double As[kGK][kGT + 1];
+    __shared__ double Bs[kGK][kGT + 1];
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const int64_t m0 = (int64_t)blockIdx.y * 64, n0 = (int64_t)blockIdx.x * 64;
+    const int64_t m0 = (int64_t)blockIdx.x * kGT, n0 = (int64_t)blockIdx.y * kGT;
     if (!ep.active(m0, n0)) return;
     const int split = blockIdx.z;
     const int64_t kb = (int64_t)split * kchunk;
     const int64_t ke = kb + kchunk < Kd ? kb + kchunk : Kd;
-    double acc[4][4] = {};
-    for (int64_t k0 = kb; k0 < ke; k0 += 16) {
-        for (int e = threadIdx.x; e < 1024; e += 256) {
-            int kk, r;
-            if (LA::kContig) {
-                kk = e & 15;
-                r = e >> 4;
-            } else {
-                r = e & 63;
-                kk = e >> 6;
-            }
-            const int64_t k = k0 + kk;
-            As[kk][r] = (m0 + r < Md && k < ke) ? la(m0 + r, k) : 0.0;
-            if (LB::kContig) {
-                kk = e & 15;
-                r = e >> 4;
-            } else {
-                r = e & 63;
-                kk = e >> 6;
-            }
-            const int64_t k2 = k0 + kk;
-            Bs[kk][r] = (n0 + r < Nd && k2 < ke) ? lb(n0 + r, k2) : 0.0;
+    // the two elements of each operand that this thread stages
+    int ka[2], ra[2], kbb[2], rb[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        const int e = threadIdx.x + 256 * u;
+        ka[u] = LA::kContig ? (e & 31) : (e >> 4);
+        ra[u] = LA::kContig ? (e >> 5) : (e & 15);
+        kbb[u] = LB::kContig ? (e & 31) : (e >> 4);
+        rb[u] = LB::kContig ? (e >> 5) : (e & 15);
+    }
+    double av[2], bv[2];
+    auto fetch = [&](int64_t k0) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            av[u] = (m0 + ra[u] < Md && k0 + ka[u] < ke) ? la(m0 + ra[u], k0 + ka[u]) : 0.0;
+            bv[u] = (n0 + rb[u] < Nd && k0 + kbb[u] < ke) ? lb(n0 + rb[u], k0 + kbb[u]) : 0.0;
+        }
+    };
+    double acc = 0.0;
+    fetch(kb);
+    for (int64_t k0 = kb; k0 < ke; k0 += kGK) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            As[ka[u]][ra[u]] = av[u];
+            Bs[kbb[u]][rb[u]] = bv[u];
         }
         __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < 16; ++kk) {
-            double av[4], bv[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                av[u] = As[kk][ty * 4 + u];
-                bv[u] = Bs[kk][tx * 4 + u];
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int v = 0; v < 4; ++v) acc[u][v] = fma(av[u], bv[v], acc[u][v]);
+        if (k0 + kGK < ke) fetch(k0 + kGK);
+        const int kn = (int)(ke - k0 < kGK ? ke - k0 : kGK);
+        if (kn == kGK) {
+#pragma unroll 8
+            for (int kk = 0; kk < kGK; ++kk) acc = fma(As[kk][ty], Bs[kk][tx], acc);
+        } else {
+            for (int kk = 0; kk < kn; ++kk) acc = fma(As[kk][ty], Bs[kk][tx], acc);
         }
         __syncthreads();
     }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const int64_t m = m0 + ty * 4 + u;
-        if (m >= Md) continue;
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            const int64_t n = n0 + tx * 4 + v;
-            if (n < Nd) ep(m, n, split, acc[u][v]);
-        }
-    }
+    const int64_t m = m0 + ty, n = n0 + tx;
+    if (m < Md && n < Nd) ep(m, n, split, acc);
 }
 
 template <class LA, class LB, class EP>
-cudaError_t gemm64(int64_t Md, int64_t Nd, int64_t Kd, int splits, LA la, LB lb, EP ep,
-                   cudaStream_t st) {
+cudaError_t gemm16(int64_t Md, int64_t Nd, int64_t Kd, int splits, LA la, LB lb, EP ep, cudaStream_t st) {
     if (Md <= 0 || Nd <= 0) return cudaSuccess;
     if (splits < 1) splits = 1;
-    int64_t kchunk = (Kd + splits - 1) / splits;
-    kchunk = (kchunk + 15) / 16 * 16;
-    if (kchunk < 16) kchunk = 16;
-    dim3 grid((unsigned)((Nd + 63) / 64), (unsigned)((Md + 63) / 64), (unsigned)splits);
-    (k_gemm64<<<grid, 256, 0, st>>>(Md, Nd, Kd, kchunk, la, lb, ep), nk::note_launch());
+    const int64_t kchunk = (Kd + splits - 1) / splits;
+    dim3 grid((unsigned)((Md + kGT - 1) / kGT), (unsigned)((Nd + kGT - 1) / kGT), (unsigned)splits);
+    (k_gemm16<<<grid, 256, 0, st>>>(Md, Nd, Kd, kchunk > 0 ? kchunk : 1, la, lb, ep), nk::note_launch());
     return cudaGetLastError();
 }
 
@@ -102,23 +98,22 @@ cudaError_t gemm64(int64_t Md, int64_t Nd, int64_t Kd, int splits, LA la, LB lb,
 // B' = [S, 1]: P[j<M][i<N] is the W block, P[j][N] the b block and P[M][i]
 // the a block of J^T g.
 
-struct VjpA {
+struct VjpA {  // A'(j, k) = T_kj (j < M) or 1
     static constexpr bool kContig = false;
-    const double *T, *g, *shift;
-    double scale;
+    const double *T;
     int M;
-    __device__ double operator()(int64_t j, int64_t k) const {
-        const double gk = scale * (g[k] - (shift ? *shift : 0.0));
-        return (j < M ? T[(size_t)k * M + j] : 1.0) * gk;
-    }
+    __device__ double operator()(int64_t j, int64_t k) const { return j < M ? T[(size_t)k * M + j] : 1.0; }
 };
 
-struct AugS_kn {  // B'(i, k) = s_ki (i < N) or 1, i contiguous
+struct AugSg_kn {  // g'_k B'(i, k), g'_k = scale (g_k - shift), B' = s_ki (i < N) or 1, i contiguous
     static constexpr bool kContig = false;
     const int8_t *s;
+    const double *g, *shift;
+    double scale;
     int N;
     __device__ double operator()(int64_t i, int64_t k) const {
-        return i < N ? (double)s[(size_t)k * N + i] : 1.0;
+        const double gk = scale * (g[k] - (shift ? *shift : 0.0));
+        return i < N ? (double)s[(size_t)k * N + i] * gk : gk;
     }
 };
 
@@ -138,8 +133,14 @@ __global__ void k_vjp_reduce(int N, int M, int splits, const double *__restrict_
     if (idx >= plane) return;
     const int j = (int)(idx / (N + 1)), i = (int)(idx % (N + 1));
     if (j == M && i == N) return;
-    double s = 0.0;
-    for (int sp = 0; sp < splits; ++sp) s += P[(size_t)sp * plane + idx];
+    // four chains over the splits, so that their loads and adds overlap
+    double q[4] = {0.0, 0.0, 0.0, 0.0};
+    int sp = 0;
+    for (; sp + 3 < splits; sp += 4)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) q[u] += P[(size_t)(sp + u) * plane + idx];
+    for (; sp < splits; ++sp) q[0] += P[(size_t)sp * plane + idx];
+    const double s = (q[0] + q[1]) + (q[2] + q[3]);
     if (j == M)
         out[i] = s;
     else if (i == N)
@@ -148,11 +149,14 @@ __global__ void k_vjp_reduce(int N, int M, int splits, const double *__restrict_
         out[N + M + (size_t)j * N + i] = s;
 }
 
+// Splits of the K = Ns range: about four blocks per SM (the FP64 pipe is full
+// with two), at least 8 samples each and at most 128 partial planes.
 int vjp_splits(int N, int M, int64_t Ns) {
-    const int64_t tiles = ((M + 1 + 63) / 64) * ((N + 1 + 63) / 64);
-    int64_t sp = (1216 + tiles - 1) / tiles;  // ~8 blocks per SM on 152 SMs
-    const int64_t maxsp = (Ns + 255) / 256;   // at least 256 samples per split
+    const int64_t tiles = (int64_t)((M + 1 + kGT - 1) / kGT) * ((N + 1 + kGT - 1) / kGT);
+    int64_t sp = (608 + tiles - 1) / tiles;
+    const int64_t maxsp = (Ns + 7) / 8;
     if (sp > maxsp) sp = maxsp;
+    if (sp > 128) sp = 128;
     if (sp < 1) sp = 1;
     return (int)sp;
 }
@@ -276,7 +280,7 @@ struct EpSyrk {
     double *C;
     int64_t n;
     double scale, eps;
-    __device__ bool active(int64_t m0, int64_t n0) const { return n0 <= m0 + 63; }
+    __device__ bool active(int64_t m0, int64_t n0) const { return n0 <= m0 + kGT - 1; }
     __device__ void operator()(int64_t m, int64_t q, int, double v) const {
         if (q > m) return;
         const double r = v * scale + (m == q ? eps : 0.0);
@@ -479,7 +483,7 @@ struct PanelLoad {  // L(r, c) = A[(off + r) n + k + c], c contiguous
 struct EpTrailing {
     double *A;
     int64_t n, off;
-    __device__ bool active(int64_t m0, int64_t n0) const { return n0 <= m0 + 63; }
+    __device__ bool active(int64_t m0, int64_t n0) const { return n0 <= m0 + kGT - 1; }
     __device__ void operator()(int64_t r, int64_t q, int, double v) const {
         if (q > r) return;
         A[(size_t)(off + r) * n + off + q] -= v;
@@ -775,12 +779,12 @@ cudaError_t launch_vjp(int N, int M, int64_t Ns, const int8_t *s, const double *
                        double g_scale, const double *g_shift, double *partial, double *out,
                        cudaStream_t st) {
     const int sp = vjp_splits(N, M, Ns);
-    VjpA la{T, g, g_shift, g_scale, M};
-    AugS_kn lb{s, N};
+    VjpA la{T, M};
+    AugSg_kn lb{s, g, g_shift, g_scale, N};
     const int64_t plane = (int64_t)(M + 1) * (N + 1);
     EpPartial ep{partial, N + 1, plane};
     const int slot = prof_begin(NK_PROF_JVP_VJP, st);
-    cudaError_t err = gemm64(M + 1, N + 1, Ns, sp, la, lb, ep, st);
+    cudaError_t err = gemm16(M + 1, N + 1, Ns, sp, la, lb, ep, st);
     if (err != cudaSuccess) return err;
     (k_vjp_reduce<<<nblk(plane, 256), 256, 0, st>>>(N, M, sp, partial, out), nk::note_launch());
     prof_end(slot, st, 2.0 * (double)Ns * (N + 1) * (double)(M + 1));
@@ -793,7 +797,7 @@ cudaError_t launch_jvp(int N, int M, int64_t Ns, const int8_t *s, const double *
     VAug lb{v, N, M};
     EpStore ep{U, M + 1};
     const int slot = prof_begin(NK_PROF_JVP_VJP, st);
-    cudaError_t err = gemm64(Ns, M + 1, N + 1, 1, la, lb, ep, st);
+    cudaError_t err = gemm16(Ns, M + 1, N + 1, 1, la, lb, ep, st);
     if (err != cudaSuccess) return err;
     (k_rowdot_aug<<<nblk(Ns, 8), 256, 0, st>>>(M, Ns, T, U, out), nk::note_launch());
     prof_end(slot, st, 2.0 * (double)Ns * (N + 1) * (double)(M + 1) + 2.0 * (double)Ns * (M + 1));
@@ -845,7 +849,7 @@ cudaError_t launch_syrk_t(const double *A, int64_t rows, int64_t cols, double sc
                           double *C, cudaStream_t st) {
     ColMajorA la{A, cols};
     EpSyrk ep{C, cols, scale, eps};
-    return gemm64(cols, cols, rows, 1, la, la, ep, st);
+    return gemm16(cols, cols, rows, 1, la, la, ep, st);
 }
 
 cudaError_t launch_gram_samplespace(int N, int M, int64_t Ns, const int8_t *s, const double *T,
@@ -880,7 +884,7 @@ cudaError_t launch_cholesky(double *A, int64_t n, int *info, cudaStream_t st) {
             PanelLoad pl{A, n, k + kb, k};
             EpTrailing ep{A, n, k + kb};
             slot = prof_begin(NK_PROF_CHOL_UPDATE, st);
-            cudaError_t err = gemm64(rest, rest, kb, 1, pl, pl, ep, st);
+            cudaError_t err = gemm16(rest, rest, kb, 1, pl, pl, ep, st);
             prof_end(slot, st, (double)kb * rest * (double)(rest + 1));
             if (err != cudaSuccess) return err;
         }

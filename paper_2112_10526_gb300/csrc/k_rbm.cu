@@ -1032,52 +1032,35 @@ __global__ void __launch_bounds__(eloc_warps(kU) * 32) k_eloc_batched(ElocBK P) 
 
 // --------------------------------------------------------- batched theta ---
 
-// T[k][j] = tanh(b_j + sum_i W_ji s_ki): 64 x 64 output tile per block,
-// 256 threads with 4 x 4 outputs each, FP64 FMA.
+// T[k][j] = tanh(b_j + sum_i W_ji s_ki): 16 x 16 output tile per block, one
+// output per thread, FP64 FMA (bound by the FP64 pipe: see k_gemm16).
 __global__ void __launch_bounds__(256) k_theta_tanh(int N, int M, const double *__restrict__ b,
                                                     const double *__restrict__ W,
                                                     const int8_t *__restrict__ s, int64_t B,
                                                     double *__restrict__ T) {
-    __shared__ double Sa[16][64 + 1];
-    __shared__ double Wb[16][64 + 1];
+    __shared__ double Sa[32][16 + 1];
+    __shared__ double Wb[32][16 + 1];
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const int64_t k0 = (int64_t)blockIdx.y * 64;
-    const int j0 = blockIdx.x * 64;
-    double acc[4][4] = {};
-    for (int i0 = 0; i0 < N; i0 += 16) {
-        for (int e = threadIdx.x; e < 16 * 64; e += 256) {
-            const int ii = e & 15, rr = e >> 4;
+    const int64_t k0 = (int64_t)blockIdx.x * 16;
+    const int j0 = blockIdx.y * 16;
+    double acc = 0.0;
+    for (int i0 = 0; i0 < N; i0 += 32) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int e = threadIdx.x + 256 * u, ii = e & 31, rr = e >> 5;
             const int64_t kk = k0 + rr;
             const int jj = j0 + rr, ic = i0 + ii;
             Sa[ii][rr] = (kk < B && ic < N) ? (double)s[(size_t)kk * N + ic] : 0.0;
             Wb[ii][rr] = (jj < M && ic < N) ? W[(size_t)jj * N + ic] : 0.0;
         }
         __syncthreads();
-#pragma unroll
-        for (int ii = 0; ii < 16; ++ii) {
-            double av[4], bv[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                av[u] = Sa[ii][ty * 4 + u];
-                bv[u] = Wb[ii][tx * 4 + u];
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int v = 0; v < 4; ++v) acc[u][v] = fma(av[u], bv[v], acc[u][v]);
-        }
+        const int n = N - i0 < 32 ? N - i0 : 32;
+        for (int ii = 0; ii < n; ++ii) acc = fma(Sa[ii][ty], Wb[ii][tx], acc);
         __syncthreads();
     }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const int64_t kk = k0 + ty * 4 + u;
-        if (kk >= B) continue;
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            const int jj = j0 + tx * 4 + v;
-            if (jj < M) T[(size_t)kk * M + jj] = tanh(acc[u][v] + b[jj]);
-        }
-    }
+    const int64_t kk = k0 + ty;
+    const int jj = j0 + tx;
+    if (kk < B && jj < M) T[(size_t)kk * M + jj] = tanh(acc + b[jj]);
 }
 
 template <typename R>
@@ -1278,7 +1261,7 @@ template cudaError_t launch_eloc<float>(const Tables<float> &, const ElocArgs &,
 cudaError_t launch_theta_tanh(int N, int M, const double *b, const double *W, const int8_t *s,
                               int64_t B, double *T, cudaStream_t st) {
     if (B <= 0) return cudaSuccess;
-    dim3 grid((M + 63) / 64, (unsigned)((B + 63) / 64));
+    dim3 grid((unsigned)((B + 15) / 16), (M + 15) / 16);
     (k_theta_tanh<<<grid, 256, 0, st>>>(N, M, b, W, s, B, T), nk::note_launch());
     return cudaGetLastError();
 }

@@ -47,8 +47,19 @@ constexpr int kAB = kBM * kBK * 2;             // A tile, bytes
 constexpr int kBB = kBN * kBK * 2;             // one B slice tile, bytes
 constexpr int kSgOutLd = kBN + 1;
 
+// The unsliced operands of a product: A row r, column k = s[r][k] (1 at k =
+// N), B row c, column k = X[c * ldx + k]; transposed: A row r, column k =
+// s[k][r] (1 at r = N), B row c, column k = X[k * ldx + c] g[k] (X = 1 at c =
+// ldx).
+struct SgRaw {
+    const int8_t *s;
+    const double *X, *g;
+    int64_t ldx;
+    int N, transposed;
+};
+
 struct SgArgs {
-    int64_t rows, cols;
+    int64_t rows, cols, K;
     int kchunks, SB;
     int kc_split;         // K-chunks per split (blockIdx.z)
     int nstages, stage_bytes;
@@ -61,7 +72,31 @@ struct SgArgs {
     const double *T;      // mode 3: T [rows][Mt]; t'_col = T[col] for col < Mt, 1 at col = Mt
     int Mt;
     int *err;
+    SgRaw raw;
+    int drop;             // low bits left out of the recombined product; -1: ten (window10)
 };
+
+// Columns whose exponent is outside this range (an infinity or a NaN among
+// the entries, or values whose products could leave the FP64 range) are not
+// cut into slices but multiplied out in FP64 by the epilogue.
+__host__ __device__ inline bool flagged_exp(int e) { return e > 900 || (e < -900 && e > -100000); }
+
+// Output (row, col) over k in [k0, k1) in FP64, from the unsliced operands.
+__device__ __noinline__ double raw_product(const SgRaw &w, int64_t row, int64_t col, int64_t k0, int64_t k1) {
+    double acc = 0.0;
+    for (int64_t k = k0; k < k1; ++k) {
+        double a, b;
+        if (w.transposed) {
+            a = row < w.N ? (double)w.s[(size_t)k * w.N + row] : 1.0;
+            b = (col < w.ldx ? w.X[(size_t)k * w.ldx + col] : 1.0) * w.g[k];
+        } else {
+            a = k < w.N ? (double)w.s[(size_t)row * w.N + k] : 1.0;
+            b = w.X[(size_t)col * w.ldx + k];
+        }
+        acc = fma(a, b, acc);
+    }
+    return acc;
+}
 
 // Smem: nstages x (A tile + SB B-slice tiles), reused by the staged output
 // tile after the MMAs.  With SB <= 4 two stages and 256 TMEM columns let two
@@ -193,7 +228,12 @@ __global__ void __launch_bounds__(kSgThreads, 2)
                     for (int t = 0; t < kMaxSB; ++t) d[t] = t < SB ? __float2int_rn(__uint_as_float(r[t][j])) : 0;
                     // V 2^(f_n - 56) with V = sum_t D_t 2^(8 (7 - t))
                     const int fn = __shfl_sync(0xffffffffu, fj_lane, j);
-                    const double v = window_to_double(sgemm_window10(d), fn - 46);
+                    double v = a.drop >= 0 ? window_to_double(sgemm_window(d, a.drop), fn - 56 + a.drop)
+                                           : window_to_double(sgemm_window10(d), fn - 46);
+                    if (flagged_exp(fn) && row_ok && n0 + c8 + j < a.cols) {
+                        const int64_t k1 = (int64_t)kc1 * kBK;
+                        v = raw_product(a.raw, row, n0 + c8 + j, (int64_t)kc0 * kBK, k1 < a.K ? k1 : a.K);
+                    }
                     if (a.mode == 3)
                         racc = fma(v, tv[j], racc);
                     else
@@ -701,13 +741,14 @@ __global__ void k_pm1_cols(const int8_t *__restrict__ s, int64_t Ns, int N, int6
     }
 }
 
-// Largest binary exponent of |x| (frexp convention, |x| < 2^e); -100000 for 0.
+// Largest binary exponent of |x| (frexp convention, |x| < 2^e); -100000 for
+// 0, 100000 for an infinity or a NaN.
 __device__ __forceinline__ int exp_of(double x) {
     int b;
     unsigned long long m;
     bool n;
     split_bits(x, b, m, n);
-    return m ? b - 1022 : -100000;
+    return b == 2047 ? 100000 : (m ? b - 1022 : -100000);
 }
 
 // Slice one value with row exponent e into SB bytes (sign applied).
@@ -1163,12 +1204,13 @@ bool make_sliced_map(CUtensorMap *map, const __nv_bfloat16 *p, int64_t rows, int
 
 // C (mode) A B^T + bias: A BF16 [rows][ldA] (K used), B slices [SB][cols][ldB].
 // ksplit > 1 (mode 0 only): split z of the K range writes C + z split_stride.
+// wide (NK_F64): the recombination keeps every bit that K leaves room for.
 // mode 3: C [rows][ldc >= col tiles] receives, per 64-column tile, the row
 // products sum_col R[row][col] t'_col with t' = [T[row][0 .. Mt-1], 1, 0 ...].
 cudaError_t sgemm(const __nv_bfloat16 *A, int64_t rows, int64_t ldA, const __nv_bfloat16 *Bsl, const int *expB,
                   int64_t cols, int64_t ldB, int64_t K, int SB, double *C, int64_t ldc, int mode,
-                  const double *bias, int *err, cudaStream_t st, const double *T = nullptr, int Mt = 0,
-                  int ksplit = 1, int64_t split_stride = 0) {
+                  const double *bias, int *err, cudaStream_t st, const SgRaw &raw, bool wide,
+                  const double *T = nullptr, int Mt = 0, int ksplit = 1, int64_t split_stride = 0) {
     if (rows <= 0 || cols <= 0 || K <= 0) return cudaSuccess;
     if (SB < 1 || SB > kMaxSB || rows > (1LL << 31) - kBM || cols > (1LL << 31) - kBN) return cudaErrorInvalidValue;
     if (ksplit < 1 || (ksplit > 1 && mode != 0) || (mode == 3 && T == nullptr)) return cudaErrorInvalidValue;
@@ -1181,8 +1223,8 @@ cudaError_t sgemm(const __nv_bfloat16 *A, int64_t rows, int64_t ldA, const __nv_
     const int kc_split = (kchunks + ksplit - 1) / ksplit;
     uint32_t tcols = 32;
     while (tcols < (uint32_t)(SB * kBN)) tcols <<= 1;
-    SgArgs a{rows, cols, kchunks, SB, kc_split, sgemm_stages(SB), kAB + SB * kBB, tcols, expB, C, ldc,
-             split_stride, mode, bias, T, Mt, err};
+    SgArgs a{rows, cols, K, kchunks, SB, kc_split, sgemm_stages(SB), kAB + SB * kBB, tcols, expB, C, ldc,
+             split_stride, mode, bias, T, Mt, err, raw, wide ? window_drop((int64_t)kc_split * kBK) : -1};
     dim3 grid(nblk(cols, kBN), nblk(rows, kBM), (unsigned)((kchunks + kc_split - 1) / kc_split));
     (k_sgemm<<<grid, kSgThreads, sgemm_smem_bytes(SB), st>>>(ma, mb, a), nk::note_launch());
     return cudaGetLastError();
@@ -1320,7 +1362,7 @@ size_t tc_theta_ws_bytes(int N, int M, int64_t B) {
 
 // theta [B][M] = S W^T + b with W sliced 7 ways: exact up to 2^-56 of max|W_j|.
 cudaError_t launch_theta_tc(int N, int M, const double *b, const double *W, const int8_t *s, int64_t B,
-                            double *theta, int *err, void *ws, cudaStream_t st, int64_t ldtheta) {
+                            double *theta, int *err, void *ws, cudaStream_t st, int64_t ldtheta, bool wide) {
     if (B <= 0) return cudaSuccess;
     const int64_t ld = pad8(N);
     char *p = static_cast<char *>(ws);
@@ -1335,7 +1377,8 @@ cudaError_t launch_theta_tc(int N, int M, const double *b, const double *W, cons
     (k_pm1_rows<<<nblk(B * ld, 256), 256, 0, st>>>(s, B, N, 0, ld, As), nk::note_launch());
     (k_slice_long_rows<<<M, 128, 0, st>>>(W, N, M, N, nullptr, kMaxSB, ld, Ws, ew), nk::note_launch());
     const int slot = prof_begin(NK_PROF_JVP_VJP, st);
-    cudaError_t e = sgemm(As, B, ld, Ws, ew, M, ld, N, kMaxSB, theta, ldtheta > 0 ? ldtheta : M, 0, b, err, st);
+    cudaError_t e = sgemm(As, B, ld, Ws, ew, M, ld, N, kMaxSB, theta, ldtheta > 0 ? ldtheta : M, 0, b, err, st,
+                          SgRaw{s, W, nullptr, N, N, 0}, wide);
     prof_end(slot, st, 2.0 * (double)B * N * (double)M, sgemm_flops(B, M, N, kMaxSB));
     return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -1381,7 +1424,7 @@ cudaError_t launch_jacobian_operands(int N, int64_t Ns, const int8_t *s, void *o
 // products taken in the S-GEMM epilogue per 64-column tile and summed after.
 cudaError_t launch_jvp_tc(int N, int M, int64_t Ns, const int8_t *s, const double *T, const double *v,
                           double *out, int SB, int *err, void *ws, cudaStream_t st, const void *opA,
-                          const void *Thl, const int *skip) {
+                          const void *Thl, const int *skip, bool wide) {
     const int64_t ld = pad8(N + 1);
     char *p = static_cast<char *>(ws);
     auto take = [&](size_t bytes) {
@@ -1421,7 +1464,8 @@ cudaError_t launch_jvp_tc(int N, int M, int64_t Ns, const int8_t *s, const doubl
     }
     const int slot = prof_begin(NK_PROF_JVP_VJP, st);
     cudaError_t e = persistent ? jvp4(As, Ns, ld, Vs, ev, M + 1, ld, N + 1, Thl, M, P, err, st, skip)
-                               : sgemm(As, Ns, ld, Vs, ev, M + 1, ld, N + 1, SB, P, ntc, 3, nullptr, err, st, T, M);
+                               : sgemm(As, Ns, ld, Vs, ev, M + 1, ld, N + 1, SB, P, ntc, 3, nullptr, err, st,
+                                       SgRaw{s, Vp, nullptr, N + 1, N, 0}, wide, T, M);
     prof_end(slot, st, 2.0 * (double)Ns * (N + 1) * (double)(M + 1),
              sgemm_flops(Ns, M + 1, N + 1, persistent ? kJvSB : SB));
     if (e != cudaSuccess) return e;
@@ -1438,11 +1482,13 @@ constexpr int kMaxKSplit = 16;
 // CTAs: the share of the last wave's slots that hold work, less 1 % per extra
 // split (its partial output is written and summed), best over 1 .. 8 splits
 // of at least 4 K-chunks each.
+// At least as many as keep a split within 65536 samples (exact FP32 levels).
 static int pick_ksplit(int64_t tiles, int64_t kchunks, int64_t slots) {
-    int best = 1;
+    const int least = (int)((kchunks + 1023) / 1024);
+    int best = least;
     double best_score = -1.0;
-    for (int ks = 1; ks <= kMaxKSplit; ++ks) {
-        if (ks > 1 && kchunks / ks < 4) break;
+    for (int ks = least; ks <= kMaxKSplit; ++ks) {
+        if (ks > least && kchunks / ks < 4) break;
         const int64_t ctas = tiles * ks, waves = (ctas + slots - 1) / slots;
         const double score = (double)ctas / (double)(waves * slots) - 0.01 * (ks - 1);
         if (score > best_score + 1e-12) best_score = score, best = ks;
@@ -1478,7 +1524,7 @@ cudaError_t launch_colexp_t(int M, int64_t Ns, const double *T, int *colexpT, vo
 cudaError_t launch_vjp_tc(int N, int M, int64_t Ns, const int8_t *s, const double *T, const double *g,
                           double scale, const double *shift, double *out, int SB, int *err, void *ws,
                           cudaStream_t st, const int *colexpT, const void *opT, const void *Thl,
-                          const int *skip) {
+                          const int *skip, bool wide) {
     const int64_t ld = pad8(Ns);
     char *p = static_cast<char *>(ws);
     auto take = [&](size_t bytes) {
@@ -1565,7 +1611,8 @@ cudaError_t launch_vjp_tc(int N, int M, int64_t Ns, const int8_t *s, const doubl
     const int kc_split = (int)((kchunks + ks - 1) / ks);
     ks = (int)((kchunks + kc_split - 1) / kc_split);  // splits the kernel launches
     const int slot = prof_begin(NK_PROF_JVP_VJP, st);
-    e = sgemm(St, N + 1, ld, Gs, eg, M + 1, ld, Ns, SB, PT, M + 1, 0, nullptr, err, st, nullptr, 0, ks, tot);
+    e = sgemm(St, N + 1, ld, Gs, eg, M + 1, ld, Ns, SB, PT, M + 1, 0, nullptr, err, st, SgRaw{s, T, gp, M, N, 1}, wide, nullptr, 0,
+              ks, tot);
     prof_end(slot, st, 2.0 * (double)Ns * (N + 1) * (double)(M + 1), sgemm_flops(N + 1, M + 1, Ns, SB));
     if (e != cudaSuccess) return e;
     (k_scatter_vjp<<<nblk(tot, 256), 256, 0, st>>>(N, M, ks, PT, out), nk::note_launch());

@@ -207,6 +207,7 @@ struct SolveWs {
     int *colexpT;     // NK_MIXED CG: column exponents of tanh(theta), [M + 1]
     void *colexp_ws;
     void *opA, *opT;  // NK_MIXED CG: the +-1 product operands, built once per solve
+    bool tcp;         // Jacobian products on the tensor cores (NK_MIXED; NK_F64 by size)
     void *thl;        // NK_MIXED CG: tanh(theta) as FP32 pairs, built once per solve
     bool ops_ready;   // opA / opT / thl hold the operands of the samples being solved for
     const int *skip;  // NK_MIXED CG: its converged flag (the products then do nothing)
@@ -218,16 +219,25 @@ size_t tcm_bytes(int N, int M, int64_t B) {
     return a > b ? (a > c ? a : c) : (b > c ? b : c);
 }
 
+// The products' workspace: tensor-core (tcp) or FP64 (partials of J^T g, U of J v).
+void carve_products(Carver &c, SolveWs &w, int N, int M, int64_t Ns, int precision, bool need_U) {
+    w.tcp = precision == NK_MIXED || nk::f64_on_tensor(N, M, Ns);
+    if (w.tcp) {
+        w.tcm = c.take<char>(tcm_bytes(N, M, Ns));
+        return;
+    }
+    w.partial = c.take<double>(nk::vjp_partial_doubles(N, M, Ns));
+    if (need_U) w.U = c.take<double>((size_t)Ns * (M + 1));
+}
+
 void carve_solve(Carver &c, SolveWs &w, int N, int M, int64_t Ns, int solver, int precision) {
     const int64_t Np = n_params(N, M);
     w = SolveWs{};
-    w.partial = c.take<double>(nk::vjp_partial_doubles(N, M, Ns));
+    carve_products(c, w, N, M, Ns, precision, solver != NK_SOLVER_CHOLESKY && solver != NK_SOLVER_SVD);
     w.dotp = c.take<double>(nk::dot_partial_doubles(Np > Ns ? Np : Ns) + 8);
     w.sc = c.take<double>(8);
     w.flags = c.take<int>(4);
-    if (precision == NK_MIXED) w.tcm = c.take<char>(tcm_bytes(N, M, Ns));
     if (solver == NK_SOLVER_CG) {
-        w.U = c.take<double>((size_t)Ns * (M + 1));
         w.w = c.take<double>(Ns);
         w.x = c.take<double>(Np);
         w.r = c.take<double>(Np);
@@ -251,7 +261,6 @@ void carve_solve(Carver &c, SolveWs &w, int N, int M, int64_t Ns, int solver, in
         const bool ss = solver == NK_SOLVER_SVD_SAMPLESPACE;
         const int64_t n = ss ? Ns : Np;
         if (ss) {
-            w.U = c.take<double>((size_t)Ns * (M + 1));
             w.w = c.take<double>(Ns);
             w.rowmean = c.take<double>(2 * Ns + 1);
             w.tmp = c.take<double>(Np);
@@ -272,7 +281,6 @@ void carve_solve(Carver &c, SolveWs &w, int N, int M, int64_t Ns, int solver, in
         w.kept = c.take<int>(4);
         w.info = c.take<int>(2);
     } else {
-        w.U = c.take<double>((size_t)Ns * (M + 1));
         w.w = c.take<double>(Ns);
         w.K = c.take<double>((size_t)Ns * Ns);
         w.rowmean = c.take<double>(2 * Ns + 1);  // row means, grand mean, centring coefficients
@@ -295,19 +303,20 @@ constexpr double kJacobiTol = 1e-14;
 
 cudaError_t jvp_any(int N, int M, int64_t Ns, const int8_t *s, const double *T, const double *v, SolveWs &w,
                     double *out, int precision, int slices, cudaStream_t st) {
-    if (precision == NK_MIXED)
-        return nk::launch_jvp_tc(N, M, Ns, s, T, v, out, slices, w.tcerr, w.tcm, st, w.ops_ready ? w.opA : nullptr,
-                                 w.ops_ready ? w.thl : nullptr, w.ops_ready ? w.skip : nullptr);
+    if (w.tcp)
+        return nk::launch_jvp_tc(N, M, Ns, s, T, v, out, precision == NK_MIXED ? slices : kExactSlices, w.tcerr, w.tcm, st, w.ops_ready ? w.opA : nullptr,
+                                 w.ops_ready ? w.thl : nullptr, w.ops_ready ? w.skip : nullptr, precision == NK_F64);
     return nk::launch_jvp(N, M, Ns, s, T, v, w.U, out, st);
 }
 
 cudaError_t vjp_any(int N, int M, int64_t Ns, const int8_t *s, const double *T, const double *g, double scale,
                     const double *shift, SolveWs &w, double *out, int precision, int slices, cudaStream_t st,
                     const int *colexpT = nullptr) {
-    if (precision == NK_MIXED)
-        return nk::launch_vjp_tc(N, M, Ns, s, T, g, scale, shift, out, slices, w.tcerr, w.tcm, st, colexpT,
+    if (w.tcp)
+        return nk::launch_vjp_tc(N, M, Ns, s, T, g, scale, shift, out, precision == NK_MIXED ? slices : kExactSlices,
+                                 w.tcerr, w.tcm, st, colexpT,
                                  w.ops_ready ? w.opT : nullptr, w.ops_ready ? w.thl : nullptr,
-                                 w.ops_ready ? w.skip : nullptr);
+                                 w.ops_ready ? w.skip : nullptr, precision == NK_F64);
     return nk::launch_vjp(N, M, Ns, s, T, g, scale, shift, w.partial, out, st);
 }
 
@@ -441,7 +450,7 @@ nk_status run_solve(nk_ctx *ctx, int N, int M, int64_t Ns, const int8_t *s, cons
         } else {
             // the dense S + eps I from the centred Jacobian
             NK_CU(nk::launch_fill(Ns, 1.0, w.ones, st), "svd mean");
-            NK_CU(nk::launch_vjp(N, M, Ns, s, T, w.ones, 1.0 / (double)Ns, nullptr, w.partial, w.mean, st),
+            NK_CU(vjp_any(N, M, Ns, s, T, w.ones, 1.0 / (double)Ns, nullptr, w, w.mean, precision, kExactSlices, st),
                   "svd mean");
             NK_CU(nk::launch_jacobian_rows(N, M, s, T, 0, Ns, w.mean, w.dJ, st), "svd dJ");
             if (tc)
@@ -486,7 +495,7 @@ nk_status run_solve(nk_ctx *ctx, int N, int M, int64_t Ns, const int8_t *s, cons
     }
     if (solver == NK_SOLVER_CHOLESKY) {
         NK_CU(nk::launch_fill(Ns, 1.0, w.ones, st), "chol");
-        NK_CU(nk::launch_vjp(N, M, Ns, s, T, w.ones, 1.0 / (double)Ns, nullptr, w.partial, w.mean, st),
+        NK_CU(vjp_any(N, M, Ns, s, T, w.ones, 1.0 / (double)Ns, nullptr, w, w.mean, precision, kExactSlices, st),
               "chol mean");
         NK_CU(nk::launch_jacobian_rows(N, M, s, T, 0, Ns, w.mean, w.dJ, st), "chol dJ");
         NK_CU(cudaMemsetAsync(w.info, 0, 2 * sizeof(int), st), "chol");
@@ -559,17 +568,17 @@ nk_status run_sweeps(nk_ctx *ctx, const nk::Tables<R> &t, const nk::SweepArgs &a
     return NK_OK;
 }
 
-// T = tanh(theta) of a batch: FP64 CUDA-core GEMM (NK_F64) or the FP64-exact
-// tensor-core product (NK_MIXED, needs tcm).
-nk_status batch_T(nk_ctx *ctx, const nk_rbm *rbm, const int8_t *s, int64_t B, double *T, bool mixed, void *tcm,
-                  cudaStream_t st) {
+// T = tanh(theta) of a batch: the FP64-exact tensor-core product with tcm
+// (NK_MIXED, large NK_F64 batches), FP64 CUDA cores without.
+nk_status batch_T(nk_ctx *ctx, const nk_rbm *rbm, const int8_t *s, int64_t B, double *T, void *tcm,
+                  cudaStream_t st, int precision) {
     const int N = rbm->N, M = rbm->M;
     const double *b = rbm->params + N, *W = rbm->params + N + M;
-    if (!mixed) {
+    if (!tcm) {
         NK_CU(nk::launch_theta_tanh(N, M, b, W, s, B, T, st), "theta");
         return NK_OK;
     }
-    NK_CU(nk::launch_theta_tc(N, M, b, W, s, B, T, ctx->tc_err, tcm, st), "theta");
+    NK_CU(nk::launch_theta_tc(N, M, b, W, s, B, T, ctx->tc_err, tcm, st, 0, precision == NK_F64), "theta");
     NK_CU(nk::launch_tanh_inplace(B * M, T, st), "tanh");
     return NK_OK;
 }
@@ -787,12 +796,12 @@ nk_status nk_rbm_logpsi(nk_ctx *ctx, const nk_rbm *rbm, int32_t precision, const
     return with_workspace(ctx, [&](Carver &c, bool run) -> nk_status {
         nk::Tables<double> t{};
         carve_tables(c, t, rbm, 0, nullptr, false, false);
-        const bool mixed = precision == NK_MIXED;
-        double *theta = mixed ? c.take<double>((size_t)B * M) : nullptr;
-        void *tcm = mixed ? c.take<char>(nk::tc_theta_ws_bytes(N, M, B)) : nullptr;
+        const bool tcp = precision == NK_MIXED || nk::f64_on_tensor(N, M, B);
+        double *theta = tcp ? c.take<double>((size_t)B * M) : nullptr;
+        void *tcm = tcp ? c.take<char>(nk::tc_theta_ws_bytes(N, M, B)) : nullptr;
         if (!run) return NK_OK;
-        if (mixed) {
-            NK_CU(nk::launch_theta_tc(N, M, t.b, t.W, s, B, theta, ctx->tc_err, tcm, st), "theta");
+        if (tcp) {
+            NK_CU(nk::launch_theta_tc(N, M, t.b, t.W, s, B, theta, ctx->tc_err, tcm, st, 0, precision == NK_F64), "theta");
             NK_CU(nk::launch_logpsi_theta(N, M, t.a, theta, s, B, logpsi_out, st), "logpsi");
             return NK_OK;
         }
@@ -948,24 +957,23 @@ nk_status nk_jacobian(nk_ctx *ctx, const nk_rbm *rbm, int32_t precision, const i
     const int N = rbm->N, M = rbm->M;
     const int64_t Np = n_params(N, M);
     return with_workspace(ctx, [&](Carver &c, bool run) -> nk_status {
-        double *T = c.take<double>((size_t)(centered ? Ns : rows) * M);
+        // T of the rows written, or of every sample when their mean is needed
+        const int8_t *st_s = centered ? s : s + (size_t)row0 * N;
+        const int64_t nT = centered ? Ns : rows;
+        double *T = c.take<double>((size_t)nT * M);
         double *mean = centered ? c.take<double>(Np) : nullptr;
         double *ones = centered ? c.take<double>(Ns) : nullptr;
-        double *partial = centered ? c.take<double>(nk::vjp_partial_doubles(N, M, Ns)) : nullptr;
+        SolveWs w{};
+        carve_products(c, w, N, M, nT, NK_F64, false);
+        w.tcerr = ctx->tc_err;
         if (!run) return NK_OK;
-        const double *b = rbm->params + N, *W = rbm->params + N + M;
+        nk_status bt = batch_T(ctx, rbm, st_s, nT, T, w.tcm, st, NK_F64);
+        if (bt != NK_OK) return bt;
         if (centered) {
-            NK_CU(nk::launch_theta_tanh(N, M, b, W, s, Ns, T, st), "theta");
             NK_CU(nk::launch_fill(Ns, 1.0, ones, st), "ones");
-            NK_CU(nk::launch_vjp(N, M, Ns, s, T, ones, 1.0 / (double)Ns, nullptr, partial, mean, st),
-                  "mean");
-            NK_CU(nk::launch_jacobian_rows(N, M, s, T, row0, rows, mean, O_out, st), "jacobian");
-        } else {
-            NK_CU(nk::launch_theta_tanh(N, M, b, W, s + (size_t)row0 * N, rows, T, st), "theta");
-            NK_CU(nk::launch_jacobian_rows(N, M, s + (size_t)row0 * N, T, 0, rows, nullptr, O_out, st),
-                  "jacobian");
+            NK_CU(vjp_any(N, M, Ns, s, T, ones, 1.0 / (double)Ns, nullptr, w, mean, NK_F64, kExactSlices, st), "mean");
         }
-        (void)Np;
+        NK_CU(nk::launch_jacobian_rows(N, M, st_s, T, centered ? row0 : 0, rows, mean, O_out, st), "jacobian");
         return NK_OK;
     });
 }
@@ -986,12 +994,10 @@ nk_status nk_vjp(nk_ctx *ctx, const nk_rbm *rbm, int32_t precision, const int8_t
     return with_workspace(ctx, [&](Carver &c, bool run) -> nk_status {
         double *T = c.take<double>((size_t)Ns * M);
         SolveWs w{};
-        w.partial = c.take<double>(nk::vjp_partial_doubles(N, M, Ns));
-        const bool mixed = precision == NK_MIXED;
-        w.tcm = mixed ? c.take<char>(tcm_bytes(N, M, Ns)) : nullptr;
+        carve_products(c, w, N, M, Ns, precision, false);
         w.tcerr = ctx->tc_err;
         if (!run) return NK_OK;
-        nk_status bt = batch_T(ctx, rbm, s, Ns, T, mixed, w.tcm, st);
+        nk_status bt = batch_T(ctx, rbm, s, Ns, T, w.tcm, st, precision);
         if (bt != NK_OK) return bt;
         NK_CU(vjp_any(N, M, Ns, s, T, gvec, 1.0, nullptr, w, out, precision, kMatvecSlices, st), "vjp");
         return NK_OK;
@@ -1014,12 +1020,10 @@ nk_status nk_jvp(nk_ctx *ctx, const nk_rbm *rbm, int32_t precision, const int8_t
     return with_workspace(ctx, [&](Carver &c, bool run) -> nk_status {
         double *T = c.take<double>((size_t)Ns * M);
         SolveWs w{};
-        w.U = c.take<double>((size_t)Ns * (M + 1));
-        const bool mixed = precision == NK_MIXED;
-        w.tcm = mixed ? c.take<char>(tcm_bytes(N, M, Ns)) : nullptr;
+        carve_products(c, w, N, M, Ns, precision, true);
         w.tcerr = ctx->tc_err;
         if (!run) return NK_OK;
-        nk_status bt = batch_T(ctx, rbm, s, Ns, T, mixed, w.tcm, st);
+        nk_status bt = batch_T(ctx, rbm, s, Ns, T, w.tcm, st, precision);
         if (bt != NK_OK) return bt;
         NK_CU(jvp_any(N, M, Ns, s, T, v, w, out, precision, kMatvecSlices, st), "jvp");
         return NK_OK;
@@ -1042,14 +1046,12 @@ nk_status nk_force(nk_ctx *ctx, const nk_rbm *rbm, int32_t precision, const int8
     return with_workspace(ctx, [&](Carver &c, bool run) -> nk_status {
         double *T = c.take<double>((size_t)Ns * M);
         SolveWs w{};
-        w.partial = c.take<double>(nk::vjp_partial_doubles(N, M, Ns));
+        carve_products(c, w, N, M, Ns, precision, false);
         double *st3 = c.take<double>(4);
         double *gv = c.take<double>(Ns);
-        const bool mixed = precision == NK_MIXED;
-        w.tcm = mixed ? c.take<char>(tcm_bytes(N, M, Ns)) : nullptr;
         w.tcerr = ctx->tc_err;
         if (!run) return NK_OK;
-        nk_status bt = batch_T(ctx, rbm, s, Ns, T, mixed, w.tcm, st);
+        nk_status bt = batch_T(ctx, rbm, s, Ns, T, w.tcm, st, precision);
         if (bt != NK_OK) return bt;
         NK_CU(nk::launch_stats(eloc, Ns, 1, st3, st), "stats");
         NK_CU(nk::launch_make_force_g(Ns, eloc, st3, gv, st), "force g");
@@ -1092,15 +1094,12 @@ nk_status nk_qgt_matvec(nk_ctx *ctx, const nk_qgt *q, double diag_shift, const d
     return with_workspace(ctx, [&](Carver &c, bool run) -> nk_status {
         double *T = c.take<double>((size_t)Ns * M);
         SolveWs w{};
-        w.partial = c.take<double>(nk::vjp_partial_doubles(N, M, Ns));
+        carve_products(c, w, N, M, Ns, q->precision, true);
         w.dotp = c.take<double>(nk::dot_partial_doubles(Ns) + 8);
-        w.U = c.take<double>((size_t)Ns * (M + 1));
         w.w = c.take<double>(Ns);
-        const bool mixed = q->precision == NK_MIXED;
-        w.tcm = mixed ? c.take<char>(tcm_bytes(N, M, Ns)) : nullptr;
         w.tcerr = ctx->tc_err;
         if (!run) return NK_OK;
-        nk_status bt = batch_T(ctx, rbm, q->s, Ns, T, mixed, w.tcm, st);
+        nk_status bt = batch_T(ctx, rbm, q->s, Ns, T, w.tcm, st, q->precision);
         if (bt != NK_OK) return bt;
         NK_CU(qgt_onthefly(N, M, Ns, q->s, T, v, diag_shift, w, out, st, q->precision), "qgt matvec");
         return NK_OK;
@@ -1157,7 +1156,7 @@ nk_status nk_sr_solve(nk_ctx *ctx, const nk_rbm *rbm, int32_t precision, const i
         carve_solve(c, w, N, M, Ns, solver, precision);
         w.tcerr = ctx->tc_err;
         if (!run) return NK_OK;
-        nk_status bt = batch_T(ctx, rbm, s, Ns, T, precision == NK_MIXED, w.tcm, st);
+        nk_status bt = batch_T(ctx, rbm, s, Ns, T, w.tcm, st, precision);
         if (bt != NK_OK) return bt;
         return run_solve(ctx, N, M, Ns, s, T, F, solver, diag_shift, cg_tol, cg_maxiter, w,
                          delta_out, info_out, resid_out, st, precision, precision == NK_MIXED);
@@ -1328,7 +1327,7 @@ nk_status nk_symm_jacobian(nk_ctx *ctx, const nk_rbm_symm *symm, int32_t precisi
         nk_status e = symm_expand_checked(ctx, symm, plain, st);
         if (e != NK_OK) return e;
         nk_rbm r{N, M, plain};
-        if ((e = batch_T(ctx, &r, s, Ns, T, mixed, tcm, st)) != NK_OK) return e;
+        if ((e = batch_T(ctx, &r, s, Ns, T, tcm, st, precision)) != NK_OK) return e;
         NK_CU(nk::launch_symm_jacobian(N, symm->alpha, symm->n_group, symm->perms, s, T, Ns, O_out, st),
               "symmetric jacobian");
         return NK_OK;

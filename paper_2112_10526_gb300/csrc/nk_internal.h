@@ -215,7 +215,10 @@ size_t tc_theta_ws_bytes(int N, int M, int64_t B);
 // theta [B][M] = S W^T + b, exact to 2^-56 of max|W_j| (7 slices); row r of
 // theta at theta + r * ldtheta (0: M).
 cudaError_t launch_theta_tc(int N, int M, const double *b, const double *W, const int8_t *s, int64_t B,
-                            double *theta, int *err, void *ws, cudaStream_t st, int64_t ldtheta = 0);
+                            double *theta, int *err, void *ws, cudaStream_t st, int64_t ldtheta = 0,
+                            bool wide = false);
+// wide, here and in the products below (NK_F64): the slices' sums are turned
+// into FP64 with every bit that the length of the sums leaves room for.
 // The +-1 operands of the two Jacobian products depend on the samples only:
 // a solve that repeats the products (CG) builds them once.  opA: [S, 1] as
 // BF16 [Ns][pad8(N + 1)] (J v); opT: [S, 1]^T as BF16 [N + 1][pad8(Ns)] (J^T g).
@@ -233,7 +236,7 @@ size_t tc_jvp_ws_bytes(int N, int M, int64_t Ns);
 // is set (the converged flag of a CG whose loop still runs to its next poll).
 cudaError_t launch_jvp_tc(int N, int M, int64_t Ns, const int8_t *s, const double *T, const double *v,
                           double *out, int SB, int *err, void *ws, cudaStream_t st, const void *opA = nullptr,
-                          const void *Thl = nullptr, const int *skip = nullptr);
+                          const void *Thl = nullptr, const int *skip = nullptr, bool wide = false);
 size_t tc_vjp_ws_bytes(int N, int M, int64_t Ns);
 // colexpT (optional, [M + 1], from launch_colexp_t): the column exponents of
 // tanh(theta), so that the slices of (T' o g')^T take their exponents from
@@ -244,9 +247,20 @@ size_t tc_vjp_ws_bytes(int N, int M, int64_t Ns);
 cudaError_t launch_vjp_tc(int N, int M, int64_t Ns, const int8_t *s, const double *T, const double *g,
                           double scale, const double *shift, double *out, int SB, int *err, void *ws,
                           cudaStream_t st, const int *colexpT = nullptr, const void *opT = nullptr,
-                          const void *Thl = nullptr, const int *skip = nullptr);
+                          const void *Thl = nullptr, const int *skip = nullptr, bool wide = false);
 size_t tc_colexp_ws_bytes(int M, int64_t Ns);
 cudaError_t launch_colexp_t(int M, int64_t Ns, const double *T, int *colexpT, void *ws, cudaStream_t st);
+
+// NK_F64 products with the configurations (theta, J v, J^T g; about N M B
+// multiply-adds) run as 7-slice tensor-core products from this size on, and
+// on the FP64 pipe below.  Both have FP64-level errors (the slices hold 56
+// bits of the largest entry of each operand row and their sums are exact); the
+// FP64 pipe retires 2 multiply-adds a clock and SM, so the 12 to 20 us of
+// slicing, products and sums pay from about 4M multiply-adds.  More than 2^20
+// samples would not fit the K splits of J^T g.
+inline bool f64_on_tensor(int N, int M, int64_t B) {
+    return (double)N * (double)M * (double)B >= 4e6 && B <= (1 << 20);
+}
 
 // vector helpers
 cudaError_t launch_axpby(int64_t n, double alpha, const double *x, double beta, double *y,
