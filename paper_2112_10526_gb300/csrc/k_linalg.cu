@@ -1,7 +1,6 @@
 // FP64 linear algebra of the VMC step: sample statistics, Jacobian products
 // (vjp / jvp, App. B.1), the stored centred Jacobian, QGT products and
-// Gram matrices (App. B.2 / B.3), blocked Cholesky and triangular solves
-// (Sec. 3.5, direct solver), and the CG / SGD vector kernels.
+// Gram matrices (App. B.2 / B.3), and the CG / SGD vector kernels.
 //
 // Every reduction runs in a fixed order (split-K partials summed in split
 // order, tree reductions with a fixed shape), so results are bitwise
@@ -409,141 +408,6 @@ __global__ void k_center_rows(int64_t n, const double *__restrict__ r, double in
 }
 
 
-// ------------------------------------------------------------- Cholesky ---
-
-constexpr int kNB = 64;
-
-// Factor the kb x kb diagonal block at (k, k) in shared memory.
-__global__ void k_potrf_diag(double *__restrict__ A, int64_t n, int64_t k, int kb,
-                             int *__restrict__ info) {
-    __shared__ double L[kNB][kNB + 1];
-    const int t = threadIdx.x;
-    for (int r = 0; r < kb; ++r)
-        if (t < kb) L[r][t] = A[(size_t)(k + r) * n + k + t];
-    __syncthreads();
-    for (int c = 0; c < kb; ++c) {
-        if (t == 0) {
-            double d = L[c][c];
-            if (!(d > 0.0)) {
-                if (info) atomicCAS(info, 0, (int)(k + c + 1));  // the first failure
-                d = 1e-300;
-            }
-            L[c][c] = sqrt(d);
-        }
-        __syncthreads();
-        if (t > c && t < kb) L[t][c] /= L[c][c];
-        __syncthreads();
-        if (t > c && t < kb) {
-            const double ltc = L[t][c];
-            for (int q = c + 1; q <= t; ++q) L[t][q] -= ltc * L[q][c];
-        }
-        __syncthreads();
-    }
-    for (int r = 0; r < kb; ++r)
-        if (t <= r && t < kb) A[(size_t)(k + r) * n + k + t] = L[r][t];
-}
-
-// Rows below the diagonal block: A[r, k:k+kb] <- A[r, k:k+kb] L_kk^{-T}.
-__global__ void k_trsm_panel(double *__restrict__ A, int64_t n, int64_t k, int kb) {
-    __shared__ double L[kNB][kNB + 1];
-    __shared__ double X[kNB][kNB + 1];
-    const int t = threadIdx.x;
-    const int64_t r0 = k + kb + (int64_t)blockIdx.x * kNB;
-    for (int r = 0; r < kb; ++r)
-        if (t < kb) L[r][t] = A[(size_t)(k + r) * n + k + t];
-    for (int r = 0; r < kNB; ++r) {
-        const int64_t row = r0 + r;
-        if (t < kb) X[r][t] = row < n ? A[(size_t)row * n + k + t] : 0.0;
-    }
-    __syncthreads();
-    const int64_t row = r0 + t;
-    if (row < n) {
-        for (int c = 0; c < kb; ++c) {
-            double v = X[t][c];
-            for (int j = 0; j < c; ++j) v -= X[t][j] * L[c][j];
-            X[t][c] = v / L[c][c];
-        }
-    }
-    __syncthreads();
-    for (int r = 0; r < kNB; ++r) {
-        const int64_t rr = r0 + r;
-        if (rr < n && t < kb) A[(size_t)rr * n + k + t] = X[r][t];
-    }
-}
-
-struct PanelLoad {  // L(r, c) = A[(off + r) n + k + c], c contiguous
-    static constexpr bool kContig = true;
-    const double *A;
-    int64_t n, off, k;
-    __device__ double operator()(int64_t r, int64_t c) const {
-        return A[(size_t)(off + r) * n + k + c];
-    }
-};
-
-struct EpTrailing {
-    double *A;
-    int64_t n, off;
-    __device__ bool active(int64_t m0, int64_t n0) const { return n0 <= m0 + kGT - 1; }
-    __device__ void operator()(int64_t r, int64_t q, int, double v) const {
-        if (q > r) return;
-        A[(size_t)(off + r) * n + off + q] -= v;
-    }
-};
-
-// Forward substitution on the diagonal block: y_k = L_kk^{-1} b_k.
-__global__ void k_trsv_diag_lower(const double *__restrict__ A, int64_t n, int64_t k, int kb,
-                                  double *__restrict__ b) {
-    __shared__ double y[kNB];
-    const int t = threadIdx.x;
-    if (t < kb) y[t] = b[k + t];
-    __syncthreads();
-    for (int c = 0; c < kb; ++c) {
-        if (t == 0) y[c] /= A[(size_t)(k + c) * n + k + c];
-        __syncthreads();
-        if (t > c && t < kb) y[t] -= A[(size_t)(k + t) * n + k + c] * y[c];
-        __syncthreads();
-    }
-    if (t < kb) b[k + t] = y[t];
-}
-
-// b[r] -= sum_{c in block} L[r][k + c] y[k + c] for rows r >= k + kb.
-__global__ void k_trsv_update_lower(const double *__restrict__ A, int64_t n, int64_t k, int kb,
-                                    double *__restrict__ b) {
-    const int lane = threadIdx.x & 31;
-    const int64_t r = k + kb + (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (r >= n) return;
-    double acc = 0.0;
-    for (int c = lane; c < kb; c += 32) acc += A[(size_t)r * n + k + c] * b[k + c];
-    acc = warp_sum(acc);
-    if (lane == 0) b[r] -= acc;
-}
-
-// Back substitution on the diagonal block: x_k = L_kk^{-T} y_k.
-__global__ void k_trsv_diag_upper(const double *__restrict__ A, int64_t n, int64_t k, int kb,
-                                  double *__restrict__ b) {
-    __shared__ double x[kNB];
-    const int t = threadIdx.x;
-    if (t < kb) x[t] = b[k + t];
-    __syncthreads();
-    for (int c = kb - 1; c >= 0; --c) {
-        if (t == 0) x[c] /= A[(size_t)(k + c) * n + k + c];
-        __syncthreads();
-        if (t < c) x[t] -= A[(size_t)(k + c) * n + k + t] * x[c];
-        __syncthreads();
-    }
-    if (t < kb) b[k + t] = x[t];
-}
-
-// b[r] -= sum_{c in block} L[k + c][r] x[k + c] for rows r < k.
-__global__ void k_trsv_update_upper(const double *__restrict__ A, int64_t n, int64_t k, int kb,
-                                    double *__restrict__ b) {
-    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= k) return;
-    double acc = 0.0;
-    for (int c = 0; c < kb; ++c) acc += A[(size_t)(k + c) * n + r] * b[k + c];
-    b[r] -= acc;
-}
-
 // ------------------------------------------------------------ statistics ---
 
 // Block-wide compensated sum (Neumaier per thread, TwoSum tree); every
@@ -869,44 +733,6 @@ cudaError_t launch_center_gram(int64_t Ns, double *K, double *rowmean, double ep
     (k_row_mean<<<nblk(Ns, 8), 256, 0, st>>>(Ns, K, rowmean), nk::note_launch());
     (k_mean_into<<<1, 1024, 0, st>>>(Ns, rowmean), nk::note_launch());
     launch_double_center(Ns, K, rowmean, eps, true, st);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_cholesky(double *A, int64_t n, int *info, cudaStream_t st) {
-    for (int64_t k = 0; k < n; k += kNB) {
-        const int kb = (int)(n - k < kNB ? n - k : kNB);
-        const int64_t rest = n - k - kb;
-        int slot = prof_begin(NK_PROF_CHOL_PANEL, st);
-        (k_potrf_diag<<<1, kNB, 0, st>>>(A, n, k, kb, info), nk::note_launch());
-        if (rest > 0) (k_trsm_panel<<<nblk(rest, kNB), kNB, 0, st>>>(A, n, k, kb), nk::note_launch());
-        prof_end(slot, st, (double)kb * kb * kb / 3.0 + (double)rest * kb * kb);
-        if (rest > 0) {
-            PanelLoad pl{A, n, k + kb, k};
-            EpTrailing ep{A, n, k + kb};
-            slot = prof_begin(NK_PROF_CHOL_UPDATE, st);
-            cudaError_t err = gemm16(rest, rest, kb, 1, pl, pl, ep, st);
-            prof_end(slot, st, (double)kb * rest * (double)(rest + 1));
-            if (err != cudaSuccess) return err;
-        }
-    }
-    return cudaGetLastError();
-}
-
-cudaError_t launch_cholesky_solve(const double *L, int64_t n, double *b, cudaStream_t st) {
-    const int slot = prof_begin(NK_PROF_TRSV, st);
-    for (int64_t k = 0; k < n; k += kNB) {
-        const int kb = (int)(n - k < kNB ? n - k : kNB);
-        (k_trsv_diag_lower<<<1, kNB, 0, st>>>(L, n, k, kb, b), nk::note_launch());
-        const int64_t rest = n - k - kb;
-        if (rest > 0) (k_trsv_update_lower<<<nblk(rest, 8), 256, 0, st>>>(L, n, k, kb, b), nk::note_launch());
-    }
-    const int64_t last = ((n - 1) / kNB) * kNB;
-    for (int64_t k = last; k >= 0; k -= kNB) {
-        const int kb = (int)(n - k < kNB ? n - k : kNB);
-        (k_trsv_diag_upper<<<1, kNB, 0, st>>>(L, n, k, kb, b), nk::note_launch());
-        if (k > 0) (k_trsv_update_upper<<<nblk(k, 256), 256, 0, st>>>(L, n, k, kb, b), nk::note_launch());
-    }
-    prof_end(slot, st, 2.0 * (double)n * (double)n);
     return cudaGetLastError();
 }
 

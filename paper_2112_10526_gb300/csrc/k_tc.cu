@@ -100,66 +100,6 @@ __global__ void k_slice_rows(const double *__restrict__ A, int64_t lda, int64_t 
     slice_row_warp(x0, x1, lane, rows, r, S, out, expo);
 }
 
-// Columns p of rows r0 .. r0 + kr - 1 (kr <= 64) of X [.][ldx] -> S BF16
-// integer slices out[s][p][0..63] (zero beyond kr) with the column exponent
-// expo[p] (max over those rows): the transposed counterpart of k_slice_rows,
-// same digits.  One block per 32 columns, staged through shared memory.
-__global__ void __launch_bounds__(256) k_slice_cols(const double *__restrict__ X, int64_t ldx, int64_t r0, int kr,
-                                                    int64_t ncols, int S, __nv_bfloat16 *__restrict__ out,
-                                                    int *__restrict__ expo) {
-    __shared__ double tile[kTileK][33];
-    __shared__ int ex[32];
-    const int tid = threadIdx.x;
-    const int64_t p0 = (int64_t)blockIdx.x * 32;
-    for (int idx = tid; idx < kTileK * 32; idx += 256) {
-        const int r = idx >> 5, c = idx & 31;
-        tile[r][c] = (r < kr && p0 + c < ncols) ? X[(size_t)(r0 + r) * ldx + p0 + c] : 0.0;
-    }
-    __syncthreads();
-    if (tid < 32) {
-        int e = -100000;
-        for (int r = 0; r < kTileK; ++r) {
-            int b;
-            unsigned long long m;
-            bool n;
-            split_bits(tile[r][tid], b, m, n);
-            if (m) e = max(e, b - 1022);
-        }
-        e = e == -100000 ? 0 : e;
-        ex[tid] = e;
-        if (p0 + tid < ncols) expo[p0 + tid] = e;
-    }
-    __syncthreads();
-    for (int idx = tid; idx < kTileK * 32; idx += 256) {
-        const int c = idx >> 6, r = idx & 63;
-        if (p0 + c >= ncols) continue;
-        int b;
-        unsigned long long m;
-        bool n;
-        split_bits(tile[r][c], b, m, n);
-        unsigned long long y = 0;
-        if (m) {
-            const int sh = b - 1075 + 8 * S - ex[c];
-            y = sh >= 0 ? (m << sh) : (sh <= -64 ? 0ULL : (m >> (-sh)));
-        }
-        for (int q = 0; q < S; ++q) {
-            const int d = (int)((y >> (8 * (S - 1 - q))) & 0xFFULL);
-            out[((size_t)q * ncols + p0 + c) * kTileK + r] = __int2bfloat16_rn(n ? -d : d);
-        }
-    }
-}
-
-// C <- scale C + eps I on the lower triangle.
-__global__ void k_scale_shift_lower(double *__restrict__ C, int64_t n, double scale, double eps) {
-    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    for (int64_t i = blockIdx.y; i < n; i += gridDim.y) {
-        if (j > i || j >= n) continue;
-        double v = C[(size_t)i * n + j] * scale;
-        if (i == j) v += eps;
-        C[(size_t)i * n + j] = v;
-    }
-}
-
 // ------------------------------------------------------------- the GEMM ---
 //
 // Warp-specialised kernel over output strips: a CTA owns up to `chunk` (<= 8)
@@ -626,6 +566,52 @@ __global__ void __launch_bounds__(32 * kTrtriWarps) k_trtri64(const double *__re
     Linv[(size_t)i * kNB + lane + 32] = x1;
 }
 
+// Rows below the diagonal block: X = A L_kk^-T by substitution in FP64, the
+// result written back and, in the same pass, as S slices (out [S][rows][64],
+// exponents expo[rows]) for the updates to come.  With y_c = x_c l_cc and V_cj
+// = l_cj / l_jj the substitution is y_c = a_c - sum_{j < c} y_j V_cj: one
+// shuffle and one FMA a step on the chain, the scaling by 1 / l_cc at the end.
+// One warp per row, lanes holding columns lane and lane + 32, 8 rows a CTA at
+// a time.
+// Against the product with the inverted block (k_trtri64 + k_slice_rows +
+// k_ozaki_gemm + k_slice_rows: about 28 us on the panel chain): substitution
+// is backward stable whatever the block's condition, takes one launch, and
+// about 4 us while the rows fit one wave of the FP64 pipe (4 rows an SM), 50 us
+// at 8192 rows.  kTrsmRows is where the two meet; NK_F64 takes the
+// substitution at every size.
+constexpr int64_t kTrsmRows = 3072;
+
+__global__ void __launch_bounds__(256) k_trsm_rows(double *__restrict__ A, int64_t n, int64_t k, int64_t rows, int S,
+                                                   __nv_bfloat16 *__restrict__ out, int *__restrict__ expo) {
+    __shared__ double V[kNB * kLd];
+    __shared__ double rd[kNB];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    if (t < kNB) rd[t] = 1.0 / A[(size_t)(k + t) * n + k + t];
+    __syncthreads();
+    for (int e = t; e < kNB * kNB; e += 256) {
+        const int c = e >> 6, j = e & 63;
+        V[c * kLd + j] = j < c ? A[(size_t)(k + c) * n + k + j] * rd[j] : 0.0;
+    }
+    __syncthreads();
+    for (int64_t r = (int64_t)blockIdx.x * 8 + warp; r < rows; r += (int64_t)gridDim.x * 8) {
+        double *row = A + (size_t)(k + kNB + r) * n + k;
+        double y0 = row[lane], y1 = row[lane + 32];
+#pragma unroll 8
+        for (int c = 0; c < 32; ++c) {
+            const double yc = __shfl_sync(0xffffffffu, y0, c);
+            y0 = fma(-yc, V[lane * kLd + c], y0);
+            y1 = fma(-yc, V[(lane + 32) * kLd + c], y1);
+        }
+#pragma unroll 8
+        for (int c = 32; c < 64; ++c)
+            y1 = fma(-__shfl_sync(0xffffffffu, y1, c - 32), V[(lane + 32) * kLd + c], y1);
+        const double x0 = y0 * rd[lane], x1 = y1 * rd[lane + 32];
+        row[lane] = x0;
+        row[lane + 32] = x1;
+        slice_row_warp(x0, x1, lane, rows, r, S, out, expo);
+    }
+}
+
 // ---------------------------------------------- triangular solves with L ---
 //
 // One cooperative launch per direction.  CTA b owns block rows b, b + G, ...
@@ -668,8 +654,41 @@ __device__ bool wait_solved(const double *y, int lane, int valid, double &a, dou
     }
 }
 
+// One step of refinement of z = M acc, M = L_ii^-1 (or its transpose) as
+// computed: z += M (acc - L z), so that the block solve is as accurate as
+// substitution with L_ii whatever its condition (NK_F64).  Thread (r, q) holds
+// 16 entries of row r of M (m) and of L (l); v: its row's entry of z, summed
+// over the four threads of the row.  zs, rs: 64 doubles of shared memory each.
+__device__ __forceinline__ double refine_block(const double (&m)[16], const double (&l)[16], double v, int r, int q,
+                                               const double *acc, double *zs, double *rs) {
+    if (q == 0) zs[r] = v;
+    __syncthreads();
+    double a = 0.0, b = 0.0;
+#pragma unroll
+    for (int u = 0; u < 16; u += 2) {
+        a = fma(l[u], zs[q * 16 + u], a);
+        b = fma(l[u + 1], zs[q * 16 + u + 1], b);
+    }
+    double lz = a + b;
+    lz += __shfl_xor_sync(0xffffffffu, lz, 1);
+    lz += __shfl_xor_sync(0xffffffffu, lz, 2);
+    if (q == 0) rs[r] = acc[r] - lz;
+    __syncthreads();
+    a = b = 0.0;
+#pragma unroll
+    for (int u = 0; u < 16; u += 2) {
+        a = fma(m[u], rs[q * 16 + u], a);
+        b = fma(m[u + 1], rs[q * 16 + u + 1], b);
+    }
+    double dz = a + b;
+    dz += __shfl_xor_sync(0xffffffffu, dz, 1);
+    dz += __shfl_xor_sync(0xffffffffu, dz, 2);
+    return v + dz;
+}
+
 // L y = b: y (sentinel-filled) receives the solution; b is read and refilled
 // with the sentinel for the backward solve.
+template <bool kRefine>
 __global__ void __launch_bounds__(kTrsvThreads) k_trsv_fwd(const double *__restrict__ L, int64_t n,
                                                            const double *__restrict__ Linv, double *b, double *y,
                                                            int *err) {
@@ -729,6 +748,17 @@ __global__ void __launch_bounds__(kTrsvThreads) k_trsv_fwd(const double *__restr
             double v = ya + yb;
             v += __shfl_xor_sync(0xffffffffu, v, 1);
             v += __shfl_xor_sync(0xffffffffu, v, 2);
+            if (kRefine) {
+                __shared__ double zs[kNB], rs[kNB];
+                double m[16], l[16];
+#pragma unroll
+                for (int u = 0; u < 16; ++u) {
+                    const int c = q * 16 + u;
+                    m[u] = inv[r * kNB + c];
+                    l[u] = (r < kb && c <= r) ? L[(size_t)(r0 + r) * n + r0 + c] : 0.0;
+                }
+                v = refine_block(m, l, v, r, q, acc, zs, rs);
+            }
             if (q == 0 && r < kb) __stcg(y + r0 + r, v);
         }
         __syncthreads();  // inv and acc are reused by the CTA's next row
@@ -737,6 +767,7 @@ __global__ void __launch_bounds__(kTrsvThreads) k_trsv_fwd(const double *__restr
 
 // L^T x = y: y holds the forward solution; x goes to b (sentinel-filled by
 // the forward solve).  Block rows are solved from the last to the first.
+template <bool kRefine>
 __global__ void __launch_bounds__(kTrsvThreads) k_trsv_bwd(const double *__restrict__ L, int64_t n,
                                                            const double *__restrict__ Linv, double *b,
                                                            const double *y, int *err) {
@@ -806,6 +837,17 @@ __global__ void __launch_bounds__(kTrsvThreads) k_trsv_bwd(const double *__restr
             double x = xa + xb;
             x += __shfl_xor_sync(0xffffffffu, x, 1);
             x += __shfl_xor_sync(0xffffffffu, x, 2);
+            if (kRefine) {
+                __shared__ double zs[kNB], rs[kNB];
+                double m[16], l[16];
+#pragma unroll
+                for (int u = 0; u < 16; ++u) {
+                    const int r = q * 16 + u;
+                    m[u] = inv[r * kNB + c];
+                    l[u] = (r < kb && r >= c) ? L[(size_t)(c0 + r) * n + c0 + c] : 0.0;
+                }
+                x = refine_block(m, l, x, c, q, acc, zs, rs);
+            }
             if (q == 0 && c < kb) __stcg(b + c0 + c, x);
         }
         __syncthreads();  // inv, part_s and acc are reused by the CTA's next row
@@ -984,20 +1026,45 @@ TcWs carve_tc(void *ws, int64_t n) {
 namespace {
 
 // Factor panel k (columns k0 .. k0 + kb - 1) whose block column is up to date:
-// diagonal block + inverse, L_panel = A_panel L_kk^-T, slices of L_panel.
-// With an aux stream (cs non-null), the panel rows below the diagonal block
-// are sliced there, beside the diagonal block's factorisation and inverse:
-// the slicing depends only on the narrow update that precedes the panel.
+// diagonal block, L_panel = A_panel L_kk^-T, slices of L_panel, and the inverse
+// of the diagonal block for the triangular solves.
+// By substitution (k_trsm_rows; `exact`, or few rows) the inverse is off the
+// chain: with an aux stream (cs non-null) it runs there, and `joined` says that
+// the aux stream must be joined before the inverses are read.  As a product
+// with the inverse, the rows below the diagonal block are sliced on the aux
+// stream beside the diagonal block's factorisation: the slicing depends only
+// on the narrow update that precedes the panel.
 cudaError_t panel_step(double *A, int64_t n, int64_t k0, int *info, int *err, TcWs &w, __nv_bfloat16 *Lsl,
-                       int *Lexp, cudaStream_t st, const CholStreams *cs) {
+                       int *Lexp, cudaStream_t st, const CholStreams *cs, bool exact, bool &joined) {
     const int S = kMaxSlices;
     const int kb = (int)(n - k0 < kNB ? n - k0 : kNB);
     const int64_t rest = n - k0 - kb;
     double *Linv = w.Linv + (size_t)(k0 / kNB) * kNB * kNB;
     double *panel = A + (size_t)(k0 + kb) * n + k0;
     cudaError_t e = cudaSuccess;
-    const bool fork = cs != nullptr && cs->aux != nullptr && rest > 0;
-    if (fork) {
+    const bool aux = cs != nullptr && cs->aux != nullptr;
+    if (exact || rest <= kTrsmRows) {
+        int slot = prof_begin(NK_PROF_CHOL_PANEL, st);
+        (k_potrf64<<<1, kPotrfThreads, 0, st>>>(A, n, k0, kb, info), nk::note_launch());
+        cudaStream_t is = st;
+        if (aux && rest > 0) {
+            e = cudaEventRecord(cs->ev_fork, st);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(cs->aux, cs->ev_fork, 0);
+            if (e != cudaSuccess) return e;
+            is = cs->aux;
+            joined = false;
+        }
+        // (the slices of the inverse that the kernel also writes are not used here)
+        (k_trtri64<<<kNB / kTrtriWarps, 32 * kTrtriWarps, 0, is>>>(A, n, k0, kb, Linv, S, w.Bsl, w.expB),
+         nk::note_launch());
+        if (rest > 0) {
+            const unsigned grid = nblk(rest, 8) < 304 ? nblk(rest, 8) : 304;
+            (k_trsm_rows<<<grid, 256, 0, st>>>(A, n, k0, rest, S, Lsl, Lexp), nk::note_launch());
+        }
+        prof_end(slot, st, 2.0 * (double)kb * kb * kb / 3.0 + (double)rest * kb * kb);
+        return cudaGetLastError();
+    }
+    if (aux) {
         e = cudaEventRecord(cs->ev_fork, st);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(cs->aux, cs->ev_fork, 0);
         if (e != cudaSuccess) return e;
@@ -1006,6 +1073,7 @@ cudaError_t panel_step(double *A, int64_t n, int64_t k0, int *info, int *err, Tc
         prof_end(aslot, cs->aux, 0.0);
         if (e == cudaSuccess) e = cudaEventRecord(cs->ev_join, cs->aux);
         if (e != cudaSuccess) return e;
+        joined = true;
     }
     // timing classes: the FP64 diagonal-block kernels and the slicing count
     // as the panel, the tensor-core panel product with the trailing updates
@@ -1014,10 +1082,9 @@ cudaError_t panel_step(double *A, int64_t n, int64_t k0, int *info, int *err, Tc
     // the inverse and its slices (the B operand of the panel solve)
     (k_trtri64<<<kNB / kTrtriWarps, 32 * kTrtriWarps, 0, st>>>(A, n, k0, kb, Linv, S, w.Bsl, w.expB),
      nk::note_launch());
-    if (rest > 0)
-        e = fork ? cudaStreamWaitEvent(st, cs->ev_join, 0) : launch_slice_rows(panel, n, rest, kb, S, Lsl, Lexp, st);
+    e = aux ? cudaStreamWaitEvent(st, cs->ev_join, 0) : launch_slice_rows(panel, n, rest, kb, S, Lsl, Lexp, st);
     prof_end(slot, st, 2.0 * (double)kb * kb * kb / 3.0);
-    if (rest > 0 && e == cudaSuccess) {
+    if (e == cudaSuccess) {
         slot = prof_begin(NK_PROF_CHOL_UPDATE, st);
         e = launch_ozaki_gemm(Lsl, Lexp, rest, w.Bsl, w.expB, kb, S, panel, n, 0, false, err, st);
         // the triangular solve L21 = A21 L11^-T: rest kb^2 flops in FP64
@@ -1032,7 +1099,7 @@ cudaError_t panel_step(double *A, int64_t n, int64_t k0, int *info, int *err, Tc
 }  // namespace
 
 cudaError_t launch_cholesky_tc(double *A, int64_t n, int *info, int *err, void *ws, cudaStream_t st,
-                               const CholStreams *cs) {
+                               const CholStreams *cs, bool exact) {
     // Step k, with panel k factored and sliced:
     //   side stream: the narrow update (block column k+1 by panel k), then
     //     panel k+1 (factor, invert, solve, slice);
@@ -1050,7 +1117,8 @@ cudaError_t launch_cholesky_tc(double *A, int64_t n, int *info, int *err, void *
     const bool two = cs != nullptr && cs->side != nullptr;
     cudaStream_t side = two ? cs->side : nullptr, ps = two ? cs->side : st;
     cudaEvent_t ev_wide = two ? cs->ev_wide : nullptr, ev_panel = two ? cs->ev_panel : nullptr;
-    e = panel_step(A, n, 0, info, err, w, buf[0], bexp[0], st, cs);
+    bool joined = true;
+    e = panel_step(A, n, 0, info, err, w, buf[0], bexp[0], st, cs, exact, joined);
     if (e != cudaSuccess) return e;
     for (int64_t k = 0; k + 1 < nb; ++k) {
         const int64_t k0 = k * kNB;
@@ -1071,7 +1139,8 @@ cudaError_t launch_cholesky_tc(double *A, int64_t n, int *info, int *err, void *
         prof_end(slot, ps, 2.0 * kNB * ((double)rest * kb1 - 0.5 * (double)kb1 * (kb1 - 1)),
                  ozaki_mma_flops(rest, kb1, S, true));
         if (e != cudaSuccess) return e;
-        e = panel_step(A, n, k0 + kNB, info, err, w, buf[(k + 1) & 1], bexp[(k + 1) & 1], ps, cs);
+        e = panel_step(A, n, k0 + kNB, info, err, w, buf[(k + 1) & 1], bexp[(k + 1) & 1], ps, cs, exact,
+                       joined);
         if (e != cudaSuccess) return e;
         if (two) {
             e = cudaEventRecord(ev_panel, side);
@@ -1092,19 +1161,26 @@ cudaError_t launch_cholesky_tc(double *A, int64_t n, int *info, int *err, void *
             if (e != cudaSuccess) return e;
         }
     }
+    if (!joined) {  // the inverted diagonal blocks
+        e = cudaEventRecord(cs->ev_join, cs->aux);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(st, cs->ev_join, 0);
+        if (e != cudaSuccess) return e;
+    }
     return cudaGetLastError();
 }
 
 cudaError_t launch_cholesky_solve_tc(const double *L, int64_t n, const void *ws, double *b, int *err,
-                                     cudaStream_t st) {
+                                     cudaStream_t st, bool exact) {
     if (n <= 0) return cudaSuccess;
     TcWs w = carve_tc(const_cast<void *>(ws), n);
     const int nb = (int)((n + kNB - 1) / kNB);
     int dev = 0, sms = 0, per_sm_f = 0, per_sm_b = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_f, k_trsv_fwd, kTrsvThreads, 0);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_b, k_trsv_bwd, kTrsvThreads, 0);
+    const void *fwd = exact ? (const void *)k_trsv_fwd<true> : (const void *)k_trsv_fwd<false>;
+    const void *bwd = exact ? (const void *)k_trsv_bwd<true> : (const void *)k_trsv_bwd<false>;
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_f, fwd, kTrsvThreads, 0);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_b, bwd, kTrsvThreads, 0);
     if (e != cudaSuccess) return e;
     // at most one CTA per SM: the resident grid needs no more, and blocks
     // rows then spread over the SMs' load bandwidth
@@ -1116,10 +1192,10 @@ cudaError_t launch_cholesky_solve_tc(const double *L, int64_t n, const void *ws,
     const double *Linv = w.Linv;
     double *y = w.y;
     void *args[] = {(void *)&L, (void *)&n, (void *)&Linv, (void *)&b, (void *)&y, (void *)&err};
-    e = cudaLaunchCooperativeKernel((const void *)k_trsv_fwd, dim3(gf), dim3(kTrsvThreads), args, 0, st);
+    e = cudaLaunchCooperativeKernel(fwd, dim3(gf), dim3(kTrsvThreads), args, 0, st);
     nk::note_launch();
     if (e != cudaSuccess) return e;
-    e = cudaLaunchCooperativeKernel((const void *)k_trsv_bwd, dim3(gb), dim3(kTrsvThreads), args, 0, st);
+    e = cudaLaunchCooperativeKernel(bwd, dim3(gb), dim3(kTrsvThreads), args, 0, st);
     nk::note_launch();
     prof_end(slot, st, 2.0 * (double)n * (double)n);
     return e != cudaSuccess ? e : cudaGetLastError();
@@ -1128,30 +1204,6 @@ cudaError_t launch_cholesky_solve_tc(const double *L, int64_t n, const void *ws,
 // Lower triangle of K = T T^T by tensor cores with S slices per 64-column
 // chunk of T [Ns][M], then the Jacobian-row Gram s.s + t.t + (t.t)(s.s)
 // written to both triangles.
-// Lower triangle of C = scale X^T X + eps I for X [rows][ncols] (row stride
-// ncols): 64 rows of X per tensor-core pass, each sliced by columns (one
-// exponent per column and pass) and accumulated in FP64.
-cudaError_t launch_gram_cols_tc(const double *X, int64_t rows, int64_t ncols, double scale, double eps, double *C,
-                                int *err, void *ws, cudaStream_t st) {
-    if (rows <= 0 || ncols <= 0) return cudaSuccess;
-    TcWs w = carve_tc(ws, ncols);
-    const int S = kMaxSlices;
-    const int slot = prof_begin(NK_PROF_GRAM, st);
-    cudaError_t e = cudaSuccess;
-    for (int64_t r0 = 0; r0 < rows && e == cudaSuccess; r0 += kTileK) {
-        const int kr = (int)(rows - r0 < kTileK ? rows - r0 : kTileK);
-        (k_slice_cols<<<nblk(ncols, 32), 256, 0, st>>>(X, ncols, r0, kr, ncols, S, w.Asl, w.expA), nk::note_launch());
-        e = launch_ozaki_gemm(w.Asl, w.expA, ncols, w.Asl, w.expA, ncols, S, C, ncols, r0 == 0 ? 0 : 2, true, err, st);
-    }
-    if (e == cudaSuccess) {
-        const dim3 grid(nblk(ncols, 256), (unsigned)(ncols < 65535 ? ncols : 65535));
-        (k_scale_shift_lower<<<grid, 256, 0, st>>>(C, ncols, scale, eps), nk::note_launch());
-    }
-    prof_end(slot, st, (double)rows * ncols * (double)(ncols + 1),
-             (double)((rows + kTileK - 1) / kTileK) * ozaki_mma_flops(ncols, ncols, S, true));
-    return e != cudaSuccess ? e : cudaGetLastError();
-}
-
 cudaError_t launch_gram_tc(int N, int M, int64_t Ns, const int8_t *s, const double *T, int S, double *K,
                            int *err, void *ws, cudaStream_t st) {
     TcWs w = carve_tc(ws, Ns);

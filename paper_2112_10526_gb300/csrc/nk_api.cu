@@ -202,7 +202,8 @@ struct SolveWs {
     double *V, *ev, *evmax, *z, *gpart;
     void *eig;
     int *kept;
-    void *tc;   // tensor-core slices and inverted diagonal blocks (NK_MIXED)
+    void *tc;   // tensor-core slices and inverted diagonal blocks
+    void *syrk; // slices and partials of the dense S
     void *tcm;  // tensor-core Jacobian-product workspace (NK_MIXED)
     int *colexpT;     // NK_MIXED CG: column exponents of tanh(theta), [M + 1]
     void *colexp_ws;
@@ -256,7 +257,8 @@ void carve_solve(Carver &c, SolveWs &w, int N, int M, int64_t Ns, int solver, in
         w.mean = c.take<double>(Np);
         w.ones = c.take<double>(Ns);
         w.info = c.take<int>(2);
-        if (precision == NK_MIXED) w.tc = c.take<char>(nk::tc_chol_ws_bytes(Np));
+        w.tc = c.take<char>(nk::tc_chol_ws_bytes(Np));
+        w.syrk = c.take<char>(nk::syrk_ws_bytes(Ns, Np));
     } else if (solver == NK_SOLVER_SVD || solver == NK_SOLVER_SVD_SAMPLESPACE) {
         const bool ss = solver == NK_SOLVER_SVD_SAMPLESPACE;
         const int64_t n = ss ? Ns : Np;
@@ -264,12 +266,12 @@ void carve_solve(Carver &c, SolveWs &w, int N, int M, int64_t Ns, int solver, in
             w.w = c.take<double>(Ns);
             w.rowmean = c.take<double>(2 * Ns + 1);
             w.tmp = c.take<double>(Np);
-            if (precision == NK_MIXED) w.tc = c.take<char>(nk::tc_chol_ws_bytes(Ns));
+            if (nk::gram_on_tensor(precision, M, Ns)) w.tc = c.take<char>(nk::tc_chol_ws_bytes(Ns));
         } else {
             w.dJ = c.take<double>((size_t)Ns * Np);
             w.mean = c.take<double>(Np);
             w.ones = c.take<double>(Ns);
-            if (precision == NK_MIXED) w.tc = c.take<char>(nk::tc_chol_ws_bytes(Np));
+            w.syrk = c.take<char>(nk::syrk_ws_bytes(Ns, Np));
         }
         w.K = c.take<double>((size_t)n * n);
         w.V = c.take<double>((size_t)n * n);
@@ -286,7 +288,7 @@ void carve_solve(Carver &c, SolveWs &w, int N, int M, int64_t Ns, int solver, in
         w.rowmean = c.take<double>(2 * Ns + 1);  // row means, grand mean, centring coefficients
         w.tmp = c.take<double>(Np);
         w.info = c.take<int>(2);
-        if (precision == NK_MIXED) w.tc = c.take<char>(nk::tc_chol_ws_bytes(Ns));
+        w.tc = c.take<char>(nk::tc_chol_ws_bytes(Ns));
     }
 }
 
@@ -441,7 +443,7 @@ nk_status run_solve(nk_ctx *ctx, int N, int M, int64_t Ns, const int8_t *s, cons
         NK_CU(cudaMemsetAsync(w.info, 0, 2 * sizeof(int), st), "svd");
         if (ss) {
             // the centred sample-space Gram X X^T, X = dJ / sqrt(Ns), no shift
-            if (tc) {
+            if (nk::gram_on_tensor(precision, M, Ns)) {
                 NK_CU(nk::launch_gram_tc(N, M, Ns, s, T, 7, w.K, w.info + 1, w.tc, st), "svd gram");
                 NK_CU(nk::launch_center_gram(Ns, w.K, w.rowmean, 0.0, st), "svd gram");
             } else {
@@ -453,11 +455,7 @@ nk_status run_solve(nk_ctx *ctx, int N, int M, int64_t Ns, const int8_t *s, cons
             NK_CU(vjp_any(N, M, Ns, s, T, w.ones, 1.0 / (double)Ns, nullptr, w, w.mean, precision, kExactSlices, st),
                   "svd mean");
             NK_CU(nk::launch_jacobian_rows(N, M, s, T, 0, Ns, w.mean, w.dJ, st), "svd dJ");
-            if (tc)
-                NK_CU(nk::launch_gram_cols_tc(w.dJ, Ns, Np, 1.0 / (double)Ns, eps, w.K, w.info + 1, w.tc, st),
-                      "svd S");
-            else
-                NK_CU(nk::launch_syrk_t(w.dJ, Ns, Np, 1.0 / (double)Ns, eps, w.K, st), "svd S");
+            NK_CU(nk::launch_syrk(w.dJ, Ns, Np, 1.0 / (double)Ns, eps, w.K, w.info + 1, w.syrk, st), "svd S");
         }
         int sweeps = 0;
         double rel = 0.0;
@@ -499,41 +497,25 @@ nk_status run_solve(nk_ctx *ctx, int N, int M, int64_t Ns, const int8_t *s, cons
               "chol mean");
         NK_CU(nk::launch_jacobian_rows(N, M, s, T, 0, Ns, w.mean, w.dJ, st), "chol dJ");
         NK_CU(cudaMemsetAsync(w.info, 0, 2 * sizeof(int), st), "chol");
-        if (tc)
-            NK_CU(nk::launch_gram_cols_tc(w.dJ, Ns, Np, 1.0 / (double)Ns, eps, w.S, w.info + 1, w.tc, st),
-                  "chol gram");
-        else
-            NK_CU(nk::launch_syrk_t(w.dJ, Ns, Np, 1.0 / (double)Ns, eps, w.S, st), "chol syrk");
-        if (tc)
-            NK_CU(nk::launch_cholesky_tc(w.S, Np, w.info, w.info + 1, w.tc, st, &cs),
-                  "chol factor");
-        else
-            NK_CU(nk::launch_cholesky(w.S, Np, w.info, st), "chol factor");
+        NK_CU(nk::launch_syrk(w.dJ, Ns, Np, 1.0 / (double)Ns, eps, w.S, w.info + 1, w.syrk, st), "chol S");
+        NK_CU(nk::launch_cholesky_tc(w.S, Np, w.info, w.info + 1, w.tc, st, &cs, !tc), "chol factor");
         NK_CU(nk::launch_axpby(Np, 1.0, F, 0.0, delta, st), "chol");
-        if (tc)
-            NK_CU(nk::launch_cholesky_solve_tc(w.S, Np, w.tc, delta, w.info + 1, st), "chol solve");
-        else
-            NK_CU(nk::launch_cholesky_solve(w.S, Np, delta, st), "chol solve");
+        NK_CU(nk::launch_cholesky_solve_tc(w.S, Np, w.tc, delta, w.info + 1, st, !tc), "chol solve");
         return sync_check ? check_factor(ctx, w.info, st) : NK_OK;
     }
     // sample space: delta = (F - X^T (X X^T + eps I)^{-1} X F) / eps, X = dJ / sqrt(Ns)
     const double isq = 1.0 / std::sqrt((double)Ns);
     NK_CU(cudaMemsetAsync(w.info, 0, 2 * sizeof(int), st), "ss");
-    if (tc) {
+    if (nk::gram_on_tensor(precision, M, Ns)) {
         NK_CU(nk::launch_gram_tc(N, M, Ns, s, T, 7, w.K, w.info + 1, w.tc, st), "ss gram");
         NK_CU(nk::launch_center_gram(Ns, w.K, w.rowmean, eps, st), "ss gram");
-        NK_CU(nk::launch_cholesky_tc(w.K, Ns, w.info, w.info + 1, w.tc, st, &cs),
-              "ss factor");
     } else {
         NK_CU(nk::launch_gram_samplespace(N, M, Ns, s, T, eps, w.K, w.rowmean, st), "ss gram");
-        NK_CU(nk::launch_cholesky(w.K, Ns, w.info, st), "ss factor");
     }
+    NK_CU(nk::launch_cholesky_tc(w.K, Ns, w.info, w.info + 1, w.tc, st, &cs, !tc), "ss factor");
     NK_CU(jvp_any(N, M, Ns, s, T, F, w, w.w, precision, kExactSlices, st), "ss XF");
     NK_CU(nk::launch_center(Ns, w.w, w.dotp, isq, st), "ss XF");
-    if (tc)
-        NK_CU(nk::launch_cholesky_solve_tc(w.K, Ns, w.tc, w.w, w.info + 1, st), "ss solve");
-    else
-        NK_CU(nk::launch_cholesky_solve(w.K, Ns, w.w, st), "ss solve");
+    NK_CU(nk::launch_cholesky_solve_tc(w.K, Ns, w.tc, w.w, w.info + 1, st, !tc), "ss solve");
     NK_CU(nk::launch_center(Ns, w.w, w.dotp, isq, st), "ss Xty");
     NK_CU(vjp_any(N, M, Ns, s, T, w.w, 1.0, nullptr, w, w.tmp, precision, kExactSlices, st), "ss Xty");
     NK_CU(nk::launch_axpby(Np, 1.0 / eps, F, 0.0, delta, st), "ss delta");
@@ -1387,7 +1369,8 @@ nk_status nk_symm_sr_step(nk_ctx *ctx, nk_rbm_symm *symm, const nk_ham *ham, nk_
         double *nrm = c.take<double>(2);
         double *dotp = c.take<double>(nk::dot_partial_doubles(Np) + 8);
         int *info = c.take<int>(2);
-        void *tc = mixed ? c.take<char>(nk::tc_chol_ws_bytes(Np)) : nullptr;
+        void *tc = c.take<char>(nk::tc_chol_ws_bytes(Np));
+        void *syrk = c.take<char>(nk::syrk_ws_bytes(Ns, Np));
         if (!run) return NK_OK;
         nk_status e = symm_expand_checked(ctx, symm, plain, st);
         if (e != NK_OK) return e;
@@ -1403,18 +1386,10 @@ nk_status nk_symm_sr_step(nk_ctx *ctx, nk_rbm_symm *symm, const nk_ham *ham, nk_
         NK_CU(nk::launch_gemv_t(O, Ns, Np, gv, 1.0, partial, F, st), "force");
         // S + eps I = dJ^T dJ / Ns + eps I, Cholesky, two triangular solves
         NK_CU(cudaMemsetAsync(info, 0, 2 * sizeof(int), st), "chol");
-        if (mixed) {
-            NK_CU(nk::launch_gram_cols_tc(O, Ns, Np, 1.0 / (double)Ns, cfg->diag_shift, S, info + 1, tc, st), "gram");
-            NK_CU(nk::launch_cholesky_tc(S, Np, info, info + 1, tc, st, &cs), "factor");
-        } else {
-            NK_CU(nk::launch_syrk_t(O, Ns, Np, 1.0 / (double)Ns, cfg->diag_shift, S, st), "syrk");
-            NK_CU(nk::launch_cholesky(S, Np, info, st), "factor");
-        }
+        NK_CU(nk::launch_syrk(O, Ns, Np, 1.0 / (double)Ns, cfg->diag_shift, S, info + 1, syrk, st), "S");
+        NK_CU(nk::launch_cholesky_tc(S, Np, info, info + 1, tc, st, &cs, !mixed), "factor");
         NK_CU(nk::launch_axpby(Np, 1.0, F, 0.0, mean, st), "solve");  // mean <- F, solved in place
-        if (mixed)
-            NK_CU(nk::launch_cholesky_solve_tc(S, Np, tc, mean, info + 1, st), "solve");
-        else
-            NK_CU(nk::launch_cholesky_solve(S, Np, mean, st), "solve");
+        NK_CU(nk::launch_cholesky_solve_tc(S, Np, tc, mean, info + 1, st, !mixed), "solve");
         NK_CU(nk::launch_dot(Np, F, F, dotp, nrm, st), "norm");
         NK_CU(nk::launch_dot(Np, mean, mean, dotp, nrm + 1, st), "norm");
         NK_CU(nk::launch_sgd(Np, cfg->lr, mean, symm->params, st), "update");
@@ -1467,7 +1442,7 @@ nk_status check_complex_out(const double *p, const char *name) {
 struct TdvpWs {
     int8_t *samples;
     double *eloc, *stats4, *O, *mean, *R, *g, *F, *rhs, *S, *V, *ev, *evmax, *z, *gpart, *partial;
-    void *eig;
+    void *eig, *tc, *syrk;
     int *info, *kept;
     unsigned long long *acc;
 };
@@ -1487,12 +1462,13 @@ nk_status tdvp_slope(nk_ctx *ctx, int N, int M, const double *p, const nk_ham *h
     NK_CU(nk::launch_cforce_g(Ns, w.eloc, w.stats4, w.g, st), "force g");
     NK_CU(nk::launch_gemv_t(w.R, 2 * Ns, n, w.g, 1.0, w.partial, w.F, st), "force");
     NK_CU(nk::launch_tdvp_rhs(Np, w.F, cfg->real_time, w.rhs, st), "rhs");
-    NK_CU(nk::launch_syrk_t(w.R, 2 * Ns, n, 1.0 / (double)Ns, cfg->diag_shift, w.S, st), "qgt");
+    const nk::CholStreams cs{ctx->side, ctx->aux, ctx->ev[0], ctx->ev[1], ctx->ev[2], ctx->ev[3]};
+    NK_CU(cudaMemsetAsync(w.info, 0, 2 * sizeof(int), st), "qgt");
+    NK_CU(nk::launch_syrk(w.R, 2 * Ns, n, 1.0 / (double)Ns, cfg->diag_shift, w.S, w.info + 1, w.syrk, st), "qgt");
     if (cfg->solver == NK_SOLVER_CHOLESKY) {
-        NK_CU(cudaMemsetAsync(w.info, 0, 2 * sizeof(int), st), "chol");
-        NK_CU(nk::launch_cholesky(w.S, n, w.info, st), "chol");
+        NK_CU(nk::launch_cholesky_tc(w.S, n, w.info, w.info + 1, w.tc, st, &cs, true), "chol");
         NK_CU(nk::launch_axpby(n, 1.0, w.rhs, 0.0, x, st), "chol");
-        NK_CU(nk::launch_cholesky_solve(w.S, n, x, st), "chol solve");
+        NK_CU(nk::launch_cholesky_solve_tc(w.S, n, w.tc, x, w.info + 1, st, true), "chol solve");
         return check_factor(ctx, w.info, st);
     }
     int sweeps = 0;
@@ -1633,6 +1609,8 @@ nk_status nk_tdvp_step(nk_ctx *ctx, nk_crbm *rbm, const nk_ham *ham, nk_chains *
         w.partial = c.take<double>(nk::gemv_t_partial_doubles(2 * Ns, n));
         w.info = c.take<int>(2);
         w.acc = c.take<unsigned long long>(C);
+        w.tc = c.take<char>(nk::tc_chol_ws_bytes(n));
+        w.syrk = c.take<char>(nk::syrk_ws_bytes(2 * Ns, n));
         if (svd) {
             w.V = c.take<double>((size_t)n * n);
             w.ev = c.take<double>(n);

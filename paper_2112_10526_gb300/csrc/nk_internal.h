@@ -174,11 +174,6 @@ cudaError_t launch_gram_samplespace(int N, int M, int64_t Ns, const int8_t *s, c
 // (lower triangle written); rowmean holds 2 Ns + 1 doubles of scratch.
 cudaError_t launch_center_gram(int64_t Ns, double *K, double *rowmean, double eps, cudaStream_t st);
 
-// In-place lower Cholesky of an n x n matrix (lda = n); info: device int.
-cudaError_t launch_cholesky(double *A, int64_t n, int *info, cudaStream_t st);
-// Solve L L^T x = b in place (b -> x).
-cudaError_t launch_cholesky_solve(const double *L, int64_t n, double *b, cudaStream_t st);
-
 // ---- tensor-core products (k_tc.cu) ---------------------------------------
 // FP64 rows -> S BF16 integer slices [S][rows][64] + row exponents.
 size_t slice_elems(int64_t rows, int S);
@@ -195,20 +190,34 @@ struct CholStreams {
     cudaStream_t side, aux;
     cudaEvent_t ev_wide, ev_panel, ev_fork, ev_join;
 };
-// cs null: everything on st.
+// cs null: everything on st.  exact (NK_F64): panels by FP64 substitution and
+// block solves refined, so that the factor and the solution are backward
+// stable whatever the condition of the diagonal blocks; else large panels are
+// products with the inverted diagonal block.
 cudaError_t launch_cholesky_tc(double *A, int64_t n, int *info, int *err, void *ws, cudaStream_t st,
-                               const CholStreams *cs = nullptr);
+                               const CholStreams *cs, bool exact);
 // Forward and backward solves with the factor of launch_cholesky_tc (one
 // cooperative launch each); err receives 6 / 7 if a block-row wait timed out.
 cudaError_t launch_cholesky_solve_tc(const double *L, int64_t n, const void *ws, double *b, int *err,
-                                     cudaStream_t st);
+                                     cudaStream_t st, bool exact);
 cudaError_t launch_gram_tc(int N, int M, int64_t Ns, const int8_t *s, const double *T, int S, double *K,
                            int *err, void *ws, cudaStream_t st);
-// Lower triangle of C = scale X^T X + eps I (X [rows][ncols]) by 7-slice
-// tensor-core products, 64 rows of X per pass; ws as for launch_cholesky_tc(ncols).
-cudaError_t launch_gram_cols_tc(const double *X, int64_t rows, int64_t ncols, double scale, double eps, double *C,
-                                int *err, void *ws, cudaStream_t st);
-
+// Lower triangle of C = scale X^T X + eps I (X [rows][n]) by 7-slice
+// tensor-core products of any length (k_syrk.cu); ws of tc_syrk_ws_bytes.
+size_t tc_syrk_ws_bytes(int64_t rows, int64_t n);
+cudaError_t launch_syrk_tc(const double *X, int64_t rows, int64_t n, double scale, double eps, double *C, int *err,
+                           void *ws, cudaStream_t st);
+// Whether S = X^T X takes the tensor cores: from about 10M multiply-adds on
+// (33 us on the FP64 pipe, 2 a clock and SM; exponents, slices, product and sum
+// take about 25 us at that size).
+inline bool syrk_on_tensor(int64_t rows, int64_t n) { return 0.5 * (double)rows * (double)n * (double)n >= 1e7; }
+// Either of the two by that rule (ws may be null for the FP64 pipe).
+inline cudaError_t launch_syrk(const double *X, int64_t rows, int64_t n, double scale, double eps, double *C,
+                               int *err, void *ws, cudaStream_t st) {
+    return syrk_on_tensor(rows, n) ? launch_syrk_tc(X, rows, n, scale, eps, C, err, ws, st)
+                                   : launch_syrk_t(X, rows, n, scale, eps, C, st);
+}
+inline size_t syrk_ws_bytes(int64_t rows, int64_t n) { return syrk_on_tensor(rows, n) ? tc_syrk_ws_bytes(rows, n) : 0; }
 
 // ---- tensor-core products with the configurations (k_sgemm.cu) -------------
 size_t tc_theta_ws_bytes(int N, int M, int64_t B);
@@ -258,6 +267,14 @@ cudaError_t launch_colexp_t(int M, int64_t Ns, const double *T, int *colexpT, vo
 // FP64 pipe retires 2 multiply-adds a clock and SM, so the 12 to 20 us of
 // slicing, products and sums pay from about 4M multiply-adds.  More than 2^20
 // samples would not fit the K splits of J^T g.
+inline bool f64_on_tensor(int N, int M, int64_t B);
+
+// The sample-space Gram T T^T of NK_F64 (Ns^2 M / 2 multiply-adds): the same
+// trade.
+inline bool gram_on_tensor(int precision, int M, int64_t Ns) {
+    return precision == NK_MIXED || 0.5 * (double)Ns * (double)Ns * (double)M >= 1e7;
+}
+
 inline bool f64_on_tensor(int N, int M, int64_t B) {
     return (double)N * (double)M * (double)B >= 4e6 && B <= (1 << 20);
 }
