@@ -89,6 +89,29 @@ __global__ void k_spectral_filter(int64_t n, const double *__restrict__ w, const
     if (keep && kept) atomicAdd(kept, 1);
 }
 
+// out[0] = trace of S [n][n] (one block, fixed order).
+__global__ void __launch_bounds__(1024) k_trace(int64_t n, const double *__restrict__ S, double *__restrict__ out) {
+    __shared__ double red[32];
+    double v = 0.0;
+    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) v += S[(size_t)i * n + i];
+    v = warp_sum(v);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        v = warp_sum(red[threadIdx.x]);
+        if (threadIdx.x == 0) *out = v;
+    }
+}
+
+// Lower triangle of out = S - (coef trace) I.
+__global__ void k_shifted_copy(int64_t n, const double *__restrict__ S, double coef, const double *__restrict__ trace,
+                               double *__restrict__ out) {
+    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, i = blockIdx.y;
+    if (i >= n || j > i) return;
+    const double v = S[(size_t)i * n + j];
+    out[(size_t)i * n + j] = i == j ? v - coef * *trace : v;
+}
+
 namespace cg = cooperative_groups;
 
 // All sweeps in one cooperative launch (every CTA resident).  Per sweep the
@@ -255,6 +278,13 @@ cudaError_t launch_jacobi_coop(double *A, double *V, int64_t n, int max_sweeps, 
     e = cudaLaunchCooperativeKernel((const void *)k_jacobi_coop, dim3(G), dim3(256), args, 0, st);
     nk::note_launch();
     return e;
+}
+
+cudaError_t launch_shifted_copy(int64_t n, const double *S, double coef, double *trace, double *out, cudaStream_t st) {
+    if (n > 65535) return cudaErrorInvalidValue;
+    (k_trace<<<1, 1024, 0, st>>>(n, S, trace), nk::note_launch());
+    (k_shifted_copy<<<dim3(nblk(n, 256), (unsigned)n), 256, 0, st>>>(n, S, coef, trace, out), nk::note_launch());
+    return cudaGetLastError();
 }
 
 cudaError_t launch_symmetrize_lower(int64_t n, double *A, cudaStream_t st) {

@@ -317,6 +317,8 @@ cudaError_t launch_sub_colmean(int64_t rows, int64_t cols, const double *mean, d
 size_t eig_ws_bytes(int64_t n);
 cudaError_t launch_symmetrize_lower(int64_t n, double *A, cudaStream_t st);
 cudaError_t launch_identity(int64_t n, double *V, cudaStream_t st);
+// trace (device scratch) = tr S; lower triangle of out = S - (coef tr S) I.
+cudaError_t launch_shifted_copy(int64_t n, const double *S, double coef, double *trace, double *out, cudaStream_t st);
 // All sweeps in one cooperative launch, until the relative off-diagonal
 // norm is <= tol or max_sweeps; out2 = (sweeps taken, final norm).
 cudaError_t launch_jacobi_coop(double *A, double *V, int64_t n, int max_sweeps, double tol, void *ws, double *out2,
