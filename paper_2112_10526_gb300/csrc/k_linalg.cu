@@ -6,6 +6,7 @@
 // order, tree reductions with a fixed shape), so results are bitwise
 // reproducible from run to run.
 
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include "nk_common.cuh"
@@ -125,6 +126,22 @@ struct EpPartial {
     }
 };
 
+// sum of n values `stride` apart: eight loads and four chains in flight (the
+// sum waits on memory and on dependent FP64 adds).
+__device__ __forceinline__ double sum_strided(const double *__restrict__ p, int64_t stride, int n) {
+    double q[4] = {0.0, 0.0, 0.0, 0.0};
+    int b = 0;
+    for (; b + 7 < n; b += 8) {
+        double v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = p[(size_t)(b + u) * stride];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) q[u] += v[u] + v[u + 4];
+    }
+    for (; b < n; ++b) q[b & 3] += p[(size_t)b * stride];
+    return (q[0] + q[1]) + (q[2] + q[3]);
+}
+
 __global__ void k_vjp_reduce(int N, int M, int splits, const double *__restrict__ P,
                              double *__restrict__ out) {
     const int64_t plane = (int64_t)(M + 1) * (N + 1);
@@ -132,14 +149,7 @@ __global__ void k_vjp_reduce(int N, int M, int splits, const double *__restrict_
     if (idx >= plane) return;
     const int j = (int)(idx / (N + 1)), i = (int)(idx % (N + 1));
     if (j == M && i == N) return;
-    // four chains over the splits, so that their loads and adds overlap
-    double q[4] = {0.0, 0.0, 0.0, 0.0};
-    int sp = 0;
-    for (; sp + 3 < splits; sp += 4)
-#pragma unroll
-        for (int u = 0; u < 4; ++u) q[u] += P[(size_t)(sp + u) * plane + idx];
-    for (; sp < splits; ++sp) q[0] += P[(size_t)sp * plane + idx];
-    const double s = (q[0] + q[1]) + (q[2] + q[3]);
+    const double s = sum_strided(P + idx, plane, splits);
     if (j == M)
         out[i] = s;
     else if (i == N)
@@ -149,13 +159,14 @@ __global__ void k_vjp_reduce(int N, int M, int splits, const double *__restrict_
 }
 
 // Splits of the K = Ns range: about four blocks per SM (the FP64 pipe is full
-// with two), at least 8 samples each and at most 128 partial planes.
+// with two), at least 8 samples each and at most 32 partial planes (their sum
+// waits on memory: 19 us for 128 planes).
 int vjp_splits(int N, int M, int64_t Ns) {
     const int64_t tiles = (int64_t)((M + 1 + kGT - 1) / kGT) * ((N + 1 + kGT - 1) / kGT);
     int64_t sp = (608 + tiles - 1) / tiles;
     const int64_t maxsp = (Ns + 7) / 8;
     if (sp > maxsp) sp = maxsp;
-    if (sp > 128) sp = 128;
+    if (sp > 32) sp = 32;
     if (sp < 1) sp = 1;
     return (int)sp;
 }
@@ -243,27 +254,40 @@ __global__ void k_gemv_rows(const double *__restrict__ A, int64_t rows, int64_t 
     if (lane == 0) y[r] = acc;
 }
 
-constexpr int kGemvTRows = 256;
+// Rows per partial sum: about four blocks of 256 columns per SM, at most 32
+// partials (or 256 rows each), at least 16 rows.
+int64_t gemv_t_rows(int64_t rows, int64_t cols) {
+    const int64_t bc = (cols + 255) / 256;
+    int64_t parts = 608 / (bc > 0 ? bc : 1);
+    if (parts > 32) parts = 32;
+    if (parts < (rows + 255) / 256) parts = (rows + 255) / 256;
+    const int64_t r = (rows + parts - 1) / parts;
+    return r < 16 ? 16 : r;
+}
 
-// partial[b][c] = sum over rows of chunk b of A[r][c] x[r]
-__global__ void k_gemv_t_partial(const double *__restrict__ A, int64_t rows, int64_t cols,
+// partial[b][c] = sum over rows of chunk b (nr rows) of A[r][c] x[r]
+__global__ void k_gemv_t_partial(const double *__restrict__ A, int64_t rows, int64_t cols, int64_t nr,
                                  const double *__restrict__ x, double *__restrict__ partial) {
     const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t r0 = (int64_t)blockIdx.y * kGemvTRows;
+    const int64_t r0 = (int64_t)blockIdx.y * nr;
     if (c >= cols) return;
-    const int64_t r1 = r0 + kGemvTRows < rows ? r0 + kGemvTRows : rows;
-    double acc = 0.0;
-    for (int64_t r = r0; r < r1; ++r) acc += A[(size_t)r * cols + c] * x[r];
-    partial[(size_t)blockIdx.y * cols + c] = acc;
+    const int64_t r1 = r0 + nr < rows ? r0 + nr : rows;
+    double p = 0.0, q = 0.0;
+    int64_t r = r0;
+#pragma unroll 4
+    for (; r + 1 < r1; r += 2) {
+        p = fma(A[(size_t)r * cols + c], x[r], p);
+        q = fma(A[(size_t)(r + 1) * cols + c], x[r + 1], q);
+    }
+    if (r < r1) p = fma(A[(size_t)r * cols + c], x[r], p);
+    partial[(size_t)blockIdx.y * cols + c] = p + q;
 }
 
 __global__ void k_sum_partials(int64_t cols, int nparts, const double *__restrict__ partial,
                                double scale, double *__restrict__ y) {
     const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= cols) return;
-    double acc = 0.0;
-    for (int b = 0; b < nparts; ++b) acc += partial[(size_t)b * cols + c];
-    y[c] = scale * acc;
+    y[c] = scale * sum_strided(partial + c, cols, nparts);
 }
 
 // ----------------------------------------------------------- SYRK (J^T J) --
@@ -410,28 +434,6 @@ __global__ void k_center_rows(int64_t n, const double *__restrict__ r, double in
 
 // ------------------------------------------------------------ statistics ---
 
-// Block-wide compensated sum (Neumaier per thread, TwoSum tree); every
-// thread returns the total.
-__device__ double block_comp_sum(double s, double c) {
-    __shared__ double ss[1024], cc[1024];
-    const int t = threadIdx.x;
-    ss[t] = s;
-    cc[t] = c;
-    __syncthreads();
-    for (int w = blockDim.x >> 1; w > 0; w >>= 1) {
-        if (t < w) {
-            double r, e;
-            two_sum(ss[t], ss[t + w], r, e);
-            ss[t] = r;
-            cc[t] = cc[t] + cc[t + w] + e;
-        }
-        __syncthreads();
-    }
-    const double out = ss[0] + cc[0];
-    __syncthreads();
-    return out;
-}
-
 __device__ __forceinline__ void neumaier_add(double &s, double &c, double x) {
     double r, e;
     two_sum(s, x, r, e);
@@ -439,44 +441,116 @@ __device__ __forceinline__ void neumaier_add(double &s, double &c, double x) {
     c += e;
 }
 
-__global__ void __launch_bounds__(1024) k_stats(const double *__restrict__ e, int64_t Ns,
-                                                int n_chains, double *__restrict__ out) {
-    double s = 0.0, c = 0.0;
-    for (int64_t k = threadIdx.x; k < Ns; k += blockDim.x) neumaier_add(s, c, e[k]);
-    const double mean = block_comp_sum(s, c) / (double)Ns;
-    s = 0.0;
-    c = 0.0;
-    for (int64_t k = threadIdx.x; k < Ns; k += blockDim.x) {
+__device__ __forceinline__ void comp_merge(double &s, double &c, double s2, double c2) {
+    double r, e;
+    two_sum(s, s2, r, e);
+    s = r;
+    c = c + c2 + e;
+}
+
+// The statistics run on one cluster of eight blocks: the compensated sums cost
+// 7 FP64 operations a sample and one SM retires 2 lanes a clock (91 us for
+// 16384 samples, 650 us for 65536 on a single block of 1024 threads).  Their
+// partial sums meet in distributed shared memory.  256 threads a block: with
+// 1024 the sum over a block (8 FP64 operations a level, quantity and warp) took
+// longer than the samples.
+constexpr int kStatCtas = 8, kStatThreads = 256;
+
+// Compensated sums of nq quantities over all threads of the cluster, in a
+// fixed order (lanes, warps, blocks); every thread returns the totals in s.
+template <int nq>
+__device__ void cluster_comp_sum(double (&s)[nq], double (&c)[nq]) {
+    constexpr int kWarps = kStatThreads / 32;
+    static_assert(kWarps == 8 && kStatCtas == 8, "the last sums run over 8 lanes");
+    __shared__ double2 part[nq][kWarps];
+    __shared__ double2 tot[nq];
+    __shared__ double all[nq];
+    cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int q = 0; q < nq; ++q)
+            comp_merge(s[q], c[q], __shfl_down_sync(0xffffffffu, s[q], o), __shfl_down_sync(0xffffffffu, c[q], o));
+    if (lane == 0)
+#pragma unroll
+        for (int q = 0; q < nq; ++q) part[q][warp] = make_double2(s[q], c[q]);
+    __syncthreads();
+    // warp q sums quantity q over the block's warps, then over the blocks
+    if (warp < nq) {
+        double2 v = part[warp][lane & 7];
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1)
+            comp_merge(v.x, v.y, __shfl_down_sync(0xffffffffu, v.x, o), __shfl_down_sync(0xffffffffu, v.y, o));
+        if (lane == 0) tot[warp] = v;
+    }
+    cl.sync();
+    if (warp < nq) {
+        double2 v = *cl.map_shared_rank(&tot[warp], lane & 7);
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1)
+            comp_merge(v.x, v.y, __shfl_down_sync(0xffffffffu, v.x, o), __shfl_down_sync(0xffffffffu, v.y, o));
+        if (lane == 0) all[warp] = v.x + v.y;
+    }
+    cl.sync();  // the totals are read before they are written again
+#pragma unroll
+    for (int q = 0; q < nq; ++q) s[q] = all[q];
+}
+
+__global__ void __cluster_dims__(kStatCtas, 1, 1) __launch_bounds__(kStatThreads)
+    k_stats(const double *__restrict__ e, int64_t Ns, int n_chains, double *__restrict__ out) {
+    const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+    double s1[1] = {0.0}, c1[1] = {0.0};
+    for (int64_t k = gid; k < Ns; k += step) neumaier_add(s1[0], c1[0], e[k]);
+    cluster_comp_sum(s1, c1);
+    const double mean = s1[0] / (double)Ns;
+    // sum (e - mean)^2, and over the chains the sums of (m - mean) and (m -
+    // mean)^2, m the chain's mean
+    double s[3] = {0.0, 0.0, 0.0}, c[3] = {0.0, 0.0, 0.0};
+    for (int64_t k = gid; k < Ns; k += step) {
         const double d = e[k] - mean;
-        neumaier_add(s, c, d * d);
+        neumaier_add(s[0], c[0], d * d);
     }
-    const double var = block_comp_sum(s, c) / (double)Ns;
-    double err;
     const int64_t per = n_chains > 0 ? Ns / n_chains : 0;
-    if (n_chains > 1 && per >= 2 && per * n_chains == Ns) {
-        // chain means, their mean and variance
-        s = 0.0;
-        c = 0.0;
-        for (int64_t ch = threadIdx.x; ch < n_chains; ch += blockDim.x) {
+    const bool chains = n_chains > 1 && per >= 2 && per * n_chains == Ns;
+    if (chains && per <= 32) {  // a thread per chain
+        for (int64_t ch = gid; ch < n_chains; ch += step) {
             double a = 0.0, ac = 0.0;
             for (int64_t q = 0; q < per; ++q) neumaier_add(a, ac, e[ch * per + q]);
-            neumaier_add(s, c, (a + ac) / (double)per);
+            const double d = (a + ac) / (double)per - mean;
+            neumaier_add(s[1], c[1], d);
+            neumaier_add(s[2], c[2], d * d);
         }
-        const double cm = block_comp_sum(s, c) / (double)n_chains;
-        s = 0.0;
-        c = 0.0;
-        for (int64_t ch = threadIdx.x; ch < n_chains; ch += blockDim.x) {
+    } else if (chains) {  // a warp per chain
+        const int lane = threadIdx.x & 31;
+        for (int64_t ch = gid >> 5; ch < n_chains; ch += step >> 5) {
             double a = 0.0, ac = 0.0;
-            for (int64_t q = 0; q < per; ++q) neumaier_add(a, ac, e[ch * per + q]);
-            const double d = (a + ac) / (double)per - cm;
-            neumaier_add(s, c, d * d);
+            for (int64_t q = lane; q < per; q += 32) neumaier_add(a, ac, e[ch * per + q]);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+                comp_merge(a, ac, __shfl_down_sync(0xffffffffu, a, o), __shfl_down_sync(0xffffffffu, ac, o));
+            if (lane == 0) {
+                const double d = (a + ac) / (double)per - mean;
+                neumaier_add(s[1], c[1], d);
+                neumaier_add(s[2], c[2], d * d);
+            }
         }
-        const double vcm = block_comp_sum(s, c) / (double)n_chains;
-        err = sqrt(vcm / (double)n_chains);
-    } else {
-        err = sqrt(var / (double)Ns);
     }
-    if (threadIdx.x == 0) {
+    if (chains) {
+        cluster_comp_sum(s, c);
+    } else {
+        double sv[1] = {s[0]}, cv[1] = {c[0]};
+        cluster_comp_sum(sv, cv);
+        s[0] = sv[0];
+    }
+    if (gid == 0) {
+        const double var = s[0] / (double)Ns;
+        double err = sqrt(var / (double)Ns);
+        if (chains) {
+            // variance of the chain means about their own mean
+            const double cm = s[1] / (double)n_chains, v = s[2] / (double)n_chains - cm * cm;
+            err = sqrt((v < 0.0 ? 0.0 : v) / (double)n_chains);
+        }
         out[0] = mean;
         out[1] = var;
         out[2] = err;
@@ -631,7 +705,7 @@ void launch_double_center(int64_t n, double *K, double *r, double eps, bool lowe
 // ============================================================ launchers ====
 
 cudaError_t launch_stats(const double *e, int64_t Ns, int n_chains, double *out, cudaStream_t st) {
-    (k_stats<<<1, 1024, 0, st>>>(e, Ns, n_chains, out), nk::note_launch());
+    (k_stats<<<kStatCtas, kStatThreads, 0, st>>>(e, Ns, n_chains, out), nk::note_launch());
     return cudaGetLastError();
 }
 
@@ -692,17 +766,17 @@ cudaError_t launch_gemv_rows(const double *A, int64_t rows, int64_t cols, const 
 }
 
 size_t gemv_t_partial_doubles(int64_t rows, int64_t cols) {
-    return (size_t)((rows + kGemvTRows - 1) / kGemvTRows) * (size_t)cols;
+    const int64_t nr = gemv_t_rows(rows, cols);
+    return (size_t)((rows + nr - 1) / nr) * (size_t)cols;
 }
 
 cudaError_t launch_gemv_t(const double *A, int64_t rows, int64_t cols, const double *x,
                           double scale, double *partial, double *y, cudaStream_t st) {
-    const int64_t nb = (rows + kGemvTRows - 1) / kGemvTRows;
+    const int64_t nr = gemv_t_rows(rows, cols), nb = (rows + nr - 1) / nr;
     for (int64_t b0 = 0; b0 < nb; b0 += 65535) {
         const int64_t bb = nb - b0 < 65535 ? nb - b0 : 65535;
         dim3 grid(nblk(cols, 256), (unsigned)bb);
-        (k_gemv_t_partial<<<grid, 256, 0, st>>>(A + (size_t)b0 * kGemvTRows * cols,
-                                               rows - b0 * kGemvTRows, cols, x + b0 * kGemvTRows,
+        (k_gemv_t_partial<<<grid, 256, 0, st>>>(A + (size_t)b0 * nr * cols, rows - b0 * nr, cols, nr, x + b0 * nr,
                                                partial + (size_t)b0 * cols), nk::note_launch());
     }
     (k_sum_partials<<<nblk(cols, 256), 256, 0, st>>>(cols, (int)nb, partial, scale, y), nk::note_launch());

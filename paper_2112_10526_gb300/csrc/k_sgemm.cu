@@ -751,16 +751,23 @@ __device__ __forceinline__ int exp_of(double x) {
     return b == 2047 ? 100000 : (m ? b - 1022 : -100000);
 }
 
+// m 2^sh, sh > -64: truncated, or with `round` to nearest (only values below
+// 2^(e - 3) are shifted right, so rounding up does not reach 2^e).
+__device__ __forceinline__ unsigned long long grid_bits(unsigned long long m, int sh, bool round) {
+    if (sh >= 0) return m << sh;
+    if (sh <= -64) return 0ULL;
+    return (m >> (-sh)) + (round ? (m >> (-sh - 1)) & 1ULL : 0ULL);
+}
+
 // Slice one value with row exponent e into SB bytes (sign applied).
-__device__ __forceinline__ void slice_value(double x, int e, int SB, __nv_bfloat16 *out, int64_t plane) {
+__device__ __forceinline__ void slice_value(double x, int e, int SB, __nv_bfloat16 *out, int64_t plane, bool round) {
     int b;
     unsigned long long m;
     bool neg;
     split_bits(x, b, m, neg);
     unsigned long long y = 0;
     if (m) {
-        const int sh = b - 1075 + 8 * SB - e;
-        y = sh >= 0 ? (m << sh) : (sh <= -64 ? 0ULL : m >> (-sh));
+        y = grid_bits(m, b - 1075 + 8 * SB - e, round);
     }
     for (int t = 0; t < SB; ++t) {
         const int d = (int)((y >> (8 * (SB - 1 - t))) & 0xFFULL);
@@ -771,7 +778,7 @@ __device__ __forceinline__ void slice_value(double x, int e, int SB, __nv_bfloat
 // slice_value for two neighbouring values of one row, written as BF16 pairs
 // (4-byte stores, so that a warp writes whole 128-byte lines per plane).
 __device__ __forceinline__ void slice_pair(double x0, double x1, int e, int SB, __nv_bfloat162 *out,
-                                           int64_t plane2) {
+                                           int64_t plane2, bool round) {
     unsigned long long y[2] = {0ULL, 0ULL};
     bool neg[2];
     const double x[2] = {x0, x1};
@@ -781,8 +788,7 @@ __device__ __forceinline__ void slice_pair(double x0, double x1, int e, int SB, 
         unsigned long long m;
         split_bits(x[h], b, m, neg[h]);
         if (m) {
-            const int sh = b - 1075 + 8 * SB - e;
-            y[h] = sh >= 0 ? (m << sh) : (sh <= -64 ? 0ULL : m >> (-sh));
+            y[h] = grid_bits(m, b - 1075 + 8 * SB - e, round);
         }
     }
     for (int t = 0; t < SB; ++t) {
@@ -840,7 +846,7 @@ __global__ void k_slice_rows_h3(const double *__restrict__ X, int64_t ldx, int64
 // SB slices [SB][rows][ld] with one exponent per row.  One block per row.
 __global__ void k_slice_long_rows(const double *__restrict__ X, int64_t ldx, int64_t rows, int64_t K,
                                   const double *__restrict__ aug, int SB, int64_t ld,
-                                  __nv_bfloat16 *__restrict__ out, int *__restrict__ expo) {
+                                  __nv_bfloat16 *__restrict__ out, int *__restrict__ expo, bool round) {
     const int64_t r = blockIdx.x;
     if (r >= rows) return;
     const int64_t Ke = aug ? K + 1 : K;
@@ -863,7 +869,7 @@ __global__ void k_slice_long_rows(const double *__restrict__ X, int64_t ldx, int
     const int64_t plane = rows * ld;
     for (int64_t k = threadIdx.x; k < ld; k += blockDim.x) {
         const double x = k < Ke ? val(k) : 0.0;
-        slice_value(x, e, SB, out + (size_t)r * ld + k, plane);
+        slice_value(x, e, SB, out + (size_t)r * ld + k, plane, round);
     }
     if (threadIdx.x == 0) expo[r] = e;
 }
@@ -875,7 +881,7 @@ __global__ void k_fill_int(int64_t n, int v, int *__restrict__ x) {
 
 // Exponent of every row j <= M of (T' o g)^T: max over samples k of
 // |t'_kj g'_k|, t'_kM = 1, g'_k = scale (g_k - shift).  Blocks of 32 rows x
-// 256 samples, combined with atomicMax (-100000 marks an all-zero row).
+// kColexpRows samples, combined with atomicMax (-100000 marks an all-zero row).
 // g'_k = scale (g_k - shift) and its exponent (|g'_k| < 2^ge_k).
 __global__ void k_scale_g(int64_t Ns, const double *__restrict__ g, double scale, const double *__restrict__ shift,
                           double *__restrict__ gp, int *__restrict__ ge) {
@@ -889,17 +895,25 @@ __global__ void k_scale_g(int64_t Ns, const double *__restrict__ g, double scale
 // Column exponents of T' o g' (column j of (T' o g')^T): an upper bound
 // max_k (exp(T'_kj) + exp(g'_k)) of the exact exponent, at most one above it,
 // taken with integer operations only.
-__global__ void k_tg_colexp(const double *__restrict__ T, const int *__restrict__ ge, int64_t Ns, int M,
-                            int *__restrict__ expo) {
-    const int j = blockIdx.x * 32 + threadIdx.x;
-    const int64_t k0 = (int64_t)blockIdx.y * 256;
+constexpr int kColexpRows = 64;  // 8 rows a thread, all in flight
+__global__ void __launch_bounds__(256) k_tg_colexp(const double *__restrict__ T, const int *__restrict__ ge, int64_t Ns,
+                                                   int M, int *__restrict__ expo) {
+    const int j = blockIdx.y * 32 + threadIdx.x;
+    const int64_t k0 = (int64_t)blockIdx.x * kColexpRows + threadIdx.y;
     int ex = -100000;
     if (j <= M) {
-        const int64_t kend = k0 + 256 < Ns ? k0 + 256 : Ns;
-#pragma unroll 4
-        for (int64_t k = k0 + threadIdx.y; k < kend; k += blockDim.y) {  // loads of 4 rows in flight
-            const int et = j < M ? exp_of(T[(size_t)k * M + j]) : 1, eg = ge[k];
-            if (et != -100000 && eg != -100000) ex = max(ex, et + eg);
+        double v[8];
+        int eg[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int64_t k = k0 + 8 * u;
+            v[u] = k < Ns && j < M ? __ldg(T + (size_t)k * M + j) : 0.5;
+            eg[u] = k < Ns ? __ldg(ge + k) : -100000;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int et = j < M ? exp_of(v[u]) : 1;
+            if (et != -100000 && eg[u] != -100000) ex = max(ex, et + eg[u]);
         }
     }
     __shared__ int red[8][32];
@@ -946,7 +960,7 @@ __global__ void k_colexp_bound(int M, const int *__restrict__ colexpT, const int
 constexpr int kTgPitch = 65;
 __global__ void __launch_bounds__(256) k_tg_slice(const double *__restrict__ T, const double *__restrict__ gp,
                                                   int64_t Ns, int M, int SB, int64_t ld, int vec,
-                                                  const int *__restrict__ expo, __nv_bfloat16 *__restrict__ out) {
+                                                  const int *__restrict__ expo, __nv_bfloat16 *__restrict__ out, bool round) {
     __shared__ double tile[64 * kTgPitch];  // [k][j]
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t k0 = (int64_t)blockIdx.x * 64;
@@ -984,7 +998,7 @@ __global__ void __launch_bounds__(256) k_tg_slice(const double *__restrict__ T, 
         if (SB == 4)
             slice_pair4(x0, x1, e, reinterpret_cast<uint32_t *>(out + (size_t)jj * ld + k), plane2);
         else
-            slice_pair(x0, x1, e, SB, reinterpret_cast<__nv_bfloat162 *>(out + (size_t)jj * ld + k), plane2);
+            slice_pair(x0, x1, e, SB, reinterpret_cast<__nv_bfloat162 *>(out + (size_t)jj * ld + k), plane2, round);
     }
 }
 
@@ -1375,7 +1389,7 @@ cudaError_t launch_theta_tc(int N, int M, const double *b, const double *W, cons
     auto *Ws = reinterpret_cast<__nv_bfloat16 *>(take((size_t)kMaxSB * M * ld * 2));
     auto *ew = reinterpret_cast<int *>(take((size_t)M * 4));
     (k_pm1_rows<<<nblk(B * ld, 256), 256, 0, st>>>(s, B, N, 0, ld, As), nk::note_launch());
-    (k_slice_long_rows<<<M, 128, 0, st>>>(W, N, M, N, nullptr, kMaxSB, ld, Ws, ew), nk::note_launch());
+    (k_slice_long_rows<<<M, 128, 0, st>>>(W, N, M, N, nullptr, kMaxSB, ld, Ws, ew, wide), nk::note_launch());
     const int slot = prof_begin(NK_PROF_JVP_VJP, st);
     cudaError_t e = sgemm(As, B, ld, Ws, ew, M, ld, N, kMaxSB, theta, ldtheta > 0 ? ldtheta : M, 0, b, err, st,
                           SgRaw{s, W, nullptr, N, N, 0}, wide);
@@ -1454,7 +1468,7 @@ cudaError_t launch_jvp_tc(int N, int M, int64_t Ns, const int8_t *s, const doubl
         (k_slice_rows_h3<<<M + 1, 128, 0, st>>>(Vp, N + 1, M + 1, N + 1, ld, reinterpret_cast<uint32_t *>(Vs), ev),
          nk::note_launch());
     else
-        (k_slice_long_rows<<<M + 1, 128, 0, st>>>(Vp, N + 1, M + 1, N + 1, nullptr, SB, ld, Vs, ev),
+        (k_slice_long_rows<<<M + 1, 128, 0, st>>>(Vp, N + 1, M + 1, N + 1, nullptr, SB, ld, Vs, ev, wide),
          nk::note_launch());
     if (persistent && Thl == nullptr) {
         void *own = take(tc_split_t_bytes(M, Ns));
@@ -1484,7 +1498,8 @@ constexpr int kMaxKSplit = 16;
 // of at least 4 K-chunks each.
 // At least as many as keep a split within 65536 samples (exact FP32 levels).
 static int pick_ksplit(int64_t tiles, int64_t kchunks, int64_t slots) {
-    const int least = (int)((kchunks + 1023) / 1024);
+    const int64_t want = (kchunks + 1023) / 1024;
+    const int least = want < kMaxKSplit ? (int)want : kMaxKSplit;
     int best = least;
     double best_score = -1.0;
     for (int ks = least; ks <= kMaxKSplit; ++ks) {
@@ -1516,7 +1531,7 @@ cudaError_t launch_colexp_t(int M, int64_t Ns, const double *T, int *colexpT, vo
     int *zero = static_cast<int *>(ws);
     (k_fill_int<<<nblk(Ns, 256), 256, 0, st>>>(Ns, 0, zero), nk::note_launch());
     (k_fill_int<<<nblk(M + 1, 256), 256, 0, st>>>(M + 1, -100000, colexpT), nk::note_launch());
-    (k_tg_colexp<<<dim3(nblk(M + 1, 32), nblk(Ns, 256)), dim3(32, 8), 0, st>>>(T, zero, Ns, M, colexpT),
+    (k_tg_colexp<<<dim3(nblk(Ns, kColexpRows), nblk(M + 1, 32)), dim3(32, 8), 0, st>>>(T, zero, Ns, M, colexpT),
      nk::note_launch());
     return cudaGetLastError();
 }
@@ -1580,10 +1595,10 @@ cudaError_t launch_vjp_tc(int N, int M, int64_t Ns, const int8_t *s, const doubl
          nk::note_launch());
     } else {
         (k_fill_int<<<nblk(M + 1, 256), 256, 0, st>>>(M + 1, -100000, eg), nk::note_launch());
-        (k_tg_colexp<<<dim3(nblk(M + 1, 32), nblk(Ns, 256)), dim3(32, 8), 0, st>>>(T, ge, Ns, M, eg),
+        (k_tg_colexp<<<dim3(nblk(Ns, kColexpRows), nblk(M + 1, 32)), dim3(32, 8), 0, st>>>(T, ge, Ns, M, eg),
          nk::note_launch());
         const int vec = (M % 2 == 0) && ((reinterpret_cast<uintptr_t>(T) & 15) == 0);
-        (k_tg_slice<<<dim3(nblk(ld, 64), nblk(M + 1, 64)), 256, 0, st>>>(T, gp, Ns, M, SB, ld, vec, eg, Gs),
+        (k_tg_slice<<<dim3(nblk(ld, 64), nblk(M + 1, 64)), 256, 0, st>>>(T, gp, Ns, M, SB, ld, vec, eg, Gs, wide),
          nk::note_launch());
     }
     // split the long K = Ns range so that the last wave of CTAs is nearly
