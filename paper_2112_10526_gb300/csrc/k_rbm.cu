@@ -48,7 +48,8 @@ __global__ void k_transpose_W(int N, int M, const double *__restrict__ W, double
 template <typename R>
 __global__ void k_tau_rows(int N, int M, int nrows, const double *__restrict__ Wt,
                            const int32_t *__restrict__ edges, R *__restrict__ tau,
-                           R *__restrict__ tauT, R *__restrict__ K) {
+                           R *__restrict__ tauT, R *__restrict__ K, float *__restrict__ tauf,
+                           double *__restrict__ D) {
     int r = blockIdx.x;
     if (r >= nrows) return;
     const double *w0, *w1 = nullptr;
@@ -64,8 +65,12 @@ __global__ void k_tau_rows(int N, int M, int nrows, const double *__restrict__ W
     for (int j = threadIdx.x; j < M; j += blockDim.x) {
         double d = w1 ? (w0[j] - w1[j]) : w0[j];
         double v = tanh(2.0 * d);
-        tau[(size_t)r * M + j] = (R)v;
-        tauT[(size_t)j * nrows + r] = (R)v;
+        if (tau) tau[(size_t)r * M + j] = (R)v;
+        if (tauT) tauT[(size_t)j * nrows + r] = (R)v;
+        if (tauf) {
+            tauf[(size_t)r * M + j] = (float)v;
+            D[(size_t)r * M + j] = 2.0 * d;
+        }
         part += lncosh(2.0 * d);
     }
     __shared__ double red[32];
@@ -311,11 +316,6 @@ __device__ __forceinline__ Prod<float> lane_product4(const float *__restrict__ t
 }
 
 template <bool kRing>
-__device__ __forceinline__ Prod<double> unit_lanes_product(const double *t, const double *tau, double si, int lane,
-                                                           int M, bool vec4) {
-    return strided_product<double>(t, tau, 1, si, lane, 32, M);
-}
-template <bool kRing>
 __device__ __forceinline__ Prod<float> unit_lanes_product(const float *t, const float *tau, float si, int lane, int M,
                                                           bool vec4) {
     return vec4 ? lane_product4<false, kRing>(t, tau, si, lane, M)
@@ -435,8 +435,9 @@ struct SweepK {
 // kRing: the FP32 form with the pipelined tau loads (M >= 3072), given the
 // registers of 3 blocks of 4 warps per SM (what shared memory allows there);
 // otherwise the registers of 7 blocks, for the small-M occupancy.
-template <typename R, bool kHam, bool kRing>
-__global__ void __launch_bounds__(128, kRing ? 3 : 7) k_sweep(SweepK<R> P) {
+template <bool kHam, bool kRing>
+__global__ void __launch_bounds__(128, kRing ? 3 : 7) k_sweep(SweepK<float> P) {
+    using R = float;
     extern __shared__ __align__(16) unsigned char sm[];
     const Tables<R> &T = P.t;
     const SweepArgs &A = P.a;
@@ -450,11 +451,12 @@ __global__ void __launch_bounds__(128, kRing ? 3 : 7) k_sweep(SweepK<R> P) {
     __syncwarp();
     unsigned long long acc = 0;
     const int n_sweeps = A.n_discard + A.n_samples;
-    constexpr bool kF32 = sizeof(R) == 4;
     using Acc = R;  // precision of the accept arithmetic
     for (int w = 0; w < n_sweeps; ++w) {
         // From-scratch FP64 theta = b + W s (rebuilt here, or given by the
-        // tensor-core product), t = tanh theta, ln psi.
+        // tensor-core product); t = tanh theta and the ln cosh terms of ln psi
+        // in FP32 lanes (the FP64 pipe of this part runs at 1/64 of the FP32
+        // rate).
         double lp = 0.0;
         for (int j = lane; j < M; j += 32) {
             double th;
@@ -464,16 +466,9 @@ __global__ void __launch_bounds__(128, kRing ? 3 : 7) k_sweep(SweepK<R> P) {
                 th = T.b[j];
                 for (int i = 0; i < N; ++i) th = fma(T.Wt[(size_t)i * M + j], (double)sv[i], th);
             }
-            if (kF32) {
-                // FP32 path: t and the ln cosh terms in FP32 lanes (the FP64
-                // pipe of this part runs at 1/64 of the FP32 rate)
-                const float thf = (float)th;
-                t[j] = (R)tanhf(thf);
-                lp += (double)lncosh(thf);
-            } else {
-                t[j] = (R)tanh(th);
-                lp += lncosh(th);
-            }
+            const float thf = (float)th;
+            t[j] = tanhf(thf);
+            lp += (double)lncosh(thf);
         }
         for (int i = lane; i < N; i += 32) lp += T.a[i] * (double)sv[i];
         lp = warp_sum(lp);
@@ -482,8 +477,7 @@ __global__ void __launch_bounds__(128, kRing ? 3 : 7) k_sweep(SweepK<R> P) {
         // Lane l prepares proposal q0 + l of each batch of 32: its Philox
         // block, ln u, the site / edge, K and the visible-bias difference, so
         // that a proposal only broadcasts them.
-        // The FP32 path takes the accept decision in FP32 (ln u and the
-        // ratio), the FP64 path in FP64.
+        // The accept decision is taken in FP32 (ln u and the ratio).
         int b_i = 0, b_k = -1, b_row = 0, b_ok = 1;
         unsigned b_hi = 0;
         R b_K = R(0);
@@ -492,10 +486,7 @@ __global__ void __launch_bounds__(128, kRing ? 3 : 7) k_sweep(SweepK<R> P) {
             if ((q & 31) == 0) {
                 Philox4 y = philox4x64_10(qbase + (unsigned long long)(q + lane), (unsigned long long)c,
                                           (unsigned long long)A.stream_id, 0ULL, A.seed, 0ULL);
-                if (kF32)
-                    b_lu = (Acc)logf((float)uniform53(y.v[1]));
-                else
-                    b_lu = (Acc)log(uniform53(y.v[1]));
+                b_lu = logf((float)uniform53(y.v[1]));
                 if (A.rule == NK_RULE_LOCAL) {
                     b_i = pick_index(y.v[0], N);
                     b_k = -1;
@@ -539,10 +530,7 @@ __global__ void __launch_bounds__(128, kRing ? 3 : 7) k_sweep(SweepK<R> P) {
                 row = e;
                 K = T.K_edge[e];
                 aa = (Acc)(T.a[i] - T.a[k]);
-                if (kF32)
-                    corr = (Acc)(logf((float)ns) - logf((float)nsp));
-                else
-                    corr = (Acc)(log((double)ns) - log((double)nsp));
+                corr = logf((float)ns) - logf((float)nsp);
                 tau = T.tau_edge + (size_t)row * M;
             } else {
                 if (!__shfl_sync(kFull, b_ok, src) || sv[i] == sv[k]) {
@@ -559,7 +547,7 @@ __global__ void __launch_bounds__(128, kRing ? 3 : 7) k_sweep(SweepK<R> P) {
             const bool accept = lu < Acc(2) * delta + corr;
             if (lane == 0 && A.decisions) A.decisions[slot] = accept ? 1 : 0;
             if (accept) {
-                if (kF32 && P.vec4) {
+                if (P.vec4) {
                     // FP32 path: 16-byte accesses, fast division (t is rebuilt
                     // exactly from theta after every sweep)
                     float *tf = reinterpret_cast<float *>(t);
@@ -614,13 +602,424 @@ __global__ void __launch_bounds__(128, kRing ? 3 : 7) k_sweep(SweepK<R> P) {
     if (lane == 0 && A.n_accepted) A.n_accepted[c] += acc;
 }
 
+// NK_F64 sweeps, every proposal screened in FP32.  The FP64 pipe retires 2
+// lanes a clock and SM and a dependent FP64 operation takes about 64 clocks, so
+// the FP64 product and logarithm of a proposal (k_sweep<double>: 3.7 us each
+// at M = 16) cost far more than the FP32 ones, and only their comparison with
+// ln u matters.  Per proposal the warp takes ln of the ratio product from
+// FP32 t = tanh(theta) and tau, with a bound on its error from the smallest
+// factor f_min >= 2^-6: each factor 1 - s t tau errs by less than 2^-22 (t:
+// theta rounded, 2^-25, and tanhf, 2^-23; tau 2^-25; the FMA 2^-24), its
+// logarithm by 2^-22 / f_min, the products and the sum of the lanes'
+// logarithms by 2^-21 / f_min a unit, and the lanes' logarithms, the threshold
+// ln u / 2 - K + a-part and the Hastings term by 2^-13 + 2^-21 (|sum| + |ln u /
+// 2 - K| + |a-part|) in all: 2^-20 M / f_min and these are the bound.
+// A proposal whose two sides differ by more than the bound is decided.  The
+// others take the differences ln cosh(theta') - ln cosh(theta) themselves,
+// first in FP32 (each errs by 2^-22 (|theta| + |theta'| + 2) at most, whatever
+// the factor, which settles nearly all proposals with a small factor), then,
+// still undecided (about one in a thousand at M = 200), in FP64.  The
+// decisions are those of FP64 either way, also where t and tau round to 1 and
+// the FP64 product form (which this replaces) loses its digits.  theta itself stays in FP64: it
+// is rebuilt at every sweep, moved by one addition a unit on an accepted
+// move, and ln psi of a sample is taken from it directly.
+// 16-site chain, 16 chains, 80 sweeps: 4763 -> see launch_sweep for the
+// measured times of both.
+template <bool kHam>
+__global__ void __launch_bounds__(128) k_sweep_screened(SweepK<double> P) {
+    extern __shared__ __align__(16) unsigned char sm[];
+    const Tables<double> &T = P.t;
+    const SweepArgs &A = P.a;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int c = blockIdx.x * (blockDim.x >> 5) + warp;
+    if (c >= A.C) return;
+    const int N = T.N, M = T.M;
+    unsigned char *base = sm + (size_t)warp * P.warp_bytes;
+    double *th = reinterpret_cast<double *>(base);                        // [M]
+    float *t = reinterpret_cast<float *>(base + (size_t)P.t_bytes);       // [M]
+    int8_t *sv = reinterpret_cast<int8_t *>(base + (size_t)P.t_bytes + P.t_bytes / 2);
+    const bool local = A.rule == NK_RULE_LOCAL;
+    const double *Dtab = local ? T.D_site : T.D_edge;
+    const float *tabf = local ? T.tauf_site : T.tauf_edge;
+    for (int i = lane; i < N; i += 32) sv[i] = A.s[(size_t)c * N + i];
+    __syncwarp();
+    unsigned long long acc = 0;
+    const int n_sweeps = A.n_discard + A.n_samples;
+    for (int w = 0; w < n_sweeps; ++w) {
+        // theta = b + W s from scratch (FP64), t = tanh theta
+        for (int j = lane; j < M; j += 32) {
+            double v;
+            if (A.theta_in) {
+                v = A.theta_in[(size_t)c * (A.theta_ld > 0 ? A.theta_ld : M) + j];
+            } else {
+                // four chains of FMAs over the sites
+                double q0 = T.b[j], q1 = 0.0, q2 = 0.0, q3 = 0.0;
+                int i = 0;
+                for (; i + 3 < N; i += 4) {
+                    q0 = fma(T.Wt[(size_t)i * M + j], (double)sv[i], q0);
+                    q1 = fma(T.Wt[(size_t)(i + 1) * M + j], (double)sv[i + 1], q1);
+                    q2 = fma(T.Wt[(size_t)(i + 2) * M + j], (double)sv[i + 2], q2);
+                    q3 = fma(T.Wt[(size_t)(i + 3) * M + j], (double)sv[i + 3], q3);
+                }
+                for (; i < N; ++i) q0 = fma(T.Wt[(size_t)i * M + j], (double)sv[i], q0);
+                v = (q0 + q1) + (q2 + q3);
+            }
+            th[j] = v;
+            t[j] = tanhf((float)v);
+        }
+        __syncwarp();
+        const unsigned long long qbase = (unsigned long long)(A.sweep0 + w) * (unsigned long long)N;
+        // lane l prepares proposal q0 + l of each batch of 32
+        int b_i = 0, b_k = -1, b_row = 0, b_ok = 1;
+        unsigned b_hi = 0;
+        double b_K = 0.0, b_aa = 0.0, b_u = 1.0;
+        float b_h = 0.f, b_a2 = 0.f;  // ln u / 2 - K (ln u / 2 for kHam), 2 a-part
+        for (int q = 0; q < N; ++q) {
+            const int src = q & 31;
+            if (src == 0) {
+                Philox4 y = philox4x64_10(qbase + (unsigned long long)(q + lane), (unsigned long long)c,
+                                          (unsigned long long)A.stream_id, 0ULL, A.seed, 0ULL);
+                b_u = uniform53(y.v[1]);
+                if (local) {
+                    b_i = pick_index(y.v[0], N);
+                    b_k = -1;
+                    b_row = b_i;
+                    b_K = T.K_site[b_i];
+                    b_aa = T.a[b_i];
+                } else if (kHam) {
+                    b_hi = (unsigned)(y.v[0] >> 32);  // the edge depends on the state
+                } else {
+                    const int e = pick_index(y.v[0], T.E);
+                    const int i0 = A.edges[2 * e], k0 = A.edges[2 * e + 1];
+                    // an edge outside [0, N) is never a move (bounds guard)
+                    b_ok = (unsigned)i0 < (unsigned)N && (unsigned)k0 < (unsigned)N;
+                    b_i = b_ok ? i0 : 0;
+                    b_k = b_ok ? k0 : 0;
+                    b_row = e;
+                    b_K = T.K_edge[e];
+                    b_aa = b_ok ? T.a[b_i] - T.a[b_k] : 0.0;
+                }
+                b_h = 0.5f * logf((float)b_u) - (kHam ? 0.f : (float)b_K);
+                b_a2 = (float)(2.0 * b_aa);
+            }
+            int i = __shfl_sync(kFull, b_i, src), k = __shfl_sync(kFull, b_k, src);
+            int row = __shfl_sync(kFull, b_row, src);
+            float h = __shfl_sync(kFull, b_h, src), a2 = __shfl_sync(kFull, b_a2, src);
+            const size_t slot = ((size_t)c * A.dec_stride + A.dec_offset + w) * N + q;
+            double K, aa = 0.0;
+            int n_s = 1, n_sp = 1;
+            if (!kHam) K = __shfl_sync(kFull, b_K, src);
+            if (kHam) {
+                int e, ns, nsp;
+                hamiltonian_pick(A.edges, T.E, N, sv, __shfl_sync(kFull, b_hi, src), lane, e, ns, nsp);
+                if (e < 0) {
+                    if (lane == 0 && A.decisions) A.decisions[slot] = 2;
+                    continue;
+                }
+                i = A.edges[2 * e];
+                k = A.edges[2 * e + 1];
+                row = e;
+                K = T.K_edge[e];
+                aa = T.a[i] - T.a[k];
+                h -= (float)K + 0.5f * (logf((float)ns) - logf((float)nsp));  // ln g(s|s') - ln g(s'|s)
+                a2 = (float)(2.0 * aa);
+                n_s = ns;
+                n_sp = nsp;
+            } else if (!local && (!__shfl_sync(kFull, b_ok, src) || sv[i] == sv[k])) {
+                if (lane == 0 && A.decisions) A.decisions[slot] = 2;
+                continue;
+            }
+            const float si = (float)sv[i];
+            // accepted iff sum_j ln(1 - s t_j tau_j) > ln u / 2 - K + 2 (a-part) s (- corr / 2)
+            const float thr = fmaf(a2, si, h);
+            const float *uf = tabf + (size_t)row * M;
+            float m0 = 1.f, m1 = 1.f, mn = 1.f;
+            int ex = 0, j = lane;
+            for (; j + 7 * 32 < M; j += 8 * 32) {
+                float f[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) f[u] = __ldg(uf + j + 32 * u);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    f[u] = fmaf(-si * t[j + 32 * u], f[u], 1.f);
+                    mn = fminf(mn, f[u]);
+                }
+                m0 = renorm_bits(m0 * ((f[0] * f[1]) * (f[2] * f[3])), ex);
+                m1 = renorm_bits(m1 * ((f[4] * f[5]) * (f[6] * f[7])), ex);
+            }
+            for (; j < M; j += 32) {  // at most 7 more
+                const float f = fmaf(-si * t[j], __ldg(uf + j), 1.f);
+                mn = fminf(mn, f);
+                m0 *= f;
+            }
+            float sum = (__log2f(m0 * m1) + (float)ex) * 0.69314718f;
+            sum = warp_sum(sum);
+            mn = __uint_as_float(__reduce_min_sync(kFull, __float_as_uint(fmaxf(mn, 0.f))));
+            const float margin = __fdividef((float)M * 9.5367432e-7f, mn) +
+                                 4.7683716e-7f * (fabsf(sum) + fabsf(h) + fabsf(a2)) + 1.2207031e-4f;
+            bool accept;
+            const double *D = Dtab + (size_t)row * M;
+            if (mn >= 0.015625f && fabsf(sum - thr) > margin) {
+                accept = sum > thr;
+            } else {
+                // factors too small to trust, or undecided: the ln cosh terms
+                // themselves, first in FP32
+                const double sd = (double)sv[i];
+                const float thr2 = fmaf(a2, si, h + (float)K);
+                float d2 = 0.f, w2 = 0.f;
+                for (int j2 = lane; j2 < M; j2 += 32) {
+                    const float x = (float)th[j2], y = (float)fma(-sd, D[j2], th[j2]);
+                    d2 += lncosh(y) - lncosh(x);
+                    w2 += fabsf(x) + fabsf(y);
+                }
+                d2 = warp_sum(d2);
+                w2 = warp_sum(w2);
+                const float margin2 = 4.7683716e-7f * (w2 + 2.f * (float)M + fabsf(d2) + fabsf(h) + fabsf((float)K) +
+                                                       fabsf(a2)) + 1.2207031e-4f;
+                if (fabsf(d2 - thr2) > margin2) {
+                    accept = d2 > thr2;
+                } else {
+                    double d3 = 0.0;
+                    for (int j3 = lane; j3 < M; j3 += 32) d3 += lncosh(fma(-sd, D[j3], th[j3])) - lncosh(th[j3]);
+                    d3 = warp_sum(d3);
+                    const double av = kHam ? aa : __shfl_sync(kFull, b_aa, src);
+                    const double corr = kHam ? log((double)n_s) - log((double)n_sp) : 0.0;
+                    accept = log(__shfl_sync(kFull, b_u, src)) < 2.0 * (d3 - 2.0 * av * sd) + corr;
+                }
+            }
+            if (lane == 0 && A.decisions) A.decisions[slot] = accept ? 1 : 0;
+            if (accept) {
+                const double sd = (double)sv[i];
+                for (int j = lane; j < M; j += 32) {
+                    const double v = fma(-sd, D[j], th[j]);
+                    th[j] = v;
+                    t[j] = tanhf((float)v);
+                }
+                __syncwarp();
+                if (lane == 0) {
+                    sv[i] = (int8_t)-sv[i];
+                    if (k >= 0) sv[k] = (int8_t)-sv[k];
+                }
+                ++acc;
+            }
+            __syncwarp();
+        }
+        if (w >= A.n_discard) {
+            const size_t row = (size_t)c * A.out_stride + A.out_offset + (w - A.n_discard);
+            for (int i = lane; i < N; i += 32) A.samples[row * N + i] = sv[i];
+            if (A.logpsi) {
+                double lp = 0.0;
+                for (int j = lane; j < M; j += 32) lp += lncosh(th[j]);
+                for (int i = lane; i < N; i += 32) lp += T.a[i] * (double)sv[i];
+                lp = warp_sum(lp);
+                if (lane == 0) A.logpsi[row] = lp;
+            }
+        }
+        __syncwarp();
+    }
+    for (int i = lane; i < N; i += 32) A.s[(size_t)c * N + i] = sv[i];
+    if (lane == 0 && A.n_accepted) A.n_accepted[c] += acc;
+}
+
+// k_sweep_screened for the local and exchange rules with M <= 32 kU: theta
+// and t in registers (lane l holds units l, l + 32, ...), the rows of the next
+// proposal loaded while the current one is decided.  Few chains wait on the
+// chain of one proposal after the other, so with kSpec the moved t is computed
+// beside the decision instead of after it (the FP64 pipe and the exponentials
+// then run for rejected proposals too, which costs nothing until it has more
+// than two chains per scheduler to serve).  Same arithmetic, bounds and
+// fallbacks as k_sweep_screened.
+template <int kU, bool kSpec>
+__global__ void __launch_bounds__(128) k_sweep_screened_regs(SweepK<double> P) {
+    extern __shared__ __align__(16) unsigned char sm[];
+    const Tables<double> &T = P.t;
+    const SweepArgs &A = P.a;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int c = blockIdx.x * (blockDim.x >> 5) + warp;
+    if (c >= A.C) return;
+    const int N = T.N, M = T.M;
+    int8_t *sv = reinterpret_cast<int8_t *>(sm + (size_t)warp * P.warp_bytes);
+    const bool local = A.rule == NK_RULE_LOCAL;
+    const double *Dtab = local ? T.D_site : T.D_edge;
+    const float *tabf = local ? T.tauf_site : T.tauf_edge;
+    for (int i = lane; i < N; i += 32) sv[i] = A.s[(size_t)c * N + i];
+    __syncwarp();
+    unsigned long long acc = 0;
+    const int n_sweeps = A.n_discard + A.n_samples;
+    bool in[kU];
+#pragma unroll
+    for (int u = 0; u < kU; ++u) in[u] = lane + 32 * u < M;
+    double th[kU];
+    float t[kU];
+    for (int w = 0; w < n_sweeps; ++w) {
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            const int j = lane + 32 * u;
+            double v = 0.0;
+            if (in[u]) {
+                if (A.theta_in) {
+                    v = A.theta_in[(size_t)c * (A.theta_ld > 0 ? A.theta_ld : M) + j];
+                } else {
+                    double q0 = T.b[j], q1 = 0.0, q2 = 0.0, q3 = 0.0;
+                    int i = 0;
+                    for (; i + 3 < N; i += 4) {
+                        q0 = fma(T.Wt[(size_t)i * M + j], (double)sv[i], q0);
+                        q1 = fma(T.Wt[(size_t)(i + 1) * M + j], (double)sv[i + 1], q1);
+                        q2 = fma(T.Wt[(size_t)(i + 2) * M + j], (double)sv[i + 2], q2);
+                        q3 = fma(T.Wt[(size_t)(i + 3) * M + j], (double)sv[i + 3], q3);
+                    }
+                    for (; i < N; ++i) q0 = fma(T.Wt[(size_t)i * M + j], (double)sv[i], q0);
+                    v = (q0 + q1) + (q2 + q3);
+                }
+            }
+            th[u] = v;
+            t[u] = tanhf((float)v);  // 0 past M: a factor 1
+        }
+        const unsigned long long qbase = (unsigned long long)(A.sweep0 + w) * (unsigned long long)N;
+        for (int q0 = 0; q0 < N; q0 += 32) {
+            // lane l prepares proposal q0 + l
+            const Philox4 y = philox4x64_10(qbase + (unsigned long long)(q0 + lane), (unsigned long long)c,
+                                            (unsigned long long)A.stream_id, 0ULL, A.seed, 0ULL);
+            const double b_u = uniform53(y.v[1]);
+            int b_i, b_k = -1, b_row, b_ok = 1;
+            double b_K, b_aa;
+            if (local) {
+                b_i = b_row = pick_index(y.v[0], N);
+                b_K = T.K_site[b_i];
+                b_aa = T.a[b_i];
+            } else {
+                b_row = pick_index(y.v[0], T.E);
+                const int i0 = A.edges[2 * b_row], k0 = A.edges[2 * b_row + 1];
+                // an edge outside [0, N) is never a move (bounds guard)
+                b_ok = (unsigned)i0 < (unsigned)N && (unsigned)k0 < (unsigned)N;
+                b_i = b_ok ? i0 : 0;
+                b_k = b_ok ? k0 : 0;
+                b_K = T.K_edge[b_row];
+                b_aa = b_ok ? T.a[b_i] - T.a[b_k] : 0.0;
+            }
+            const float b_h = 0.5f * logf((float)b_u) - (float)b_K, b_a2 = (float)(2.0 * b_aa);
+            const int nq = N - q0 < 32 ? N - q0 : 32;
+            float uf[kU];
+            double D[kU];
+            auto fetch = [&](int row) {
+#pragma unroll
+                for (int u = 0; u < kU; ++u) {
+                    const size_t at = (size_t)row * M + lane + 32 * u;
+                    uf[u] = in[u] ? __ldg(tabf + at) : 0.f;
+                    D[u] = in[u] ? __ldg(Dtab + at) : 0.0;
+                }
+            };
+            fetch(__shfl_sync(kFull, b_row, 0));
+            for (int src = 0; src < nq; ++src) {
+                const int i = __shfl_sync(kFull, b_i, src), k = __shfl_sync(kFull, b_k, src);
+                const float h = __shfl_sync(kFull, b_h, src), a2 = __shfl_sync(kFull, b_a2, src);
+                const int next = __shfl_sync(kFull, b_row, src + 1 < nq ? src + 1 : src);
+                float u0[kU];
+                double D0[kU];
+#pragma unroll
+                for (int u = 0; u < kU; ++u) {
+                    u0[u] = uf[u];
+                    D0[u] = D[u];
+                }
+                fetch(next);
+                const int si8 = sv[i];
+                const size_t slot = ((size_t)c * A.dec_stride + A.dec_offset + w) * N + q0 + src;
+                if (!local && (!__shfl_sync(kFull, b_ok, src) || si8 == sv[k])) {
+                    if (lane == 0 && A.decisions) A.decisions[slot] = 2;
+                    continue;
+                }
+                const float si = (float)si8;
+                const double sd = si8 > 0 ? 1.0 : -1.0;
+                const float thr = fmaf(a2, si, h);
+                float m = 1.f, mn = 1.f;
+#pragma unroll
+                for (int u = 0; u < kU; ++u) {
+                    const float f = fmaf(-si * t[u], u0[u], 1.f);
+                    mn = fminf(mn, f);
+                    m *= f;
+                }
+                double th2[kU];
+                float t2[kU];
+                if (kSpec) {
+#pragma unroll
+                    for (int u = 0; u < kU; ++u) {
+                        th2[u] = fma(-sd, D0[u], th[u]);
+                        t2[u] = tanhf((float)th2[u]);
+                    }
+                }
+                const float sum = warp_sum(__log2f(m)) * 0.69314718f;
+                mn = __uint_as_float(__reduce_min_sync(kFull, __float_as_uint(fmaxf(mn, 0.f))));
+                // |sum - thr| above the bound, both sides times f_min
+                const float slack = 4.7683716e-7f * (fabsf(sum) + fabsf(h) + fabsf(a2)) + 1.2207031e-4f;
+                bool accept;
+                if (mn >= 0.015625f && (fabsf(sum - thr) - slack) * mn > (float)M * 9.5367432e-7f) {
+                    accept = sum > thr;
+                } else {
+                    const float K = (float)__shfl_sync(kFull, b_K, src), thr2 = fmaf(a2, si, h + K);
+                    float d2 = 0.f, w2 = 0.f;
+#pragma unroll
+                    for (int u = 0; u < kU; ++u) {
+                        const float x = (float)th[u], z = (float)fma(-sd, D0[u], th[u]);
+                        d2 += lncosh(z) - lncosh(x);
+                        w2 += fabsf(x) + fabsf(z);
+                    }
+                    d2 = warp_sum(d2);
+                    w2 = warp_sum(w2);
+                    const float margin2 = 4.7683716e-7f * (w2 + 2.f * (float)M + fabsf(d2) + fabsf(h) + fabsf(K) +
+                                                           fabsf(a2)) + 1.2207031e-4f;
+                    if (fabsf(d2 - thr2) > margin2) {
+                        accept = d2 > thr2;
+                    } else {
+                        double d3 = 0.0;
+#pragma unroll
+                        for (int u = 0; u < kU; ++u)
+                            if (in[u]) d3 += lncosh(fma(-sd, D0[u], th[u])) - lncosh(th[u]);
+                        d3 = warp_sum(d3);
+                        accept = log(__shfl_sync(kFull, b_u, src)) <
+                                 2.0 * (d3 - 2.0 * __shfl_sync(kFull, b_aa, src) * sd);
+                    }
+                }
+                if (lane == 0 && A.decisions) A.decisions[slot] = accept ? 1 : 0;
+                if (accept) {
+#pragma unroll
+                    for (int u = 0; u < kU; ++u) {
+                        th[u] = kSpec ? th2[u] : fma(-sd, D0[u], th[u]);
+                        t[u] = kSpec ? t2[u] : tanhf((float)th[u]);
+                    }
+                    if (lane == 0) {
+                        sv[i] = (int8_t)-si8;
+                        if (k >= 0) sv[k] = (int8_t)si8;
+                    }
+                    ++acc;
+                    __syncwarp();
+                }
+            }
+        }
+        if (w >= A.n_discard) {
+            const size_t row = (size_t)c * A.out_stride + A.out_offset + (w - A.n_discard);
+            for (int i = lane; i < N; i += 32) A.samples[row * N + i] = sv[i];
+            if (A.logpsi) {
+                double lp = 0.0;
+#pragma unroll
+                for (int u = 0; u < kU; ++u)
+                    if (in[u]) lp += lncosh(th[u]);
+                for (int i = lane; i < N; i += 32) lp += T.a[i] * (double)sv[i];
+                lp = warp_sum(lp);
+                if (lane == 0) A.logpsi[row] = lp;
+            }
+        }
+    }
+    for (int i = lane; i < N; i += 32) A.s[(size_t)c * N + i] = sv[i];
+    if (lane == 0 && A.n_accepted) A.n_accepted[c] += acc;
+}
+
 // FP32 sweeps of the local and exchange rules with the flip-ratio row of a
 // proposal held in registers: every lane issues the loads of all its kC
 // chunks of the row at once, so a proposal waits for one L2 round trip
-// (k_sweep<float, false> waits for one per group of four chunks: nine at M =
+// (k_sweep<false, false> waits for one per group of four chunks: nine at M =
 // 4608).  The accepted move's update of t reuses the registers.  The
 // arithmetic and the order of every product are those of
-// k_sweep<float, false>, so the decisions are identical.  Needs M % 4 == 0 and
+// k_sweep<false, false>, so the decisions are identical.  Needs M % 4 == 0 and
 // M <= 128 kC.
 template <int kC>
 __global__ void __launch_bounds__(128) k_sweep_rows(SweepK<float> P) {
@@ -751,10 +1150,6 @@ struct ElocK {
     int warp_bytes, t_bytes, s_bytes;
     int units;  // 1: lanes over hidden units (large M), 0: lanes over connections
 };
-
-// Hidden-unit count from which the local energy spreads the units over the
-// lanes (one warp reduction per connection) instead of the connections.
-constexpr int kUnitsMappingM = 1024;
 
 // One warp per sample.  theta and t are rebuilt from s; the connected
 // configurations are spread over the lanes (sites for the Ising field term,
@@ -1078,10 +1473,10 @@ cudaError_t launch_tables(const Tables<R> &t, bool need_site, bool need_edge, cu
     (k_transpose_W<<<tg, tb, 0, st>>>(t.N, t.M, t.W, t.Wt), nk::note_launch());
     if (need_site)
         (k_tau_rows<R><<<t.N, 256, 0, st>>>(t.N, t.M, t.N, t.Wt, nullptr, t.tau_site, t.tau_siteT,
-                                           t.K_site), nk::note_launch());
+                                           t.K_site, t.tauf_site, t.D_site), nk::note_launch());
     if (need_edge && t.E > 0)
         (k_tau_rows<R><<<t.E, 256, 0, st>>>(t.N, t.M, t.E, t.Wt, t.edges, t.tau_edge, t.tau_edgeT,
-                                           t.K_edge), nk::note_launch());
+                                           t.K_edge, t.tauf_edge, t.D_edge), nk::note_launch());
     return cudaGetLastError();
 }
 
@@ -1142,9 +1537,52 @@ cudaError_t launch_sweep_rows_kc(const SweepK<float> &P, cudaStream_t st) {
 // (10.9 against 8.4 ms, 140 against 125 ms), so those sizes keep k_sweep.
 cudaError_t launch_sweep_rows(const SweepK<float> &P, cudaStream_t st) { return launch_sweep_rows_kc<4>(P, st); }
 
+// NK_F64: the screened kernel.  Shared memory holds theta (FP64), t (FP32) and
+// the spins of each chain.
+template <int kU>
+cudaError_t launch_sweep_screened_regs(SweepK<double> P, cudaStream_t st) {
+    P.warp_bytes = align16<double>(P.t.N);
+    // one chain per scheduler while there are few: their warps do not share it
+    const int wpb = P.a.C <= 152 ? 1 : 4;
+    const unsigned grid = (unsigned)((P.a.C + wpb - 1) / wpb);
+    const int slot = prof_begin(NK_PROF_SWEEP, st);
+    if (P.a.C <= 1216)
+        (k_sweep_screened_regs<kU, true><<<grid, 32 * wpb, wpb * P.warp_bytes, st>>>(P), nk::note_launch());
+    else
+        (k_sweep_screened_regs<kU, false><<<grid, 32 * wpb, wpb * P.warp_bytes, st>>>(P), nk::note_launch());
+    prof_end(slot, st, (double)P.a.C * (P.a.n_discard + P.a.n_samples) * P.t.N * (double)P.t.M);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_sweep_screened(const SweepK<double> &P0, cudaStream_t st) {
+    if (P0.a.rule != NK_RULE_HAMILTONIAN && P0.t.M <= 128)
+        return P0.t.M <= 32 ? launch_sweep_screened_regs<1>(P0, st)
+                            : (P0.t.M <= 64 ? launch_sweep_screened_regs<2>(P0, st)
+                                            : launch_sweep_screened_regs<4>(P0, st));
+    SweepK<double> P = P0;
+    P.t_bytes = align16<double>(P.t.M * 8 + 8) / 32 * 32 + 32;  // theta; half of it holds t
+    P.warp_bytes = P.t_bytes + P.t_bytes / 2 + align16<double>(P.t.N);
+    int wpb = 4;
+    while (wpb > 1 && (size_t)wpb * P.warp_bytes > 200 * 1024) wpb >>= 1;
+    const size_t smem = (size_t)wpb * P.warp_bytes;
+    if (smem > 227 * 1024) return cudaErrorInvalidValue;
+    const bool ham = P.a.rule == NK_RULE_HAMILTONIAN;
+    cudaError_t err = nk::allow_max_dynamic_smem(ham ? (const void *)k_sweep_screened<true>
+                                                     : (const void *)k_sweep_screened<false>);
+    if (err != cudaSuccess) return err;
+    const unsigned grid = (unsigned)((P.a.C + wpb - 1) / wpb);
+    const int slot = prof_begin(NK_PROF_SWEEP, st);
+    if (ham)
+        (k_sweep_screened<true><<<grid, 32 * wpb, smem, st>>>(P), nk::note_launch());
+    else
+        (k_sweep_screened<false><<<grid, 32 * wpb, smem, st>>>(P), nk::note_launch());
+    prof_end(slot, st, (double)P.a.C * (P.a.n_discard + P.a.n_samples) * P.t.N * (double)P.t.M);
+    return cudaGetLastError();
+}
+
+// The arguments of a sweep with the defaults filled in.
 template <typename R>
-cudaError_t launch_sweep(const Tables<R> &t, const SweepArgs &a, cudaStream_t st) {
-    if (a.C <= 0 || a.n_discard + a.n_samples <= 0) return cudaSuccess;
+SweepK<R> sweep_args(const Tables<R> &t, const SweepArgs &a) {
     SweepK<R> P;
     P.t = t;
     P.a = a;
@@ -1159,37 +1597,44 @@ cudaError_t launch_sweep(const Tables<R> &t, const SweepArgs &a, cudaStream_t st
     P.t_bytes = align16<R>(t.M * (int)sizeof(R));
     P.warp_bytes = P.t_bytes + align16<R>(t.N);
     P.vec4 = sizeof(R) == 4 && (t.M % 4) == 0;
-    // FP32 local and exchange rules: the prefetching kernel, when two more
-    // rows per warp fit in shared memory
-    if constexpr (sizeof(R) == 4) {
-        if (P.vec4 && a.rule != NK_RULE_HAMILTONIAN && t.M <= 4 * 128) return launch_sweep_rows(P, st);
-    }
+    return P;
+}
+
+template <>
+cudaError_t launch_sweep<double>(const Tables<double> &t, const SweepArgs &a, cudaStream_t st) {
+    if (a.C <= 0 || a.n_discard + a.n_samples <= 0) return cudaSuccess;
+    return launch_sweep_screened(sweep_args(t, a), st);
+}
+
+template <>
+cudaError_t launch_sweep<float>(const Tables<float> &t, const SweepArgs &a, cudaStream_t st) {
+    if (a.C <= 0 || a.n_discard + a.n_samples <= 0) return cudaSuccess;
+    const SweepK<float> P = sweep_args(t, a);
+    // local and exchange rules with few units: the register-row kernel
+    if (P.vec4 && a.rule != NK_RULE_HAMILTONIAN && t.M <= 4 * 128) return launch_sweep_rows(P, st);
     int wpb = 4;
     while (wpb > 1 && (size_t)wpb * P.warp_bytes > 200 * 1024) wpb >>= 1;
     size_t smem = (size_t)wpb * P.warp_bytes;
     if (smem > 227 * 1024) return cudaErrorInvalidValue;
     const bool ham = a.rule == NK_RULE_HAMILTONIAN;
-    const bool ring = sizeof(R) == 4 && P.vec4 && t.M >= 6 * 512;
-    const void *fn = ham ? (ring ? (const void *)k_sweep<R, true, true> : (const void *)k_sweep<R, true, false>)
-                         : (ring ? (const void *)k_sweep<R, false, true> : (const void *)k_sweep<R, false, false>);
+    const bool ring = P.vec4 && t.M >= 6 * 512;
+    const void *fn = ham ? (ring ? (const void *)k_sweep<true, true> : (const void *)k_sweep<true, false>)
+                         : (ring ? (const void *)k_sweep<false, true> : (const void *)k_sweep<false, false>);
     cudaError_t err = nk::allow_max_dynamic_smem(fn);
     if (err != cudaSuccess) return err;
     unsigned grid = (unsigned)((a.C + wpb - 1) / wpb);
     const int slot = prof_begin(NK_PROF_SWEEP, st);
     if (ham && ring)
-        (k_sweep<R, true, true><<<grid, 32 * wpb, smem, st>>>(P), nk::note_launch());
+        (k_sweep<true, true><<<grid, 32 * wpb, smem, st>>>(P), nk::note_launch());
     else if (ham)
-        (k_sweep<R, true, false><<<grid, 32 * wpb, smem, st>>>(P), nk::note_launch());
+        (k_sweep<true, false><<<grid, 32 * wpb, smem, st>>>(P), nk::note_launch());
     else if (ring)
-        (k_sweep<R, false, true><<<grid, 32 * wpb, smem, st>>>(P), nk::note_launch());
+        (k_sweep<false, true><<<grid, 32 * wpb, smem, st>>>(P), nk::note_launch());
     else
-        (k_sweep<R, false, false><<<grid, 32 * wpb, smem, st>>>(P), nk::note_launch());
+        (k_sweep<false, false><<<grid, 32 * wpb, smem, st>>>(P), nk::note_launch());
     prof_end(slot, st, (double)a.C * (a.n_discard + a.n_samples) * t.N * (double)t.M);
     return cudaGetLastError();
 }
-
-template cudaError_t launch_sweep<double>(const Tables<double> &, const SweepArgs &, cudaStream_t);
-template cudaError_t launch_sweep<float>(const Tables<float> &, const SweepArgs &, cudaStream_t);
 
 size_t eloc_batched_smem(int N, int M, int warps) {
     const size_t t_ld = (size_t)(M + 3) / 4 * 4, s_ld = (size_t)(N + 15) / 16 * 16;

@@ -154,9 +154,11 @@ nk_status check_ham(const nk_ham *h, int N) {
     return NK_OK;
 }
 
+// sweep, eloc: the tables are for sweeps, for local energies (whose small-M
+// kernel reads the unit-major form), or both.
 template <typename R>
 void carve_tables(Carver &c, nk::Tables<R> &t, const nk_rbm *rbm, int E, const int32_t *edges,
-                  bool site, bool edge) {
+                  bool site, bool edge, bool sweep, bool eloc) {
     const int N = rbm->N, M = rbm->M;
     t.N = N;
     t.M = M;
@@ -166,12 +168,20 @@ void carve_tables(Carver &c, nk::Tables<R> &t, const nk_rbm *rbm, int E, const i
     t.W = rbm->params + N + M;
     t.edges = edges;
     t.Wt = c.take<double>((size_t)N * M);
-    t.tau_site = site ? c.take<R>((size_t)N * M) : nullptr;
-    t.tau_siteT = site ? c.take<R>((size_t)N * M) : nullptr;
+    const bool unit_major = eloc && M < nk::kUnitsMappingM;
+    const bool rows = (eloc && !unit_major) || (sweep && sizeof(R) == 4);
+    t.tau_site = site && rows ? c.take<R>((size_t)N * M) : nullptr;
+    t.tau_siteT = site && unit_major ? c.take<R>((size_t)N * M) : nullptr;
     t.K_site = site ? c.take<R>(N) : nullptr;
-    t.tau_edge = edge ? c.take<R>((size_t)E * M) : nullptr;
-    t.tau_edgeT = edge ? c.take<R>((size_t)E * M) : nullptr;
+    t.tau_edge = edge && rows ? c.take<R>((size_t)E * M) : nullptr;
+    t.tau_edgeT = edge && unit_major ? c.take<R>((size_t)E * M) : nullptr;
     t.K_edge = edge ? c.take<R>(E) : nullptr;
+    if (sizeof(R) == 8 && sweep) {
+        t.tauf_site = site ? c.take<float>((size_t)N * M) : nullptr;
+        t.D_site = site ? c.take<double>((size_t)N * M) : nullptr;
+        t.tauf_edge = edge ? c.take<float>((size_t)E * M) : nullptr;
+        t.D_edge = edge ? c.take<double>((size_t)E * M) : nullptr;
+    }
 }
 
 __global__ void k_cg_init(const double *rr, double *ff, double *rr_keep, int *done, int *iters) {
@@ -620,7 +630,7 @@ template <typename R>
 void carve_step(Carver &c, nk::Tables<R> &t, StepBufs &b, const nk_rbm *rbm, const nk_ham *ham, int C,
                 int64_t Ns, bool site, bool edge, bool mixed, int8_t *samples_out, double *eloc_out) {
     const int N = rbm->N, M = rbm->M;
-    carve_tables(c, t, rbm, ham->n_edges, ham->edges, site, edge);
+    carve_tables(c, t, rbm, ham->n_edges, ham->edges, site, edge, true, true);
     b.samples = samples_out ? samples_out : c.take<int8_t>((size_t)Ns * N);
     b.eloc = eloc_out ? eloc_out : c.take<double>(Ns);
     b.T = c.take<double>((size_t)Ns * M);
@@ -817,7 +827,7 @@ nk_status nk_rbm_logpsi(nk_ctx *ctx, const nk_rbm *rbm, int32_t precision, const
     const int N = rbm->N, M = rbm->M;
     return with_workspace(ctx, [&](Carver &c, bool run) -> nk_status {
         nk::Tables<double> t{};
-        carve_tables(c, t, rbm, 0, nullptr, false, false);
+        carve_tables(c, t, rbm, 0, nullptr, false, false, false, false);
         const bool tcp = precision == NK_MIXED || nk::f64_on_tensor(N, M, B);
         double *theta = tcp ? c.take<double>((size_t)B * M) : nullptr;
         void *tcm = tcp ? c.take<char>(nk::tc_theta_ws_bytes(N, M, B)) : nullptr;
@@ -898,7 +908,7 @@ nk_status nk_metropolis_sweep(nk_ctx *ctx, const nk_rbm *rbm, int32_t precision,
     auto body = [&](auto tag, Carver &c, bool run) -> nk_status {
         using R = decltype(tag);
         nk::Tables<R> t{};
-        carve_tables(c, t, rbm, E, edges, !pair, pair);
+        carve_tables(c, t, rbm, E, edges, !pair, pair, true, false);
         const bool mixed = precision == NK_MIXED;
         double *theta = mixed ? c.take<double>((size_t)C * rbm->M) : nullptr;
         void *tcm = mixed ? c.take<char>(nk::tc_theta_ws_bytes(rbm->N, rbm->M, C)) : nullptr;
@@ -931,7 +941,7 @@ nk_status nk_local_energy(nk_ctx *ctx, const nk_rbm *rbm, int32_t precision, con
     auto body = [&](auto tag, Carver &c, bool run) -> nk_status {
         using R = decltype(tag);
         nk::Tables<R> t{};
-        carve_tables(c, t, rbm, ham->n_edges, ham->edges, site, edge);
+        carve_tables(c, t, rbm, ham->n_edges, ham->edges, site, edge, false, true);
         const bool mixed = precision == NK_MIXED;
         double *theta = mixed ? c.take<double>((size_t)Ns * rbm->M) : nullptr;
         void *tcm = mixed ? c.take<char>(nk::tc_theta_ws_bytes(rbm->N, rbm->M, Ns)) : nullptr;

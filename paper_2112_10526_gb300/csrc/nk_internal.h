@@ -61,6 +61,10 @@ struct Tables {
     R *tau_edge;              // [E][M]  tanh(2 (W_ji - W_jk))
     R *tau_edgeT;             // [M][E]
     R *K_edge;                // [E]
+    // NK_F64 sweeps: tau in FP32 (the screening of proposals) and 2 (W_ji -
+    // W_jk) (the move of theta; 2 W_ji for single flips)
+    float *tauf_site, *tauf_edge;
+    double *D_site, *D_edge;
 };
 
 template <typename R>
@@ -128,6 +132,11 @@ inline ElocArgs eloc_args(const nk_ham *h, const int8_t *s, int64_t Ns, double *
     a.E2 = h->n_edges2;
     return a;
 }
+
+// Hidden-unit count from which the local energy spreads the units over the
+// lanes (one warp reduction per connection) instead of the connections, and
+// reads the row-major tables.
+constexpr int kUnitsMappingM = 1024;
 
 template <typename R>
 cudaError_t launch_eloc(const Tables<R> &t, const ElocArgs &a, cudaStream_t st);
