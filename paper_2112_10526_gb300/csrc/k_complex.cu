@@ -5,11 +5,11 @@
 // theta, tanh theta s^T] (holomorphic, Eq. eq:log-derivative-O) and the
 // realified Jacobian whose Gram gives the real embedding of the complex QGT.
 //
-// Complex numbers are double2 (x = real, y = imaginary part); everything is
-// FP64 on CUDA cores.  One warp per chain or sample, hidden units over the
-// lanes, theta in shared memory.  Log-ratios are differences of ln cosh term
-// by term on the moved activations (no tanh tables): complex ln cosh is cheap
-// next to keeping the phase of a running product right.
+// Complex numbers are double2 (x = real, y = imaginary part); results are FP64
+// on CUDA cores.  One warp per chain or sample, theta in shared memory.  A
+// Metropolis decision needs only the sign of a real difference, which FP32
+// with an error bound settles for nearly every proposal; the local energies
+// take each amplitude ratio as one product over the hidden units.
 
 #include <cuda_runtime.h>
 
@@ -151,16 +151,40 @@ struct CSweepArgs {
     unsigned stream_id;
     int8_t *samples;  // [C][n_samples][N]
     unsigned long long *n_accepted;
+    int warp_bytes;
 };
 
+// Re ln cosh z + ln 2 in FP32 (g.x) and a bound on its error (g.y):
+// |x| + ln(w) / 2 with w = |1 + e^{-2y}|^2 = (1 - E)^2 + 4 E cos^2 Im z, E =
+// e^{-2 |x|}, x = Re z.  Rounding z, the exponential, the cosine and the
+// square leave w within 2^-18 (1 + |x| + |y|) (relative to w it is that over
+// w, also through the poles' growth of the derivative, 2 / sqrt w), the
+// logarithm and the sum within 2^-22 (1 + |x|).  No bound (infinite) below w =
+// 2^-6, near the zeros of cosh, and for a NaN.
+__device__ __forceinline__ float2 re_lncosh_bounded(double2 z) {
+    const float x = fabsf((float)z.x), y = (float)z.y;
+    const float E = expf(-2.f * x), c = cosf(y), o = 1.f - E;
+    const float w = fmaf(4.f * E * c, c, o * o);
+    const float e = __fdividef(3.8146973e-6f * (1.f + x + fabsf(y)), w);
+    return make_float2(x + 0.5f * logf(w), w >= 0.015625f ? e : __int_as_float(0x7F800000));
+}
+
+// One warp per chain.  The move is accepted iff ln u < 2 Re[ln psi(s') - ln
+// psi(s)].  Both sides are first taken in FP32 from Re ln cosh of the moved
+// units (that of the present ones is kept), with the sum of the units' error
+// bounds: a difference above it decides.  Otherwise (about one proposal in a
+// few thousand at M = 20) the FP64 log-ratio of clog_ratio decides, which
+// used to be taken for every proposal: two complex ln cosh a unit, some 150
+// FP64 operations each on a pipe of 2 lanes a clock and SM.  theta stays in
+// FP64.  20 sites, M = 20, 1024 chains, 24 sweeps: 11.4 ms before.
 __global__ void __launch_bounds__(128) k_crbm_sweep(CSweepArgs A) {
     extern __shared__ __align__(16) unsigned char sm[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int c = blockIdx.x * (blockDim.x >> 5) + warp;
     const int N = A.N, M = A.M;
-    const size_t wb = ((size_t)M * sizeof(double2) + (size_t)N + 15) / 16 * 16;
-    double2 *th = reinterpret_cast<double2 *>(sm + warp * wb);
-    int8_t *sv = reinterpret_cast<int8_t *>(th + M);
+    double2 *th = reinterpret_cast<double2 *>(sm + (size_t)warp * A.warp_bytes);
+    float2 *g = reinterpret_cast<float2 *>(th + M);  // Re ln cosh theta + ln 2 and its error bound
+    int8_t *sv = reinterpret_cast<int8_t *>(g + M);
     if (c >= A.C) return;
     for (int i = lane; i < N; i += 32) sv[i] = A.s[(size_t)c * N + i];
     __syncwarp();
@@ -168,35 +192,81 @@ __global__ void __launch_bounds__(128) k_crbm_sweep(CSweepArgs A) {
     unsigned long long acc = 0;
     for (int w = 0; w < A.n_discard + A.n_samples; ++w) {
         hidden(v, N, M, sv, th, lane);
+        for (int j = lane; j < M; j += 32) g[j] = re_lncosh_bounded(th[j]);  // the lane's own units
         __syncwarp();
         const unsigned long long qbase = (unsigned long long)(A.sweep0 + w) * (unsigned long long)N;
+        int b_i = 0, b_k = 0, b_ok = 1;
+        double b_u = 1.0;
+        float b_h = 0.f, b_a2 = 0.f;  // ln u / 2, 2 Re(a_i - a_k)
         for (int q = 0; q < N; ++q) {
-            const Philox4 y = philox4x64_10(qbase + (unsigned long long)q, (unsigned long long)c,
-                                            (unsigned long long)A.stream_id, 0ULL, A.seed, 0ULL);
-            int sites[2], n;
-            if (A.rule == NK_RULE_LOCAL) {
-                sites[0] = pick_index(y.v[0], N);
-                n = 1;
-            } else {
-                const int e = pick_index(y.v[0], A.E);
-                const int i0 = A.edges[2 * e], k0 = A.edges[2 * e + 1];
-                if ((unsigned)i0 >= (unsigned)N || (unsigned)k0 >= (unsigned)N || sv[i0] == sv[k0]) continue;
-                sites[0] = i0;
-                sites[1] = k0;
-                n = 2;
+            const int src = q & 31;
+            if (src == 0) {  // lane l prepares proposal q + l
+                const Philox4 y = philox4x64_10(qbase + (unsigned long long)(q + lane), (unsigned long long)c,
+                                                (unsigned long long)A.stream_id, 0ULL, A.seed, 0ULL);
+                b_u = uniform53(y.v[1]);
+                b_h = 0.5f * logf((float)b_u);
+                if (A.rule == NK_RULE_LOCAL) {
+                    b_i = pick_index(y.v[0], N);
+                    b_a2 = (float)(2.0 * v.a[b_i].x);
+                } else {
+                    const int e = pick_index(y.v[0], A.E);
+                    const int i0 = A.edges[2 * e], k0 = A.edges[2 * e + 1];
+                    b_ok = (unsigned)i0 < (unsigned)N && (unsigned)k0 < (unsigned)N;
+                    b_i = b_ok ? i0 : 0;
+                    b_k = b_ok ? k0 : 0;
+                    b_a2 = b_ok ? (float)(2.0 * (v.a[b_i].x - v.a[b_k].x)) : 0.f;
+                }
             }
-            const double2 d = clog_ratio(v, N, M, sv, th, sites, n, lane);
-            const double lu = log(uniform53(y.v[1]));
-            if (lu < 2.0 * d.x) {
-                for (int j = lane; j < M; j += 32) {
-                    double2 t = th[j];
-                    for (int r = 0; r < n; ++r) {
-                        const double s2 = 2.0 * (double)sv[sites[r]];
-                        const double2 wj = v.W[(size_t)j * N + sites[r]];
-                        t.x -= s2 * wj.x;
-                        t.y -= s2 * wj.y;
+            int sites[2] = {__shfl_sync(0xffffffffu, b_i, src), __shfl_sync(0xffffffffu, b_k, src)};
+            const float h = __shfl_sync(0xffffffffu, b_h, src), a2 = __shfl_sync(0xffffffffu, b_a2, src);
+            const int ok = __shfl_sync(0xffffffffu, b_ok, src);
+            const int n = A.rule == NK_RULE_LOCAL ? 1 : 2;
+            if (n == 2 && (!ok || sv[sites[0]] == sv[sites[1]])) continue;
+            const double s0 = 2.0 * (double)sv[sites[0]];
+            auto moved = [&](int j) {
+                double2 t = th[j];
+                const double2 w0 = v.W[(size_t)j * N + sites[0]];
+                t.x = fma(-s0, w0.x, t.x);
+                t.y = fma(-s0, w0.y, t.y);
+                if (n == 2) {  // s_k = -s_i
+                    const double2 w1 = v.W[(size_t)j * N + sites[1]];
+                    t.x = fma(s0, w1.x, t.x);
+                    t.y = fma(s0, w1.y, t.y);
+                }
+                return t;
+            };
+            // sum_j Re[ln cosh theta' - ln cosh theta] > ln u / 2 + 2 Re(a-part) s
+            const float thr = fmaf(a2, (float)sv[sites[0]], h);
+            float d = 0.f, err = 0.f;
+            float2 g0 = make_float2(0.f, 0.f);
+            double2 t0 = make_double2(0.0, 0.0);
+            for (int j = lane; j < M; j += 32) {
+                t0 = moved(j);
+                g0 = re_lncosh_bounded(t0);
+                d += g0.x - g[j].x;
+                err += g0.y + g[j].y + 4.7683716e-7f * (fabsf(g0.x) + fabsf(g[j].x));
+            }
+            d = warp_sum(d);
+            err = warp_sum(err) + 4.7683716e-7f * (fabsf(h) + fabsf(a2)) + 1.9073486e-6f;
+            bool accept;
+            if (fabsf(d - thr) > err) {  // false for an infinite bound and for NaNs
+                accept = d > thr;
+            } else {
+                const double2 d2 = clog_ratio(v, N, M, sv, th, sites, n, lane);
+                accept = log(__shfl_sync(0xffffffffu, b_u, src)) < 2.0 * d2.x;
+            }
+            if (accept) {
+                if (M <= 32) {  // the lane's only unit is still in registers
+                    if (lane < M) {
+                        th[lane] = t0;
+                        g[lane] = g0;
                     }
-                    th[j] = t;
+                } else {
+                    for (int j = lane; j < M; j += 32) {
+                        const double2 t = moved(j);
+                        th[j] = t;
+                        g[j] = re_lncosh_bounded(t);
+                    }
                 }
                 __syncwarp();
                 if (lane == 0)
@@ -221,54 +291,151 @@ __global__ void __launch_bounds__(128) k_crbm_sweep(CSweepArgs A) {
 // element (+-2 J_e, Marshall sign on the nearest-neighbour class) per
 // antiparallel edge.  out: complex [Ns].
 
+// An amplitude ratio is a product over the hidden units: with p_j = 1 / (1 +
+// e^{-2 theta_j}) and q_j = 1 - p_j = 1 / (1 + e^{2 theta_j}),
+//     cosh(theta_j - d_j) / cosh theta_j = e^{-d_j} p_j + e^{d_j} q_j,
+// which has no cancellation of its own (both terms are positive for real
+// arguments; a small sum is a theta_j - d_j near a zero of cosh, where ln cosh
+// is as sensitive).  e^{+-2 W_ji} come from a table (one exponential per weight
+// instead of two complex ln cosh per weight and sample), so a term costs 12
+// FP64 operations for a flip and 20 for a pair against about 300.  Lanes run
+// over the connected configurations, the tables are unit-major as W is, so the
+// lanes' loads coalesce and no reduction is needed per ratio.  20 sites, M =
+// 20, 4096 samples: 1.7 ms before.
 struct CElocArgs {
     int N, M, E, E2, kind, marshall;
     double J, J2, h;
     const double *p;
+    const double2 *ep, *em;  // e^{2 W}, e^{-2 W}, [M][N]
     const int32_t *edges;
     const int8_t *s;
     int64_t Ns;
     double *eloc;
+    int warp_bytes, pq_bytes, s_bytes;
+    int compact;  // the antiparallel edges are listed in shared memory first
 };
+
+__global__ void k_crbm_exp_tables(int64_t n, const double2 *__restrict__ W, double2 *__restrict__ ep,
+                                  double2 *__restrict__ em) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    double sn, cs;
+    sincos(2.0 * W[i].y, &sn, &cs);
+    const double a = exp(2.0 * W[i].x), b = exp(-2.0 * W[i].x);
+    ep[i] = make_double2(a * cs, a * sn);
+    em[i] = make_double2(b * cs, -b * sn);
+}
+
+// 1 / (1 + e^{-2z}) and 1 / (1 + e^{2z}), from the exponential that does not
+// grow: with y = +-z, Re y >= 0, w = e^{-2y}: 1 / (1 + w) and w / (1 + w).
+__device__ __forceinline__ void logistic_pair(double2 z, double2 &p, double2 &q) {
+    const bool neg = z.x < 0.0;
+    const double2 y = neg ? make_double2(-z.x, -z.y) : z;
+    const double2 w = cexp(make_double2(-2.0 * y.x, -2.0 * y.y));
+    const double2 o = make_double2(1.0 + w.x, w.y);
+    const double inv = 1.0 / (o.x * o.x + o.y * o.y);
+    const double2 a = make_double2(o.x * inv, -o.y * inv), b = cmul(w, a);
+    p = neg ? b : a;
+    q = neg ? a : b;
+}
 
 __global__ void __launch_bounds__(128) k_crbm_eloc(CElocArgs A) {
     extern __shared__ __align__(16) unsigned char sm[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t k = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
     const int N = A.N, M = A.M, E1 = A.E - A.E2;
-    const size_t wb = ((size_t)M * sizeof(double2) + (size_t)N + 15) / 16 * 16;
-    double2 *th = reinterpret_cast<double2 *>(sm + warp * wb);
-    int8_t *sv = reinterpret_cast<int8_t *>(th + M);
+    unsigned char *base = sm + (size_t)warp * A.warp_bytes;
+    double2 *pq = reinterpret_cast<double2 *>(base);  // [M][2]
+    int8_t *sv = reinterpret_cast<int8_t *>(base + A.pq_bytes);
+    int *list = reinterpret_cast<int *>(base + A.pq_bytes + A.s_bytes);
     if (k >= A.Ns) return;
     for (int i = lane; i < N; i += 32) sv[i] = A.s[(size_t)k * N + i];
     __syncwarp();
     const CView v = cview(A.p, N, M);
-    hidden(v, N, M, sv, th, lane);
+    hidden(v, N, M, sv, pq, lane);  // theta in pq[0 .. M - 1]
     __syncwarp();
+    // (p, q) of the units from the last to the first block of 32: a block's
+    // theta is read by its lanes before pairs are written over it
+    for (int j0 = (M - 1) / 32 * 32; j0 >= 0; j0 -= 32) {
+        const int j = j0 + lane;
+        double2 p = make_double2(0.0, 0.0), q = p;
+        if (j < M) logistic_pair(pq[j], p, q);
+        __syncwarp();
+        if (j < M) {
+            pq[2 * j] = p;
+            pq[2 * j + 1] = q;
+        }
+        __syncwarp();
+    }
     double diag = 0.0;
     for (int e = lane; e < A.E; e += 32) {
         const int i = A.edges[2 * e], kk = A.edges[2 * e + 1];
         if ((unsigned)i < (unsigned)N && (unsigned)kk < (unsigned)N)
             diag += (e < E1 ? A.J : A.J2) * (double)sv[i] * (double)sv[kk];
     }
-    diag = warp_sum(diag);
-    double2 off = make_double2(0.0, 0.0);
-    if (A.kind == NK_TFIM) {
-        for (int i = 0; i < N; ++i) {
-            const int site[1] = {i};
-            const double2 r = cexp(clog_ratio(v, N, M, sv, th, site, 1, lane));
-            off = cadd(off, cscale(r, -A.h));
+    // the connected configurations: the N sites, or the antiparallel edges
+    // (all edges, the parallel ones skipped, where the list does not fit)
+    int n = A.kind == NK_TFIM ? N : A.E;
+    if (A.compact) {
+        n = 0;
+        for (int e0 = 0; e0 < A.E; e0 += 32) {
+            const int e = e0 + lane;
+            bool f = false;
+            if (e < A.E) {
+                const int i = A.edges[2 * e], kk = A.edges[2 * e + 1];
+                f = (unsigned)i < (unsigned)N && (unsigned)kk < (unsigned)N && sv[i] != sv[kk];
+            }
+            const unsigned mask = __ballot_sync(0xffffffffu, f);
+            if (f) list[n + __popc(mask & ((1u << lane) - 1u))] = e;
+            n += __popc(mask);
         }
-    } else {
-        for (int e = 0; e < A.E; ++e) {
-            const int i = A.edges[2 * e], kk = A.edges[2 * e + 1];
-            if ((unsigned)i >= (unsigned)N || (unsigned)kk >= (unsigned)N || sv[i] == sv[kk]) continue;
-            const int pair[2] = {i, kk};
-            const double el = e < E1 ? (A.marshall ? -2.0 * A.J : 2.0 * A.J) : 2.0 * A.J2;
-            const double2 r = cexp(clog_ratio(v, N, M, sv, th, pair, 2, lane));
-            off = cadd(off, cscale(r, el));
-        }
+        __syncwarp();
     }
+    double2 off = make_double2(0.0, 0.0);
+    for (int x = lane; x < n; x += 32) {
+        int i = x, kk = -1;
+        double el = -A.h;
+        if (A.kind != NK_TFIM) {
+            const int e = A.compact ? list[x] : x;
+            i = A.edges[2 * e];
+            kk = A.edges[2 * e + 1];
+            if (!A.compact && ((unsigned)i >= (unsigned)N || (unsigned)kk >= (unsigned)N || sv[i] == sv[kk])) continue;
+            el = e < E1 ? (A.marshall ? -2.0 * A.J : 2.0 * A.J) : 2.0 * A.J2;
+        }
+        // d_j = 2 s_i (W_ji - W_jk): e^{-d} is em for s_i = 1, ep for s_i = -1
+        const bool up = sv[i] > 0;
+        const double2 *dn = (up ? A.em : A.ep), *gr = (up ? A.ep : A.em);
+        double2 r = make_double2(1.0, 0.0);
+        int ex = 0;
+        for (int j = 0; j < M; ++j) {
+            const size_t at = (size_t)j * N;
+            double2 a = dn[at + i], b = gr[at + i];
+            if (kk >= 0) {
+                a = cmul(a, gr[at + kk]);
+                b = cmul(b, dn[at + kk]);
+            }
+            const double2 p = pq[2 * j], q = pq[2 * j + 1];
+            const double2 f = make_double2(fma(b.x, q.x, -b.y * q.y) + fma(a.x, p.x, -a.y * p.y),
+                                           fma(b.x, q.y, b.y * q.x) + fma(a.x, p.y, a.y * p.x));
+            r = cmul(r, f);
+            // keep the product's exponent within +-240
+            const int eb = max((__double2hiint(r.x) >> 20) & 0x7FF, (__double2hiint(r.y) >> 20) & 0x7FF) - 1023;
+            if ((eb > 240 && eb < 1024) || (eb < -240 && eb > -1023)) {
+                r.x = ldexp(r.x, -eb);
+                r.y = ldexp(r.y, -eb);
+                ex += eb;
+            }
+        }
+        // e^{-2 s_i (a_i - a_k)} 2^ex
+        double2 av = v.a[i];
+        if (kk >= 0) av = csub(av, v.a[kk]);
+        const double sg = up ? -2.0 : 2.0;
+        double2 z = cscale(av, sg);
+        z.x += (double)ex * 0.69314718055994530942;
+        off = cadd(off, cscale(cmul(r, cexp(z)), el));
+    }
+    off = warp_csum(off);
+    diag = warp_sum(diag);
     if (lane == 0) reinterpret_cast<double2 *>(A.eloc)[k] = make_double2(diag + off.x, off.y);
 }
 
@@ -300,13 +467,24 @@ __global__ void k_crbm_jacobian(int N, int M, const double *__restrict__ p, cons
     }
 }
 
-// Column means of a complex [rows][cols] matrix: one thread per column.
-__global__ void k_ccolmean(int64_t rows, int64_t cols, const double2 *__restrict__ O, double2 *__restrict__ mean) {
-    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= cols) return;
+// Column means of a complex [rows][cols] matrix: 32 columns a block, 32 threads
+// a column (one thread a column waited on its loads: 0.8 ms for 440 columns of
+// 4096 rows), summed in a fixed order.
+__global__ void __launch_bounds__(1024) k_ccolmean(int64_t rows, int64_t cols, const double2 *__restrict__ O,
+                                                   double2 *__restrict__ mean) {
+    __shared__ double2 part[32][33];
+    const int c = threadIdx.x & 31, y = threadIdx.x >> 5;
+    const int64_t q = (int64_t)blockIdx.x * 32 + c;
     double2 acc = make_double2(0.0, 0.0);
-    for (int64_t k = 0; k < rows; ++k) acc = cadd(acc, O[(size_t)k * cols + q]);
-    mean[q] = cscale(acc, 1.0 / (double)rows);
+    if (q < cols) {
+#pragma unroll 4
+        for (int64_t k = y; k < rows; k += 32) acc = cadd(acc, O[(size_t)k * cols + q]);
+    }
+    part[c][y] = acc;
+    __syncthreads();
+    const double2 v = warp_csum(part[y][c]);  // warp y sums column y of the block
+    const int64_t qo = (int64_t)blockIdx.x * 32 + y;
+    if (c == 0 && qo < cols) mean[qo] = cscale(v, 1.0 / (double)rows);
 }
 
 // The realified centred Jacobian R [2 rows][2 cols]: with dO = X + i Y
@@ -428,26 +606,43 @@ cudaError_t launch_crbm_sweep(int N, int M, const double *p, int rule, int E, co
                               int64_t sweep0, int n_discard, int n_samples, uint64_t seed, uint32_t stream_id,
                               int8_t *samples, unsigned long long *n_accepted, cudaStream_t st) {
     if (C <= 0) return cudaSuccess;
-    CSweepArgs a{N, M, E, rule, C, p, edges, s, sweep0, n_discard, n_samples, seed, stream_id, samples, n_accepted};
-    const size_t smem = 4 * cwarp_bytes(N, M);
+    const int wb = (int)(((size_t)M * (sizeof(double2) + sizeof(float2)) + (size_t)N + 15) / 16 * 16);
+    CSweepArgs a{N, M, E, rule, C, p, edges, s, sweep0, n_discard, n_samples, seed, stream_id, samples, n_accepted,
+                 wb};
+    int wpb = 4;
+    while (wpb > 1 && (size_t)wpb * wb > 227 * 1024) wpb >>= 1;
+    if ((size_t)wpb * wb > 227 * 1024) return cudaErrorInvalidValue;
     cudaError_t e = nk::allow_max_dynamic_smem((const void *)k_crbm_sweep);
     if (e != cudaSuccess) return e;
     const int slot = prof_begin(NK_PROF_SWEEP, st);
-    (k_crbm_sweep<<<nblk(C, 4), 128, smem, st>>>(a), nk::note_launch());
+    (k_crbm_sweep<<<nblk(C, wpb), 32 * wpb, (size_t)wpb * wb, st>>>(a), nk::note_launch());
     prof_end(slot, st, (double)C * (n_discard + n_samples) * N * (double)M);
     return cudaGetLastError();
 }
 
+size_t crbm_eloc_ws_bytes(int N, int M) { return (size_t)2 * N * M * sizeof(double2); }
+
 cudaError_t launch_crbm_eloc(int N, int M, const double *p, const nk_ham *ham, const int8_t *s, int64_t Ns,
-                             double *eloc, cudaStream_t st) {
+                             double *eloc, void *ws, cudaStream_t st) {
     if (Ns <= 0) return cudaSuccess;
+    const int64_t nw = (int64_t)N * M;
+    double2 *ep = static_cast<double2 *>(ws), *em = ep + nw;
+    (k_crbm_exp_tables<<<nblk(nw, 256), 256, 0, st>>>(nw, reinterpret_cast<const double2 *>(p) + N + M, ep, em),
+     nk::note_launch());
+    const bool pairs = ham->kind != NK_TFIM;
+    const int pq = M * 2 * (int)sizeof(double2), sb = (N + 15) / 16 * 16;
+    const size_t lb = ((size_t)ham->n_edges * 4 + 15) / 16 * 16;
+    const bool compact = pairs && (size_t)pq + sb + lb <= 100 * 1024;
+    const size_t wb = (size_t)pq + sb + (compact ? lb : 0);
+    int wpb = 4;
+    while (wpb > 1 && wpb * wb > 227 * 1024) wpb >>= 1;
+    if (wpb * wb > 227 * 1024) return cudaErrorInvalidValue;
     CElocArgs a{N, M, ham->n_edges, ham->n_edges2, ham->kind, ham->marshall, ham->J, ham->J2, ham->h,
-                p, ham->edges, s, Ns, eloc};
-    const size_t smem = 4 * cwarp_bytes(N, M);
+                p, ep, em, ham->edges, s, Ns, eloc, (int)wb, pq, sb, compact ? 1 : 0};
     cudaError_t e = nk::allow_max_dynamic_smem((const void *)k_crbm_eloc);
     if (e != cudaSuccess) return e;
     const int slot = prof_begin(NK_PROF_ELOC, st);
-    (k_crbm_eloc<<<nblk(Ns, 4), 128, smem, st>>>(a), nk::note_launch());
+    (k_crbm_eloc<<<nblk(Ns, wpb), 32 * wpb, wpb * wb, st>>>(a), nk::note_launch());
     prof_end(slot, st, (double)Ns * (ham->kind == NK_TFIM ? N : 0.5 * ham->n_edges) * (double)M);
     return cudaGetLastError();
 }
@@ -463,7 +658,7 @@ cudaError_t launch_crbm_jacobian(int N, int M, const double *p, const int8_t *s,
 }
 
 cudaError_t launch_crealify(int64_t rows, int64_t cols, const double *O, double *mean, double *R, cudaStream_t st) {
-    (k_ccolmean<<<nblk(cols, 128), 128, 0, st>>>(rows, cols, reinterpret_cast<const double2 *>(O),
+    (k_ccolmean<<<nblk(cols, 32), 1024, 0, st>>>(rows, cols, reinterpret_cast<const double2 *>(O),
                                                  reinterpret_cast<double2 *>(mean)), nk::note_launch());
     (k_realify<<<nblk(rows * cols, 256), 256, 0, st>>>(rows, cols, reinterpret_cast<const double2 *>(O),
                                                        reinterpret_cast<const double2 *>(mean), R), nk::note_launch());

@@ -1492,7 +1492,7 @@ nk_status check_complex_out(const double *p, const char *name) {
 struct TdvpWs {
     int8_t *samples;
     double *eloc, *stats4, *O, *mean, *R, *g, *F, *rhs, *S, *V, *ev, *evmax, *z, *gpart, *partial;
-    void *eig, *tc, *syrk;
+    void *eig, *tc, *syrk, *exps;
     int *info, *kept;
     unsigned long long *acc;
 };
@@ -1505,7 +1505,7 @@ nk_status tdvp_slope(nk_ctx *ctx, int N, int M, const double *p, const nk_ham *h
                                 n_discard, cfg->n_samples, cfg->seed, cfg->stream_id, w.samples, w.acc, st),
           "sweep");
     chains->sweeps_done += n_discard + cfg->n_samples;
-    NK_CU(nk::launch_crbm_eloc(N, M, p, ham, w.samples, Ns, w.eloc, st), "local energy");
+    NK_CU(nk::launch_crbm_eloc(N, M, p, ham, w.samples, Ns, w.eloc, w.exps, st), "local energy");
     NK_CU(nk::launch_cstats(Ns, w.eloc, w.stats4, st), "stats");
     NK_CU(nk::launch_crbm_jacobian(N, M, p, w.samples, Ns, w.O, st), "jacobian");
     NK_CU(nk::launch_crealify(Ns, Np, w.O, w.mean, w.R, st), "realify");
@@ -1596,10 +1596,13 @@ nk_status nk_crbm_local_energy(nk_ctx *ctx, const nk_crbm *rbm, const nk_ham *ha
     if (Ns == 0) return NK_OK;
     NK_DEV(s, "s");
     if ((st0 = check_complex_out(eloc_out, "eloc_out")) != NK_OK) return st0;
-    if (g_plan_only) return NK_OK;
-    NK_CU(nk::launch_crbm_eloc(rbm->N, rbm->M, rbm->params, ham, s, Ns, eloc_out, (cudaStream_t)stream),
-          "local energy");
-    return NK_OK;
+    return with_workspace(ctx, [&](Carver &c, bool run) -> nk_status {
+        void *exps = c.take<char>(nk::crbm_eloc_ws_bytes(rbm->N, rbm->M));
+        if (!run) return NK_OK;
+        NK_CU(nk::launch_crbm_eloc(rbm->N, rbm->M, rbm->params, ham, s, Ns, eloc_out, exps, (cudaStream_t)stream),
+              "local energy");
+        return NK_OK;
+    });
 }
 
 nk_status nk_crbm_jacobian(nk_ctx *ctx, const nk_crbm *rbm, const int8_t *s, int64_t Ns, double *O_out,
@@ -1665,6 +1668,7 @@ nk_status nk_tdvp_step(nk_ctx *ctx, nk_crbm *rbm, const nk_ham *ham, nk_chains *
         w.acc = c.take<unsigned long long>(C);
         w.tc = c.take<char>(nk::tc_chol_ws_bytes(n));
         w.syrk = c.take<char>(nk::syrk_ws_bytes(2 * Ns, n));
+        w.exps = c.take<char>(nk::crbm_eloc_ws_bytes(N, M));
         if (svd) {
             w.V = c.take<double>((size_t)n * n);
             w.ev = c.take<double>(n);

@@ -345,8 +345,9 @@ cudaError_t launch_crbm_logpsi(int N, int M, const double *p, const int8_t *s, i
 cudaError_t launch_crbm_sweep(int N, int M, const double *p, int rule, int E, const int32_t *edges, int C, int8_t *s,
                               int64_t sweep0, int n_discard, int n_samples, uint64_t seed, uint32_t stream_id,
                               int8_t *samples, unsigned long long *n_accepted, cudaStream_t st);
+size_t crbm_eloc_ws_bytes(int N, int M);  // the tables e^{+-2 W}
 cudaError_t launch_crbm_eloc(int N, int M, const double *p, const nk_ham *ham, const int8_t *s, int64_t Ns,
-                             double *eloc, cudaStream_t st);
+                             double *eloc, void *ws, cudaStream_t st);
 cudaError_t launch_crbm_jacobian(int N, int M, const double *p, const int8_t *s, int64_t Ns, double *O,
                                  cudaStream_t st);
 // mean: complex [cols] scratch; R [2 rows][2 cols] the realified centred O.
