@@ -76,11 +76,6 @@ struct SgArgs {
     int drop;             // low bits left out of the recombined product; -1: ten (window10)
 };
 
-// Columns whose exponent is outside this range (an infinity or a NaN among
-// the entries, or values whose products could leave the FP64 range) are not
-// cut into slices but multiplied out in FP64 by the epilogue.
-__host__ __device__ inline bool flagged_exp(int e) { return e > 900 || (e < -900 && e > -100000); }
-
 // Output (row, col) over k in [k0, k1) in FP64, from the unsliced operands.
 __device__ __noinline__ double raw_product(const SgRaw &w, int64_t row, int64_t col, int64_t k0, int64_t k1) {
     double acc = 0.0;
@@ -841,6 +836,46 @@ __global__ void k_slice_rows_h3(const double *__restrict__ X, int64_t ldx, int64
     if (threadIdx.x == 0) expo[r] = e;
 }
 
+// Rows of X [rows][K] into 5 FP16 slices of digits in base 4096 (each in
+// [-2048, 2048], exact in FP16) of the integers y = x 2^(bits - e), |x| < 2^e:
+// bits 59, rounded to nearest (NK_F64), or 56, truncated: the integers of the
+// 7-slice products, so that NK_MIXED activations keep their every bit.  out
+// [5][rows][ld], one block per row; rows whose exponent is flagged get zeros.
+__global__ void k_slice_rows_h5(const double *__restrict__ X, int64_t rows, int64_t K, int64_t ld, int bits,
+                                __half *__restrict__ out, int *__restrict__ expo) {
+    const int64_t r = blockIdx.x;
+    if (r >= rows) return;
+    int ex = -100000;
+    for (int64_t k = threadIdx.x; k < K; k += blockDim.x) ex = max(ex, exp_of(X[(size_t)r * K + k]));
+    __shared__ int red[4];
+    ex = __reduce_max_sync(0xffffffffu, ex);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ex;
+    __syncthreads();
+    ex = max(max(red[0], red[1]), max(red[2], red[3]));
+    const int e = ex == -100000 ? 0 : ex;
+    const int64_t plane = rows * ld;
+    for (int64_t k = threadIdx.x; k < ld; k += blockDim.x) {
+        long long y = 0;
+        if (k < K && !flagged_exp(e)) {
+            int b;
+            unsigned long long m;
+            bool neg;
+            split_bits(X[(size_t)r * K + k], b, m, neg);
+            const long long u = m ? (long long)grid_bits(m, b - 1075 + bits - e, bits != 56) : 0;
+            y = neg ? -u : u;
+        }
+        __half *o = out + (size_t)r * ld + k;
+#pragma unroll
+        for (int t = 4; t >= 1; --t) {
+            const int d = (int)((y + 2048) & 4095) - 2048;
+            y = (y - d) >> 12;
+            o[(size_t)t * plane] = __int2half_rn(d);
+        }
+        o[0] = __int2half_rn((int)y);
+    }
+    if (threadIdx.x == 0) expo[r] = e;
+}
+
 // Rows of a row-major FP64 matrix (row r, column k: X[r * ldx + k] for k < K;
 // with augment, column K holds aug[r] and the operand has K + 1 columns) ->
 // SB slices [SB][rows][ld] with one exponent per row.  One block per row.
@@ -1370,13 +1405,14 @@ double sgemm_flops(int64_t rows, int64_t cols, int64_t K, int SB) {
 
 size_t tc_theta_ws_bytes(int N, int M, int64_t B) {
     const int64_t ld = pad8(N);
-    return ((size_t)B * ld * 2 + 255) / 256 * 256 + ((size_t)kMaxSB * M * ld * 2 + 255) / 256 * 256 +
+    return ((size_t)B * ld * 2 + 255) / 256 * 256 + ((size_t)5 * M * ld * 2 + 255) / 256 * 256 +
            ((size_t)M * 4 + 255) / 256 * 256 + 256;
 }
 
-// theta [B][M] = S W^T + b with W sliced 7 ways: exact up to 2^-56 of max|W_j|.
+// theta [B][M] = S W^T + b with W in 5 FP16 slices (k_theta.cu).
 cudaError_t launch_theta_tc(int N, int M, const double *b, const double *W, const int8_t *s, int64_t B,
-                            double *theta, int *err, void *ws, cudaStream_t st, int64_t ldtheta, bool wide) {
+                            double *theta, int *err, void *ws, cudaStream_t st, int64_t ldtheta, bool wide,
+                            bool sliced) {
     if (B <= 0) return cudaSuccess;
     const int64_t ld = pad8(N);
     char *p = static_cast<char *>(ws);
@@ -1385,15 +1421,16 @@ cudaError_t launch_theta_tc(int N, int M, const double *b, const double *W, cons
         p += (bytes + 255) / 256 * 256;
         return q;
     };
-    auto *As = reinterpret_cast<__nv_bfloat16 *>(take((size_t)B * ld * 2));
-    auto *Ws = reinterpret_cast<__nv_bfloat16 *>(take((size_t)kMaxSB * M * ld * 2));
+    auto *As = reinterpret_cast<__half *>(take((size_t)B * ld * 2));
+    auto *Ws = reinterpret_cast<__half *>(take((size_t)5 * M * ld * 2));
     auto *ew = reinterpret_cast<int *>(take((size_t)M * 4));
     (k_pm1_rows<<<nblk(B * ld, 256), 256, 0, st>>>(s, B, N, 0, ld, As), nk::note_launch());
-    (k_slice_long_rows<<<M, 128, 0, st>>>(W, N, M, N, nullptr, kMaxSB, ld, Ws, ew, wide), nk::note_launch());
+    if (!sliced) (k_slice_rows_h5<<<M, 128, 0, st>>>(W, M, N, ld, wide ? 59 : 56, Ws, ew), nk::note_launch());
     const int slot = prof_begin(NK_PROF_JVP_VJP, st);
-    cudaError_t e = sgemm(As, B, ld, Ws, ew, M, ld, N, kMaxSB, theta, ldtheta > 0 ? ldtheta : M, 0, b, err, st,
-                          SgRaw{s, W, nullptr, N, N, 0}, wide);
-    prof_end(slot, st, 2.0 * (double)B * N * (double)M, sgemm_flops(B, M, N, kMaxSB));
+    cudaError_t e = launch_theta_product(As, B, ld, Ws, ew, M, N, b, theta, ldtheta > 0 ? ldtheta : M,
+                                         wide ? 59 : 56, s, W, err,
+                                         st);
+    prof_end(slot, st, 2.0 * (double)B * N * (double)M, sgemm_flops(B, M, N, 5));
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 

@@ -585,7 +585,7 @@ nk_status run_sweeps(nk_ctx *ctx, const nk::Tables<R> &t, const nk::SweepArgs &a
     }
     const int total = a.n_discard + a.n_samples;
     for (int w = 0; w < total; ++w) {
-        NK_CU(nk::launch_theta_tc(t.N, t.M, t.b, t.W, a.s, a.C, theta, ctx->tc_err, tcm, st), "theta");
+        NK_CU(nk::launch_theta_tc(t.N, t.M, t.b, t.W, a.s, a.C, theta, ctx->tc_err, tcm, st, 0, false, w > 0), "theta");
         nk::SweepArgs b = a;
         b.sweep0 = a.sweep0 + w;
         b.n_discard = w < a.n_discard ? 1 : 0;
@@ -660,7 +660,8 @@ nk_status run_sweeps_theta(nk_ctx *ctx, const nk::Tables<R> &t, const nk::Tables
         // sample 0's rows serve as scratch until its own theta arrives)
         const int q = w - 1 - nd;
         double *th = b.theta + (size_t)(q > 0 ? q : 0) * M;
-        NK_CU(nk::launch_theta_tc(N, M, t.b, t.W, a.s, C, th, ctx->tc_err, b.tcm, st, (int64_t)ns * M), "theta");
+        NK_CU(nk::launch_theta_tc(N, M, t.b, t.W, a.s, C, th, ctx->tc_err, b.tcm, st, (int64_t)ns * M, false, w > 0),
+              "theta");
         if (w == total) break;
         nk::SweepArgs sa = a;
         sa.sweep0 = a.sweep0 + w;

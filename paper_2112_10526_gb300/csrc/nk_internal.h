@@ -231,10 +231,17 @@ inline size_t syrk_ws_bytes(int64_t rows, int64_t n) { return syrk_on_tensor(row
 // ---- tensor-core products with the configurations (k_sgemm.cu) -------------
 size_t tc_theta_ws_bytes(int N, int M, int64_t B);
 // theta [B][M] = S W^T + b, exact to 2^-56 of max|W_j| (7 slices); row r of
-// theta at theta + r * ldtheta (0: M).
+// theta at theta + r * ldtheta (0: M).  sliced: ws still holds the slices of W
+// from the last call with the same N, M, B and W.
 cudaError_t launch_theta_tc(int N, int M, const double *b, const double *W, const int8_t *s, int64_t B,
                             double *theta, int *err, void *ws, cudaStream_t st, int64_t ldtheta = 0,
-                            bool wide = false);
+                            bool wide = false, bool sliced = false);
+// Its product (k_theta.cu): A the +-1 configurations in BF16 [rows][ldA], Wsl
+// the 7 slices [7][units][ldA] of W with row exponents expW; s and W (unsliced)
+// serve units whose weights the slices cannot hold.
+cudaError_t launch_theta_product(const __nv_bfloat16 *A, int64_t rows, int64_t ldA, const __nv_bfloat16 *Wsl,
+                                 const int *expW, int units, int N, const double *bias, double *out, int64_t ld,
+                                 bool wide, const int8_t *s, const double *W, int *err, cudaStream_t st);
 // wide, here and in the products below (NK_F64): the slices' sums are turned
 // into FP64 with every bit that the length of the sums leaves room for.
 // The +-1 operands of the two Jacobian products depend on the samples only:

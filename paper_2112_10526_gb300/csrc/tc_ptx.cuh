@@ -259,6 +259,11 @@ __device__ __forceinline__ void split_bits(double x, int &biased, unsigned long 
     else biased = 1;  // subnormal: value = mant 2^(1 - 1075)
 }
 
+// Operand rows whose exponent is outside this range (an infinity or a NaN among
+// the entries, or values whose products could leave the FP64 range; -100000: a
+// row of zeros) are not cut into slices but multiplied out in FP64.
+__host__ __device__ __forceinline__ bool flagged_exp(int e) { return e > 900 || (e < -900 && e > -100000); }
+
 __host__ __device__ __forceinline__ int clz64_any(unsigned long long x) {
 #ifdef __CUDA_ARCH__
     return __clzll((long long)x);

@@ -19,9 +19,10 @@ from gpu_util import cu, dev
 
 pytestmark = pytest.mark.gpu
 
-# (N, M, B): one tile and less, ragged tiles, just below and above 4e6, well above
+# (N, M, B): one tile and less, ragged tiles, just below and above 4e6, well above,
+# more tiles than SMs (clusters; an odd count of row tiles), N beyond one resident row
 SIZES = [(1, 1, 1), (16, 16, 256), (15, 17, 33), (37, 45, 1025), (50, 80, 999), (50, 80, 1000), (129, 191, 257),
-         (144, 288, 1500)]
+         (144, 288, 1500), (30, 700, 1600), (600, 100, 300), (65, 40, 5000)]
 
 
 @pytest.fixture(scope="module")
