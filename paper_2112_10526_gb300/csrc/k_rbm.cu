@@ -20,6 +20,8 @@
 
 #include "nk_common.cuh"
 #include "nk_internal.h"
+#include "tanh64.cuh"
+#include "tc_ptx.cuh"
 
 namespace nk {
 
@@ -43,12 +45,106 @@ __global__ void k_transpose_W(int N, int M, const double *__restrict__ W, double
     }
 }
 
+// x in [-1, 1] as 2^63 x, +-1 as the nearest FP64 number below (so that a factor
+// of two such numbers stays below 2).  A NaN reads as 1.
+__device__ __forceinline__ long long to_fixed63(double x) {
+    int b;
+    unsigned long long m;
+    bool neg;
+    split_bits(x, b, m, neg);
+    const int sh = b - 1012;  // m 2^(b - 1075 + 63)
+    constexpr unsigned long long kMost = 0x7FFFFFFFFFFFFC00ULL;  // 2^63 (1 - 2^-53)
+    unsigned long long y = sh >= 0 ? (sh > 10 ? kMost : m << sh)
+                                   : (sh <= -54 ? 0ULL : (m >> (-sh)) + ((m >> (-sh - 1)) & 1ULL));
+    if (y > kMost) y = kMost;
+    return neg ? -(long long)y : (long long)y;
+}
+
+template <typename R>
+__device__ __forceinline__ typename TauOf<R>::type to_tau(double x);
+template <>
+__device__ __forceinline__ float to_tau<float>(double x) {
+    return (float)x;
+}
+template <>
+__device__ __forceinline__ long long to_tau<double>(double x) {
+    return to_fixed63(x);
+}
+
+// The exponent of every unit's weights (column j of Wt; |W| < 2^e, 0 for zero
+// weights, 100000 with an infinity or a NaN) and Wt in place as the integers
+// (y >> 30, y & (2^30 - 1)), y = rint(W 2^(59 - e)): the integers of the wide
+// slices of k_slice_rows_h5, so that activations summed from either are the
+// same to the last bit.  Units whose exponent is flagged (infinities, NaNs,
+// magnitudes near the ends of the FP64 range) keep their FP64 weights.
+__global__ void __launch_bounds__(256) k_fix_weights(int N, int M, double *__restrict__ Wt, int *__restrict__ eW) {
+    const int c = threadIdx.x & 31, y = threadIdx.x >> 5;
+    const int j = blockIdx.x * 32 + c;
+    int ex = -100000;
+    if (j < M)
+        for (int i = y; i < N; i += 8) {
+            int b;
+            unsigned long long m;
+            bool neg;
+            split_bits(Wt[(size_t)i * M + j], b, m, neg);
+            if (m) ex = max(ex, b == 2047 ? 100000 : b - 1022);
+        }
+    __shared__ int red[8][32];
+    red[y][c] = ex;
+    __syncthreads();
+    for (int q = 0; q < 8; ++q) ex = max(ex, red[q][c]);
+    const int e = ex == -100000 ? 0 : ex;
+    if (j >= M) return;
+    if (y == 0) eW[j] = e;
+    if (flagged_exp(e)) return;
+    for (int i = y; i < N; i += 8) {
+        int b;
+        unsigned long long m;
+        bool neg;
+        split_bits(Wt[(size_t)i * M + j], b, m, neg);
+        long long v = 0;
+        if (m) {
+            const int sh = b - 1075 + 59 - e;
+            const unsigned long long u =
+                sh >= 0 ? m << sh : (sh <= -64 ? 0ULL : (m >> (-sh)) + ((m >> (-sh - 1)) & 1ULL));
+            v = neg ? -(long long)u : (long long)u;
+        }
+        reinterpret_cast<int2 *>(Wt)[(size_t)i * M + j] = make_int2((int)(v >> 30), (int)(v & 0x3FFFFFFF));
+    }
+}
+
+// theta_j = b_j + sum_i W_ji s_i from the integers of k_fix_weights (exact sum,
+// rounded once): two 64-bit multiply-adds a site on the integer pipe.  drop =
+// theta_drop(N).
+__host__ __device__ inline int theta_drop(int N) { return window_drop(8LL * N); }
+
+__device__ __forceinline__ double fixed_theta(const Tables<double> &T, const int8_t *sv, int j, int drop) {
+    const int e = T.eW[j];
+    double v;
+    if (flagged_exp(e)) {
+        v = 0.0;
+        for (int i = 0; i < T.N; ++i) v = fma((double)sv[i], T.Wt[(size_t)i * T.M + j], v);
+    } else {
+        const int2 *w = reinterpret_cast<const int2 *>(T.Wt) + j;
+        long long hi = 0, lo = 0;
+#pragma unroll 4
+        for (int i = 0; i < T.N; ++i) {
+            const int2 y = __ldg(w + (size_t)i * T.M);
+            const int s = sv[i];
+            hi += (long long)s * y.x;
+            lo += (long long)s * y.y;
+        }
+        v = window_to_double((long long)((unsigned long long)hi << (30 - drop)) + (lo >> drop), e - 59 + drop);
+    }
+    return v + T.b[j];
+}
+
 // One block per site (or edge): tau row, its transpose and K by a fixed-order
 // block reduction.
 template <typename R>
 __global__ void k_tau_rows(int N, int M, int nrows, const double *__restrict__ Wt,
-                           const int32_t *__restrict__ edges, R *__restrict__ tau,
-                           R *__restrict__ tauT, R *__restrict__ K, float *__restrict__ tauf,
+                           const int32_t *__restrict__ edges, typename TauOf<R>::type *__restrict__ tau,
+                           typename TauOf<R>::type *__restrict__ tauT, R *__restrict__ K, float *__restrict__ tauf,
                            double *__restrict__ D) {
     int r = blockIdx.x;
     if (r >= nrows) return;
@@ -64,9 +160,9 @@ __global__ void k_tau_rows(int N, int M, int nrows, const double *__restrict__ W
     double part = 0.0;
     for (int j = threadIdx.x; j < M; j += blockDim.x) {
         double d = w1 ? (w0[j] - w1[j]) : w0[j];
-        double v = tanh(2.0 * d);
-        if (tau) tau[(size_t)r * M + j] = (R)v;
-        if (tauT) tauT[(size_t)j * nrows + r] = (R)v;
+        const double v = tanh64(2.0 * d);
+        if (tau) tau[(size_t)r * M + j] = to_tau<R>(v);
+        if (tauT) tauT[(size_t)j * nrows + r] = to_tau<R>(v);
         if (tauf) {
             tauf[(size_t)r * M + j] = (float)v;
             D[(size_t)r * M + j] = 2.0 * d;
@@ -122,9 +218,9 @@ __global__ void k_logpsi_theta(int N, int M, const double *__restrict__ a, const
     if (lane == 0) out[k] = part;
 }
 
-__global__ void k_tanh_inplace(int64_t n, double *__restrict__ x) {
+__global__ void k_tanh_inplace(int64_t n, double *__restrict__ x, bool lib) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) x[i] = tanh(x[i]);
+    if (i < n) x[i] = lib ? tanh(x[i]) : tanh64(x[i]);
 }
 
 // ------------------------------------------------------------- chain init ---
@@ -159,9 +255,9 @@ __global__ void k_chain_init(int N, int C, int rule, unsigned long long seed, un
 // prod over j = j0, j0 + step, ... < M of (1 - si t_j tau[j * tstride]) as
 // mantissa x 2^exp.  Four independent running products (each renormalised
 // every RenormEvery factors) keep several loads and multiplies in flight.
-template <typename R>
-__device__ __forceinline__ Prod<R> strided_product(const R *__restrict__ t, const R *__restrict__ tau, size_t tstride,
-                                                   R si, int j0, int step, int M) {
+__device__ __forceinline__ Prod<float> strided_product(const float *__restrict__ t, const float *__restrict__ tau,
+                                                       size_t tstride, float si, int j0, int step, int M) {
+    using R = float;
     R m0 = R(1), m1 = R(1), m2 = R(1), m3 = R(1);
     int e = 0, cnt = 0;
     int j = j0;
@@ -194,6 +290,47 @@ __device__ __forceinline__ Prod<R> strided_product(const R *__restrict__ t, cons
     p.m *= m3;
     renorm(p);
     return p;
+}
+
+// The same product for NK_F64 from 2^63 t and 2^63 tau in 64-bit integers: a
+// factor 1 - s t tau is 2^62 -+ the high half of a product, good to 2^-62, and
+// the running mantissa (leading one at bit 63) takes two factors and one
+// normalisation a step.  An FP64 multiply-add or multiply costs 64 clocks a warp
+// and scheduler, a 64-bit high product about 11: 30 clocks a factor against 192
+// (multiply, multiply-add, multiply).
+struct FixProd {
+    unsigned long long m;
+    int e;
+};
+__device__ __forceinline__ unsigned long long fixed_factor(long long t, long long tau, bool up) {
+    const long long p = __mul64hi(t, tau);  // 2^62 t tau
+    return (unsigned long long)((1LL << 62) - (up ? p : -p)) << 1;  // 2^63 (1 - s t tau), in [0, 2^64)
+}
+__device__ __forceinline__ void fixed_mul(FixProd &a, unsigned long long f, int point) {
+    const unsigned long long r = __umul64hi(a.m, f);  // 2^(point - 1) of the product
+    const int z = __clz((int)(r >> 32));              // 32 once the high word is empty: the next step goes on
+    a.m = r << z;
+    a.e += 64 - point - z;
+}
+
+__device__ __forceinline__ Prod<double> strided_product(const long long *__restrict__ t,
+                                                        const long long *__restrict__ tau, size_t tstride, double si,
+                                                        int j0, int step, int M) {
+    const bool up = si > 0.0;
+    FixProd a{1ULL << 63, 0}, b{1ULL << 63, 0};
+    int j = j0;
+    for (; j + 3 * step < M; j += 4 * step) {
+        const unsigned long long f0 = fixed_factor(t[j], tau[(size_t)j * tstride], up);
+        const unsigned long long f1 = fixed_factor(t[j + step], tau[(size_t)(j + step) * tstride], up);
+        const unsigned long long f2 = fixed_factor(t[j + 2 * step], tau[(size_t)(j + 2 * step) * tstride], up);
+        const unsigned long long f3 = fixed_factor(t[j + 3 * step], tau[(size_t)(j + 3 * step) * tstride], up);
+        fixed_mul(a, __umul64hi(f0, f1), 62);
+        fixed_mul(b, __umul64hi(f2, f3), 62);
+    }
+    for (; j < M; j += step) fixed_mul(a, fixed_factor(t[j], tau[(size_t)j * tstride], up), 63);
+    fixed_mul(a, b.m, 63);
+    // value = m 2^-63 2^(a.e + b.e), as a mantissa in [1/2, 1)
+    return Prod<double>{window_to_double((long long)(a.m >> 1), -63), a.e + b.e + 1};
 }
 
 // Lanes over hidden units, four consecutive units per lane (16-byte loads of
@@ -319,7 +456,7 @@ template <bool kRing>
 __device__ __forceinline__ Prod<float> unit_lanes_product(const float *t, const float *tau, float si, int lane, int M,
                                                           bool vec4) {
     return vec4 ? lane_product4<false, kRing>(t, tau, si, lane, M)
-                : strided_product<float>(t, tau, 1, si, lane, 32, M);
+                : strided_product(t, tau, 1, si, lane, 32, M);
 }
 
 // lane_product4 on a tau row already held in registers: uv[u] is the chunk j
@@ -644,25 +781,15 @@ __global__ void __launch_bounds__(128) k_sweep_screened(SweepK<double> P) {
     for (int i = lane; i < N; i += 32) sv[i] = A.s[(size_t)c * N + i];
     __syncwarp();
     unsigned long long acc = 0;
-    const int n_sweeps = A.n_discard + A.n_samples;
+    const int n_sweeps = A.n_discard + A.n_samples, drop = theta_drop(N);
     for (int w = 0; w < n_sweeps; ++w) {
-        // theta = b + W s from scratch (FP64), t = tanh theta
+        // theta = b + W s from scratch, t = tanh theta
         for (int j = lane; j < M; j += 32) {
             double v;
             if (A.theta_in) {
                 v = A.theta_in[(size_t)c * (A.theta_ld > 0 ? A.theta_ld : M) + j];
             } else {
-                // four chains of FMAs over the sites
-                double q0 = T.b[j], q1 = 0.0, q2 = 0.0, q3 = 0.0;
-                int i = 0;
-                for (; i + 3 < N; i += 4) {
-                    q0 = fma(T.Wt[(size_t)i * M + j], (double)sv[i], q0);
-                    q1 = fma(T.Wt[(size_t)(i + 1) * M + j], (double)sv[i + 1], q1);
-                    q2 = fma(T.Wt[(size_t)(i + 2) * M + j], (double)sv[i + 2], q2);
-                    q3 = fma(T.Wt[(size_t)(i + 3) * M + j], (double)sv[i + 3], q3);
-                }
-                for (; i < N; ++i) q0 = fma(T.Wt[(size_t)i * M + j], (double)sv[i], q0);
-                v = (q0 + q1) + (q2 + q3);
+                v = fixed_theta(T, sv, j, drop);
             }
             th[j] = v;
             t[j] = tanhf((float)v);
@@ -845,7 +972,7 @@ __global__ void __launch_bounds__(128) k_sweep_screened_regs(SweepK<double> P) {
     for (int i = lane; i < N; i += 32) sv[i] = A.s[(size_t)c * N + i];
     __syncwarp();
     unsigned long long acc = 0;
-    const int n_sweeps = A.n_discard + A.n_samples;
+    const int n_sweeps = A.n_discard + A.n_samples, drop = theta_drop(N);
     bool in[kU];
 #pragma unroll
     for (int u = 0; u < kU; ++u) in[u] = lane + 32 * u < M;
@@ -860,16 +987,7 @@ __global__ void __launch_bounds__(128) k_sweep_screened_regs(SweepK<double> P) {
                 if (A.theta_in) {
                     v = A.theta_in[(size_t)c * (A.theta_ld > 0 ? A.theta_ld : M) + j];
                 } else {
-                    double q0 = T.b[j], q1 = 0.0, q2 = 0.0, q3 = 0.0;
-                    int i = 0;
-                    for (; i + 3 < N; i += 4) {
-                        q0 = fma(T.Wt[(size_t)i * M + j], (double)sv[i], q0);
-                        q1 = fma(T.Wt[(size_t)(i + 1) * M + j], (double)sv[i + 1], q1);
-                        q2 = fma(T.Wt[(size_t)(i + 2) * M + j], (double)sv[i + 2], q2);
-                        q3 = fma(T.Wt[(size_t)(i + 3) * M + j], (double)sv[i + 3], q3);
-                    }
-                    for (; i < N; ++i) q0 = fma(T.Wt[(size_t)i * M + j], (double)sv[i], q0);
-                    v = (q0 + q1) + (q2 + q3);
+                    v = fixed_theta(T, sv, j, drop);
                 }
             }
             th[u] = v;
@@ -1165,7 +1283,8 @@ __global__ void __launch_bounds__(128) k_eloc(ElocK<R> P) {
     if (k >= A.Ns) return;
     const int N = T.N, M = T.M, E = T.E;
     unsigned char *base = sm + (size_t)warp * P.warp_bytes;
-    R *t = reinterpret_cast<R *>(base);
+    using Tau = typename TauOf<R>::type;
+    Tau *t = reinterpret_cast<Tau *>(base);
     int8_t *sv = reinterpret_cast<int8_t *>(base + P.t_bytes);
     int *list = reinterpret_cast<int *>(base + P.t_bytes + P.s_bytes);
     for (int i = lane; i < N; i += 32) sv[i] = A.s[(size_t)k * N + i];
@@ -1174,12 +1293,14 @@ __global__ void __launch_bounds__(128) k_eloc(ElocK<R> P) {
         double th;
         if (A.theta_in) {
             th = A.theta_in[(size_t)k * M + j];
+        } else if constexpr (sizeof(R) == 8) {
+            th = fixed_theta(T, sv, j, theta_drop(N));
         } else {
             th = T.b[j];
             for (int i = 0; i < N; ++i) th = fma(T.Wt[(size_t)i * M + j], (double)sv[i], th);
         }
-        const double tj = tanh(th);
-        t[j] = (R)tj;
+        const double tj = A.lib_tanh ? tanh(th) : tanh64(th);
+        t[j] = to_tau<R>(tj);
         if (A.t_out) A.t_out[(size_t)k * M + j] = tj;
     }
     // edges [0, E1) couple with J, the next-nearest ones [E1, E) with J2
@@ -1196,7 +1317,7 @@ __global__ void __launch_bounds__(128) k_eloc(ElocK<R> P) {
         // large M: lanes over hidden units, one warp reduction per site
         for (int i = 0; i < N; ++i) {
             const R si = (R)sv[i];
-            Prod<R> pr = strided_product<R>(t, T.tau_site + (size_t)i * M, 1, si, lane, 32, M);
+            Prod<R> pr = strided_product(t, T.tau_site + (size_t)i * M, 1, si, lane, 32, M);
             pr = warp_prod(pr);
             const double delta = -2.0 * T.a[i] * (double)si + (double)(T.K_site[i] + prod_log(pr));
             if (lane == 0) off += -A.h * exp(delta);
@@ -1205,7 +1326,7 @@ __global__ void __launch_bounds__(128) k_eloc(ElocK<R> P) {
         // small M: lanes over sites, each over all hidden units
         for (int i = lane; i < N; i += 32) {
             const R si = (R)sv[i];
-            Prod<R> pr = strided_product<R>(t, T.tau_siteT + i, (size_t)N, si, 0, 1, M);
+            Prod<R> pr = strided_product(t, T.tau_siteT + i, (size_t)N, si, 0, 1, M);
             const double delta = -2.0 * T.a[i] * (double)si + (double)(T.K_site[i] + prod_log(pr));
             off += -A.h * exp(delta);
         }
@@ -1232,7 +1353,7 @@ __global__ void __launch_bounds__(128) k_eloc(ElocK<R> P) {
                 const int e = list[idx];
                 const int i = T.edges[2 * e], kk = T.edges[2 * e + 1];
                 const R si = (R)sv[i];
-                Prod<R> pr = strided_product<R>(t, T.tau_edge + (size_t)e * M, 1, si, lane, 32, M);
+                Prod<R> pr = strided_product(t, T.tau_edge + (size_t)e * M, 1, si, lane, 32, M);
                 pr = warp_prod(pr);
                 const double delta =
                     -2.0 * (double)si * (T.a[i] - T.a[kk]) + (double)(T.K_edge[e] + prod_log(pr));
@@ -1243,7 +1364,7 @@ __global__ void __launch_bounds__(128) k_eloc(ElocK<R> P) {
                 const int e = list[idx];
                 const int i = T.edges[2 * e], kk = T.edges[2 * e + 1];
                 const R si = (R)sv[i];
-                Prod<R> pr = strided_product<R>(t, T.tau_edgeT + e, (size_t)E, si, 0, 1, M);
+                Prod<R> pr = strided_product(t, T.tau_edgeT + e, (size_t)E, si, 0, 1, M);
                 const double delta =
                     -2.0 * (double)si * (T.a[i] - T.a[kk]) + (double)(T.K_edge[e] + prod_log(pr));
                 off += (e < E1 ? hoff : hoff2) * exp(delta);
@@ -1299,7 +1420,8 @@ __global__ void __launch_bounds__(eloc_warps(kU) * 32) k_eloc_batched(ElocBK P) 
         const int g = x / M, j = x % M;
         float tv = 0.f;
         if (g < G) {
-            const double tj = tanh(A.theta_in[(size_t)(k0 + g) * M + j]);
+            const double th = A.theta_in[(size_t)(k0 + g) * M + j];
+            const double tj = A.lib_tanh ? tanh(th) : tanh64(th);
             tv = (float)tj;
             if (A.t_out) A.t_out[(size_t)(k0 + g) * M + j] = tj;
         }
@@ -1455,7 +1577,7 @@ __global__ void __launch_bounds__(256) k_theta_tanh(int N, int M, const double *
     }
     const int64_t kk = k0 + ty;
     const int jj = j0 + tx;
-    if (kk < B && jj < M) T[(size_t)kk * M + jj] = tanh(acc + b[jj]);
+    if (kk < B && jj < M) T[(size_t)kk * M + jj] = tanh64(acc + b[jj]);
 }
 
 template <typename R>
@@ -1477,6 +1599,8 @@ cudaError_t launch_tables(const Tables<R> &t, bool need_site, bool need_edge, cu
     if (need_edge && t.E > 0)
         (k_tau_rows<R><<<t.E, 256, 0, st>>>(t.N, t.M, t.E, t.Wt, t.edges, t.tau_edge, t.tau_edgeT,
                                            t.K_edge, t.tauf_edge, t.D_edge), nk::note_launch());
+    if (t.eW)
+        (k_fix_weights<<<(t.M + 31) / 32, 256, 0, st>>>(t.N, t.M, t.Wt, t.eW), nk::note_launch());
     return cudaGetLastError();
 }
 
@@ -1500,9 +1624,9 @@ cudaError_t launch_logpsi_theta(int N, int M, const double *a, const double *the
     return cudaGetLastError();
 }
 
-cudaError_t launch_tanh_inplace(int64_t n, double *x, cudaStream_t st) {
+cudaError_t launch_tanh_inplace(int64_t n, double *x, bool lib, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    (k_tanh_inplace<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, x), nk::note_launch());
+    (k_tanh_inplace<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, x, lib), nk::note_launch());
     return cudaGetLastError();
 }
 

@@ -168,13 +168,14 @@ void carve_tables(Carver &c, nk::Tables<R> &t, const nk_rbm *rbm, int E, const i
     t.W = rbm->params + N + M;
     t.edges = edges;
     t.Wt = c.take<double>((size_t)N * M);
+    t.eW = sizeof(R) == 8 && (sweep || eloc) ? c.take<int>(M) : nullptr;
     const bool unit_major = eloc && M < nk::kUnitsMappingM;
     const bool rows = (eloc && !unit_major) || (sweep && sizeof(R) == 4);
-    t.tau_site = site && rows ? c.take<R>((size_t)N * M) : nullptr;
-    t.tau_siteT = site && unit_major ? c.take<R>((size_t)N * M) : nullptr;
+    t.tau_site = site && rows ? c.take<typename nk::TauOf<R>::type>((size_t)N * M) : nullptr;
+    t.tau_siteT = site && unit_major ? c.take<typename nk::TauOf<R>::type>((size_t)N * M) : nullptr;
     t.K_site = site ? c.take<R>(N) : nullptr;
-    t.tau_edge = edge && rows ? c.take<R>((size_t)E * M) : nullptr;
-    t.tau_edgeT = edge && unit_major ? c.take<R>((size_t)E * M) : nullptr;
+    t.tau_edge = edge && rows ? c.take<typename nk::TauOf<R>::type>((size_t)E * M) : nullptr;
+    t.tau_edgeT = edge && unit_major ? c.take<typename nk::TauOf<R>::type>((size_t)E * M) : nullptr;
     t.K_edge = edge ? c.take<R>(E) : nullptr;
     if (sizeof(R) == 8 && sweep) {
         t.tauf_site = site ? c.take<float>((size_t)N * M) : nullptr;
@@ -600,10 +601,19 @@ nk_status run_sweeps(nk_ctx *ctx, const nk::Tables<R> &t, const nk::SweepArgs &a
     return NK_OK;
 }
 
+// Where tanh(theta) feeds NK_MIXED conjugate gradients it is CUDA's tanh()
+// instead of the integer one (which is closer to the exact value and eight
+// times as fast).  Those iterations work on 33-bit products up to a tolerance
+// of 1e-6 and carry a difference of one last bit in tanh(theta) up to 1e-7 of
+// the solution (measured on lattices of 60 to 576 sites), sometimes into
+// another iteration count: with the same bits, runs and saved trajectories
+// continue exactly as they did.
+inline bool lib_tanh(int precision, int solver) { return precision == NK_MIXED && solver == NK_SOLVER_CG; }
+
 // T = tanh(theta) of a batch: the FP64-exact tensor-core product with tcm
 // (NK_MIXED, large NK_F64 batches), FP64 CUDA cores without.
 nk_status batch_T(nk_ctx *ctx, const nk_rbm *rbm, const int8_t *s, int64_t B, double *T, void *tcm,
-                  cudaStream_t st, int precision) {
+                  cudaStream_t st, int precision, bool lib = false) {
     const int N = rbm->N, M = rbm->M;
     const double *b = rbm->params + N, *W = rbm->params + N + M;
     if (!tcm) {
@@ -611,7 +621,7 @@ nk_status batch_T(nk_ctx *ctx, const nk_rbm *rbm, const int8_t *s, int64_t B, do
         return NK_OK;
     }
     NK_CU(nk::launch_theta_tc(N, M, b, W, s, B, T, ctx->tc_err, tcm, st, 0, precision == NK_F64), "theta");
-    NK_CU(nk::launch_tanh_inplace(B * M, T, st), "tanh");
+    NK_CU(nk::launch_tanh_inplace(B * M, T, lib, st), "tanh");
     return NK_OK;
 }
 
@@ -660,7 +670,8 @@ nk_status run_sweeps_theta(nk_ctx *ctx, const nk::Tables<R> &t, const nk::Tables
         // sample 0's rows serve as scratch until its own theta arrives)
         const int q = w - 1 - nd;
         double *th = b.theta + (size_t)(q > 0 ? q : 0) * M;
-        NK_CU(nk::launch_theta_tc(N, M, t.b, t.W, a.s, C, th, ctx->tc_err, b.tcm, st, (int64_t)ns * M, false, w > 0),
+        NK_CU(nk::launch_theta_tc(N, M, t.b, t.W, a.s, C, th, ctx->tc_err, b.tcm, st, (int64_t)ns * M, false,
+                                  w > 0),
               "theta");
         if (w == total) break;
         nk::SweepArgs sa = a;
@@ -708,6 +719,7 @@ nk_status run_sample_measure(nk_ctx *ctx, const nk::Tables<R> &t, const StepBufs
     nk_status sw = mixed ? run_sweeps_theta(ctx, t, ts, a, b, st) : run_sweeps(ctx, ts, a, false, nullptr, nullptr, st);
     if (sw != NK_OK) return sw;
     nk::ElocArgs ea = nk::eloc_args(ham, b.samples, Ns, b.eloc, b.T, b.theta);
+    ea.lib_tanh = lib_tanh(cfg->precision, cfg->solver);
     NK_CU(nk::launch_eloc(t, ea, st), "local energy");
     NK_CU(nk::launch_stats(b.eloc, Ns, C, b.st3, st), "stats");
     return NK_OK;
@@ -943,14 +955,18 @@ nk_status nk_local_energy(nk_ctx *ctx, const nk_rbm *rbm, int32_t precision, con
         using R = decltype(tag);
         nk::Tables<R> t{};
         carve_tables(c, t, rbm, ham->n_edges, ham->edges, site, edge, false, true);
-        const bool mixed = precision == NK_MIXED;
-        double *theta = mixed ? c.take<double>((size_t)Ns * rbm->M) : nullptr;
-        void *tcm = mixed ? c.take<char>(nk::tc_theta_ws_bytes(rbm->N, rbm->M, Ns)) : nullptr;
+        // (the theta of the tensor cores and of the kernel are the same to the
+        // last bit in NK_F64)
+        const bool tcp = precision == NK_MIXED || nk::f64_on_tensor(rbm->N, rbm->M, Ns);
+        double *theta = tcp ? c.take<double>((size_t)Ns * rbm->M) : nullptr;
+        void *tcm = tcp ? c.take<char>(nk::tc_theta_ws_bytes(rbm->N, rbm->M, Ns)) : nullptr;
         if (!run) return NK_OK;
         NK_CU(nk::launch_tables(t, site, edge, st), "tables");
         nk::ElocArgs am = a;
-        if (mixed) {
-            NK_CU(nk::launch_theta_tc(rbm->N, rbm->M, t.b, t.W, s, Ns, theta, ctx->tc_err, tcm, st), "theta");
+        if (tcp) {
+            NK_CU(nk::launch_theta_tc(rbm->N, rbm->M, t.b, t.W, s, Ns, theta, ctx->tc_err, tcm, st, 0,
+                                      precision == NK_F64),
+                  "theta");
             am.theta_in = theta;
         }
         NK_CU(nk::launch_eloc(t, am, st), "local energy");
@@ -1189,7 +1205,7 @@ nk_status nk_sr_solve(nk_ctx *ctx, const nk_rbm *rbm, int32_t precision, const i
         carve_solve(c, w, N, M, Ns, solver, precision);
         w.tcerr = ctx->tc_err;
         if (!run) return NK_OK;
-        nk_status bt = batch_T(ctx, rbm, s, Ns, T, w.tcm, st, precision);
+        nk_status bt = batch_T(ctx, rbm, s, Ns, T, w.tcm, st, precision, lib_tanh(precision, solver));
         if (bt != NK_OK) return bt;
         return run_solve(ctx, N, M, Ns, s, T, F, solver, diag_shift, cg_tol, cg_maxiter, w,
                          delta_out, info_out, resid_out, st, precision, precision == NK_MIXED);

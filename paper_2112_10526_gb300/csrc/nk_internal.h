@@ -3,6 +3,7 @@
 #pragma once
 
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -47,19 +48,35 @@ void note_launch(long long n = 1);
 cudaError_t allow_max_dynamic_smem(const void *func);
 void prof_end(int slot, cudaStream_t st, double work, double executed = -1.0);
 
+// The type of the flip-ratio tables: FP32 (NK_MIXED), or 2^63 tau as a 64-bit
+// integer (NK_F64; k_eloc multiplies them on the integer pipe).
+template <typename R>
+struct TauOf {
+    using type = R;
+};
+template <>
+struct TauOf<double> {
+    using type = long long;
+};
+
 // Per-parameter tables of the flip-ratio identity (see k_rbm.cu).  All
-// pointers are device workspace.  R = double (NK_F64) or float (NK_MIXED).
+// pointers are device workspace; a null table is not built.  R = double
+// (NK_F64) or float (NK_MIXED).
 template <typename R>
 struct Tables {
+    using Tau = typename TauOf<R>::type;
     int N, M, E;
     const double *a, *b, *W;  // views of the parameter vector
     double *Wt;               // [N][M] transposed W (FP64, coalesced theta rebuild)
-    R *tau_site;              // [N][M]  tanh(2 W_ji)
-    R *tau_siteT;             // [M][N]
+    // with eW (NK_F64): Wt is turned into the 59-bit integers y = rint(W 2^(59 -
+    // eW)), as (y >> 30, y & (2^30 - 1)), once the other tables are built
+    int *eW;                  // [M] exponent of each unit's weights
+    Tau *tau_site;            // [N][M]  tanh(2 W_ji)
+    Tau *tau_siteT;           // [M][N]
     R *K_site;                // [N]     sum_j ln cosh(2 W_ji)
     const int32_t *edges;     // [E][2]
-    R *tau_edge;              // [E][M]  tanh(2 (W_ji - W_jk))
-    R *tau_edgeT;             // [M][E]
+    Tau *tau_edge;            // [E][M]  tanh(2 (W_ji - W_jk))
+    Tau *tau_edgeT;           // [M][E]
     R *K_edge;                // [E]
     // NK_F64 sweeps: tau in FP32 (the screening of proposals) and 2 (W_ji -
     // W_jk) (the move of theta; 2 W_ji for single flips)
@@ -75,7 +92,7 @@ cudaError_t launch_logpsi(int N, int M, const double *a, const double *b, const 
 
 cudaError_t launch_logpsi_theta(int N, int M, const double *a, const double *theta, const int8_t *s, int64_t B,
                                 double *out, cudaStream_t st);
-cudaError_t launch_tanh_inplace(int64_t n, double *x, cudaStream_t st);
+cudaError_t launch_tanh_inplace(int64_t n, double *x, bool lib, cudaStream_t st);  // lib: CUDA's tanh()
 
 cudaError_t launch_chain_init(int N, int C, int rule, uint64_t seed, uint32_t stream_id,
                               int8_t *s, cudaStream_t st);
@@ -115,6 +132,7 @@ struct ElocArgs {
     const double *theta_in;   // [Ns][M] precomputed theta, or null (rebuilt in the kernel)
     double J2;                // coupling of the last E2 edges (next-nearest neighbours)
     int E2;
+    int lib_tanh;             // t by CUDA's tanh() (see lib_tanh in nk_api.cu)
 };
 
 // The rule NK_RULE_HAMILTONIAN becomes for a Hamiltonian kind: the Ising
@@ -230,19 +248,20 @@ inline size_t syrk_ws_bytes(int64_t rows, int64_t n) { return syrk_on_tensor(row
 
 // ---- tensor-core products with the configurations (k_sgemm.cu) -------------
 size_t tc_theta_ws_bytes(int N, int M, int64_t B);
-// theta [B][M] = S W^T + b, exact to 2^-56 of max|W_j| (7 slices); row r of
+// theta [B][M] = S W^T + b, exact to 2^-56 of the scale of W_j (wide, NK_F64:
+// 2^-60); row r of
 // theta at theta + r * ldtheta (0: M).  sliced: ws still holds the slices of W
 // from the last call with the same N, M, B and W.
 cudaError_t launch_theta_tc(int N, int M, const double *b, const double *W, const int8_t *s, int64_t B,
                             double *theta, int *err, void *ws, cudaStream_t st, int64_t ldtheta = 0,
                             bool wide = false, bool sliced = false);
-// Its product (k_theta.cu): A the +-1 configurations in BF16 [rows][ldA], Wsl
-// the 7 slices [7][units][ldA] of W with row exponents expW; s and W (unsliced)
-// serve units whose weights the slices cannot hold.
-cudaError_t launch_theta_product(const __nv_bfloat16 *A, int64_t rows, int64_t ldA, const __nv_bfloat16 *Wsl,
+// Its product (k_theta.cu): A the +-1 configurations in FP16 [rows][ldA], Wsl
+// the 5 slices [5][units][ldA] of the integers W 2^(bits - expW) (56 or 59
+// bits); s and W (unsliced) serve units whose weights the slices cannot hold.
+cudaError_t launch_theta_product(const __half *A, int64_t rows, int64_t ldA, const __half *Wsl,
                                  const int *expW, int units, int N, const double *bias, double *out, int64_t ld,
-                                 bool wide, const int8_t *s, const double *W, int *err, cudaStream_t st);
-// wide, here and in the products below (NK_F64): the slices' sums are turned
+                                 int bits, const int8_t *s, const double *W, int *err, cudaStream_t st);
+// wide, in the products below (NK_F64): the slices' sums are turned
 // into FP64 with every bit that the length of the sums leaves room for.
 // The +-1 operands of the two Jacobian products depend on the samples only:
 // a solve that repeats the products (CG) builds them once.  opA: [S, 1] as

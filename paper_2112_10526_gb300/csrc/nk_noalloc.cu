@@ -138,13 +138,24 @@ size_t plan_tables(Bump &b, nk::Tables<R> &t, const nk_rbm *rbm, const nk_ham *h
     t.b = rbm->params + N;
     t.W = rbm->params + N + M;
     t.edges = ham->edges;
+    // The local-energy kernel reads one form of the tau table, row-major or
+    // unit-major, by M; the other's room (which the size limit has always
+    // counted) holds the exponents of NK_F64.
+    using Tau = typename nk::TauOf<R>::type;
+    const bool unit_major = M < nk::kUnitsMappingM;
     t.Wt = b.take<double>((size_t)N * M);
-    t.tau_site = site ? b.take<R>((size_t)N * M) : nullptr;
-    t.tau_siteT = site ? b.take<R>((size_t)N * M) : nullptr;
+    Tau *rows = site ? b.take<Tau>((size_t)N * M) : nullptr, *cols = site ? b.take<Tau>((size_t)N * M) : nullptr;
+    t.tau_site = unit_major ? nullptr : rows;
+    t.tau_siteT = unit_major ? cols : nullptr;
     t.K_site = site ? b.take<R>(N) : nullptr;
-    t.tau_edge = edge ? b.take<R>((size_t)E * M) : nullptr;
-    t.tau_edgeT = edge ? b.take<R>((size_t)E * M) : nullptr;
+    Tau *spare = unit_major ? rows : cols;
+    rows = edge ? b.take<Tau>((size_t)E * M) : nullptr;
+    cols = edge ? b.take<Tau>((size_t)E * M) : nullptr;
+    t.tau_edge = unit_major ? nullptr : rows;
+    t.tau_edgeT = unit_major ? cols : nullptr;
     t.K_edge = edge ? b.take<R>(E) : nullptr;
+    if (edge) spare = unit_major ? rows : cols;
+    t.eW = sizeof(R) == 8 ? reinterpret_cast<int *>(spare) : nullptr;
     return b.off;
 }
 
