@@ -1434,6 +1434,28 @@ cudaError_t launch_theta_tc(int N, int M, const double *b, const double *W, cons
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
+cudaError_t launch_theta_pairs(int N, int M, const double *b, const double *W, const int8_t *s, int64_t B,
+                               void *Thl, int *colexpT, int *err, void *ws, cudaStream_t st) {
+    if (B <= 0) return cudaSuccess;
+    const int64_t ld = pad8(N);
+    char *p = static_cast<char *>(ws);
+    auto take = [&](size_t bytes) {
+        char *q = p;
+        p += (bytes + 255) / 256 * 256;
+        return q;
+    };
+    auto *As = reinterpret_cast<__half *>(take((size_t)B * ld * 2));
+    auto *Ws = reinterpret_cast<__half *>(take((size_t)5 * M * ld * 2));
+    auto *ew = reinterpret_cast<int *>(take((size_t)M * 4));
+    (k_fill_int<<<nblk(M + 1, 256), 256, 0, st>>>(M + 1, -100000, colexpT), nk::note_launch());
+    (k_pm1_rows<<<nblk(B * ld, 256), 256, 0, st>>>(s, B, N, 0, ld, As), nk::note_launch());
+    (k_slice_rows_h5<<<M, 128, 0, st>>>(W, M, N, ld, 56, Ws, ew), nk::note_launch());
+    const int slot = prof_begin(NK_PROF_JVP_VJP, st);
+    cudaError_t e = launch_theta_product(As, B, ld, Ws, ew, M, N, b, nullptr, M, 56, s, W, err, st, Thl, colexpT);
+    prof_end(slot, st, 2.0 * (double)B * N * (double)M, sgemm_flops(B, M, N, 5));
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 size_t tc_jvp_ws_bytes(int N, int M, int64_t Ns) {
     const int64_t ld = pad8(N + 1), ntc = (M + 1 + kBN - 1) / kBN;
     return ((size_t)Ns * ld * 2 + 255) / 256 * 256 + ((size_t)kMaxSB * (M + 1) * ld * 2 + 255) / 256 * 256 +
@@ -1548,6 +1570,11 @@ static int pick_ksplit(int64_t tiles, int64_t kchunks, int64_t slots) {
     return best;
 }
 
+bool pairs_suffice(int64_t Ns) {
+    const int64_t kchunks = (Ns + kBK - 1) / kBK;
+    return (kchunks + kH3MaxK / kBK - 1) / (kH3MaxK / kBK) <= kMaxKSplit;
+}
+
 size_t tc_vjp_ws_bytes(int N, int M, int64_t Ns) {
     const int64_t ld = pad8(Ns);
     return ((size_t)(N + 1) * ld * 2 + 255) / 256 * 256 + ((size_t)kMaxSB * (M + 1) * ld * 2 + 255) / 256 * 256 +
@@ -1594,7 +1621,7 @@ cudaError_t launch_vjp_tc(int N, int M, int64_t Ns, const int8_t *s, const doubl
     const int64_t kchunks = (Ns + kBK - 1) / kBK;
     // 4 slices' accuracy (the CG products) through the persistent kernel on 3
     // FP16 slices of 11-bit digits (33 bits), in units of at most 8192 samples
-    const bool h3 = SB == 4 && (kchunks + kH3MaxK / kBK - 1) / (kH3MaxK / kBK) <= kMaxKSplit;
+    const bool h3 = SB == 4 && pairs_suffice(Ns);
     if (h3 && opT)
         St = static_cast<__nv_bfloat16 *>(const_cast<void *>(opT));  // FP16 bits
     else if (h3)

@@ -20,6 +20,11 @@
 // against about 1 us of L2 latency).  The tile kernel this replaces (k_sgemm:
 // one 128 x 64 tile a CTA, nothing overlapping its drain) took 19 us for 1024 x
 // 200 x 100 and 4.70 ms for 65536 x 4608 x 576.
+// The epilogue writes theta in FP64, or (for the products of NK_MIXED that read
+// tanh(theta) as FP32 pairs) t' = [tanh(theta), 1] straight into the tile order
+// of k_tc4, with the exponents of its columns: the 24 x 24 lattice's 302 M
+// activations then cross HBM once instead of six times (theta, tanh, exponents
+// and two passes of pairs: 11 ms).
 // Every wait is bounded; a time-out records a code, drains the copies and MMAs
 // in flight and returns.
 
@@ -29,6 +34,7 @@
 
 #include "nk_common.cuh"
 #include "nk_internal.h"
+#include "tanh64.cuh"
 #include "tc_ptx.cuh"
 
 namespace nk {
@@ -57,7 +63,9 @@ struct ThetaArgs {
     int bits, drop;      // V 2^(expW - bits), its lowest `drop` bits left out
     const int *expW;     // [units]
     const double *bias;  // [units]
-    double *out;         // [rows][ld]
+    double *out;         // [rows][ld], or null:
+    float4 *pairs;       // t' as FP32 pairs, tile-major (launch_split_t)
+    int *colexp;         // [units + 1], -100000 before: exponents of the columns of t'
     int64_t ld;
     const int8_t *s;     // [rows][N] and W [units][N]: the units whose exponent is flagged
     const double *W;
@@ -81,6 +89,7 @@ __device__ __forceinline__ long long window_of(const uint32_t (&r)[kHS], int dro
     return (long long)((unsigned long long)hi << (24 - drop)) + (lo >> drop);
 }
 
+template <bool kPairs>
 __global__ void __launch_bounds__(kHThreads, 1)
     k_theta(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, ThetaArgs a) {
     extern __shared__ unsigned char smem_raw[];
@@ -250,6 +259,9 @@ __global__ void __launch_bounds__(kHThreads, 1)
                 break;
             }
             tc_fence_after();
+            // columns of t' that this warp's tile holds; the column of ones is `units`
+            int held = -100000;
+            if (kPairs) held = n0 + (lane & 7) <= a.units ? __ldcg(a.colexp + n0 + (lane & 7)) : 0;
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 uint32_t r[kHS][4];
@@ -262,6 +274,7 @@ __global__ void __launch_bounds__(kHThreads, 1)
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&acc_empty[b]);
                 }
+                float2 pr[4];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     uint32_t d[kHS];
@@ -269,9 +282,33 @@ __global__ void __launch_bounds__(kHThreads, 1)
                     for (int g = 0; g < kHS; ++g) d[g] = r[g][j];
                     const int e = __shfl_sync(0xffffffffu, e_lane, 4 * h + j);
                     double v = window_to_double(window_of(d, a.drop), e - a.bits + a.drop);
-                    if (flagged_exp(e) && m0 + lane < a.rows && n0 + 4 * h + j < a.units)
-                        v = raw_theta(a, m0 + lane, n0 + 4 * h + j);
-                    stage[lane * 4 + (j ^ ((lane >> 2) & 3))] = v;
+                    const int unit = n0 + 4 * h + j;
+                    if (flagged_exp(e) && m0 + lane < a.rows && unit < a.units) v = raw_theta(a, m0 + lane, unit);
+                    if (kPairs) {
+                        // t', 0 past the last row and past the column of ones
+                        const double b = __shfl_sync(0xffffffffu, bv[h], j);  // lane j holds unit 4 h + j
+                        double t = unit < a.units ? tanh64(v + b) : (unit == a.units ? 1.0 : 0.0);
+                        if (m0 + lane >= a.rows) t = 0.0;
+                        pr[j] = fp32_pair(t);
+                        const int be = (__double2hiint(t) >> 20) & 0x7FF;
+                        int ex = be == 0 ? -100000 : (be == 2047 ? 100000 : be - 1022);
+                        ex = __reduce_max_sync(0xffffffffu, ex);
+                        if (lane == 4 * h + j && unit <= a.units && ex > held) atomicMax(a.colexp + unit, ex);
+                    } else {
+                        stage[lane * 4 + (j ^ ((lane >> 2) & 3))] = v;
+                    }
+                }
+                if (kPairs) {
+                    // 64-unit tiles of 32 column pairs x 128 rows
+                    const int u0 = n0 + 4 * h;
+                    const int64_t mt = t / a.n_nt * C + rank;
+                    if (mt * kHM < a.rows) {
+                        float4 *dst = a.pairs + ((size_t)(mt * (a.n_nt / 2) + (u0 >> 6)) * 32 + ((u0 & 63) >> 1)) * kHM +
+                                      q * 32 + lane;
+                        __stcs(dst, make_float4(pr[0].x, pr[0].y, pr[1].x, pr[1].y));
+                        __stcs(dst + kHM, make_float4(pr[2].x, pr[2].y, pr[3].x, pr[3].y));
+                    }
+                    continue;
                 }
                 __syncwarp();
                 const int u = n0 + 4 * h + cc;
@@ -304,7 +341,8 @@ __global__ void __launch_bounds__(kHThreads, 1)
 
 cudaError_t launch_theta_product(const __half *A, int64_t rows, int64_t ldA, const __half *Wsl,
                                  const int *expW, int units, int N, const double *bias, double *out, int64_t ld,
-                                 int bits, const int8_t *s, const double *W, int *err, cudaStream_t st) {
+                                 int bits, const int8_t *s, const double *W, int *err, cudaStream_t st,
+                                 void *pairs, int *colexp) {
     if (rows <= 0 || units <= 0) return cudaSuccess;
     if (N > 4096 || rows > (1LL << 31) - 2 * kHM) return cudaErrorInvalidValue;
     EncodeTiledFn fn = encode_fn();
@@ -325,7 +363,8 @@ cudaError_t launch_theta_product(const __half *A, int64_t rows, int64_t ldA, con
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return cudaErrorInvalidValue;
     }
-    cudaError_t e = nk::allow_max_dynamic_smem((const void *)k_theta);
+    const void *kern = pairs ? (const void *)k_theta<true> : (const void *)k_theta<false>;
+    cudaError_t e = nk::allow_max_dynamic_smem(kern);
     int dev = 0, sms = 0;
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -336,7 +375,10 @@ cudaError_t launch_theta_product(const __half *A, int64_t rows, int64_t ldA, con
     a.N = N;
     a.kchunks = (N + kHK - 1) / kHK;
     a.resident = a.kchunks <= kHResident ? 1 : 0;
-    a.n_nt = (units + kHN - 1) / kHN;
+    // pairs: whole 64-unit tiles with the column of ones
+    a.n_nt = pairs ? (units + 1 + 63) / 64 * 2 : (units + kHN - 1) / kHN;
+    a.pairs = static_cast<float4 *>(pairs);
+    a.colexp = colexp;
     // |V| <= N 2^bits in 63 bits; 56-bit integers drop ten bits whatever N is
     a.bits = bits;
     a.drop = bits == 56 ? 10 : window_drop(8 * (int64_t)N);
@@ -374,7 +416,7 @@ cudaError_t launch_theta_product(const __half *A, int64_t rows, int64_t ldA, con
         if (C > 1) {
             int fit = 0;
             cfg.gridDim = dim3((unsigned)(ncl * C));
-            e = cudaOccupancyMaxActiveClusters(&fit, (const void *)k_theta, &cfg);
+            e = cudaOccupancyMaxActiveClusters(&fit, kern, &cfg);
             if (e != cudaSuccess) return e;
             if (fit < 1) continue;  // no cluster fits: single CTAs
             if (fit < ncl) ncl = fit;
@@ -383,7 +425,8 @@ cudaError_t launch_theta_product(const __half *A, int64_t rows, int64_t ldA, con
         a.per = (a.tiles + ncl - 1) / ncl;
         ncl = (a.tiles + a.per - 1) / a.per;
         cfg.gridDim = dim3((unsigned)(ncl * C));
-        e = cudaLaunchKernelEx(&cfg, k_theta, ma, mb, a);
+        e = pairs ? cudaLaunchKernelEx(&cfg, k_theta<true>, ma, mb, a)
+                  : cudaLaunchKernelEx(&cfg, k_theta<false>, ma, mb, a);
         nk::note_launch();
         return e != cudaSuccess ? e : cudaGetLastError();
     }

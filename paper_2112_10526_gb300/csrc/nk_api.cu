@@ -221,6 +221,7 @@ struct SolveWs {
     void *opA, *opT;  // NK_MIXED CG: the +-1 product operands, built once per solve
     bool tcp;         // Jacobian products on the tensor cores (NK_MIXED; NK_F64 by size)
     void *thl;        // NK_MIXED CG: tanh(theta) as FP32 pairs, built once per solve
+    bool pairs;       // thl and colexpT hold tanh(theta) of the samples; there is no T in FP64
     bool ops_ready;   // opA / opT / thl hold the operands of the samples being solved for
     const int *skip;  // NK_MIXED CG: its converged flag (the products then do nothing)
     int *tcerr; // sticky tensor-core error word of the context
@@ -319,7 +320,7 @@ cudaError_t jvp_any(int N, int M, int64_t Ns, const int8_t *s, const double *T, 
                     double *out, int precision, int slices, cudaStream_t st) {
     if (w.tcp)
         return nk::launch_jvp_tc(N, M, Ns, s, T, v, out, precision == NK_MIXED ? slices : kExactSlices, w.tcerr, w.tcm, st, w.ops_ready ? w.opA : nullptr,
-                                 w.ops_ready ? w.thl : nullptr, w.ops_ready ? w.skip : nullptr, precision == NK_F64);
+                                 w.ops_ready || w.pairs ? w.thl : nullptr, w.ops_ready ? w.skip : nullptr, precision == NK_F64);
     return nk::launch_jvp(N, M, Ns, s, T, v, w.U, out, st);
 }
 
@@ -328,8 +329,8 @@ cudaError_t vjp_any(int N, int M, int64_t Ns, const int8_t *s, const double *T, 
                     const int *colexpT = nullptr) {
     if (w.tcp)
         return nk::launch_vjp_tc(N, M, Ns, s, T, g, scale, shift, out, precision == NK_MIXED ? slices : kExactSlices,
-                                 w.tcerr, w.tcm, st, colexpT,
-                                 w.ops_ready ? w.opT : nullptr, w.ops_ready ? w.thl : nullptr,
+                                 w.tcerr, w.tcm, st, w.pairs ? w.colexpT : colexpT,
+                                 w.ops_ready ? w.opT : nullptr, w.ops_ready || w.pairs ? w.thl : nullptr,
                                  w.ops_ready ? w.skip : nullptr, precision == NK_F64);
     return nk::launch_vjp(N, M, Ns, s, T, g, scale, shift, w.partial, out, st);
 }
@@ -725,6 +726,26 @@ nk_status run_sample_measure(nk_ctx *ctx, const nk::Tables<R> &t, const StepBufs
     return NK_OK;
 }
 
+// tanh(theta) for the one-off products of nk_vjp, nk_jvp and nk_qgt_matvec: as
+// FP32 pairs where those read nothing else (NK_MIXED), else T in FP64.
+double *carve_T(Carver &c, SolveWs &w, int N, int M, int64_t Ns, int precision) {
+    w.pairs = precision == NK_MIXED && nk::pairs_suffice(Ns);
+    if (!w.pairs) return c.take<double>((size_t)Ns * M);
+    w.thl = c.take<char>(nk::tc_split_t_bytes(M, Ns));
+    w.colexpT = c.take<int>(M + 1);
+    return nullptr;
+}
+
+nk_status fill_T(nk_ctx *ctx, const nk_rbm *rbm, const int8_t *s, int64_t Ns, double *T, SolveWs &w, int precision,
+                 cudaStream_t st) {
+    if (!w.pairs) return batch_T(ctx, rbm, s, Ns, T, w.tcm, st, precision);
+    const int N = rbm->N, M = rbm->M;
+    NK_CU(nk::launch_theta_pairs(N, M, rbm->params + N, rbm->params + N + M, s, Ns, w.thl, w.colexpT, ctx->tc_err,
+                                 w.tcm, st),
+          "theta");
+    return NK_OK;
+}
+
 nk_status check_solver(int solver, double eps, double tol, int maxiter) {
     if (solver != NK_SOLVER_CG && solver != NK_SOLVER_CHOLESKY && solver != NK_SOLVER_CHOLESKY_SAMPLESPACE &&
         solver != NK_SOLVER_SVD && solver != NK_SOLVER_SVD_SAMPLESPACE)
@@ -1041,12 +1062,12 @@ nk_status nk_vjp(nk_ctx *ctx, const nk_rbm *rbm, int32_t precision, const int8_t
     cudaStream_t st = (cudaStream_t)stream;
     const int N = rbm->N, M = rbm->M;
     return with_workspace(ctx, [&](Carver &c, bool run) -> nk_status {
-        double *T = c.take<double>((size_t)Ns * M);
         SolveWs w{};
+        double *T = carve_T(c, w, N, M, Ns, precision);
         carve_products(c, w, N, M, Ns, precision, false);
         w.tcerr = ctx->tc_err;
         if (!run) return NK_OK;
-        nk_status bt = batch_T(ctx, rbm, s, Ns, T, w.tcm, st, precision);
+        nk_status bt = fill_T(ctx, rbm, s, Ns, T, w, precision, st);
         if (bt != NK_OK) return bt;
         NK_CU(vjp_any(N, M, Ns, s, T, gvec, 1.0, nullptr, w, out, precision, kMatvecSlices, st), "vjp");
         return NK_OK;
@@ -1067,12 +1088,12 @@ nk_status nk_jvp(nk_ctx *ctx, const nk_rbm *rbm, int32_t precision, const int8_t
     cudaStream_t st = (cudaStream_t)stream;
     const int N = rbm->N, M = rbm->M;
     return with_workspace(ctx, [&](Carver &c, bool run) -> nk_status {
-        double *T = c.take<double>((size_t)Ns * M);
         SolveWs w{};
+        double *T = carve_T(c, w, N, M, Ns, precision);
         carve_products(c, w, N, M, Ns, precision, true);
         w.tcerr = ctx->tc_err;
         if (!run) return NK_OK;
-        nk_status bt = batch_T(ctx, rbm, s, Ns, T, w.tcm, st, precision);
+        nk_status bt = fill_T(ctx, rbm, s, Ns, T, w, precision, st);
         if (bt != NK_OK) return bt;
         NK_CU(jvp_any(N, M, Ns, s, T, v, w, out, precision, kMatvecSlices, st), "jvp");
         return NK_OK;
@@ -1141,14 +1162,14 @@ nk_status nk_qgt_matvec(nk_ctx *ctx, const nk_qgt *q, double diag_shift, const d
     const nk_rbm *rbm = q->rbm;
     const int N = rbm->N, M = rbm->M;
     return with_workspace(ctx, [&](Carver &c, bool run) -> nk_status {
-        double *T = c.take<double>((size_t)Ns * M);
         SolveWs w{};
+        double *T = carve_T(c, w, N, M, Ns, q->precision);
         carve_products(c, w, N, M, Ns, q->precision, true);
         w.dotp = c.take<double>(nk::dot_partial_doubles(Ns) + 8);
         w.w = c.take<double>(Ns);
         w.tcerr = ctx->tc_err;
         if (!run) return NK_OK;
-        nk_status bt = batch_T(ctx, rbm, q->s, Ns, T, w.tcm, st, q->precision);
+        nk_status bt = fill_T(ctx, rbm, q->s, Ns, T, w, q->precision, st);
         if (bt != NK_OK) return bt;
         NK_CU(qgt_onthefly(N, M, Ns, q->s, T, v, diag_shift, w, out, st, q->precision), "qgt matvec");
         return NK_OK;

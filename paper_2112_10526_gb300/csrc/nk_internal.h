@@ -260,7 +260,15 @@ cudaError_t launch_theta_tc(int N, int M, const double *b, const double *W, cons
 // bits); s and W (unsliced) serve units whose weights the slices cannot hold.
 cudaError_t launch_theta_product(const __half *A, int64_t rows, int64_t ldA, const __half *Wsl,
                                  const int *expW, int units, int N, const double *bias, double *out, int64_t ld,
-                                 int bits, const int8_t *s, const double *W, int *err, cudaStream_t st);
+                                 int bits, const int8_t *s, const double *W, int *err, cudaStream_t st,
+                                 void *pairs = nullptr, int *colexp = nullptr);
+// t' = [tanh(theta), 1] of the batch as the FP32 pairs of launch_split_t and its
+// column exponents [M + 1] (launch_colexp_t), without theta in memory (out null
+// in the product); ws of tc_theta_ws_bytes.
+cudaError_t launch_theta_pairs(int N, int M, const double *b, const double *W, const int8_t *s, int64_t B,
+                               void *Thl, int *colexpT, int *err, void *ws, cudaStream_t st);
+// Whether J v and J^T g of NK_MIXED read tanh(theta) through those pairs alone.
+bool pairs_suffice(int64_t Ns);
 // wide, in the products below (NK_F64): the slices' sums are turned
 // into FP64 with every bit that the length of the sums leaves room for.
 // The +-1 operands of the two Jacobian products depend on the samples only:

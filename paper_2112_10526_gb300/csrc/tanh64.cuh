@@ -280,5 +280,24 @@ __host__ __device__ __forceinline__ double tanh64_with(double theta, const ulong
 
 __device__ __forceinline__ double tanh64(double theta) { return tanh64_with(theta, g_tanh_table); }
 
+// t as an FP32 pair, h = fl32(t) and l = fl32(t - h) (t - h is exact in FP64),
+// with integer operations only for |t| in [2^-64, 1]: the top 24 bits of the
+// mantissa rounded to nearest even, and the signed rest.
+__device__ __forceinline__ float2 fp32_pair(double t) {
+    const unsigned long long bits = (unsigned long long)__double_as_longlong(t);
+    const int be = (int)((bits >> 52) & 0x7FF);
+    if (be < 1023 - 64 || be > 1023) {
+        const float h = __double2float_rn(t);
+        return make_float2(h, __double2float_rn(t - (double)h));
+    }
+    const uint32_t sign = (uint32_t)(bits >> 63) << 31;
+    const uint32_t top = (uint32_t)(bits >> 29) & 0x7FFFFFU, rest = (uint32_t)bits & 0x1FFFFFFFU;
+    const uint32_t up = rest > 0x10000000U || (rest == 0x10000000U && (top & 1U)) ? 1U : 0U;
+    const uint32_t h = ((uint32_t)(be - 896) << 23) + top + up;  // a carry lifts the exponent
+    const int low = (int)rest - (int)(up << 29);                 // t - h in units of 2^(be - 1075)
+    const float l = __fmul_rn(__int2float_rn(low), __uint_as_float((uint32_t)(be - 948) << 23));
+    return make_float2(__uint_as_float(sign | h), __uint_as_float(__float_as_uint(l) ^ sign));
+}
+
 }  // namespace
 }  // namespace nk
