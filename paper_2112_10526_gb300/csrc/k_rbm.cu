@@ -459,48 +459,50 @@ __device__ __forceinline__ Prod<float> unit_lanes_product(const float *t, const 
                 : strided_product(t, tau, 1, si, lane, 32, M);
 }
 
-// lane_product4 on a tau row already held in registers: uv[u] is the chunk j
-// = 4 lane + 128 u (zero past M).  The groups, renormalisations and tail are
-// those of lane_product4, in the same order, so the result is identical; only
-// the loads are gone (the caller issues all of them at once, one L2 round
-// trip per row instead of one per group of four).
+// frexp by the exponent bits where they are those of a normal number.
+__device__ __forceinline__ void renorm_fast(Prod<float> &p) {
+    const int b = __float_as_int(p.m), be = (b >> 23) & 0xFF;
+    if (be - 1u < 254u) {
+        p.e += be - 126;
+        p.m = __int_as_float((b & 0x807FFFFF) | 0x3F000000);
+    } else {
+        renorm(p);
+    }
+}
+
+// lane_product4 on t and a tau row already held in registers: chunk u is units j
+// = 4 lane + 128 u .. j + 3 (zero past M).  The groups, renormalisations and tail
+// are those of lane_product4, in the same order, so the result is identical.
 template <int kC>
-__device__ __forceinline__ Prod<float> lane_product4_regs(const float *__restrict__ t, const float4 (&uv)[kC],
-                                                          float si, int lane, int M) {
+__device__ __forceinline__ Prod<float> lane_product4_regs(const float4 (&tv)[kC], const float4 (&uv)[kC], float si,
+                                                          int lane, int M) {
     float m0 = 1.f, m1 = 1.f;
-    int e = 0;
-    int j = 4 * lane, G = 0;
+    int e = 0, G = 0;
+    const int j = 4 * lane;
 #pragma unroll
     for (int g = 0; g < kC / 4; ++g) {
-        if (j + 3 * 128 < M) {
-            float4 tv[4];
+        if (j + 512 * g + 3 * 128 < M) {
 #pragma unroll
-            for (int u = 0; u < 4; ++u) tv[u] = *reinterpret_cast<const float4 *>(t + j + u * 128);
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const float4 w = uv[4 * g + u];
-                m0 *= fmaf(-si * tv[u].x, w.x, 1.f) * fmaf(-si * tv[u].y, w.y, 1.f);
-                m1 *= fmaf(-si * tv[u].z, w.z, 1.f) * fmaf(-si * tv[u].w, w.w, 1.f);
+            for (int u = 4 * g; u < 4 * g + 4; ++u) {
+                m0 *= fmaf(-si * tv[u].x, uv[u].x, 1.f) * fmaf(-si * tv[u].y, uv[u].y, 1.f);
+                m1 *= fmaf(-si * tv[u].z, uv[u].z, 1.f) * fmaf(-si * tv[u].w, uv[u].w, 1.f);
             }
             m0 = renorm_bits(m0, e);
             m1 = renorm_bits(m1, e);
-            j += 4 * 128;
             ++G;
         }
     }
 #pragma unroll
     for (int u = 0; u < kC; ++u) {
-        if (u >= 4 * G && 4 * lane + 128 * u < M) {
-            const float4 tv = *reinterpret_cast<const float4 *>(t + 4 * lane + 128 * u);
-            const float4 w = uv[u];
-            m0 *= fmaf(-si * tv.x, w.x, 1.f) * fmaf(-si * tv.y, w.y, 1.f);
-            m1 *= fmaf(-si * tv.z, w.z, 1.f) * fmaf(-si * tv.w, w.w, 1.f);
+        if (u >= 4 * G && j + 128 * u < M) {
+            m0 *= fmaf(-si * tv[u].x, uv[u].x, 1.f) * fmaf(-si * tv[u].y, uv[u].y, 1.f);
+            m1 *= fmaf(-si * tv[u].z, uv[u].z, 1.f) * fmaf(-si * tv[u].w, uv[u].w, 1.f);
         }
     }
     Prod<float> p{m0, e};
-    renorm(p);
+    renorm_fast(p);
     p.m *= m1;
-    renorm(p);
+    renorm_fast(p);
     return p;
 }
 
@@ -1131,14 +1133,31 @@ __global__ void __launch_bounds__(128) k_sweep_screened_regs(SweepK<double> P) {
     if (lane == 0 && A.n_accepted) A.n_accepted[c] += acc;
 }
 
-// FP32 sweeps of the local and exchange rules with the flip-ratio row of a
-// proposal held in registers: every lane issues the loads of all its kC
-// chunks of the row at once, so a proposal waits for one L2 round trip
-// (k_sweep<false, false> waits for one per group of four chunks: nine at M =
-// 4608).  The accepted move's update of t reuses the registers.  The
-// arithmetic and the order of every product are those of
-// k_sweep<false, false>, so the decisions are identical.  Needs M % 4 == 0 and
-// M <= 128 kC.
+// FP32 sweeps of the local and exchange rules at few units (M % 4 == 0, M <=
+// 128 kC): t = tanh(theta) in registers, the rows of flip ratios of the next
+// kSweepAhead proposals on their way into a ring in shared memory (cp.async; a
+// lane reads back only the 16-byte chunks it copied).  The proposals come from
+// Philox alone, so the rows are known ahead; an exchange row is fetched if its
+// spins differ at that time (and loaded on demand if they have come to differ
+// since).  A chain then waits for nothing but its own arithmetic: with 1024
+// chains there are two warps a scheduler, and the row's L2 round trip and the
+// shared-memory round trips of t were most of a proposal.  The arithmetic and
+// the order of every product are those of k_sweep, so the decisions are
+// identical.  ln psi is summed only where it is asked for.
+// 10 x 10 lattice, M = 200, 1024 chains: 66 us a sweep with the row loaded when
+// its proposal came up, 55 now: some 160 instructions a proposal at 6.5 cycles
+// each, the latency of one dependent on the next.
+constexpr int kSweepAhead = 4;
+
+__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int n>
+__device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(n) : "memory");
+}
+
 template <int kC>
 __global__ void __launch_bounds__(128) k_sweep_rows(SweepK<float> P) {
     extern __shared__ __align__(16) unsigned char sm[];
@@ -1149,8 +1168,10 @@ __global__ void __launch_bounds__(128) k_sweep_rows(SweepK<float> P) {
     if (c >= A.C) return;
     const int N = T.N, M = T.M;
     unsigned char *base = sm + (size_t)warp * P.warp_bytes;
-    float *t = reinterpret_cast<float *>(base);
-    int8_t *sv = reinterpret_cast<int8_t *>(base + P.t_bytes);
+    float *ring = reinterpret_cast<float *>(base);  // [kSweepAhead][M]
+    int4 *prop_i = reinterpret_cast<int4 *>(base + (size_t)kSweepAhead * P.t_bytes);  // [32]
+    float4 *prop_f = reinterpret_cast<float4 *>(prop_i + 32);                         // [32]
+    int8_t *sv = reinterpret_cast<int8_t *>(prop_f + 32);
     const bool local = A.rule == NK_RULE_LOCAL;
     const float *tab = local ? T.tau_site : T.tau_edge;
     for (int i = lane; i < N; i += 32) sv[i] = A.s[(size_t)c * N + i];
@@ -1158,95 +1179,134 @@ __global__ void __launch_bounds__(128) k_sweep_rows(SweepK<float> P) {
     unsigned long long acc = 0;
     const int n_sweeps = A.n_discard + A.n_samples;
     for (int w = 0; w < n_sweeps; ++w) {
-        double lp = 0.0;
-        for (int j = lane; j < M; j += 32) {
-            double th;
-            if (A.theta_in) {
-                th = A.theta_in[(size_t)c * (A.theta_ld > 0 ? A.theta_ld : M) + j];
-            } else {
-                th = T.b[j];
-                for (int i = 0; i < N; ++i) th = fma(T.Wt[(size_t)i * M + j], (double)sv[i], th);
+        const bool want_lp = A.logpsi != nullptr && w >= A.n_discard;
+        uint8_t *decisions =
+            A.decisions ? A.decisions + ((size_t)c * A.dec_stride + A.dec_offset + w) * N : nullptr;
+        const double *th = A.theta_in + (size_t)c * (A.theta_ld > 0 ? A.theta_ld : M);
+        float4 t[kC];
+#pragma unroll
+        for (int u = 0; u < kC; ++u) {
+            const int j = 4 * lane + 128 * u;
+            t[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (j < M) {
+                const double2 a = *reinterpret_cast<const double2 *>(th + j);
+                const double2 b = *reinterpret_cast<const double2 *>(th + j + 2);
+                t[u] = make_float4(tanhf((float)a.x), tanhf((float)a.y), tanhf((float)b.x), tanhf((float)b.y));
             }
-            const float thf = (float)th;
-            t[j] = tanhf(thf);
-            lp += (double)lncosh(thf);
         }
-        for (int i = lane; i < N; i += 32) lp += T.a[i] * (double)sv[i];
-        lp = warp_sum(lp);
-        __syncwarp();
+        double lp = 0.0;
+        if (want_lp) {
+            for (int j = lane; j < M; j += 32) lp += (double)lncosh((float)th[j]);
+            for (int i = lane; i < N; i += 32) lp += T.a[i] * (double)sv[i];
+            lp = warp_sum(lp);
+        }
         const unsigned long long qbase = (unsigned long long)(A.sweep0 + w) * (unsigned long long)N;
-        int b_i = 0, b_k = -1, b_row = 0, b_ok = 1;
-        float b_K = 0.f, b_aa = 0.f, b_lu = 0.f;
-        for (int q = 0; q < N; ++q) {
-            const int src = q & 31;
-            if (src == 0) {
-                Philox4 y = philox4x64_10(qbase + (unsigned long long)(q + lane), (unsigned long long)c,
-                                          (unsigned long long)A.stream_id, 0ULL, A.seed, 0ULL);
-                b_lu = logf((float)uniform53(y.v[1]));
-                if (local) {
-                    b_i = pick_index(y.v[0], N);
-                    b_k = -1;
-                    b_row = b_i;
-                    b_K = T.K_site[b_i];
-                    b_aa = (float)T.a[b_i];
-                } else {
-                    const int e = pick_index(y.v[0], T.E);
-                    const int i0 = A.edges[2 * e], k0 = A.edges[2 * e + 1];
-                    // an edge outside [0, N) is never a move (bounds guard)
-                    b_ok = (unsigned)i0 < (unsigned)N && (unsigned)k0 < (unsigned)N;
-                    b_i = b_ok ? i0 : 0;
-                    b_k = b_ok ? k0 : 0;
-                    b_row = e;
-                    b_K = T.K_edge[e];
-                    b_aa = b_ok ? (float)(T.a[b_i] - T.a[b_k]) : 0.f;
-                }
+        for (int q0 = 0; q0 < N; q0 += 32) {
+            // lane l prepares proposal q0 + l
+            const Philox4 y = philox4x64_10(qbase + (unsigned long long)(q0 + lane), (unsigned long long)c,
+                                            (unsigned long long)A.stream_id, 0ULL, A.seed, 0ULL);
+            const float b_lu = logf((float)uniform53(y.v[1]));
+            int4 pi;    // site i (-1: never a move), site k (-1: single flip), row, -
+            float4 pf;  // ln u, K, a-part, -
+            if (local) {
+                const int i = pick_index(y.v[0], N);
+                pi = make_int4(i, -1, i, 0);
+                pf = make_float4(b_lu, T.K_site[i], (float)T.a[i], 0.f);
+            } else {
+                const int row = pick_index(y.v[0], T.E);
+                const int i0 = A.edges[2 * row], k0 = A.edges[2 * row + 1];
+                // an edge outside [0, N) is never a move (bounds guard)
+                const bool in = (unsigned)i0 < (unsigned)N && (unsigned)k0 < (unsigned)N;
+                pi = make_int4(in ? i0 : -1, k0, row, 0);
+                pf = make_float4(b_lu, T.K_edge[row], in ? (float)(T.a[i0] - T.a[k0]) : 0.f, 0.f);
             }
-            const int i = __shfl_sync(kFull, b_i, src), k = __shfl_sync(kFull, b_k, src);
-            const int row = __shfl_sync(kFull, b_row, src);
-            const float K = __shfl_sync(kFull, b_K, src), aa = __shfl_sync(kFull, b_aa, src);
-            const float lu = __shfl_sync(kFull, b_lu, src);
-            const int ok = __shfl_sync(kFull, b_ok, src);
-            const size_t slot = ((size_t)c * A.dec_stride + A.dec_offset + w) * N + q;
-            if (!local && (!ok || sv[i] == sv[k])) {
-                if (lane == 0 && A.decisions) A.decisions[slot] = 2;
-                continue;
-            }
-            const float d0 = -2.f * aa * (float)sv[i];
-            const float si = (float)sv[i];
-            float4 uv[kC];
-            const float *row_p = tab + (size_t)row * M;
-#pragma unroll
-            for (int u = 0; u < kC; ++u) {
-                const int j = 4 * lane + 128 * u;
-                uv[u] = j < M ? __ldg(reinterpret_cast<const float4 *>(row_p + j)) : make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-            Prod<float> pr = lane_product4_regs<kC>(t, uv, si, lane, M);
-            pr = warp_prod_normalised(pr);
-            const float delta = d0 + (K + prod_log(pr));
-            const bool accept = lu < 2.f * delta;
-            if (lane == 0 && A.decisions) A.decisions[slot] = accept ? 1 : 0;
-            if (accept) {
-#pragma unroll
-                for (int u = 0; u < kC; ++u) {
-                    const int j = 4 * lane + 128 * u;
-                    if (j >= M) continue;
-                    float4 tv = *reinterpret_cast<const float4 *>(t + j);
-                    const float v0 = si * uv[u].x, v1 = si * uv[u].y, v2 = si * uv[u].z, v3 = si * uv[u].w;
-                    tv.x = __fdividef(tv.x - v0, fmaf(-tv.x, v0, 1.f));
-                    tv.y = __fdividef(tv.y - v1, fmaf(-tv.y, v1, 1.f));
-                    tv.z = __fdividef(tv.z - v2, fmaf(-tv.z, v2, 1.f));
-                    tv.w = __fdividef(tv.w - v3, fmaf(-tv.w, v3, 1.f));
-                    *reinterpret_cast<float4 *>(t + j) = tv;
-                }
-                __syncwarp();
-                if (lane == 0) {
-                    sv[i] = (int8_t)-sv[i];
-                    if (k >= 0) sv[k] = (int8_t)-sv[k];
-                }
-                lp += (double)delta;
-                ++acc;
-            }
+            // handed on through shared memory: two loads a proposal instead of
+            // seven shuffles
             __syncwarp();
+            prop_i[lane] = pi;
+            prop_f[lane] = pf;
+            __syncwarp();
+            const int nq = N - q0 < 32 ? N - q0 : 32;
+            unsigned fetched = 0;  // bit src: the row of proposal src is in (or on its way to) the ring
+            auto prefetch = [&](int src) {
+                if (src < nq) {
+                    const int4 p = prop_i[src];
+                    if (local || (p.x >= 0 && sv[p.x] != sv[p.y])) {  // warp-uniform
+                        const float *row_p = tab + (size_t)p.z * M;
+                        float *dst = ring + (size_t)(src % kSweepAhead) * (P.t_bytes / 4);
+#pragma unroll
+                        for (int u = 0; u < kC; ++u) {
+                            const int j = 4 * lane + 128 * u;
+                            if (j < M) cp_async16(dst + j, row_p + j);
+                        }
+                        fetched |= 1u << src;
+                    }
+                }
+                cp_async_commit();  // one group a proposal, empty or not
+            };
+#pragma unroll
+            for (int src = 0; src < kSweepAhead - 1; ++src) prefetch(src);
+            for (int src = 0; src < nq; ++src) {
+                prefetch(src + kSweepAhead - 1);
+                // this proposal's row has landed (those of the later ones may be under
+                // way), also if it is no move any more: its slot is refilled next
+                cp_async_wait<kSweepAhead - 1>();
+                const int4 p = prop_i[src];
+                const int i = p.x, k = p.y;
+                const int si8 = i >= 0 ? sv[i] : 0;
+                if (!local && (i < 0 || si8 == sv[k])) {
+                    if (decisions && lane == 0) decisions[q0 + src] = 2;
+                    continue;
+                }
+                float4 uv[kC];
+                if ((fetched >> src) & 1u) {
+                    const float *row_s = ring + (size_t)(src % kSweepAhead) * (P.t_bytes / 4);
+#pragma unroll
+                    for (int u = 0; u < kC; ++u) {
+                        const int j = 4 * lane + 128 * u;
+                        uv[u] = j < M ? *reinterpret_cast<const float4 *>(row_s + j) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    }
+                } else {
+                    const float *row_p = tab + (size_t)p.z * M;
+#pragma unroll
+                    for (int u = 0; u < kC; ++u) {
+                        const int j = 4 * lane + 128 * u;
+                        uv[u] = j < M ? __ldg(reinterpret_cast<const float4 *>(row_p + j))
+                                      : make_float4(0.f, 0.f, 0.f, 0.f);
+                    }
+                }
+                const float si = (float)si8;
+                const float4 pf = prop_f[src];
+                const float d0 = -2.f * pf.z * si;
+                Prod<float> pr = lane_product4_regs<kC>(t, uv, si, lane, M);
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1) {  // as warp_prod_normalised
+                    pr.m *= __shfl_xor_sync(kFull, pr.m, off);
+                    pr.e += __shfl_xor_sync(kFull, pr.e, off);
+                }
+                renorm_fast(pr);
+                const float delta = d0 + (pf.y + prod_log(pr));
+                const bool accept = pf.x < 2.f * delta;
+                if (decisions && lane == 0) decisions[q0 + src] = accept ? 1 : 0;
+                if (accept) {
+#pragma unroll
+                    for (int u = 0; u < kC; ++u) {
+                        const float v0 = si * uv[u].x, v1 = si * uv[u].y, v2 = si * uv[u].z, v3 = si * uv[u].w;
+                        t[u].x = __fdividef(t[u].x - v0, fmaf(-t[u].x, v0, 1.f));
+                        t[u].y = __fdividef(t[u].y - v1, fmaf(-t[u].y, v1, 1.f));
+                        t[u].z = __fdividef(t[u].z - v2, fmaf(-t[u].z, v2, 1.f));
+                        t[u].w = __fdividef(t[u].w - v3, fmaf(-t[u].w, v3, 1.f));
+                    }
+                    if (lane == 0) {
+                        sv[i] = (int8_t)-si8;
+                        if (!local) sv[k] = (int8_t)si8;  // it held -s_i
+                    }
+                    if (want_lp) lp += (double)delta;
+                    ++acc;
+                    __syncwarp();
+                }
+            }
+            cp_async_wait<0>();  // the ring's slots start over with the next batch
         }
         if (w >= A.n_discard) {
             const size_t row = (size_t)c * A.out_stride + A.out_offset + (w - A.n_discard);
@@ -1637,13 +1697,13 @@ cudaError_t launch_chain_init(int N, int C, int rule, uint64_t seed, uint32_t st
     return cudaGetLastError();
 }
 
-// The register-row sweep for kC chunks of 128 floats per lane.
+// The register sweep for up to kC chunks of 128 units.
 template <int kC>
-cudaError_t launch_sweep_rows_kc(const SweepK<float> &P, cudaStream_t st) {
-    int wpb = 4;
-    while (wpb > 1 && (size_t)wpb * P.warp_bytes > 200 * 1024) wpb >>= 1;
+cudaError_t launch_sweep_rows(SweepK<float> P, cudaStream_t st) {
+    P.warp_bytes = kSweepAhead * P.t_bytes + 1024 + align16<float>(P.t.N);
+    // two warps a block spread few chains more evenly over the SMs
+    const int wpb = P.a.C <= 4864 ? 2 : 4;
     const size_t smem = (size_t)wpb * P.warp_bytes;
-    if (smem > 227 * 1024) return cudaErrorInvalidValue;
     cudaError_t err = nk::allow_max_dynamic_smem((const void *)k_sweep_rows<kC>);
     if (err != cudaSuccess) return err;
     const unsigned grid = (unsigned)((P.a.C + wpb - 1) / wpb);
@@ -1652,14 +1712,6 @@ cudaError_t launch_sweep_rows_kc(const SweepK<float> &P, cudaStream_t st) {
     prof_end(slot, st, (double)P.a.C * (P.a.n_discard + P.a.n_samples) * P.t.N * (double)P.t.M);
     return cudaGetLastError();
 }
-
-// FP32 local and exchange rules with M % 4 == 0 and M <= 512: the
-// register-row kernel (4 chunks a lane, 72 registers, the occupancy of
-// k_sweep).  Measured on GB300: 0.62 against 0.71 ms a step at M = 200; at
-// M = 1600 (16 chunks, 161 registers) and M = 4608 (36 chunks, 254
-// registers) the larger register footprint made it slower than k_sweep
-// (10.9 against 8.4 ms, 140 against 125 ms), so those sizes keep k_sweep.
-cudaError_t launch_sweep_rows(const SweepK<float> &P, cudaStream_t st) { return launch_sweep_rows_kc<4>(P, st); }
 
 // NK_F64: the screened kernel.  Shared memory holds theta (FP64), t (FP32) and
 // the spins of each chain.
@@ -1734,8 +1786,10 @@ template <>
 cudaError_t launch_sweep<float>(const Tables<float> &t, const SweepArgs &a, cudaStream_t st) {
     if (a.C <= 0 || a.n_discard + a.n_samples <= 0) return cudaSuccess;
     const SweepK<float> P = sweep_args(t, a);
-    // local and exchange rules with few units: the register-row kernel
-    if (P.vec4 && a.rule != NK_RULE_HAMILTONIAN && t.M <= 4 * 128) return launch_sweep_rows(P, st);
+    // local and exchange rules with few units and theta given: t in registers
+    if (P.vec4 && a.rule != NK_RULE_HAMILTONIAN && t.M <= 4 * 128 && a.theta_in)
+        return t.M <= 128 ? launch_sweep_rows<1>(P, st)
+                          : (t.M <= 256 ? launch_sweep_rows<2>(P, st) : launch_sweep_rows<4>(P, st));
     int wpb = 4;
     while (wpb > 1 && (size_t)wpb * P.warp_bytes > 200 * 1024) wpb >>= 1;
     size_t smem = (size_t)wpb * P.warp_bytes;
