@@ -416,26 +416,82 @@ __global__ void __launch_bounds__(kPThreads, 1)
 
 constexpr int kNB = 64;
 
-// Factor the kb x kb diagonal block at (k, k) in place (lower).  One CTA of
-// 256 threads holds the block in shared memory (continued by the identity
-// beyond kb) and factors it column by column with a look-ahead of one:
-//   * warp 0 carries the dependency chain (lanes hold rows lane and
-//     lane + 32): it updates column c+1 with the finished column c in
-//     registers, broadcasts the pivot d_{c+1} by shuffle, and scales column
-//     c+1 by d_{c+1}^-1/2;
-//   * meanwhile six warps (none on warp 0's SM sub-partition) apply column c
-//     to the columns right of c+1: a_rq -= l_rc l_qc, c+2 <= q <= r, over a
-//     packed table of the lower triangle ordered by column q descending
-//     (entries with q >= x are its first (64 - x)(65 - x)/2), four entries
-//     per thread at a time so that their FMA chains overlap.
-// One barrier per column; kb^3/6 FMAs.  On this part a dependent FP64
-// operation takes tens of cycles and an FP64 reciprocal square root hundreds
-// (pairing columns to share one did not pay: the longer FP64 sequence per
-// pair cost more), so the chain per column is one FMA, one shuffle, one
-// rsqrt and one multiply, with the positivity test done on the bit pattern.
-constexpr int kPotrfThreads = 256;
+// Factor the kb x kb diagonal block at (k, k) in place (lower), in 64-bit fixed
+// point, as L D L^T with the square roots taken at the end.  An SM does two FP64
+// lanes a cycle, a warp's FP64 instruction is some 64 cycles in flight, and a
+// block is 64 dependent pivots and kb^3/6 multiply-adds: integers are several
+// times faster at both.
+// With row and column i scaled by 2^-k_i so that a_ii is in [1/4, 1), every entry
+// of a positive definite block and of what is left of it after each column lies
+// in (-1, 1): entries are 2^60 a.  Column c (u = L D) is normalised by the even
+// power of two that takes its pivot to M = d 2^(2 f) in [1/4, 1): |u 2^f| <=
+// sqrt(M) < 1 is held to 2^-62, y = 1 / M and (u 2^f) y, both below 4, to 2^-60,
+// and a product of the last two enters the block to 2^-59: sqrt(a_ii a_jj) 2^-59
+// an operation, where FP64's backward error is 2^-53 of it.
+// One CTA holds the block in shared memory (continued by the identity beyond
+// kb).  Phase p does at the same time
+//   * warp 0: d_{p+1} by columns p - 1 and p and its reciprocal, the chain that
+//     all else follows;
+//   * warps 1 and 2 (a row a lane): column p normalised and divided, column p +
+//     1 by columns p - 1 and p;
+//   * twenty warps (one of them on the chain's scheduler): column p - 1 applied
+//     to the columns right of p + 1.  A thread keeps its three entries of the
+//     lower triangle in registers, in order of their columns from the last, so
+//     that whole warps finish as the columns do; a column goes back to shared
+//     memory when it is the next in work.
+// and ends with its one barrier.  A block that leaves these bounds (not positive
+// definite, or a pivot below 2^-52 of its diagonal entry, which FP64 could not
+// tell from zero either) is done over in FP64, column by column.
+// 30 us a block of 64, 46 as a Cholesky in FP64.  What is left: loading and storing
+// it 5 us; 63 phases of 700 cycles while few columns are left, which is the chain
+// (a third of it the reciprocal), and 1000 at first, the multiplications of the
+// bulk: a 32 x 32 -> 64-bit product holds a scheduler's pipe for some ten cycles,
+// half of what the FP64 multiply-add it replaces takes.
+constexpr int kPotrfThreads = 896;
 constexpr int kLd = kNB + 1;
 constexpr int kTriEntries = kNB * (kNB - 1) / 2 + 0;  // (r, q) with 1 <= q <= r <= 63: 2016
+
+// 2^60 a 2^-sh to nearest; |.| >= 2^60, infinities and NaN come back as 2^62.
+__device__ __forceinline__ long long to_fixed60(double a, int sh) {
+    const unsigned long long bits = (unsigned long long)__double_as_longlong(a);
+    const int b = (int)(bits >> 52) & 0x7ff;
+    const unsigned long long m = (bits & 0xfffffffffffffULL) | (b ? 1ULL << 52 : 0ULL);
+    const int s = (b ? b : 1) - 1075 + 60 - sh;  // 2^60 a 2^-sh = m 2^s
+    if (b == 2047 || s > 7) return m ? 1LL << 62 : 0;
+    const unsigned long long v = s >= 0 ? m << s : s < -54 ? 0ULL : ((m >> (-s - 1)) + 1) >> 1;
+    return (bits >> 63) ? -(long long)v : (long long)v;
+}
+
+__device__ __forceinline__ float rcp_approx(float x) {  // to 2^-23
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// A number of 63 bits as hi 2^31 + lo, 0 <= lo < 2^31, and x y 2^-62 without the
+// product of the low halves (from 0 to 2 below): three 32 x 32-bit products, 32
+// cycles a warp.  (__mul64hi takes as long, but wants the operands' signs mended
+// each time, where halves are split once: 35 us a block with it.)
+__device__ __forceinline__ int2 halves(long long x) { return make_int2((int)(x >> 31), (int)x & 0x7fffffff); }
+
+__device__ __forceinline__ long long mul62(int2 x, int2 y) {
+    return (long long)x.x * y.x + (((long long)x.x * y.y + (long long)x.y * y.x) >> 31);
+}
+
+// y = 2^60 / x for x = X 2^-60 in [1/4, 1): the FP32 reciprocal y0 and one
+// third-order step, y0 + y0 (e + e^2) with e = 1 - x y0 (|e| < 2^-21, so the
+// rest is below 2^-63).
+__device__ __forceinline__ unsigned long long fixed_reciprocal(unsigned long long X) {
+    const uint32_t xh = (uint32_t)(X >> 28), xl = (uint32_t)X & 0xfffffffu;
+    const uint32_t y0 = __float2uint_rn(rcp_approx((float)xh) * 2305843009213693952.0f);  // 2^29 / x: 2^61 / xh
+    const long long e = (1LL << 61) - (long long)((unsigned long long)xh * y0 + (((unsigned long long)xl * y0) >> 28));
+    const int e40 = (int)(e >> 21);                             // 2^40 e
+    const long long h = e + ((long long)e40 * e40 >> 19);       // 2^61 (e + e^2)
+    const int hh = (int)(h >> 16);
+    const long long yh =  // 2^74 y0 (e + e^2)
+        (long long)hh * (long long)y0 + (long long)(((unsigned long long)((uint32_t)h & 0xffffu) * y0) >> 16);
+    return ((unsigned long long)y0 << 31) + (unsigned long long)(yh >> 14);
+}
 
 __host__ __device__ constexpr int tri_from(int x) {  // packed entries with column q >= x (1 <= x <= 64)
     return (64 - x) * (65 - x) / 2;
@@ -446,74 +502,166 @@ __device__ __forceinline__ bool positive_finite(double x) {  // integer compares
     return bits > 0 && bits < 0x7FF0000000000000LL;
 }
 
-__global__ void __launch_bounds__(kPotrfThreads) k_potrf64(double *__restrict__ A, int64_t n, int64_t k, int kb,
-                                                           int *__restrict__ info) {
-    __shared__ double L[kNB * kLd];
-    __shared__ uint16_t tab[kTriEntries];
-    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-    for (int e = t; e < kNB * kNB; e += kPotrfThreads) {
-        const int r = e >> 6, c = e & 63;
-        L[r * kLd + c] = (r < kb && c <= r) ? A[(size_t)(k + r) * n + k + c] : (r == c ? 1.0 : 0.0);
-    }
-    // column q (1 .. 63) owns entries [(63 - q)(64 - q)/2, +64 - q): rows q .. 63
-    if (t >= 1 && t < kNB) {
-        const int q = t, s0 = (63 - q) * (64 - q) / 2;
-        for (int r = q; r < kNB; ++r) tab[s0 + r - q] = (uint16_t)((r << 8) | q);
-    }
-    const int r0 = lane, r1 = lane + 32;
-    // warp 0: pivot of column c from d (its updated diagonal) and the scaling
-    // of the column's rows below, held as v0 (row r0) and v1 (row r1)
-    auto pivot_scale = [&](int c, double d, double v0, double v1) {
+// The block in FP64 (shared memory L, lower triangle), column by column.
+__device__ __noinline__ void potrf64_f64(double *L, int64_t k, int kb, int *info) {
+    for (int c = 0; c < kNB; ++c) {
+        double d = L[c * kLd + c];
         if (!positive_finite(d)) {
-            if (lane == 0 && info && c < kb) atomicCAS(info, 0, (int)(k + c + 1));  // the first failure
+            if (threadIdx.x == 0 && info && c < kb) atomicCAS(info, 0, (int)(k + c + 1));  // the first failure
             d = 1e-300;
         }
         const double rs = rsqrt(d);
-        if (r0 >= c) L[r0 * kLd + c] = r0 == c ? d * rs : v0 * rs;
-        if (r1 >= c) L[r1 * kLd + c] = r1 == c ? d * rs : v1 * rs;
+        __syncthreads();
+        for (int r = c + threadIdx.x; r < kNB; r += blockDim.x) L[r * kLd + c] = (r == c ? d : L[r * kLd + c]) * rs;
+        __syncthreads();
+        for (int e = threadIdx.x; e < kNB * kNB; e += blockDim.x) {
+            const int r = e >> 6, q = e & 63;
+            if (q > c && r >= q) L[r * kLd + q] = fma(-L[r * kLd + c], L[q * kLd + c], L[r * kLd + q]);
+        }
+        __syncthreads();
+    }
+}
+
+__global__ void __launch_bounds__(kPotrfThreads) k_potrf64(double *__restrict__ A, int64_t n, int64_t k, int kb,
+                                                           int *__restrict__ info) {
+    __shared__ long long L[kNB * kLd];  // 2^60 u below the diagonal, 2^60 a right of the columns in work
+    __shared__ int2 un[2][kNB];         // u 2^f of the last two columns (2^62 of it)
+    __shared__ int2 ln[2][kNB];         // and that divided by M (2^60)
+    __shared__ int2 ybuf[2];
+    __shared__ long long dd[kNB];
+    __shared__ double rs[kNB];
+    __shared__ int fbuf[2], ke[kNB];
+    __shared__ uint16_t tab[kTriEntries];
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    constexpr int kEach = (kNB * kNB + kPotrfThreads - 1) / kPotrfThreads;
+    double a[kEach];
+#pragma unroll
+    for (int i = 0; i < kEach; ++i) {
+        const int e = t + i * kPotrfThreads, r = e >> 6, c = e & 63;
+        a[i] = e < kNB * kNB && r < kb && c <= r ? A[(size_t)(k + r) * n + k + c] : r == c ? 0.5 : 0.0;
+    }
+#pragma unroll
+    for (int i = 0; i < kEach; ++i) {
+        const int e = t + i * kPotrfThreads, r = e >> 6, c = e & 63;
+        if (e >= kNB * kNB) break;
+        if (r == c) {
+            int x = (__double2hiint(a[i]) >> 20) - 1022;  // a < 2^x
+            if (x < -800 || x > 800) x = 0;               // (also what is not positive: such a block ends in FP64)
+            ke[r] = r < kb ? (x + 1) >> 1 : 0;            // 2 k_i is x or x + 1
+        }
+        // column q (1 .. 63) owns entries [(63 - q)(64 - q)/2, +64 - q): rows q .. 63
+        if (c >= 1 && r >= c) tab[(63 - c) * (64 - c) / 2 + r - c] = (uint16_t)((r << 8) | c);
+    }
+    __syncthreads();
+    bool out = false;
+#pragma unroll
+    for (int i = 0; i < kEach; ++i) {
+        const int e = t + i * kPotrfThreads, r = e >> 6, c = e & 63;
+        if (e >= kNB * kNB) break;
+        const long long v = to_fixed60(a[i], ke[r] + ke[c]);
+        out |= v >= 1LL << 60 || v <= -(1LL << 60) || (r == c && v < 1LL << 58);
+        L[r * kLd + c] = v;
+    }
+    // warp 0: the pivot of column c, its reciprocal and its power of two
+    int2 y = make_int2(0, 0);
+    int f = 0;
+    auto pivot = [&](int c, long long d) {
+        if (d < 256) {
+            out = true;
+            d = 1LL << 59;
+        }
+        f = (__clzll(d) - 4) >> 1;  // d 2^(2 f) in [2^58, 2^60)
+        y = halves((long long)fixed_reciprocal((unsigned long long)d << (2 * f)));
+        if (lane == 0) {
+            ybuf[c & 1] = y;
+            fbuf[c & 1] = f;
+            dd[c] = d;
+        }
     };
+    // bulk warps: 3, and 5 up without the chain's scheduler (8, 12, ...); 4 last
+    constexpr int kBulk = 20 * 32, kOwn = 3;
+    static_assert(kBulk * kOwn >= tri_from(3), "a thread has three entries");
+    const bool bulk = warp >= 3 && ((warp & 3) || warp == 4);
+    const int rank = warp == 4 ? 19 : warp - 3 - (warp >> 2);  // 3, 5, 6, 7, 9 ..: 0 ..
     __syncthreads();
-    if (warp == 0) pivot_scale(0, L[0], L[r0 * kLd], L[r1 * kLd]);
+    long long own[kOwn] = {};
+    int at[kOwn] = {};
+    long long u0 = 0;  // columns: the row's entry of column p
+    int2 un0 = make_int2(0, 0);  // and its normalised one of column p - 1
+    if (warp == 0) {
+        pivot(0, L[0]);
+    } else if (warp <= 2) {
+        u0 = L[(t - 32) * kLd];
+    } else if (bulk) {
+#pragma unroll
+        for (int i = 0; i < kOwn; ++i) {
+            const int e = i * kBulk + rank * 32 + lane;
+            at[i] = e < tri_from(3) ? tab[e] : 0;  // (0: column 0, never written back)
+            own[i] = L[(at[i] >> 8) * kLd + (at[i] & 255)];
+        }
+    }
     __syncthreads();
-    // bulk workers: warps 1-3 and 5-7
-    const int bulk_rank = warp == 0 || warp == 4 ? -1 : (warp < 4 ? warp - 1 : warp - 2) * 32 + lane;
-    constexpr int kBulkThreads = 6 * 32;
-    for (int c = 0; c + 1 < kNB; ++c) {
+    for (int p = 0; p + 1 < kNB; ++p) {
+        const int2 *uprev = un[(p + 1) & 1], *lprev = ln[(p + 1) & 1];
+        const int c1 = p + 1;
         if (warp == 0) {
-            // column c+1 by the finished column c, in registers
-            const double lq = L[(c + 1) * kLd + c];
-            const double v0 = r0 > c ? fma(-L[r0 * kLd + c], lq, L[r0 * kLd + c + 1]) : 0.0;
-            const double v1 = r1 > c ? fma(-L[r1 * kLd + c], lq, L[r1 * kLd + c + 1]) : 0.0;
-            const double d = c + 1 < 32 ? __shfl_sync(0xffffffffu, v0, c + 1) : __shfl_sync(0xffffffffu, v1, c - 31);
-            pivot_scale(c + 1, d, v0, v1);
-        } else if (bulk_rank >= 0) {
-            // four entries at a time, loads first: their FMA chains overlap (a
-            // store could alias the next loads as far as the compiler knows)
-            const int ne = tri_from(c + 2);
-            for (int e0 = bulk_rank; e0 < ne; e0 += 4 * kBulkThreads) {
-                int at[4];
-                double acc[4], x[4], y[4];
+            const int2 u = halves(L[c1 * kLd + p] << (f + 2));
+            long long a = L[c1 * kLd + c1];
+            if (p > 0) a -= mul62(uprev[c1], lprev[c1]);
+            const long long u2 = (long long)u.x * u.x + (((long long)u.x * u.y) >> 30);
+            pivot(c1, a - mul62(halves(u2), y));
+        } else if (warp <= 2) {
+            if (32 * warp > c1) {  // rows of this warp are left
+                const int r = t - 32, fp = fbuf[p & 1] + 2;
+                const int2 yp = ybuf[p & 1];
+                const int2 lq = halves(mul62(halves(L[c1 * kLd + p] << fp), yp));
+                const long long ul = (long long)((unsigned long long)u0 << fp);
+                const int2 u = halves(ul);
+                long long v = L[r * kLd + c1];
+                if (p > 0) v -= mul62(un0, lprev[c1]);
+                out |= r > p && ((ul >> fp) != u0 || ul >= 1LL << 62 || ul <= -(1LL << 62));
+                un[p & 1][r] = u;
+                ln[p & 1][r] = halves(mul62(u, yp));
+                un0 = u;
+                u0 = v - mul62(u, lq);
+                // (the pivot's row is warp 0's: it reads the entry meanwhile)
+                if (r > c1) L[r * kLd + c1] = u0;
+            }
+        } else if (bulk && p > 0) {
+            const int ne = tri_from(p + 2);
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int e = e0 + u * kBulkThreads;
-                    const int rq = e < ne ? tab[e] : ((63 << 8) | 63), r = rq >> 8, q = rq & 255;
-                    at[u] = e < ne ? r * kLd + q : -1;
-                    acc[u] = L[r * kLd + q];
-                    x[u] = L[r * kLd + c];
-                    y[u] = L[q * kLd + c];
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) acc[u] = fma(-x[u], y[u], acc[u]);
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    if (at[u] >= 0) L[at[u]] = acc[u];
+            for (int i = 0; i < kOwn; ++i) {
+                if (i * kBulk + rank * 32 >= ne) break;  // warp-uniform
+                own[i] -= mul62(uprev[at[i] >> 8], lprev[at[i] & 255]);
+                if ((at[i] & 255) == p + 2) L[(at[i] >> 8) * kLd + p + 2] = own[i];
             }
         }
         __syncthreads();
     }
+    if (t < kNB) rs[t] = rsqrt((double)dd[t]);
+    if (__syncthreads_or(out)) {
+        double *Lf = reinterpret_cast<double *>(L);
+        for (int e = t; e < kNB * kNB; e += kPotrfThreads) {
+            const int r = e >> 6, c = e & 63;
+            Lf[r * kLd + c] = (r < kb && c <= r) ? A[(size_t)(k + r) * n + k + c] : (r == c ? 1.0 : 0.0);
+        }
+        __syncthreads();
+        potrf64_f64(Lf, k, kb, info);
+        for (int e = t; e < kNB * kNB; e += kPotrfThreads) {
+            const int r = e >> 6, c = e & 63;
+            if (r < kb && c <= r) A[(size_t)(k + r) * n + k + c] = Lf[r * kLd + c];
+        }
+        return;
+    }
+    // l = u / sqrt(d): 2^60 u 2^-60 2^(k_r + k_c) / sqrt(2^60 d 2^-60 2^(2 k_c))
     for (int e = t; e < kNB * kNB; e += kPotrfThreads) {
         const int r = e >> 6, c = e & 63;
-        if (r < kb && c <= r) A[(size_t)(k + r) * n + k + c] = L[r * kLd + c];
+        if (r < kb && c <= r) {
+            const double l = (double)(r == c ? dd[c] : L[r * kLd + c]) * rs[c];
+            // (times 2^(k_r - 30) on the exponent: |l| is 0 or above 2^-31)
+            A[(size_t)(k + r) * n + k + c] =
+                l == 0.0 ? 0.0 : __hiloint2double(__double2hiint(l) + ((ke[r] - 30) << 20), __double2loint(l));
+        }
     }
 }
 

@@ -55,3 +55,19 @@ def test_direct_solve_residual(ctx, N, M, Ns, prec, eps, solver):
     # the sample-space form subtracts vectors of size ||F|| / eps
     size = np.linalg.norm(A) * (np.linalg.norm(x) + (np.linalg.norm(F) / eps if solver != "cholesky" else 0.0))
     assert np.linalg.norm(A @ x - F) <= 8 * n * 2.0 ** -53 * (size + np.linalg.norm(F))
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+@pytest.mark.parametrize("at", [7, 40, 62])
+def test_a_block_without_a_factor(ctx, bad, at):
+    """A bias or weight of a hidden unit that is not a number reaches S through the
+    unit's activations: the diagonal block leaves the fixed-point range and is done in
+    FP64, where it spreads as it does in any Cholesky factorisation."""
+    N, M, Ns = 7, 7, 65
+    p, s, _, F = _system(N, M, Ns)
+    p[at] = bad
+    if np.isinf(bad):  # an infinite weight: infinity - infinity somewhere
+        p[N + M:N + M + N] = bad
+    delta = torch.empty(p.size, dtype=torch.float64, device=dev())
+    nk.nk_sr_solve(ctx, cu(p), N, M, cu(s), cu(F), delta, solver="cholesky", diag_shift=0.01)
+    assert torch.isnan(delta).all()
