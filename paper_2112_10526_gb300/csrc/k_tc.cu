@@ -115,6 +115,11 @@ __global__ void k_slice_rows(const double *__restrict__ A, int64_t lda, int64_t 
 //     lane quarter) and 8 columns, loads its C entries a tile ahead, and
 //     turns the S accumulators into FP64 by exact integer recombination
 //     before writing C back.
+// A tile's epilogue takes the longest (6000 cycles on 16 warps, against 1800 of
+// MMAs and 2000 of FP64 additions, two lanes a cycle): whole tiles test no entry,
+// C moves 16 bytes a lane where its rows allow it, and L2 is asked for a row's
+// segment once, which took 170 instructions an entry to 98 and the trailing
+// update of a 8064 x 8064 matrix from 228 to 194 us.
 // Strips (lower triangle only when `lower`) are numbered row by row.  CTAs
 // are short-lived on purpose: kernels of a higher-priority stream (the
 // Cholesky look-ahead) get SMs as strips retire.  mbarriers hand buffers
@@ -133,6 +138,7 @@ struct OzArgs {
     int64_t n_nb;         // tile columns
     int chunk;            // tiles per strip: 1, 2, 4 or 8
     int chunk_log2;
+    int vec;              // pairs of C's entries are 16-byte aligned
 };
 
 constexpr int kPN = 32;                      // tile columns
@@ -313,42 +319,60 @@ __global__ void __launch_bounds__(kPThreads, 1)
         // --------------------------------------------------------- epilogue
         // Lane l turns TMEM lane 32q + l (tile row 32q + l) into FP64 for the
         // warp's 8 columns and parks the values in its shared block
-        // [32 rows][8 columns] (column index XOR (row / 2) mod 8: conflict-free
-        // for both access patterns); C is then read and written with lane l on
-        // row 4k + l / 8, column l mod 8 (k = 0 .. 7), 64-byte row segments.
+        // [32 rows][8 columns], 16 bytes at a time (pair index XOR (row / 2) mod
+        // 4: conflict-free for both access patterns); C is then read and written
+        // with lane l on row 8k + l / 4, columns 2 (l mod 4) and the next (k = 0
+        // .. 3), 64-byte row segments.
         const int q = warp & 3;                 // TMEM lane quarter = tile rows 32q .. 32q + 31
         const int c0 = ((warp - 2) >> 2) * kPColsPerWarp;  // the warp's 8 tile columns
         const uint32_t lane_base = (uint32_t)(q * 32) << 16;
-        double *stage = reinterpret_cast<double *>(sE) + (warp - 2) * 32 * kPColsPerWarp;
+        double2 *stage = reinterpret_cast<double2 *>(sE) + (warp - 2) * 32 * (kPColsPerWarp / 2);
         const int64_t row = m0 + q * 32 + lane;
         const int ei = row < a.rows ? a.expA[row] : 0;
-        const int rr = lane >> 3, cc = lane & 7;
-        const int64_t row_c = m0 + q * 32 + rr;  // + 4k: the rows this lane reads and writes in C
+        const int rr = lane >> 2, cc = 2 * (lane & 3);
+        const int64_t row_c = m0 + q * 32 + rr;  // + 8k: the rows this lane reads and writes in C
+        const int64_t step = 8 * a.ldc;
         auto on = [&](int64_t r, int64_t col) { return r < a.rows && col < a.cols && !(a.lower && col > r); };
-        auto load_c = [&](int i, double (&cv)[8]) {
+        // tiles that lie in C (and below its diagonal) whole need no test of their entries
+        auto whole = [&](int i) {
+            const int64_t end = (nb0 + i + 1) * kPN;
+            return m0 + kTileM <= a.rows && end <= a.cols && !(a.lower && end > m0 + 1);
+        };
+        auto load_c = [&](int i, double2 (&cv)[4]) {
             const int64_t col = (nb0 + i) * kPN + c0 + cc;
+            const double *p = a.C + (size_t)row_c * a.ldc + col;
+            if (a.mode == 0) {
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const int64_t r = row_c + 4 * k;
-                cv[k] = (a.mode != 0 && on(r, col)) ? a.C[(size_t)r * a.ldc + col] : 0.0;
+                for (int k = 0; k < 4; ++k) cv[k] = make_double2(0.0, 0.0);
+            } else if (whole(i)) {
+                if (a.vec) {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) cv[k] = *reinterpret_cast<const double2 *>(p + k * step);
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) cv[k] = make_double2(p[k * step], p[k * step + 1]);
+                }
+            } else {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int64_t r = row_c + 8 * k;
+                    cv[k] = make_double2(on(r, col) ? p[k * step] : 0.0, on(r, col + 1) ? p[k * step + 1] : 0.0);
+                }
             }
         };
         // column exponents (lane & 7 holds column c0 + (lane & 7)), broadcast by shuffles
         auto load_f = [&](int i) {
-            const int64_t col = (nb0 + i) * kPN + c0 + cc;
+            const int64_t col = (nb0 + i) * kPN + c0 + (lane & 7);
             return col < a.cols ? a.expB[col] : 0;
         };
-        const long long flip = a.mode == 1 ? (long long)0x8000000000000000ULL : 0LL;
+        const int flip = a.mode == 1 ? (int)0x80000000 : 0;  // of the sign in the upper half
         if (a.mode != 0) {
             // the strip's C entries (at most 128 x 256 FP64 per CTA) into L2 up
-            // front, so that the per-tile loads below wait on L2, not on HBM
+            // front, so that the per-tile loads below wait on L2, not on HBM:
+            // a lane per row of the warp's 8 columns
             for (int i = 0; i < count; ++i) {
-                const int64_t col = (nb0 + i) * kPN + c0 + cc;
-#pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    const int64_t r = row_c + 4 * k;
-                    if (on(r, col)) prefetch_l2(a.C + (size_t)r * a.ldc + col);
-                }
+                const int64_t col = (nb0 + i) * kPN + c0;
+                if (on(row, col)) prefetch_l2(a.C + (size_t)row * a.ldc + col);
             }
         }
         for (int i = 0; i < count; ++i) {
@@ -356,7 +380,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
             const uint32_t use = (uint32_t)(i >> 1);
             // this tile's C entries and column exponents are in flight while
             // the accumulators fill and drain; C is needed only at the end
-            double cv[8];
+            double2 cv[4];
             load_c(i, cv);
             const int fj_lane = load_f(i);
             int ok = 1;
@@ -375,6 +399,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
                     if (gi < S)
                         tmem_ld2(tmem + (uint32_t)b * kPAccCols + lane_base + (uint32_t)(gi * kPN + c0 + c4), r[gi]);
                 tmem_wait_ld();
+                double v[2];
 #pragma unroll
                 for (int j = 0; j < 2; ++j) {
                     int d[kMaxSlices];
@@ -382,24 +407,31 @@ __global__ void __launch_bounds__(kPThreads, 1)
                     for (int gi = 0; gi < kMaxSlices; ++gi)
                         d[gi] = gi < S ? __float2int_rn(__uint_as_float(r[gi][j])) : 0;
                     // V 2^sc with V = sum_g D_g 2^(8 (8 - g)); C - R as C + (-R)
-                    const int sc = ei + __shfl_sync(0xffffffffu, fj_lane, c4 + j) - 64;
-                    const double v = __longlong_as_double(
-                        __double_as_longlong(window_to_double(ozaki_window8(d), sc + 8)) ^ flip);
-                    const int c = c4 + j;
-                    stage[lane * 8 + (c ^ ((lane >> 1) & 7))] = v;
+                    const int sc = ei + __shfl_sync(0xffffffffu, fj_lane, c4 + j) - 56;
+                    const double x = window_to_double_seldom(ozaki_window8(d), sc);
+                    v[j] = __hiloint2double(__double2hiint(x) ^ flip, __double2loint(x));
                 }
+                stage[lane * 4 + ((c4 >> 1) ^ ((lane >> 1) & 3))] = make_double2(v[0], v[1]);
             }
             // the accumulators are drained: hand the buffer back before the C traffic
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&acc_empty[b]);
             const int64_t col = (nb0 + i) * kPN + c0 + cc;
+            double *p = a.C + (size_t)row_c * a.ldc + col;
+            const bool all = whole(i);
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const int rl = 4 * k + rr;
-                const double v = stage[rl * 8 + (cc ^ ((rl >> 1) & 7))];
-                const int64_t r = row_c + 4 * k;
-                if (on(r, col)) a.C[(size_t)r * a.ldc + col] = cv[k] + v;  // C reads as 0 in mode 0
+            for (int k = 0; k < 4; ++k) {
+                const int rl = 8 * k + rr;
+                const double2 v = stage[rl * 4 + ((lane & 3) ^ ((rl >> 1) & 3))];
+                const double x = cv[k].x + v.x, y = cv[k].y + v.y;  // C reads as 0 in mode 0
+                if (all && a.vec) {
+                    *reinterpret_cast<double2 *>(p + k * step) = make_double2(x, y);
+                } else {
+                    const int64_t r = row_c + 8 * k;
+                    if (on(r, col)) p[k * step] = x;
+                    if (on(r, col + 1)) p[k * step + 1] = y;
+                }
             }
             __syncwarp();
         }
@@ -1088,7 +1120,8 @@ cudaError_t launch_ozaki_gemm_strided(const __nv_bfloat16 *Asl, const int *expA,
     const void *kern = S == kMaxSlices ? (const void *)k_ozaki_gemm<kMaxSlices> : (const void *)k_ozaki_gemm<0>;
     cudaError_t e = nk::allow_max_dynamic_smem(kern);
     if (e != cudaSuccess) return e;
-    OzArgs a{rows, cols, S, expA, expB, C, ldc, mode, lower ? 1 : 0, err, (cols + kPN - 1) / kPN, 1, 0};
+    OzArgs a{rows, cols, S, expA, expB, C, ldc, mode, lower ? 1 : 0, err, (cols + kPN - 1) / kPN, 1, 0,
+             ldc % 2 == 0 && reinterpret_cast<uintptr_t>(C) % 16 == 0};
     const int64_t n_mb = (rows + kTileM - 1) / kTileM;
     // strips of up to 8 tiles amortise a CTA's A slices over its tiles; a
     // product with few tiles per SM (the panel solve and the narrow update of

@@ -348,6 +348,27 @@ __host__ __device__ __forceinline__ double window_to_double(long long x, int sc)
     return v;
 }
 
+// The same on 32-bit halves, with zero and the ends of the exponent range in a
+// branch that is seldom taken: some 25 instructions where the form above has 35,
+// for an epilogue bound by them (half a warp a cycle and scheduler).
+__device__ __forceinline__ double window_to_double_seldom(long long x, int sc) {
+    const long long s = x >> 63;
+    const unsigned long long m = (unsigned long long)((x ^ s) - s);
+    const uint32_t mh = (uint32_t)(m >> 32), ml = (uint32_t)m;
+    const bool low = mh == 0;
+    const uint32_t a = low ? ml : mh, b = low ? 0u : ml;
+    const int z = __clz((int)a);
+    const uint32_t hi = __funnelshift_l(b, a, z), lo = b << (z & 31);  // leading one at bit 63 (m != 0)
+    const int eb = (low ? 1054 : 1086) - z + sc;
+    const unsigned long long r = ((((unsigned long long)hi << 32) | lo) >> 11) + ((lo >> 10) & 1u);
+    unsigned long long bits = r + ((unsigned long long)((uint32_t)(eb - 1) << 20) << 32);
+    if (a == 0u || (unsigned)(eb - 1) >= 2045u) {
+        const int ef = eb + (int)(r >> 53);
+        bits = (a == 0u || ef < 1) ? 0ULL : (ef > 2046 ? 0x7FF0000000000000ULL : bits);
+    }
+    return __longlong_as_double((long long)(bits | ((unsigned long long)s & 0x8000000000000000ULL)));
+}
+
 // The four FP32 levels of a 4-slice product (exact integers, |D_t| < 2^22)
 // as the signed 64-bit V = D_0 2^24 + D_1 2^16 + D_2 2^8 + D_3.  One FP32 add
 // of 1.5 2^23 turns a level into the bit pattern 0x4B400000 + D_t (ulp 1 in
