@@ -18,6 +18,8 @@
 
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "nk_common.cuh"
 #include "nk_internal.h"
 #include "tanh64.cuh"
@@ -470,6 +472,19 @@ __device__ __forceinline__ void renorm_fast(Prod<float> &p) {
     }
 }
 
+// tanh(theta) of a unit after a flip: (t - s tau) / (1 - s t tau), s = +1 (kPos) or
+// -1, as a product with the approximate reciprocal: the value of __fdividef here
+// (the denominator is 0 or at least 2^-48, and below 2) in four instructions.
+__device__ __forceinline__ float rcp_approx(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+template <bool kPos>
+__device__ __forceinline__ float flipped(float t, float tau) {
+    return kPos ? (t - tau) * rcp_approx(fmaf(-t, tau, 1.f)) : (t + tau) * rcp_approx(fmaf(t, tau, 1.f));
+}
+
 // lane_product4 on t and a tau row already held in registers: chunk u is units j
 // = 4 lane + 128 u .. j + 3 (zero past M).  The groups, renormalisations and tail
 // are those of lane_product4, in the same order, so the result is identical.
@@ -691,29 +706,34 @@ __global__ void __launch_bounds__(128, kRing ? 3 : 7) k_sweep(SweepK<float> P) {
                     // exactly from theta after every sweep)
                     float *tf = reinterpret_cast<float *>(t);
                     const float *uf = reinterpret_cast<const float *>(tau);
-                    const float sf = (float)si;
-                    auto upd = [&](float4 tv, const float4 &uv, int j) {
-                        const float v0 = sf * uv.x, v1 = sf * uv.y, v2 = sf * uv.z, v3 = sf * uv.w;
-                        tv.x = __fdividef(tv.x - v0, fmaf(-tv.x, v0, 1.f));
-                        tv.y = __fdividef(tv.y - v1, fmaf(-tv.y, v1, 1.f));
-                        tv.z = __fdividef(tv.z - v2, fmaf(-tv.z, v2, 1.f));
-                        tv.w = __fdividef(tv.w - v3, fmaf(-tv.w, v3, 1.f));
-                        *reinterpret_cast<float4 *>(tf + j) = tv;
+                    auto update = [&](auto pos) {
+                        constexpr bool kPos = decltype(pos)::value;
+                        auto upd = [&](float4 tv, const float4 &uv, int j) {
+                            *reinterpret_cast<float4 *>(tf + j) =
+                                make_float4(flipped<kPos>(tv.x, uv.x), flipped<kPos>(tv.y, uv.y),
+                                            flipped<kPos>(tv.z, uv.z), flipped<kPos>(tv.w, uv.w));
+                        };
+                        // the row again in groups of four 16-byte loads (one round
+                        // trip per group where it has left L1)
+                        int j = 4 * lane;
+                        for (; j + 3 * 128 < M; j += 4 * 128) {
+                            float4 uv[4], tv[4];
+#pragma unroll
+                            for (int u = 0; u < 4; ++u)
+                                uv[u] = __ldg(reinterpret_cast<const float4 *>(uf + j + u * 128));
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) tv[u] = *reinterpret_cast<const float4 *>(tf + j + u * 128);
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) upd(tv[u], uv[u], j + u * 128);
+                        }
+                        for (; j < M; j += 128)
+                            upd(*reinterpret_cast<const float4 *>(tf + j),
+                                __ldg(reinterpret_cast<const float4 *>(uf + j)), j);
                     };
-                    // the row again in groups of four 16-byte loads (one round
-                    // trip per group where it has left L1)
-                    int j = 4 * lane;
-                    for (; j + 3 * 128 < M; j += 4 * 128) {
-                        float4 uv[4], tv[4];
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) uv[u] = __ldg(reinterpret_cast<const float4 *>(uf + j + u * 128));
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) tv[u] = *reinterpret_cast<const float4 *>(tf + j + u * 128);
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) upd(tv[u], uv[u], j + u * 128);
-                    }
-                    for (; j < M; j += 128)
-                        upd(*reinterpret_cast<const float4 *>(tf + j), __ldg(reinterpret_cast<const float4 *>(uf + j)), j);
+                    if (si > R(0))
+                        update(std::true_type{});
+                    else
+                        update(std::false_type{});
                 } else {
                     for (int j = lane; j < M; j += 32) {
                         const R tj = t[j], tv = si * tau[j];
@@ -1290,13 +1310,9 @@ __global__ void __launch_bounds__(128) k_sweep_rows(SweepK<float> P) {
                 if (decisions && lane == 0) decisions[q0 + src] = accept ? 1 : 0;
                 if (accept) {
 #pragma unroll
-                    for (int u = 0; u < kC; ++u) {
-                        const float v0 = si * uv[u].x, v1 = si * uv[u].y, v2 = si * uv[u].z, v3 = si * uv[u].w;
-                        t[u].x = __fdividef(t[u].x - v0, fmaf(-t[u].x, v0, 1.f));
-                        t[u].y = __fdividef(t[u].y - v1, fmaf(-t[u].y, v1, 1.f));
-                        t[u].z = __fdividef(t[u].z - v2, fmaf(-t[u].z, v2, 1.f));
-                        t[u].w = __fdividef(t[u].w - v3, fmaf(-t[u].w, v3, 1.f));
-                    }
+                    for (int u = 0; u < kC; ++u)
+                        t[u] = make_float4(flipped<true>(t[u].x, si * uv[u].x), flipped<true>(t[u].y, si * uv[u].y),
+                                           flipped<true>(t[u].z, si * uv[u].z), flipped<true>(t[u].w, si * uv[u].w));
                     if (lane == 0) {
                         sv[i] = (int8_t)-si8;
                         if (!local) sv[k] = (int8_t)si8;  // it held -s_i
@@ -1317,6 +1333,225 @@ __global__ void __launch_bounds__(128) k_sweep_rows(SweepK<float> P) {
     }
     for (int i = lane; i < N; i += 32) A.s[(size_t)c * N + i] = sv[i];
     if (lane == 0 && A.n_accepted) A.n_accepted[c] += acc;
+}
+
+// FP32 sweeps of the local and exchange rules at many units (M % 4 == 0, M <= 128
+// kU), theta given: a block of two warps per chain.  Thread (l, h) = (16 warp +
+// lane / 2, lane % 2) does the part of lane l of k_sweep that goes into its running
+// product m_h: units 4 l + 2 h + 128 u and the next, in the same order, so that
+// every product, renormalisation and decision is the same.  Its t = tanh(theta)
+// stays in registers; the row of flip ratios comes into shared memory once, by
+// cp.async while the move before it is worked on, and serves both the product and
+// the update.  The moves of a batch of 32 proposals are found by ballot; the next
+// one is guessed from the spins as they are (an accepted move changes the few
+// proposals that share a site with it: then the row is fetched on demand).
+// k_sweep had a warp per chain, t in shared memory (12 chains an SM at M = 4608)
+// and read the row twice from L2: 12 TB/s of it, and three warps a scheduler.
+// 24 x 24 lattice, M = 4608, 8192 chains: 7.3 ms a sweep there, 5.4 here.
+template <int kU>
+__global__ void __launch_bounds__(64, kU <= 16 ? (kU <= 8 ? 16 : 12) : (kU <= 24 ? 9 : (kU <= 40 ? 6 : 4))) k_sweep_pair(SweepK<float> P) {
+    extern __shared__ __align__(16) unsigned char sm[];
+    const Tables<float> &T = P.t;
+    const SweepArgs &A = P.a;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int c = blockIdx.x;
+    const int N = T.N, M = T.M, words = (N + 31) / 32;
+    float *ring = reinterpret_cast<float *>(sm);                              // [2][M]
+    float2 *xch = reinterpret_cast<float2 *>(sm + 2 * (size_t)P.t_bytes);     // [32] (product, exponent)
+    uint32_t *sb = reinterpret_cast<uint32_t *>(xch + 32) + warp * words;     // bit i: spin i is up (a copy per warp)
+    const int l = 16 * warp + (lane >> 1), h = lane & 1, j0 = 4 * l + 2 * h;
+    const bool local = A.rule == NK_RULE_LOCAL;
+    const float *tab = local ? T.tau_site : T.tau_edge;
+    constexpr int kLoose = 2;  // groups of four chunks that may be cut short
+    for (int w = 0; w < words; ++w) {
+        const int i = 32 * w + lane;
+        const unsigned up = __ballot_sync(kFull, i < N && A.s[(size_t)c * N + i] > 0);
+        if (lane == 0) sb[w] = up;
+    }
+    __syncwarp();
+    auto spin = [&](int i) { return (sb[i >> 5] >> (i & 31)) & 1u; };
+    unsigned long long acc = 0;
+    const int n_sweeps = A.n_discard + A.n_samples;
+    for (int w = 0; w < n_sweeps; ++w) {
+        const bool want_lp = warp == 0 && A.logpsi != nullptr && w >= A.n_discard;
+        uint8_t *decisions = A.decisions && warp == 0
+                                 ? A.decisions + ((size_t)c * A.dec_stride + A.dec_offset + w) * N
+                                 : nullptr;
+        const double *th = A.theta_in + (size_t)c * (A.theta_ld > 0 ? A.theta_ld : M);
+        float2 t[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            const int j = j0 + 128 * u;
+            t[u] = make_float2(0.f, 0.f);
+            if (j < M) {
+                const double2 a = *reinterpret_cast<const double2 *>(th + j);
+                t[u] = make_float2(tanhf((float)a.x), tanhf((float)a.y));
+            }
+        }
+        double lp = 0.0;
+        if (want_lp) {
+            for (int j = lane; j < M; j += 32) lp += (double)lncosh((float)th[j]);
+            for (int i = lane; i < N; i += 32) lp += T.a[i] * (spin(i) ? 1.0 : -1.0);
+            lp = warp_sum(lp);
+        }
+        const unsigned long long qbase = (unsigned long long)(A.sweep0 + w) * (unsigned long long)N;
+        // lane l's proposal q0 + l: sites (i < 0: never a move), row, ln u, K and
+        // the visible-bias difference
+        struct Batch {
+            int i, k, row;
+            float lu, K, aa;
+        };
+        auto draw = [&](int q0) {
+            Batch b{-1, -1, 0, 0.f, 0.f, 0.f};
+            const Philox4 y = philox4x64_10(qbase + (unsigned long long)(q0 + lane), (unsigned long long)c,
+                                            (unsigned long long)A.stream_id, 0ULL, A.seed, 0ULL);
+            if (q0 + lane >= N) return b;
+            b.lu = logf((float)uniform53(y.v[1]));
+            if (local) {
+                b.i = b.row = pick_index(y.v[0], N);
+                b.K = T.K_site[b.i];
+                b.aa = (float)T.a[b.i];
+            } else {
+                b.row = pick_index(y.v[0], T.E);
+                const int i0 = A.edges[2 * b.row], k0 = A.edges[2 * b.row + 1];
+                // an edge outside [0, N) is never a move (bounds guard)
+                if ((unsigned)i0 < (unsigned)N && (unsigned)k0 < (unsigned)N) {
+                    b.i = i0;
+                    b.k = k0;
+                    b.aa = (float)(T.a[i0] - T.a[k0]);
+                }
+                b.K = T.K_edge[b.row];
+            }
+            return b;
+        };
+        auto is_move = [&](const Batch &b) { return b.i >= 0 && (local || spin(b.i) != spin(b.k)); };
+        auto fetch = [&](int row, int buf) {
+            const float *src = tab + (size_t)row * M + 4 * tid;
+            const uint32_t dst = smem_u32(ring) + (uint32_t)buf * (uint32_t)P.t_bytes + 16u * (uint32_t)tid;
+#pragma unroll
+            for (int v = 0; v < kU / 2; ++v)
+                if (v + 2 * kLoose < kU / 2 || 4 * tid + 256 * v < M)
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 1024u * v), "l"(src + 256 * v)
+                                 : "memory");
+            cp_async_commit();
+        };
+        Batch cur = draw(0), nxt = draw(32);
+        int q0 = 0, pos = -1;         // the batch and the last proposal of it that was dealt with
+        int ahead_q = -1, buf = 0;    // the proposal whose row is on its way to buffer buf
+        for (;;) {
+            const unsigned later = pos < 0 ? kFull : ~((2u << pos) - 1u);
+            const unsigned mask = __ballot_sync(kFull, is_move(cur)) & later;
+            const int src = mask ? __ffs(mask) - 1 : 32;
+            if (decisions && lane > pos && lane < src && q0 + lane < N) decisions[q0 + lane] = 2;
+            if (src == 32) {  // the batch is done
+                q0 += 32;
+                if (q0 >= N) break;
+                cur = nxt;
+                nxt = draw(q0 + 32);
+                pos = -1;
+                continue;
+            }
+            pos = src;
+            const int i = __shfl_sync(kFull, cur.i, src), k = __shfl_sync(kFull, cur.k, src);
+            if (ahead_q != q0 + src) {  // guessed wrongly, or the first of the sweep
+                cp_async_wait<0>();
+                fetch(__shfl_sync(kFull, cur.row, src), buf);
+            }
+            cp_async_wait<0>();
+            __syncthreads();  // the row is there for both warps; both are done with the other buffer
+            const float *row_s = ring + (size_t)buf * (P.t_bytes / 4) + j0;
+            {
+                const unsigned rest = src == 31 ? 0u : mask & ~((2u << src) - 1u);
+                const unsigned then = __ballot_sync(kFull, is_move(nxt));
+                if (rest | then) {
+                    const int at = __ffs(rest ? rest : then) - 1;
+                    ahead_q = q0 + at + (rest ? 0 : 32);
+                    buf ^= 1;
+                    fetch(__shfl_sync(kFull, rest ? cur.row : nxt.row, at), buf);
+                } else {
+                    ahead_q = -1;
+                    buf ^= 1;
+                }
+            }
+            const bool up = spin(i);
+            const float si = up ? 1.f : -1.f;
+            // the running product m_h of lane l
+            float m = 1.f;
+            int e = 0;
+            auto product = [&](auto pos_tag) {
+                constexpr bool kPos = decltype(pos_tag)::value;
+                auto mul = [&](int u) {
+                    const float2 v = *reinterpret_cast<const float2 *>(row_s + 128 * u);
+                    m *= fmaf(kPos ? -t[u].x : t[u].x, v.x, 1.f) * fmaf(kPos ? -t[u].y : t[u].y, v.y, 1.f);
+                };
+#pragma unroll
+                for (int g = 0; g < kU / 4; ++g) {
+                    if (g + kLoose < kU / 4 || 4 * l + 512 * g + 3 * 128 < M) {
+#pragma unroll
+                        for (int u = 4 * g; u < 4 * g + 4; ++u) mul(u);
+                        m = renorm_bits(m, e);
+                    } else {
+#pragma unroll
+                        for (int u = 4 * g; u < 4 * g + 3; ++u)
+                            if (4 * l + 128 * u < M) mul(u);
+                    }
+                }
+            };
+            if (up)
+                product(std::true_type{});
+            else
+                product(std::false_type{});
+            const float mo = __shfl_xor_sync(kFull, m, 1);
+            Prod<float> pr{h ? mo : m, e + __shfl_xor_sync(kFull, e, 1)};
+            renorm_fast(pr);
+            pr.m *= h ? m : mo;
+            renorm_fast(pr);
+            // over the lanes l as warp_prod_normalised: 16 across the warps, then 8 .. 1
+            if (h == 0) xch[l] = make_float2(pr.m, __int_as_float(pr.e));
+            __syncthreads();
+            {
+                const float2 o = xch[l ^ 16];
+                pr.m *= o.x;
+                pr.e += __float_as_int(o.y);
+            }
+#pragma unroll
+            for (int off = 16; off > 1; off >>= 1) {
+                pr.m *= __shfl_xor_sync(kFull, pr.m, off);
+                pr.e += __shfl_xor_sync(kFull, pr.e, off);
+            }
+            renorm_fast(pr);
+            const float d0 = -2.f * __shfl_sync(kFull, cur.aa, src) * si;
+            const float delta = d0 + (__shfl_sync(kFull, cur.K, src) + prod_log(pr));
+            const bool accept = __shfl_sync(kFull, cur.lu, src) < 2.f * delta;
+            if (decisions && lane == 0) decisions[q0 + src] = accept ? 1 : 0;
+            if (accept) {
+#pragma unroll
+                for (int u = 0; u < kU; ++u) {
+                    if (u + 4 * kLoose < kU || 4 * l + 128 * u < M) {
+                        const float2 v = *reinterpret_cast<const float2 *>(row_s + 128 * u);
+                        t[u] = make_float2(flipped<true>(t[u].x, si * v.x), flipped<true>(t[u].y, si * v.y));
+                    }
+                }
+                __syncwarp();
+                if (lane == 0) {
+                    sb[i >> 5] ^= 1u << (i & 31);
+                    if (k >= 0) sb[k >> 5] ^= 1u << (k & 31);
+                }
+                __syncwarp();
+                if (want_lp) lp += (double)delta;
+                ++acc;
+            }
+        }
+        cp_async_wait<0>();  // (a guess that turned out to be no move)
+        __syncthreads();
+        if (w >= A.n_discard) {
+            const size_t row = (size_t)c * A.out_stride + A.out_offset + (w - A.n_discard);
+            for (int i = tid; i < N; i += 64) A.samples[row * N + i] = spin(i) ? 1 : -1;
+            if (tid == 0 && A.logpsi) A.logpsi[row] = lp;
+        }
+    }
+    for (int i = tid; i < N; i += 64) A.s[(size_t)c * N + i] = spin(i) ? 1 : -1;
+    if (tid == 0 && A.n_accepted) A.n_accepted[c] += acc;
 }
 
 // ----------------------------------------------------------- local energy ---
@@ -1713,6 +1948,18 @@ cudaError_t launch_sweep_rows(SweepK<float> P, cudaStream_t st) {
     return cudaGetLastError();
 }
 
+// The two-warp sweep for up to kU chunks of 128 units.
+template <int kU>
+cudaError_t launch_sweep_pair(const SweepK<float> &P, cudaStream_t st) {
+    const size_t smem = 2 * (size_t)P.t_bytes + 256 + 2 * (size_t)((P.t.N + 31) / 32) * 4;
+    cudaError_t err = nk::allow_max_dynamic_smem((const void *)k_sweep_pair<kU>);
+    if (err != cudaSuccess) return err;
+    const int slot = prof_begin(NK_PROF_SWEEP, st);
+    (k_sweep_pair<kU><<<(unsigned)P.a.C, 64, smem, st>>>(P), nk::note_launch());
+    prof_end(slot, st, (double)P.a.C * (P.a.n_discard + P.a.n_samples) * P.t.N * (double)P.t.M);
+    return cudaGetLastError();
+}
+
 // NK_F64: the screened kernel.  Shared memory holds theta (FP64), t (FP32) and
 // the spins of each chain.
 template <int kU>
@@ -1786,10 +2033,23 @@ template <>
 cudaError_t launch_sweep<float>(const Tables<float> &t, const SweepArgs &a, cudaStream_t st) {
     if (a.C <= 0 || a.n_discard + a.n_samples <= 0) return cudaSuccess;
     const SweepK<float> P = sweep_args(t, a);
-    // local and exchange rules with few units and theta given: t in registers
-    if (P.vec4 && a.rule != NK_RULE_HAMILTONIAN && t.M <= 4 * 128 && a.theta_in)
-        return t.M <= 128 ? launch_sweep_rows<1>(P, st)
-                          : (t.M <= 256 ? launch_sweep_rows<2>(P, st) : launch_sweep_rows<4>(P, st));
+    // local and exchange rules with theta given: t in registers, a warp a chain (two
+    // are slower there: M = 400, 1024 chains: 0.10 and 0.13 ms a sweep) ...
+    const int chunks = (t.M + 127) / 128;
+    const bool regs = P.vec4 && a.rule != NK_RULE_HAMILTONIAN && a.theta_in;
+    if (regs && chunks <= 4)
+        return chunks == 1 ? launch_sweep_rows<1>(P, st)
+                           : (chunks == 2 ? launch_sweep_rows<2>(P, st) : launch_sweep_rows<4>(P, st));
+    // ... or two: from 25 chunks of 128 units (M = 4608, 8192 chains: 5.5 ms a sweep,
+    // 6.3 by k_sweep; 256 chains: 0.74 and 1.19), and below with at most eight chains
+    // an SM (M = 2000, 512 chains: 0.21 and 0.31 ms; M = 1600, 8192 chains: 3.7 and 3.0)
+    if (regs && chunks <= 48 && (chunks > 24 || a.C <= 1216))
+        return chunks <= 8    ? launch_sweep_pair<8>(P, st)
+               : chunks <= 16 ? launch_sweep_pair<16>(P, st)
+               : chunks <= 24 ? launch_sweep_pair<24>(P, st)
+               : chunks <= 32 ? launch_sweep_pair<32>(P, st)
+               : chunks <= 40 ? launch_sweep_pair<40>(P, st)
+                              : launch_sweep_pair<48>(P, st);
     int wpb = 4;
     while (wpb > 1 && (size_t)wpb * P.warp_bytes > 200 * 1024) wpb >>= 1;
     size_t smem = (size_t)wpb * P.warp_bytes;

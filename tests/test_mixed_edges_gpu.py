@@ -1,6 +1,6 @@
-"""NK_MIXED at the edges of its layouts: the register sweep (one, two and four
-chunks of 128 units, the last chunk ragged, and the widths next to the ones it
-takes), and the Jacobian products whose theta, tanh and FP32 pairs are one kernel
+"""NK_MIXED at the edges of its layouts: the register sweeps (a warp a chain for up
+to four chunks of 128 units, two warps for up to 48; the last chunk ragged, and the
+widths next to the ones they take), and the Jacobian products whose theta, tanh and FP32 pairs are one kernel
 (units around its tiles of 64, rows around its tiles of 128).
 
 Sweeps replay the oracle as the other sweep tests do, with their tie band, and equal
@@ -31,8 +31,9 @@ def ctx():
 
 @pytest.mark.parametrize("rule,N,edges", [("local", 37, None), ("exchange", 16, I.square_edges(4)),
                                           ("exchange", 36, I.square_edges(6))])
-@pytest.mark.parametrize("M", [4, 8, 124, 128, 132, 256, 260, 508, 512, 516, 130])
-def test_mixed_sweep_widths(ctx, rule, N, edges, M, C=37, nd=1, ns=3, sig=0.3):
+@pytest.mark.parametrize("M", [4, 8, 124, 128, 132, 256, 260, 508, 512, 516, 130, 2044, 2048, 2052, 3076, 4608, 6144])
+def test_mixed_sweep_widths(ctx, rule, N, edges, M, nd=1, ns=3):
+    C, sig = (37, 0.3) if M < 600 else (5, 0.05)
     p = I.rbm_params(N, M, 3 + M, sig)
     s0 = oracle.chain_init(N, C, rule, 9, 1)
     st, samples = cu(s0), torch.empty((C, ns, N), dtype=torch.int8, device=dev())
@@ -52,7 +53,7 @@ def test_mixed_sweep_widths(ctx, rule, N, edges, M, C=37, nd=1, ns=3, sig=0.3):
     np.testing.assert_array_equal(nacc.cpu().numpy(), (got == 1).sum(axis=(1, 2)))
     # with units of zero weight up to a width that the general sweep takes, every
     # product, sum and renormalisation is the same
-    Mw = 520
+    Mw = 6160
     pw = np.zeros(N + Mw + Mw * N)
     pw[:N + M], pw[N + Mw:N + Mw + M * N] = p[:N + M], p[N + M:]
     outs = [cu(s0), torch.empty_like(samples), torch.empty_like(lp), torch.zeros_like(nacc), torch.empty_like(dec)]
