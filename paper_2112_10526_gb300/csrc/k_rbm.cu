@@ -763,8 +763,8 @@ __global__ void __launch_bounds__(128, kRing ? 3 : 7) k_sweep(SweepK<float> P) {
 
 // NK_F64 sweeps, every proposal screened in FP32.  The FP64 pipe retires 2
 // lanes a clock and SM and a dependent FP64 operation takes about 64 clocks, so
-// the FP64 product and logarithm of a proposal (k_sweep<double>: 3.7 us each
-// at M = 16) cost far more than the FP32 ones, and only their comparison with
+// the FP64 product and logarithm of a proposal (3.7 us each at M = 16) cost far
+// more than the FP32 ones, and only their comparison with
 // ln u matters.  Per proposal the warp takes ln of the ratio product from
 // FP32 t = tanh(theta) and tau, with a bound on its error from the smallest
 // factor f_min >= 2^-6: each factor 1 - s t tau errs by less than 2^-22 (t:
@@ -782,8 +782,8 @@ __global__ void __launch_bounds__(128, kRing ? 3 : 7) k_sweep(SweepK<float> P) {
 // the FP64 product form (which this replaces) loses its digits.  theta itself stays in FP64: it
 // is rebuilt at every sweep, moved by one addition a unit on an accepted
 // move, and ln psi of a sample is taken from it directly.
-// 16-site chain, 16 chains, 80 sweeps: 4763 -> see launch_sweep for the
-// measured times of both.
+// 16-site chain, 16 chains, 80 sweeps: 4.76 ms with every proposal in FP64, 0.59
+// by the form of it with the units in registers.
 template <bool kHam>
 __global__ void __launch_bounds__(128) k_sweep_screened(SweepK<double> P) {
     extern __shared__ __align__(16) unsigned char sm[];
@@ -1691,7 +1691,7 @@ struct ElocBK {
 
 // kU tau loads in flight per lane: 4 where M is large enough that the
 // shared-memory t of kEG samples allows one CTA per SM anyway (M >= 4096),
-// else 1 (the extra registers of 4 would halve the resident CTAs).
+// else 2 (the extra registers of 4 would halve the resident CTAs).
 template <int kU>
 __global__ void __launch_bounds__(eloc_warps(kU) * 32) k_eloc_batched(ElocBK P) {
     constexpr int kEW = eloc_warps(kU);
@@ -1769,15 +1769,24 @@ __global__ void __launch_bounds__(eloc_warps(kU) * 32) k_eloc_batched(ElocBK P) 
         // The active samples of this connection as slots 0 .. cnt - 1 (in
         // increasing sample order, so every product is formed as before):
         // the loops below stop at cnt, so inactive samples cost nothing.
-        const int cnt = __popc(active);
+        // Those with s_i = +1 come first: the factors 1 - t tau of the one kind and 1 +
+        // t tau of the other then differ in the sign of an FMA's operand, and a sample
+        // takes kU chunks and their renormalisations in one go: 24 x 24 lattice, M =
+        // 4608, 65536 samples: 50.8 ms with a multiplication by the sign and the
+        // samples inside each chunk, 45.7 so (M = 1600: 3.0 ms either way).
+        unsigned ups = 0;
+#pragma unroll
+        for (int g = 0; g < kEG; ++g) ups |= (unsigned)(sv[g * P.s_ld + i] > 0) << g;
+        const int cnt = __popc(active), cnt_up = __popc(active & ups);
         float m[kEG];
         int ex[kEG];
         float sg[kEG];
         const float *tg[kEG];
         int gs[kEG];
-        unsigned rest = active;
+        unsigned rest = active & ups, down = active & ~ups;
 #pragma unroll
         for (int q = 0; q < kEG; ++q) {
+            if (!rest) rest = down, down = 0;
             const int g = rest ? __ffs(rest) - 1 : 0;
             rest &= rest - 1u;
             gs[q] = g;
@@ -1795,25 +1804,25 @@ __global__ void __launch_bounds__(eloc_warps(kU) * 32) k_eloc_batched(ElocBK P) 
             for (int u = 0; u < kU; ++u)
                 uv[u] = j0 + u * 128 < M ? __ldg(reinterpret_cast<const float4 *>(tau + j0 + u * 128))
                                          : make_float4(0.f, 0.f, 0.f, 0.f);
+            auto multiply = [&](int q, auto up) {
+                constexpr bool kUp = decltype(up)::value;
 #pragma unroll
-            for (int u = 0; u < kU; ++u) {
-                const int j = j0 + u * 128;
-                if (j >= M) break;
-#pragma unroll
-                for (int q = 0; q < kEG; ++q) {
-                    if (q >= cnt) break;
+                for (int u = 0; u < kU; ++u) {
+                    const int j = j0 + u * 128;
+                    if (j >= M) break;
                     const float4 tv = *reinterpret_cast<const float4 *>(tg[q] + j);
-                    const float ns = -sg[q];
-                    m[q] *= fmaf(ns * tv.x, uv[u].x, 1.f) * fmaf(ns * tv.y, uv[u].y, 1.f) *
-                            fmaf(ns * tv.z, uv[u].z, 1.f) * fmaf(ns * tv.w, uv[u].w, 1.f);
+                    m[q] *= fmaf(kUp ? -tv.x : tv.x, uv[u].x, 1.f) * fmaf(kUp ? -tv.y : tv.y, uv[u].y, 1.f) *
+                            fmaf(kUp ? -tv.z : tv.z, uv[u].z, 1.f) * fmaf(kUp ? -tv.w : tv.w, uv[u].w, 1.f);
+                    if (u & 1) m[q] = renorm_bits(m[q], ex[q]);  // kU is even
                 }
-                if ((j >> 7) & 1) {
+            };
 #pragma unroll
-                    for (int q = 0; q < kEG; ++q) {
-                        if (q >= cnt) break;
-                        m[q] = renorm_bits(m[q], ex[q]);
-                    }
-                }
+            for (int q = 0; q < kEG; ++q) {
+                if (q >= cnt) break;
+                if (q < cnt_up)
+                    multiply(q, std::true_type{});
+                else
+                    multiply(q, std::false_type{});
             }
         }
 #pragma unroll
@@ -2092,10 +2101,10 @@ cudaError_t launch_eloc_batched<float>(const Tables<float> &t, const ElocArgs &a
     P.t_ld = (t.M + 3) / 4 * 4;
     P.s_ld = (t.N + 15) / 16 * 16;
     const bool wide = t.M >= 4096;
-    const int warps = wide ? eloc_warps(4) : eloc_warps(1);
+    const int warps = wide ? eloc_warps(4) : eloc_warps(2);
     const size_t smem = eloc_batched_smem(t.N, t.M, warps);
     if (smem > 227 * 1024) return cudaErrorInvalidValue;
-    const void *fn = wide ? (const void *)k_eloc_batched<4> : (const void *)k_eloc_batched<1>;
+    const void *fn = wide ? (const void *)k_eloc_batched<4> : (const void *)k_eloc_batched<2>;
     cudaError_t err = nk::allow_max_dynamic_smem(fn);
     if (err != cudaSuccess) return err;
     const unsigned grid = (unsigned)((a.Ns + kEG - 1) / kEG);
@@ -2103,7 +2112,7 @@ cudaError_t launch_eloc_batched<float>(const Tables<float> &t, const ElocArgs &a
     if (wide)
         (k_eloc_batched<4><<<grid, warps * 32, smem, st>>>(P), nk::note_launch());
     else
-        (k_eloc_batched<1><<<grid, warps * 32, smem, st>>>(P), nk::note_launch());
+        (k_eloc_batched<2><<<grid, warps * 32, smem, st>>>(P), nk::note_launch());
     const double conn = a.kind == NK_TFIM ? (double)t.N : 0.5 * (double)t.E;
     prof_end(slot, st, (double)a.Ns * conn * (double)t.M);
     return cudaGetLastError();
