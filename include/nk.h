@@ -28,11 +28,15 @@
  *     (cudaMalloc, which synchronises the device).  A context is not
  *     thread-safe: use one per host thread.  Calls on one context must not
  *     overlap on different streams (they share the workspace).
- *   - precision: NK_F64 computes everything in FP64 on CUDA cores.
+ *   - precision: NK_F64 computes everything to FP64 accuracy, on the FP64
+ *     pipe or, where that is slower, on 64-bit integers and (from 4e6
+ *     multiply-adds) on 7 BF16 slices on the tensor cores; Metropolis
+ *     decisions are taken in FP32 where a bound on its error decides them and
+ *     in FP64 elsewhere.
  *     NK_MIXED keeps the Metropolis chains and local-energy ratios in FP32,
  *     rebuilds the hidden activations from scratch at every sweep with an
- *     FP64-exact tensor-core product (configurations x W cut into 7 BF16
- *     integer slices, FP32 accumulation), runs the Jacobian products on the
+ *     FP64-exact tensor-core product (configurations x W cut into 5 FP16
+ *     integer slices of 12 bits, FP32 accumulation), runs the Jacobian products on the
  *     tensor cores (in CG matvecs 3 FP16 slices of 11-bit digits, 33 bits of
  *     each operand row; 7 BF16 slices where the sample-space solve needs
  *     FP64-level products) and keeps FP64 for sample means, centring,
@@ -117,11 +121,11 @@ const char *nk_last_error(void);
 /* Library version (major*10000 + minor*100 + patch). */
 int32_t nk_version(void);
 /*
- * Sticky status of the context's tensor-core products (NK_MIXED paths):
+ * Sticky status of the context's tensor-core products:
  * waits for the context's work on `stream` and returns in *code 0, or the
  * code of the last bounded wait that timed out since the last call (the
- * results of that call are invalid): 3-5 the S-GEMM (producer, MMA issuer,
- * epilogue), 6 / 7 the forward / backward triangular solve, 12-16 the
+ * results of that call are invalid): 3-5 the S-GEMM and theta (producer, MMA
+ * issuer, epilogue), 6 / 7 the forward / backward triangular solve, 12-16 the
  * FP64-accurate product (producer, A slices, B slices, accumulator buffer,
  * epilogue).  Resets the word.
  */
@@ -447,7 +451,8 @@ nk_status nk_symm_sr_step(nk_ctx *ctx, nk_rbm_symm *symm, const nk_ham *ham, nk_
  * complex O_a = s, O_b = tanh theta, O_W = tanh theta s^T.
  * Complex arrays are interleaved (re, im) float64 pairs and must be 16-byte
  * aligned (NK_ERR_INVALID_ARG otherwise).  Parameters: [a (N); b (M); W (M x
- * N, row-major)] complex, 2 Np doubles.  Everything is FP64 on CUDA cores.
+ * N, row-major)] complex, 2 Np doubles.  Everything is to FP64 accuracy (see
+ * NK_F64).
  * Limits: N <= 4096, M <= 4096.
  */
 typedef struct {

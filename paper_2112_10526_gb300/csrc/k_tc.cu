@@ -756,8 +756,8 @@ __global__ void __launch_bounds__(32 * kTrtriWarps) k_trtri64(const double *__re
 // Against the product with the inverted block (k_trtri64 + k_slice_rows +
 // k_ozaki_gemm + k_slice_rows: about 28 us on the panel chain): substitution
 // is backward stable whatever the block's condition, takes one launch, and
-// about 4 us while the rows fit one wave of the FP64 pipe (4 rows an SM), 50 us
-// at 8192 rows.  kTrsmRows is where the two meet; NK_F64 takes the
+// 17 to 22 us up to 3072 rows (FP64 latencies, whatever the number of rows), 50
+// us at 8192.  kTrsmRows is where the two meet; NK_F64 takes the
 // substitution at every size.
 constexpr int64_t kTrsmRows = 3072;
 
