@@ -1036,11 +1036,16 @@ __global__ void __launch_bounds__(kTrsvThreads) k_trsv_bwd(const double *__restr
 
 // Lower triangle of K holds g_t = t_k . t_l; replace it (both triangles) by
 // the Gram of the Jacobian rows g_s + g_t + g_t g_s with g_s = s_k . s_l
-// (exact integer dot products of the +-1 configurations).
+// (exact integer dot products of the +-1 configurations).  The tile passes
+// through shared memory, so that both triangles are read and written in rows
+// (entry by entry from the registers of the products, 8 bytes at a stride of a
+// row: 434 us for 8192 rows, 285 so).
 __global__ void __launch_bounds__(256) k_gram_combine(int N, int64_t Ns, const int8_t *__restrict__ s,
                                                       double *__restrict__ K) {
-    __shared__ __align__(16) int8_t sa[64][132];
-    __shared__ __align__(16) int8_t sb[64][132];
+    __shared__ __align__(16) unsigned char raw[64 * 65 * 8];
+    int8_t(*sa)[132] = reinterpret_cast<int8_t(*)[132]>(raw);
+    int8_t(*sb)[132] = reinterpret_cast<int8_t(*)[132]>(raw + 64 * 132);
+    double(*tile)[65] = reinterpret_cast<double(*)[65]>(raw);  // once the configurations are done with
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
     const int64_t m0 = (int64_t)blockIdx.y * 64, n0 = (int64_t)blockIdx.x * 64;
     if (n0 > m0 + 63) return;
@@ -1067,19 +1072,27 @@ __global__ void __launch_bounds__(256) k_gram_combine(int N, int64_t Ns, const i
         }
         __syncthreads();
     }
+    auto in_lower = [&](int r, int c) { return m0 + r < Ns && n0 + c <= m0 + r; };  // then n0 + c < Ns too
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const int64_t k = m0 + ty * 4 + u;
-        if (k >= Ns) continue;
+    for (int i = 0; i < 16; ++i) {
+        const int e = threadIdx.x + 256 * i, r = e >> 6, c = e & 63;
+        tile[r][c] = in_lower(r, c) ? K[(size_t)(m0 + r) * Ns + n0 + c] : 0.0;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
-            const int64_t l = n0 + tx * 4 + v;
-            if (l >= Ns || l > k) continue;
-            const double gt = K[(size_t)k * Ns + l];
-            const double g = (double)gs[u][v] + gt + gt * (double)gs[u][v];
-            K[(size_t)k * Ns + l] = g;
-            K[(size_t)l * Ns + k] = g;
+            double &x = tile[ty * 4 + u][tx * 4 + v];
+            const double gt = x;
+            x = (double)gs[u][v] + gt + gt * (double)gs[u][v];
         }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        const int e = threadIdx.x + 256 * i, r = e >> 6, c = e & 63;
+        if (in_lower(r, c)) K[(size_t)(m0 + r) * Ns + n0 + c] = tile[r][c];
+        if (in_lower(c, r)) K[(size_t)(n0 + r) * Ns + m0 + c] = tile[c][r];
     }
 }
 
