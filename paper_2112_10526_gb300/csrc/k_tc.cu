@@ -868,25 +868,32 @@ __device__ __forceinline__ double refine_block(const double (&m)[16], const doub
 
 // L y = b: y (sentinel-filled) receives the solution; b is read and refilled
 // with the sentinel for the backward solve.
+// Row stride of the inverse in shared memory: the rows and columns that a half
+// warp reads at a time fall on different banks.
+// What bounds a block row is the FP64 pipe of its SM, 19 cycles a warp
+// instruction: 128 for the last block's product, and the sums over the lanes and
+// the product with the inverse, which take 72 each (320 and 128, and 32-way bank
+// conflicts, as sums row by row and a square product: 6.8 us a block row forward
+// and 3.8 back, 3.2 and 2.9 now, n = 8192).
+constexpr int kInvLd = kNB + 4;
+
 template <bool kRefine>
 __global__ void __launch_bounds__(kTrsvThreads) k_trsv_fwd(const double *__restrict__ L, int64_t n,
                                                            const double *__restrict__ Linv, double *b, double *y,
                                                            int *err) {
-    __shared__ double inv[kNB * kNB];
+    __shared__ double inv[kNB * kInvLd];
     __shared__ double acc[kNB];
     const int nb = (int)((n + kNB - 1) / kNB);
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     for (int i = blockIdx.x; i < nb; i += gridDim.x) {
         const int64_t r0 = (int64_t)i * kNB;
         const int kb = (int)(n - r0 < kNB ? n - r0 : kNB);
-        for (int e = t; e < kNB * kNB; e += kTrsvThreads) inv[e] = Linv[(size_t)i * kNB * kNB + e];
+        for (int e = t; e < kNB * kNB; e += kTrsvThreads)
+            inv[(e >> 6) * kInvLd + (e & 63)] = Linv[(size_t)i * kNB * kNB + e];
         // warp w: rows 8w .. 8w + 7 of the block; lanes: columns lane, lane + 32
-        double part[8], bi[8];  // bi: the right-hand side of the warp's rows, read early
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            part[u] = 0.0;
-            bi[u] = (lane == 0 && warp * 8 + u < kb) ? b[r0 + warp * 8 + u] : 0.0;
-        }
+        // (the right-hand side of row lane / 4 read early)
+        double part[8] = {};
+        const double bi = warp * 8 + (lane >> 2) < kb ? b[r0 + warp * 8 + (lane >> 2)] : 0.0;
         bool live = true;
         for (int j = 0; j < i && live; ++j) {
             const int64_t c0 = (int64_t)j * kNB;  // j < i: a full block
@@ -905,25 +912,34 @@ __global__ void __launch_bounds__(kTrsvThreads) k_trsv_fwd(const double *__restr
             for (int u = 0; u < 8; ++u)
                 if (warp * 8 + u < kb) part[u] = fma(p0[u], y0, fma(p1[u], y1, part[u]));
         }
+        // sums over the lanes, eight at a time: each exchange halves the values a
+        // lane holds, 9 additions in place of 40; lane 4 u ends with row u's
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const double sum = warp_sum(part[u]);
-            const int r = warp * 8 + u;
-            if (lane == 0) {
-                acc[r] = r < kb ? bi[u] - sum : 0.0;
-                if (r < kb) b[r0 + r] = __longlong_as_double((long long)kSolveSentinel);
+        for (int h = 4; h >= 1; h >>= 1) {
+            const bool hi = lane & (4 * h);
+#pragma unroll
+            for (int u = 0; u < h; ++u) {
+                const double give = hi ? part[u] : part[u + h], keep = hi ? part[u + h] : part[u];
+                part[u] = keep + __shfl_xor_sync(0xffffffffu, give, 4 * h);
             }
         }
+        part[0] += __shfl_xor_sync(0xffffffffu, part[0], 2);
+        part[0] += __shfl_xor_sync(0xffffffffu, part[0], 1);
+        if ((lane & 3) == 0) {
+            const int r = warp * 8 + (lane >> 2);
+            acc[r] = r < kb ? bi - part[0] : 0.0;
+            if (r < kb) b[r0 + r] = __longlong_as_double((long long)kSolveSentinel);
+        }
         __syncthreads();
-        // y_i = Linv_i acc: four threads per row, 16 columns each, in two
-        // independent FMA chains (a dependent FP64 FMA costs tens of cycles)
+        // y_i = Linv_i acc: four threads per row, every fourth column each up to
+        // the last row of the warp, in two independent FMA chains
         {
             const int r = t >> 2, q = t & 3;
             double ya = 0.0, yb = 0.0;
-#pragma unroll
-            for (int c = q * 16; c < q * 16 + 16; c += 2) {
-                ya = fma(inv[r * kNB + c], acc[c], ya);
-                yb = fma(inv[r * kNB + c + 1], acc[c + 1], yb);
+#pragma unroll 2
+            for (int c = q; c < 8 * warp + 8; c += 8) {
+                ya = fma(inv[r * kInvLd + c], acc[c], ya);
+                yb = fma(inv[r * kInvLd + c + 4], acc[c + 4], yb);
             }
             double v = ya + yb;
             v += __shfl_xor_sync(0xffffffffu, v, 1);
@@ -934,7 +950,7 @@ __global__ void __launch_bounds__(kTrsvThreads) k_trsv_fwd(const double *__restr
 #pragma unroll
                 for (int u = 0; u < 16; ++u) {
                     const int c = q * 16 + u;
-                    m[u] = inv[r * kNB + c];
+                    m[u] = inv[r * kInvLd + c];
                     l[u] = (r < kb && c <= r) ? L[(size_t)(r0 + r) * n + r0 + c] : 0.0;
                 }
                 v = refine_block(m, l, v, r, q, acc, zs, rs);
@@ -951,7 +967,7 @@ template <bool kRefine>
 __global__ void __launch_bounds__(kTrsvThreads) k_trsv_bwd(const double *__restrict__ L, int64_t n,
                                                            const double *__restrict__ Linv, double *b,
                                                            const double *y, int *err) {
-    __shared__ double inv[kNB * kNB];
+    __shared__ double inv[kNB * kInvLd];
     __shared__ double part_s[kTrsvThreads / 32][kNB];
     __shared__ double acc[kNB];
     const int nb = (int)((n + kNB - 1) / kNB);
@@ -960,7 +976,8 @@ __global__ void __launch_bounds__(kTrsvThreads) k_trsv_bwd(const double *__restr
         const int i = nb - 1 - ii;
         const int64_t c0 = (int64_t)i * kNB;
         const int kb = (int)(n - c0 < kNB ? n - c0 : kNB);
-        for (int e = t; e < kNB * kNB; e += kTrsvThreads) inv[e] = Linv[(size_t)i * kNB * kNB + e];
+        for (int e = t; e < kNB * kNB; e += kTrsvThreads)
+            inv[(e >> 6) * kInvLd + (e & 63)] = Linv[(size_t)i * kNB * kNB + e];
         // lanes: columns lane, lane + 32 of block column i; warp w: rows w, w + 8, ... of block row j
         double p0 = 0.0, p1 = 0.0;
         const bool v0 = lane < kb, v1 = lane + 32 < kb;
@@ -980,19 +997,15 @@ __global__ void __launch_bounds__(kTrsvThreads) k_trsv_bwd(const double *__restr
             }
             double xa, xb;  // x_j: lane holds rows lane, lane + 32 of block j
             live = wait_solved(b + r0, lane, kr, xa, xb, err, 7);
-            // four independent chains per column, summed after
-            double a0[4] = {0.0, 0.0, 0.0, 0.0}, a1[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
                 const int r = warp + 8 * u;  // < 64: its x is in lane r (xa) or r - 32 (xb)
                 const double xr = r < 32 ? __shfl_sync(0xffffffffu, xa, r) : __shfl_sync(0xffffffffu, xb, r - 32);
                 if (r < kr) {
-                    a0[u & 3] = fma(q0[u], xr, a0[u & 3]);
-                    a1[u & 3] = fma(q1[u], xr, a1[u & 3]);
+                    p0 = fma(q0[u], xr, p0);
+                    p1 = fma(q1[u], xr, p1);
                 }
             }
-            p0 += (a0[0] + a0[1]) + (a0[2] + a0[3]);
-            p1 += (a1[0] + a1[1]) + (a1[2] + a1[3]);
         }
         part_s[warp][lane] = p0;
         part_s[warp][lane + 32] = p1;
@@ -1004,15 +1017,15 @@ __global__ void __launch_bounds__(kTrsvThreads) k_trsv_bwd(const double *__restr
             acc[t] = t < kb ? yi - sum : 0.0;
         }
         __syncthreads();
-        // x_i = Linv_i^T acc: four threads per column, 16 rows each, in two
-        // independent FMA chains
+        // x_i = Linv_i^T acc: four threads per column, every fourth row each from
+        // the first column of the warp on, in two independent FMA chains
         {
             const int c = t >> 2, q = t & 3;
             double xa = 0.0, xb = 0.0;
-#pragma unroll
-            for (int r = q * 16; r < q * 16 + 16; r += 2) {
-                xa = fma(inv[r * kNB + c], acc[r], xa);
-                xb = fma(inv[(r + 1) * kNB + c], acc[r + 1], xb);
+#pragma unroll 2
+            for (int r = 8 * warp + q; r < kNB; r += 8) {
+                xa = fma(inv[r * kInvLd + c], acc[r], xa);
+                xb = fma(inv[(r + 4) * kInvLd + c], acc[r + 4], xb);
             }
             double x = xa + xb;
             x += __shfl_xor_sync(0xffffffffu, x, 1);
@@ -1023,7 +1036,7 @@ __global__ void __launch_bounds__(kTrsvThreads) k_trsv_bwd(const double *__restr
 #pragma unroll
                 for (int u = 0; u < 16; ++u) {
                     const int r = q * 16 + u;
-                    m[u] = inv[r * kNB + c];
+                    m[u] = inv[r * kInvLd + c];
                     l[u] = (r < kb && r >= c) ? L[(size_t)(c0 + r) * n + c0 + c] : 0.0;
                 }
                 x = refine_block(m, l, x, c, q, acc, zs, rs);
