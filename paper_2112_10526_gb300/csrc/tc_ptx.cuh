@@ -351,14 +351,20 @@ __host__ __device__ __forceinline__ double window_to_double(long long x, int sc)
 // The same on 32-bit halves, with zero and the ends of the exponent range in a
 // branch that is seldom taken: some 25 instructions where the form above has 35,
 // for an epilogue bound by them (half a warp a cycle and scheduler).
-__device__ __forceinline__ double window_to_double_seldom(long long x, int sc) {
+__host__ __device__ __forceinline__ double window_to_double_seldom(long long x, int sc) {
     const long long s = x >> 63;
     const unsigned long long m = (unsigned long long)((x ^ s) - s);
     const uint32_t mh = (uint32_t)(m >> 32), ml = (uint32_t)m;
     const bool low = mh == 0;
     const uint32_t a = low ? ml : mh, b = low ? 0u : ml;
+#ifdef __CUDA_ARCH__
     const int z = __clz((int)a);
     const uint32_t hi = __funnelshift_l(b, a, z), lo = b << (z & 31);  // leading one at bit 63 (m != 0)
+#else
+    const int z = a ? __builtin_clz(a) : 32;
+    const unsigned long long ab = (((unsigned long long)a << 32) | b) << (z & 31);
+    const uint32_t hi = (uint32_t)(ab >> 32), lo = (uint32_t)ab;
+#endif
     const int eb = (low ? 1054 : 1086) - z + sc;
     const unsigned long long r = ((((unsigned long long)hi << 32) | lo) >> 11) + ((lo >> 10) & 1u);
     unsigned long long bits = r + ((unsigned long long)((uint32_t)(eb - 1) << 20) << 32);
@@ -366,7 +372,14 @@ __device__ __forceinline__ double window_to_double_seldom(long long x, int sc) {
         const int ef = eb + (int)(r >> 53);
         bits = (a == 0u || ef < 1) ? 0ULL : (ef > 2046 ? 0x7FF0000000000000ULL : bits);
     }
-    return __longlong_as_double((long long)(bits | ((unsigned long long)s & 0x8000000000000000ULL)));
+    bits |= (unsigned long long)s & 0x8000000000000000ULL;
+    double v;
+#ifdef __CUDA_ARCH__
+    v = __longlong_as_double((long long)bits);
+#else
+    __builtin_memcpy(&v, &bits, 8);
+#endif
+    return v;
 }
 
 // The four FP32 levels of a 4-slice product (exact integers, |D_t| < 2^22)
