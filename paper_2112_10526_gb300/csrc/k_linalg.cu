@@ -463,36 +463,38 @@ __device__ __forceinline__ void comp_merge(double &s, double &c, double s2, doub
 // 16384 samples, 650 us for 65536 on a single block of 1024 threads).  Their
 // partial sums meet in distributed shared memory.  256 threads a block: with
 // 1024 the sum over a block (8 FP64 operations a level, quantity and warp) took
-// longer than the samples.
+// longer than the samples; one warp a quantity sums the block (1024 samples: 23.7
+// us, 29.8 with every warp's own sum first).
 constexpr int kStatCtas = 8, kStatThreads = 256;
 
 // Compensated sums of nq quantities over all threads of the cluster, in a
 // fixed order (lanes, warps, blocks); every thread returns the totals in s.
 template <int nq>
 __device__ void cluster_comp_sum(double (&s)[nq], double (&c)[nq]) {
-    constexpr int kWarps = kStatThreads / 32;
-    static_assert(kWarps == 8 && kStatCtas == 8, "the last sums run over 8 lanes");
-    __shared__ double2 part[nq][kWarps];
+    static_assert(kStatThreads == 256 && kStatCtas == 8, "sums of eight");
+    __shared__ double2 part[nq][kStatThreads];
     __shared__ double2 tot[nq];
     __shared__ double all[nq];
     cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-        for (int q = 0; q < nq; ++q)
-            comp_merge(s[q], c[q], __shfl_down_sync(0xffffffffu, s[q], o), __shfl_down_sync(0xffffffffu, c[q], o));
-    if (lane == 0)
-#pragma unroll
-        for (int q = 0; q < nq; ++q) part[q][warp] = make_double2(s[q], c[q]);
+    for (int q = 0; q < nq; ++q) part[q][threadIdx.x] = make_double2(s[q], c[q]);
     __syncthreads();
-    // warp q sums quantity q over the block's warps, then over the blocks
+    // warp q sums quantity q over the block (eight threads a lane first: 96 FP64
+    // instructions where every warp's own sum took 40), then over the blocks
     if (warp < nq) {
-        double2 v = part[warp][lane & 7];
+        double2 v[8];
 #pragma unroll
-        for (int o = 4; o > 0; o >>= 1)
-            comp_merge(v.x, v.y, __shfl_down_sync(0xffffffffu, v.x, o), __shfl_down_sync(0xffffffffu, v.y, o));
-        if (lane == 0) tot[warp] = v;
+        for (int u = 0; u < 8; ++u) v[u] = part[warp][32 * u + lane];
+#pragma unroll
+        for (int h = 4; h > 0; h >>= 1)
+#pragma unroll
+            for (int u = 0; u < h; ++u) comp_merge(v[u].x, v[u].y, v[u + h].x, v[u + h].y);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            comp_merge(v[0].x, v[0].y, __shfl_down_sync(0xffffffffu, v[0].x, o),
+                       __shfl_down_sync(0xffffffffu, v[0].y, o));
+        if (lane == 0) tot[warp] = v[0];
     }
     cl.sync();
     if (warp < nq) {
