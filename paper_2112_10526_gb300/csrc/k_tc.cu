@@ -457,7 +457,7 @@ constexpr int kNB = 64;
 // of a positive definite block and of what is left of it after each column lies
 // in (-1, 1): entries are 2^60 a.  Column c (u = L D) is normalised by the even
 // power of two that takes its pivot to M = d 2^(2 f) in [1/4, 1): |u 2^f| <=
-// sqrt(M) < 1 is held to 2^-62, y = 1 / M and (u 2^f) y, both below 4, to 2^-60,
+// sqrt(M) < 1 is held to 2^-62, y = 1 / M (held below 4) and (u 2^f) y to 2^-60,
 // and a product of the last two enters the block to 2^-59: sqrt(a_ii a_jj) 2^-59
 // an operation, where FP64's backward error is 2^-53 of it.
 // One CTA holds the block in shared memory (continued by the identity beyond
@@ -494,35 +494,46 @@ __device__ __forceinline__ long long to_fixed60(double a, int sh) {
     return (bits >> 63) ? -(long long)v : (long long)v;
 }
 
-__device__ __forceinline__ float rcp_approx(float x) {  // to 2^-23
+__host__ __device__ __forceinline__ float rcp_approx(float x) {  // to 2^-23
+#ifdef __CUDA_ARCH__
     float y;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
+#else
+    return 1.0f / x;
+#endif
 }
 
 // A number of 63 bits as hi 2^31 + lo, 0 <= lo < 2^31, and x y 2^-62 without the
 // product of the low halves (from 0 to 2 below): three 32 x 32-bit products, 32
 // cycles a warp.  (__mul64hi takes as long, but wants the operands' signs mended
 // each time, where halves are split once: 35 us a block with it.)
-__device__ __forceinline__ int2 halves(long long x) { return make_int2((int)(x >> 31), (int)x & 0x7fffffff); }
+__host__ __device__ __forceinline__ int2 halves(long long x) { return make_int2((int)(x >> 31), (int)x & 0x7fffffff); }
 
-__device__ __forceinline__ long long mul62(int2 x, int2 y) {
+__host__ __device__ __forceinline__ long long mul62(int2 x, int2 y) {
     return (long long)x.x * y.x + (((long long)x.x * y.y + (long long)x.y * y.x) >> 31);
 }
 
 // y = 2^60 / x for x = X 2^-60 in [1/4, 1): the FP32 reciprocal y0 and one
 // third-order step, y0 + y0 (e + e^2) with e = 1 - x y0 (|e| < 2^-21, so the
-// rest is below 2^-63).
-__device__ __forceinline__ unsigned long long fixed_reciprocal(unsigned long long X) {
+// rest is below 2^-63).  At x = 1/4, the pivots 4^k, y would be 2^62, one more
+// than `halves` holds: it is kept at 2^62 - 1, 2^-62 of itself below.
+__host__ __device__ __forceinline__ unsigned long long fixed_reciprocal(unsigned long long X) {
     const uint32_t xh = (uint32_t)(X >> 28), xl = (uint32_t)X & 0xfffffffu;
-    const uint32_t y0 = __float2uint_rn(rcp_approx((float)xh) * 2305843009213693952.0f);  // 2^29 / x: 2^61 / xh
+    const float yf = rcp_approx((float)xh) * 2305843009213693952.0f;  // 2^29 / x: 2^61 / xh
+#ifdef __CUDA_ARCH__
+    const uint32_t y0 = __float2uint_rn(yf);
+#else
+    const uint32_t y0 = (uint32_t)yf;  // at least 2^29: a whole number
+#endif
     const long long e = (1LL << 61) - (long long)((unsigned long long)xh * y0 + (((unsigned long long)xl * y0) >> 28));
     const int e40 = (int)(e >> 21);                             // 2^40 e
     const long long h = e + ((long long)e40 * e40 >> 19);       // 2^61 (e + e^2)
     const int hh = (int)(h >> 16);
     const long long yh =  // 2^74 y0 (e + e^2)
         (long long)hh * (long long)y0 + (long long)(((unsigned long long)((uint32_t)h & 0xffffu) * y0) >> 16);
-    return ((unsigned long long)y0 << 31) + (unsigned long long)(yh >> 14);
+    const unsigned long long y = ((unsigned long long)y0 << 31) + (unsigned long long)(yh >> 14);
+    return y < 0x3fffffffffffffffULL ? y : 0x3fffffffffffffffULL;
 }
 
 __host__ __device__ constexpr int tri_from(int x) {  // packed entries with column q >= x (1 <= x <= 64)
