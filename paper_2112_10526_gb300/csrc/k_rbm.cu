@@ -47,18 +47,18 @@ __global__ void k_transpose_W(int N, int M, const double *__restrict__ W, double
     }
 }
 
-// x in [-1, 1] as 2^63 x, +-1 as the nearest FP64 number below (so that a factor
-// of two such numbers stays below 2).  A NaN reads as 1.
-__device__ __forceinline__ long long to_fixed63(double x) {
+// x in [-1, 1] as 2^62 x to nearest; +-1 and every FP64 number down to 1/512 are
+// exact, so that a factor 1 - t tau of saturated units is 0 as it is in FP64 (one
+// ulp less than 1 instead made it 2^-52, which the cosh(2 W) of large weights
+// multiplies to anything).  A NaN reads as 1.
+__device__ __forceinline__ long long to_fixed62(double x) {
     int b;
     unsigned long long m;
     bool neg;
     split_bits(x, b, m, neg);
-    const int sh = b - 1012;  // m 2^(b - 1075 + 63)
-    constexpr unsigned long long kMost = 0x7FFFFFFFFFFFFC00ULL;  // 2^63 (1 - 2^-53)
-    unsigned long long y = sh >= 0 ? (sh > 10 ? kMost : m << sh)
-                                   : (sh <= -54 ? 0ULL : (m >> (-sh)) + ((m >> (-sh - 1)) & 1ULL));
-    if (y > kMost) y = kMost;
+    const int sh = b - 1013;  // m 2^(b - 1075 + 62)
+    const unsigned long long y = sh >= 0 ? (sh > 10 ? 1ULL << 62 : m << sh)
+                                         : (sh <= -54 ? 0ULL : (m >> (-sh)) + ((m >> (-sh - 1)) & 1ULL));
     return neg ? -(long long)y : (long long)y;
 }
 
@@ -70,7 +70,7 @@ __device__ __forceinline__ float to_tau<float>(double x) {
 }
 template <>
 __device__ __forceinline__ long long to_tau<double>(double x) {
-    return to_fixed63(x);
+    return to_fixed62(x);
 }
 
 // The exponent of every unit's weights (column j of Wt; |W| < 2^e, 0 for zero
@@ -294,8 +294,8 @@ __device__ __forceinline__ Prod<float> strided_product(const float *__restrict__
     return p;
 }
 
-// The same product for NK_F64 from 2^63 t and 2^63 tau in 64-bit integers: a
-// factor 1 - s t tau is 2^62 -+ the high half of a product, good to 2^-62, and
+// The same product for NK_F64 from 2^62 t and 2^62 tau in 64-bit integers: a
+// factor 1 - s t tau is 2^60 -+ the high half of a product, good to 2^-60, and
 // the running mantissa (leading one at bit 63) takes two factors and one
 // normalisation a step.  An FP64 multiply-add or multiply costs 64 clocks a warp
 // and scheduler, a 64-bit high product about 11: 30 clocks a factor against 192
@@ -305,8 +305,8 @@ struct FixProd {
     int e;
 };
 __device__ __forceinline__ unsigned long long fixed_factor(long long t, long long tau, bool up) {
-    const long long p = __mul64hi(t, tau);  // 2^62 t tau
-    return (unsigned long long)((1LL << 62) - (up ? p : -p)) << 1;  // 2^63 (1 - s t tau), in [0, 2^64)
+    const long long p = __mul64hi(t, tau) * 4;  // 2^62 t tau
+    return (1ULL << 62) - (unsigned long long)(up ? p : -p);  // 2^62 (1 - s t tau), in [0, 2^63]
 }
 __device__ __forceinline__ void fixed_mul(FixProd &a, unsigned long long f, int point) {
     const unsigned long long r = __umul64hi(a.m, f);  // 2^(point - 1) of the product
@@ -326,10 +326,10 @@ __device__ __forceinline__ Prod<double> strided_product(const long long *__restr
         const unsigned long long f1 = fixed_factor(t[j + step], tau[(size_t)(j + step) * tstride], up);
         const unsigned long long f2 = fixed_factor(t[j + 2 * step], tau[(size_t)(j + 2 * step) * tstride], up);
         const unsigned long long f3 = fixed_factor(t[j + 3 * step], tau[(size_t)(j + 3 * step) * tstride], up);
-        fixed_mul(a, __umul64hi(f0, f1), 62);
-        fixed_mul(b, __umul64hi(f2, f3), 62);
+        fixed_mul(a, __umul64hi(f0, f1), 60);
+        fixed_mul(b, __umul64hi(f2, f3), 60);
     }
-    for (; j < M; j += step) fixed_mul(a, fixed_factor(t[j], tau[(size_t)j * tstride], up), 63);
+    for (; j < M; j += step) fixed_mul(a, fixed_factor(t[j], tau[(size_t)j * tstride], up), 62);
     fixed_mul(a, b.m, 63);
     // value = m 2^-63 2^(a.e + b.e), as a mantissa in [1/2, 1)
     return Prod<double>{window_to_double((long long)(a.m >> 1), -63), a.e + b.e + 1};

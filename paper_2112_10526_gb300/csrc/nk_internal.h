@@ -48,7 +48,7 @@ void note_launch(long long n = 1);
 cudaError_t allow_max_dynamic_smem(const void *func);
 void prof_end(int slot, cudaStream_t st, double work, double executed = -1.0);
 
-// The type of the flip-ratio tables: FP32 (NK_MIXED), or 2^63 tau as a 64-bit
+// The type of the flip-ratio tables: FP32 (NK_MIXED), or 2^62 tau as a 64-bit
 // integer (NK_F64; k_eloc multiplies them on the integer pipe).
 template <typename R>
 struct TauOf {

@@ -1,0 +1,65 @@
+"""NK_F64 local energies of the Ising field where the flip ratios' factors 1 - s t tau
+(t = tanh theta, tau = tanh 2 W) are at the ends of their range, against ratios of
+cosh in extended precision.  M below and from 1024 on: the two mappings of the
+kernel."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2112_10526_gb300 import nk
+from gpu_util import cu, dev
+
+pytestmark = pytest.mark.gpu
+
+LD = np.longdouble
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    with nk.Ctx() as c:
+        yield c
+
+
+def _lncosh(x):
+    x = np.abs(x)
+    return x + np.log1p(np.exp(-2 * x)) - np.log(LD(2))
+
+
+def _params(a, b, W):
+    return np.concatenate([a, b, W.ravel()]).astype(np.float64)
+
+
+def _field(ctx, a, b, W, s):
+    """-sum_i psi(s with i flipped) / psi(s) per sample: the library's and the exact."""
+    M, N = W.shape
+    h = nk.make_ham("tfim", 0.0, 1.0, False, cu(np.array([[0, 1]], dtype=np.int32)))
+    out = torch.empty(len(s), dtype=torch.float64, device=dev())
+    nk.nk_local_energy(ctx, cu(_params(a, b, W)), N, M, h, cu(s), out, precision="f64")
+    th = b.astype(LD) + s.astype(LD) @ W.T.astype(LD)
+    ref = np.zeros(len(s), dtype=LD)
+    for i in range(N):
+        si = s[:, i].astype(LD)
+        d = 2 * si[:, None] * W[:, i].astype(LD)[None, :]
+        ref -= np.exp(-2 * a[i] * si + (_lncosh(th - d) - _lncosh(th)).sum(1))
+    return out.cpu().numpy(), ref
+
+
+@pytest.mark.parametrize("d", [25.0, 30.0, 40.0, 100.0])
+@pytest.mark.parametrize("M,at", [(1, 0), (7, 2), (7, 6), (1030, 1), (1030, 1029)])
+def test_saturated_units(ctx, M, at, d):
+    """theta = 2 W = d of one unit: t = tau = 1 in FP64, factor 0, exact ratio 1 / cosh d
+    (2.8e-11 at most); and t = 1, tau = -1, factor 2.  Tolerance: NK_F64's 1e-10."""
+    N = 2
+    g = np.random.default_rng(M)
+    a, b, W = np.zeros(N), 0.01 * g.normal(size=M), 0.01 * g.normal(size=(M, N))
+    b[at] = W[at, 0] = d / 2
+    W[at, 1] = 0.0
+    s = np.array([[1, 1], [1, -1]], dtype=np.int8)
+    got, ref = _field(ctx, a, b, W, s)  # site 0: 1 / cosh d, site 1: about 1
+    assert np.max(np.abs(got - ref)) <= 1e-10
+    b[at] = -d * 1.5  # theta = -2 d, moved to -d for s_0 = -1: cosh d / cosh 2 d; from -d to -2 d for +1
+    got, ref = _field(ctx, a, b, W, np.array([[1, 1], [-1, 1]], dtype=np.int8))
+    assert abs(got[1] - ref[1]) <= 1e-10
+    assert abs(got[0] / float(ref[0]) - 1) <= 1e-10
