@@ -315,6 +315,19 @@ __device__ __forceinline__ void fixed_mul(FixProd &a, unsigned long long f, int 
     a.e += 64 - point - z;
 }
 
+// Two factors f0, f1 (2^62 each) at once; one after the other where their product
+// is below 2^-8 and its high half would lose digits that they have (a pair of 2^-20
+// kept 22 bits).
+__device__ __forceinline__ void fixed_mul2(FixProd &a, unsigned long long f0, unsigned long long f1) {
+    const unsigned long long p = __umul64hi(f0, f1);  // 2^60 of the product
+    if ((p >> 52) != 0) {
+        fixed_mul(a, p, 60);
+    } else {
+        fixed_mul(a, f0, 62);
+        fixed_mul(a, f1, 62);
+    }
+}
+
 __device__ __forceinline__ Prod<double> strided_product(const long long *__restrict__ t,
                                                         const long long *__restrict__ tau, size_t tstride, double si,
                                                         int j0, int step, int M) {
@@ -326,8 +339,8 @@ __device__ __forceinline__ Prod<double> strided_product(const long long *__restr
         const unsigned long long f1 = fixed_factor(t[j + step], tau[(size_t)(j + step) * tstride], up);
         const unsigned long long f2 = fixed_factor(t[j + 2 * step], tau[(size_t)(j + 2 * step) * tstride], up);
         const unsigned long long f3 = fixed_factor(t[j + 3 * step], tau[(size_t)(j + 3 * step) * tstride], up);
-        fixed_mul(a, __umul64hi(f0, f1), 60);
-        fixed_mul(b, __umul64hi(f2, f3), 60);
+        fixed_mul2(a, f0, f1);
+        fixed_mul2(b, f2, f3);
     }
     for (; j < M; j += step) fixed_mul(a, fixed_factor(t[j], tau[(size_t)j * tstride], up), 62);
     fixed_mul(a, b.m, 63);

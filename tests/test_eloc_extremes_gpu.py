@@ -63,3 +63,26 @@ def test_saturated_units(ctx, M, at, d):
     got, ref = _field(ctx, a, b, W, np.array([[1, 1], [-1, 1]], dtype=np.int8))
     assert abs(got[1] - ref[1]) <= 1e-10
     assert abs(got[0] / float(ref[0]) - 1) <= 1e-10
+
+
+@pytest.mark.parametrize("d", [3.0, 5.0, 7.0, 9.0])
+@pytest.mark.parametrize("M,units", [(2, [0, 1]), (5, [0, 1, 2, 3]), (9, [4, 5, 6, 7, 8]), (1030, [3, 35]),
+                                     (1030, [64, 96, 128, 160])])
+def test_several_small_factors(ctx, M, units, d):
+    """Neighbouring factors of about 1 / cosh^2 d, which the product takes in pairs.
+
+    Tolerance: t and tau are within 2^-53, so that a factor f errs by 2^-52 / f of
+    itself; the product, the sum of logarithms K and the exponential by 2^-53 each per
+    unit, of the logarithms' sizes: M (2 + d) 2^-53.  Both twice."""
+    N = 2
+    g = np.random.default_rng(M)
+    a, b, W = 0.1 * g.normal(size=N), np.zeros(M), np.zeros((M, N))
+    W[units] = 0.5 * d
+    b[units] = 0.2 * g.normal(size=len(units))
+    s = np.array([[1, 1], [1, -1], [-1, -1]], dtype=np.int8)
+    got, ref = _field(ctx, a, b, W, s)
+    th = b + s @ W.T
+    f = [min(1 - abs(np.tanh(LD(th[k, j])) * np.tanh(2 * LD(W[j, 0]))) for j in units) for k in (0, 2)]
+    for k, fk in zip((0, 2), f):
+        tol = 2 * (len(units) * 2.0 ** -52 / float(fk) + M * (2 + d) * 2.0 ** -53)
+        assert abs(float((LD(got[k]) - ref[k]) / ref[k])) <= tol
