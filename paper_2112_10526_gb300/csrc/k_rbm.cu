@@ -308,23 +308,24 @@ __device__ __forceinline__ unsigned long long fixed_factor(long long t, long lon
     const long long p = __mul64hi(t, tau) * 4;  // 2^62 t tau
     return (1ULL << 62) - (unsigned long long)(up ? p : -p);  // 2^62 (1 - s t tau), in [0, 2^63]
 }
+// a times f 2^-point; kSmall: f may be small or 0.
+template <bool kSmall>
 __device__ __forceinline__ void fixed_mul(FixProd &a, unsigned long long f, int point) {
     const unsigned long long r = __umul64hi(a.m, f);  // 2^(point - 1) of the product
-    const int z = __clz((int)(r >> 32));              // 32 once the high word is empty: the next step goes on
+    const int z = kSmall ? min(__clzll((long long)r), 63) : __clz((int)(r >> 32));
     a.m = r << z;
     a.e += 64 - point - z;
 }
-
 // Two factors f0, f1 (2^62 each) at once; one after the other where their product
 // is below 2^-8 and its high half would lose digits that they have (a pair of 2^-20
 // kept 22 bits).
 __device__ __forceinline__ void fixed_mul2(FixProd &a, unsigned long long f0, unsigned long long f1) {
     const unsigned long long p = __umul64hi(f0, f1);  // 2^60 of the product
     if ((p >> 52) != 0) {
-        fixed_mul(a, p, 60);
+        fixed_mul<false>(a, p, 60);
     } else {
-        fixed_mul(a, f0, 62);
-        fixed_mul(a, f1, 62);
+        fixed_mul<true>(a, f0, 62);
+        fixed_mul<true>(a, f1, 62);
     }
 }
 
@@ -342,8 +343,8 @@ __device__ __forceinline__ Prod<double> strided_product(const long long *__restr
         fixed_mul2(a, f0, f1);
         fixed_mul2(b, f2, f3);
     }
-    for (; j < M; j += step) fixed_mul(a, fixed_factor(t[j], tau[(size_t)j * tstride], up), 62);
-    fixed_mul(a, b.m, 63);
+    for (; j < M; j += step) fixed_mul<true>(a, fixed_factor(t[j], tau[(size_t)j * tstride], up), 62);
+    fixed_mul<true>(a, b.m, 63);
     // value = m 2^-63 2^(a.e + b.e), as a mantissa in [1/2, 1)
     return Prod<double>{window_to_double((long long)(a.m >> 1), -63), a.e + b.e + 1};
 }

@@ -65,7 +65,7 @@ def test_saturated_units(ctx, M, at, d):
     assert abs(got[0] / float(ref[0]) - 1) <= 1e-10
 
 
-@pytest.mark.parametrize("d", [3.0, 5.0, 7.0, 9.0])
+@pytest.mark.parametrize("d", [3.0, 5.0, 7.0, 9.0, 13.0, 15.0])
 @pytest.mark.parametrize("M,units", [(2, [0, 1]), (5, [0, 1, 2, 3]), (9, [4, 5, 6, 7, 8]), (1030, [3, 35]),
                                      (1030, [64, 96, 128, 160])])
 def test_several_small_factors(ctx, M, units, d):
