@@ -50,7 +50,8 @@ __global__ void k_transpose_W(int N, int M, const double *__restrict__ W, double
 // x in [-1, 1] as 2^62 x to nearest; +-1 and every FP64 number down to 1/512 are
 // exact, so that a factor 1 - t tau of saturated units is 0 as it is in FP64 (one
 // ulp less than 1 instead made it 2^-52, which the cosh(2 W) of large weights
-// multiplies to anything).  A NaN reads as 1.
+// multiplies to anything).  A NaN reads as 1: k_eloc carries it on by itself, and
+// the table's NaNs stand in K as well.
 __device__ __forceinline__ long long to_fixed62(double x) {
     int b;
     unsigned long long m;
@@ -1598,6 +1599,7 @@ __global__ void __launch_bounds__(128) k_eloc(ElocK<R> P) {
     int *list = reinterpret_cast<int *>(base + P.t_bytes + P.s_bytes);
     for (int i = lane; i < N; i += 32) sv[i] = A.s[(size_t)k * N + i];
     __syncwarp();
+    bool nan = false;
     for (int j = lane; j < M; j += 32) {
         double th;
         if (A.theta_in) {
@@ -1610,8 +1612,13 @@ __global__ void __launch_bounds__(128) k_eloc(ElocK<R> P) {
         }
         const double tj = A.lib_tanh ? tanh(th) : tanh64(th);
         t[j] = to_tau<R>(tj);
+        if (sizeof(R) == 8) nan |= tj != tj;
         if (A.t_out) A.t_out[(size_t)k * M + j] = tj;
     }
+    // a NaN among the activations, which the integers of NK_F64 cannot hold, is
+    // added to every ratio's logarithm
+    const double poison =
+        sizeof(R) == 8 && __any_sync(kFull, nan) ? __longlong_as_double(0x7FF8000000000000LL) : 0.0;
     // edges [0, E1) couple with J, the next-nearest ones [E1, E) with J2
     const int E1 = E - A.E2;
     double diag = 0.0;
@@ -1628,7 +1635,7 @@ __global__ void __launch_bounds__(128) k_eloc(ElocK<R> P) {
             const R si = (R)sv[i];
             Prod<R> pr = strided_product(t, T.tau_site + (size_t)i * M, 1, si, lane, 32, M);
             pr = warp_prod(pr);
-            const double delta = -2.0 * T.a[i] * (double)si + (double)(T.K_site[i] + prod_log(pr));
+            const double delta = -2.0 * T.a[i] * (double)si + (double)(T.K_site[i] + prod_log(pr)) + poison;
             if (lane == 0) off += -A.h * exp(delta);
         }
     } else if (A.kind == NK_TFIM) {
@@ -1636,7 +1643,7 @@ __global__ void __launch_bounds__(128) k_eloc(ElocK<R> P) {
         for (int i = lane; i < N; i += 32) {
             const R si = (R)sv[i];
             Prod<R> pr = strided_product(t, T.tau_siteT + i, (size_t)N, si, 0, 1, M);
-            const double delta = -2.0 * T.a[i] * (double)si + (double)(T.K_site[i] + prod_log(pr));
+            const double delta = -2.0 * T.a[i] * (double)si + (double)(T.K_site[i] + prod_log(pr)) + poison;
             off += -A.h * exp(delta);
         }
     } else {
@@ -1665,7 +1672,7 @@ __global__ void __launch_bounds__(128) k_eloc(ElocK<R> P) {
                 Prod<R> pr = strided_product(t, T.tau_edge + (size_t)e * M, 1, si, lane, 32, M);
                 pr = warp_prod(pr);
                 const double delta =
-                    -2.0 * (double)si * (T.a[i] - T.a[kk]) + (double)(T.K_edge[e] + prod_log(pr));
+                    -2.0 * (double)si * (T.a[i] - T.a[kk]) + (double)(T.K_edge[e] + prod_log(pr)) + poison;
                 if (lane == 0) off += (e < E1 ? hoff : hoff2) * exp(delta);
             }
         } else {
@@ -1675,7 +1682,7 @@ __global__ void __launch_bounds__(128) k_eloc(ElocK<R> P) {
                 const R si = (R)sv[i];
                 Prod<R> pr = strided_product(t, T.tau_edgeT + e, (size_t)E, si, 0, 1, M);
                 const double delta =
-                    -2.0 * (double)si * (T.a[i] - T.a[kk]) + (double)(T.K_edge[e] + prod_log(pr));
+                    -2.0 * (double)si * (T.a[i] - T.a[kk]) + (double)(T.K_edge[e] + prod_log(pr)) + poison;
                 off += (e < E1 ? hoff : hoff2) * exp(delta);
             }
         }

@@ -86,3 +86,25 @@ def test_several_small_factors(ctx, M, units, d):
     for k, fk in zip((0, 2), f):
         tol = 2 * (len(units) * 2.0 ** -52 / float(fk) + M * (2 + d) * 2.0 ** -53)
         assert abs(float((LD(got[k]) - ref[k]) / ref[k])) <= tol
+
+
+@pytest.mark.parametrize("M,at", [(1, 0), (33, 32), (1030, 5)])
+@pytest.mark.parametrize("bad", ["bias", "weight"])
+def test_a_nan_reaches_the_energy(ctx, M, at, bad):
+    """A NaN among the parameters of a hidden unit makes every flip ratio NaN; a
+    Heisenberg configuration without a pair to exchange has none to take part in."""
+    N = 4
+    g = np.random.default_rng(M)
+    a, b, W = 0.1 * g.normal(size=N), 0.1 * g.normal(size=M), 0.1 * g.normal(size=(M, N))
+    if bad == "bias":
+        b[at] = np.nan
+    else:
+        W[at, 2] = np.nan
+    s = np.array([[1, 1, 1, 1], [1, -1, 1, -1], [1, 1, -1, -1]], dtype=np.int8)
+    edges = cu(np.array([[0, 1], [1, 2], [2, 3], [3, 0]], dtype=np.int32))
+    p = cu(_params(a, b, W))
+    out = torch.empty(len(s), dtype=torch.float64, device=dev())
+    nk.nk_local_energy(ctx, p, N, M, nk.make_ham("tfim", 1.0, 1.0, False, edges), cu(s), out, precision="f64")
+    assert torch.isnan(out).all()
+    nk.nk_local_energy(ctx, p, N, M, nk.make_ham("heis", 1.0, 0.0, False, edges), cu(s), out, precision="f64")
+    assert out.cpu().numpy()[0] == 4.0 and torch.isnan(out[1:]).all()
