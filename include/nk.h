@@ -121,10 +121,11 @@ const char *nk_last_error(void);
 /* Library version (major*10000 + minor*100 + patch). */
 int32_t nk_version(void);
 /*
- * Sticky status of the context's tensor-core products:
- * waits for the context's work on `stream` and returns in *code 0, or the
- * code of the last bounded wait that timed out since the last call (the
- * results of that call are invalid): 3-5 the S-GEMM and theta (producer, MMA
+ * Sticky status of the context's tensor-core products and triangular solves, in
+ * either precision: waits for the context's work on `stream` and returns in *code
+ * 0, or the code of the last bounded wait that timed out since the last call, other
+ * than in a call that returned NK_ERR_TIMEOUT (the results of the call that timed
+ * out are invalid): 3-5 the S-GEMM and theta (producer, MMA
  * issuer, epilogue), 6 / 7 the forward / backward triangular solve, 12-16 the
  * FP64-accurate product (producer, A slices, B slices, accumulator buffer,
  * epilogue).  Resets the word.
@@ -318,11 +319,13 @@ nk_status nk_tc_gemm(nk_ctx *ctx, int64_t rows, int64_t cols, int32_t k, const d
  * u_k^T X F).  For the two SVD solvers cg_tol is rcond (0: 1e-12); their
  * eigendecomposition is cyclic Jacobi in FP64 on CUDA cores, which reads
  * its convergence back once per sweep (synchronises the stream); n = Np or
- * Ns at most 8192.  With NK_MIXED the Cholesky factorisations run their
- * panel and trailing products on the tensor cores at FP64-level accuracy
- * (see nk_tc_gemm), and so do the Gram matrices; the call then synchronises
- * the stream and returns NK_ERR_CUDA on a failed factorisation
- * (NK_ERR_TIMEOUT on a tensor-core time-out).
+ * Ns at most 8192.  The Cholesky factorisations run their trailing products on
+ * the tensor cores at FP64-level accuracy (see nk_tc_gemm), and so do, from 1e7
+ * multiply-adds on in NK_F64, S and the Gram matrices.  Every wait of these
+ * kernels is bounded.  With NK_MIXED, and with the SVD solvers, the call
+ * synchronises the stream and returns NK_ERR_CUDA on a failed factorisation,
+ * NK_ERR_TIMEOUT on a time-out; the Cholesky solvers in NK_F64 stay asynchronous,
+ * and nk_ctx_error reports their time-outs.
  *   info_out host int32[2] or NULL: iterations (CG) or Jacobi sweeps (SVD),
  *   converged flag.
  *   resid_out host double or NULL: final relative residual (CG), or the
@@ -370,8 +373,8 @@ typedef struct {
     double f_norm;       /* ||F|| */
     double delta_norm;   /* ||delta|| */
     double solver_status; /* 0 = ok; k > 0: the Cholesky pivot k (1-based) was not
-                             positive; -1 / -2: a tensor-core product timed out
-                             waiting for its operands / its MMAs */
+                             positive; < 0: minus the code of a wait that timed out
+                             in the solve (see nk_ctx_error, which has it too) */
 } nk_sr_stats;
 
 /*

@@ -360,6 +360,20 @@ nk_status check_factor(nk_ctx *ctx, const int *info, cudaStream_t st) {
     return NK_OK;
 }
 
+// A time-out among a solve's status words (info[1]) goes to the context's sticky
+// word, for the calls that do not read the words back.
+__global__ void k_keep_timeout(const int *__restrict__ info, int *__restrict__ sticky) {
+    if (info[1]) *sticky = info[1];
+}
+
+// The end of a direct solve: its status words read back, or left to nk_ctx_error.
+nk_status end_solve(nk_ctx *ctx, const int *info, bool sync_check, cudaStream_t st) {
+    if (sync_check) return check_factor(ctx, info, st);
+    (k_keep_timeout<<<1, 1, 0, st>>>(info, ctx->tc_err), nk::note_launch());
+    NK_CU(cudaGetLastError(), "status");
+    return NK_OK;
+}
+
 // Cyclic Jacobi sweeps on the full symmetric K [n][n] (diagonalised in
 // place; V <- V J from the identity) until the relative off-diagonal norm is
 // at the rounding level or kMaxJacobiSweeps: one cooperative launch, whose
@@ -534,10 +548,8 @@ nk_status run_solve(nk_ctx *ctx, int N, int M, int64_t Ns, const int8_t *s, cons
         }
         if (host_info) host_info[0] = sweeps, host_info[1] = converged ? 1 : 0;
         if (host_resid) *host_resid = rel;
-        if (tc) {
-            nk_status f = check_factor(ctx, w.info, st);
-            if (f != NK_OK) return f;
-        }
+        nk_status f = check_factor(ctx, w.info, st);
+        if (f != NK_OK) return f;
         if (!converged)
             return fail(NK_ERR_NOT_CONVERGED, "Jacobi sweeps left a relative off-diagonal norm %g after %d sweeps",
                         rel, sweeps);
@@ -553,7 +565,7 @@ nk_status run_solve(nk_ctx *ctx, int N, int M, int64_t Ns, const int8_t *s, cons
         NK_CU(nk::launch_cholesky_tc(w.S, Np, w.info, w.info + 1, w.tc, st, &cs, !tc), "chol factor");
         NK_CU(nk::launch_axpby(Np, 1.0, F, 0.0, delta, st), "chol");
         NK_CU(nk::launch_cholesky_solve_tc(w.S, Np, w.tc, delta, w.info + 1, st, !tc), "chol solve");
-        return sync_check ? check_factor(ctx, w.info, st) : NK_OK;
+        return end_solve(ctx, w.info, sync_check, st);
     }
     // sample space: delta = (F - X^T (X X^T + eps I)^{-1} X F) / eps, X = dJ / sqrt(Ns)
     const double isq = 1.0 / std::sqrt((double)Ns);
@@ -572,7 +584,7 @@ nk_status run_solve(nk_ctx *ctx, int N, int M, int64_t Ns, const int8_t *s, cons
     NK_CU(vjp_any(N, M, Ns, s, T, w.w, 1.0, nullptr, w, w.tmp, precision, kExactSlices, st), "ss Xty");
     NK_CU(nk::launch_axpby(Np, 1.0 / eps, F, 0.0, delta, st), "ss delta");
     NK_CU(nk::launch_axpby(Np, -1.0 / eps, w.tmp, 1.0, delta, st), "ss delta");
-    return sync_check ? check_factor(ctx, w.info, st) : NK_OK;
+    return end_solve(ctx, w.info, sync_check, st);
 }
 
 // Metropolis sweeps.  NK_F64 rebuilds theta inside the sweep kernel; NK_MIXED
@@ -1493,7 +1505,7 @@ nk_status nk_symm_sr_step(nk_ctx *ctx, nk_rbm_symm *symm, const nk_ham *ham, nk_
             NK_CU(cudaGetLastError(), "acc");
         }
         chains->sweeps_done += cfg->n_discard + cfg->n_samples;
-        return mixed ? check_factor(ctx, info, st) : NK_OK;
+        return end_solve(ctx, info, mixed, st);
     };
     if (!mixed) return with_workspace(ctx, [&](Carver &c, bool run) { return body(double{}, c, run); });
     return with_workspace(ctx, [&](Carver &c, bool run) { return body(float{}, c, run); });
