@@ -300,7 +300,7 @@ __global__ void __launch_bounds__(kSgThreads, 2)
 // as FP32 pairs in shared memory (a ring of 4 tiles, an mbarrier per quarter
 // and slot), and warp (q, 0) writes the tile's row partial P[nt][row] in
 // FP64.  J^T g (mode 1) recombines V exactly in int64 and writes FP64 split-K
-// partials.  Units go round robin over the clusters.  Every wait is bounded;
+// partials.  Units go round robin over the CTAs.  Every wait is bounded;
 // a time-out sets err and drains the copies and MMAs in flight before the
 // TMEM is released.
 constexpr int kJvEpiWarps = 16;
@@ -318,9 +318,8 @@ struct Tc4Args {
     int kchunks;          // K-chunks of the whole product
     int kc_split;         // K-chunks per unit (mode 1; kchunks in mode 0)
     int ks;               // K splits
-    int n_nt, n_mg;       // column tiles; row-tile groups of C tiles
-    int C;                // CTAs per cluster (1, 2, 4): B slices multicast across them
-    int64_t groups;       // n_mg * n_nt * ks
+    int n_nt, n_mt;       // column tiles; row tiles
+    int64_t units;        // n_mt * n_nt * ks
     const int *expB;      // [n_nt * 64] (read up to the tile end; columns >= cols unused)
     const float4 *Thl;    // mode 0: t' as FP32 pairs, tile-major (launch_split_t)
     double *P;            // mode 0: [n_nt][rows]; mode 1: [ks][cols][ldp] (column-major tiles)
@@ -341,29 +340,26 @@ constexpr size_t jv_smem_bytes() {
            (size_t)(2 * kJvStages + 4 + kJvRing * 4) * 8 + 16;
 }
 
-// Unit li of cluster slot `cl` (of ncl): the cluster's row-tile group mg,
-// column tile nt and K split z, this CTA's row tile mt = mg C + rank.
-// Mode 0 walks the column tiles fastest (the A tiles of a group are reused),
-// mode 1 the row-tile groups (the B range of (nt, z) is reused from L2).
+// Unit g: row tile mt, column tile nt and K split z.  Mode 0 walks the column tiles
+// fastest (the A tiles of a row are reused), mode 1 the row tiles (the B range of
+// (nt, z) is reused from L2).
 struct Tc4Unit {
     int64_t mt;
     int nt, z;
 };
 template <int kMode>
-__device__ __forceinline__ Tc4Unit tc4_unit(const Tc4Args &a, int64_t g, uint32_t rank) {
+__device__ __forceinline__ Tc4Unit tc4_unit(const Tc4Args &a, int64_t g) {
     Tc4Unit u;
-    int64_t mg;
     if (kMode == kTcRowDot) {
-        mg = g / a.n_nt;
+        u.mt = g / a.n_nt;
         u.nt = (int)(g % a.n_nt);
         u.z = 0;
     } else {
-        mg = g % a.n_mg;
-        const int64_t r = g / a.n_mg;
+        u.mt = g % a.n_mt;
+        const int64_t r = g / a.n_mt;
         u.nt = (int)(r % a.n_nt);
         u.z = (int)(r / a.n_nt);
     }
-    u.mt = mg * a.C + rank;
     return u;
 }
 template <int kMode>
@@ -382,17 +378,13 @@ __global__ void __launch_bounds__(kJvThreads, 1)
     uint32_t *tslot = reinterpret_cast<uint32_t *>(red_full + kJvRing * 4);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tslot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int C = a.C;
-    const uint32_t rank = C > 1 ? cluster_rank() : 0u;
-    const uint16_t mask = (uint16_t)((1u << C) - 1u);
-    const int64_t cl = blockIdx.x / C, ncl = gridDim.x / C;
-    const int64_t nunits = a.groups > cl ? (a.groups - 1 - cl) / ncl + 1 : 0;
-    const int64_t n_mt = (a.rows + kBM - 1) / kBM;
+    const int64_t cta = blockIdx.x, ctas = gridDim.x;
+    const int64_t nunits = a.units > cta ? (a.units - 1 - cta) / ctas + 1 : 0;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kJvStages; ++s) {
             mbar_init(&full[s], 1);
-            mbar_init(&empty[s], (uint32_t)C);  // one commit from every CTA of the cluster
+            mbar_init(&empty[s], 1);
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&acc_full[b], 1);
@@ -404,10 +396,7 @@ __global__ void __launch_bounds__(kJvThreads, 1)
     }
     if (warp == 0) tmem_alloc(tslot, kJvTmemCols);
     tc_fence_before();
-    if (C > 1)
-        cluster_sync_all();  // the peers' barriers exist before any multicast reaches them
-    else
-        __syncthreads();
+    __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tslot;
     auto fail = [&](int code) {
@@ -417,11 +406,9 @@ __global__ void __launch_bounds__(kJvThreads, 1)
 
     if (warp == 0 && lane == 0) {
         // ---------------------------------------------------------- producer
-        // own A tile; B slices rank * 3 / C .. (rank + 1) * 3 / C - 1 to every CTA
-        const int t0 = (int)rank * kJvSB / C, t1 = ((int)rank + 1) * kJvSB / C;
         int64_t g = 0;  // K-chunks issued (all units)
         for (int64_t li = 0; li < nunits && !*abort_flag; ++li) {
-            const Tc4Unit u = tc4_unit<kMode>(a, cl + li * ncl, rank);
+            const Tc4Unit u = tc4_unit<kMode>(a, cta + li * ctas);
             const int m0 = (int)(u.mt * kBM), n0 = u.nt * kBN;
             const int kc0 = u.z * a.kc_split;
             const int kc1 = kc0 + a.kc_split < a.kchunks ? kc0 + a.kc_split : a.kchunks;
@@ -435,12 +422,7 @@ __global__ void __launch_bounds__(kJvThreads, 1)
                 unsigned char *sp = ops + (size_t)s * kJvStageBytes;
                 mbar_expect_tx(&full[s], (uint32_t)kJvStageBytes);
                 tma_load_2d(sp, &mapA, &full[s], kc * kBK, m0);
-                for (int t = t0; t < t1; ++t) {
-                    if (C > 1)
-                        tma_load_3d_mc(sp + kAB + t * kBB, &mapB, &full[s], kc * kBK, n0, t, mask);
-                    else
-                        tma_load_3d(sp + kAB + t * kBB, &mapB, &full[s], kc * kBK, n0, t);
-                }
+                for (int t = 0; t < kJvSB; ++t) tma_load_3d(sp + kAB + t * kBB, &mapB, &full[s], kc * kBK, n0, t);
             }
         }
         if (*abort_flag) {
@@ -454,7 +436,7 @@ __global__ void __launch_bounds__(kJvThreads, 1)
         int64_t g = 0;
         int64_t committed = -1;  // last unit whose accumulator commit was issued
         for (int64_t li = 0; li < nunits && !*abort_flag; ++li) {
-            const Tc4Unit u = tc4_unit<kMode>(a, cl + li * ncl, rank);
+            const Tc4Unit u = tc4_unit<kMode>(a, cta + li * ctas);
             const int kc0 = u.z * a.kc_split;
             const int kc1 = kc0 + a.kc_split < a.kchunks ? kc0 + a.kc_split : a.kchunks;
             const int b = (int)(li & 1);
@@ -478,11 +460,7 @@ __global__ void __launch_bounds__(kJvThreads, 1)
                 for (int kk = 0; kk < kBK / 16; ++kk)
                     umma_bf16(tmem + (uint32_t)b * kJvAccCols, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2),
                               idesc, (kc > kc0 || kk > 0) ? 1u : 0u);
-                // the stage is free once every CTA of the cluster has read it
-                if (C > 1)
-                    umma_commit_mc(&empty[s], mask);
-                else
-                    umma_commit(&empty[s]);
+                umma_commit(&empty[s]);
             }
             umma_commit(&acc_full[b]);
             committed = li;
@@ -500,7 +478,7 @@ __global__ void __launch_bounds__(kJvThreads, 1)
         const int q = warp & 3, grp = (warp - 2) >> 2, c0 = grp * 16;
         const uint32_t lane_base = (uint32_t)(q * 32) << 16;
         for (int64_t li = 0; li < nunits; ++li) {
-            const Tc4Unit u = tc4_unit<kMode>(a, cl + li * ncl, rank);
+            const Tc4Unit u = tc4_unit<kMode>(a, cta + li * ctas);
             const int64_t m0 = u.mt * kBM;
             const int n0 = u.nt * kBN;
             const int64_t row = m0 + q * 32 + lane;
@@ -511,18 +489,13 @@ __global__ void __launch_bounds__(kJvThreads, 1)
             // contiguous bytes, one 16-byte load per lane and column pair)
             float2 tv[16];
             if (kMode == kTcRowDot) {
-                if (u.mt < n_mt) {
-                    const float4 *src =
-                        a.Thl + (((size_t)u.mt * a.n_nt + u.nt) * (kBN / 2) + (c0 >> 1)) * kBM + q * 32 + lane;
+                const float4 *src =
+                    a.Thl + (((size_t)u.mt * a.n_nt + u.nt) * (kBN / 2) + (c0 >> 1)) * kBM + q * 32 + lane;
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const float4 v4 = __ldcs(src + (size_t)j * kBM);
-                        tv[2 * j] = make_float2(v4.x, v4.y);
-                        tv[2 * j + 1] = make_float2(v4.z, v4.w);
-                    }
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) tv[j] = make_float2(0.f, 0.f);
+                for (int j = 0; j < 8; ++j) {
+                    const float4 v4 = __ldcs(src + (size_t)j * kBM);
+                    tv[2 * j] = make_float2(v4.x, v4.y);
+                    tv[2 * j + 1] = make_float2(v4.z, v4.w);
                 }
             }
             // the warp's column exponents; mode 0 scales them against the
@@ -662,12 +635,7 @@ __global__ void __launch_bounds__(kJvThreads, 1)
         }
     }
     tc_fence_before();
-    // no peer multicasts into this CTA's shared memory or arrives on its
-    // barriers after the cluster barrier; then the TMEM goes back
-    if (C > 1)
-        cluster_sync_all();
-    else
-        __syncthreads();
+    __syncthreads();
     if (warp == 0) {
         tc_fence_after();
         tmem_dealloc(tmem, kJvTmemCols);
@@ -1279,44 +1247,22 @@ cudaError_t sgemm(const __nv_bfloat16 *A, int64_t rows, int64_t ldA, const __nv_
     return cudaGetLastError();
 }
 
-// One launch of k_tc4: as many clusters of a.C CTAs as fit at once (one CTA
-// per SM), each walking its units round robin.
+// One launch of k_tc4 on at most `ctas` CTAs (one per SM), each walking its units
+// round robin.
 template <int kMode>
-cudaError_t launch_tc4(const CUtensorMap &ma, const CUtensorMap &mb, const Tc4Args &a, cudaStream_t st) {
-    cudaError_t e = nk::allow_max_dynamic_smem((const void *)k_tc4<kMode>);
-    int dev = 0, sms = 0;
-    if (e == cudaSuccess) e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+cudaError_t launch_tc4(const CUtensorMap &ma, const CUtensorMap &mb, const Tc4Args &a, int ctas, cudaStream_t st) {
+    const cudaError_t e = nk::allow_max_dynamic_smem((const void *)k_tc4<kMode>);
     if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)a.C;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.blockDim = dim3(kJvThreads);
-    cfg.dynamicSmemBytes = jv_smem_bytes();
-    cfg.stream = st;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    int64_t ncl = sms / a.C;
-    if (a.C > 1) {
-        int fit = 0;
-        cfg.gridDim = dim3((unsigned)(ncl * a.C));
-        e = cudaOccupancyMaxActiveClusters(&fit, (const void *)k_tc4<kMode>, &cfg);
-        if (e != cudaSuccess) return e;
-        if (fit < 1) return cudaErrorInvalidConfiguration;  // the caller falls back to single CTAs
-        if (fit < ncl) ncl = fit;
-    }
-    if (ncl > a.groups) ncl = a.groups;
-    cfg.gridDim = dim3((unsigned)(ncl * a.C));
-    e = cudaLaunchKernelEx(&cfg, k_tc4<kMode>, ma, mb, a);
-    nk::note_launch();
-    return e != cudaSuccess ? e : cudaGetLastError();
+    const unsigned grid = (unsigned)(ctas < a.units ? ctas : a.units);
+    (k_tc4<kMode><<<grid, kJvThreads, jv_smem_bytes(), st>>>(ma, mb, a), nk::note_launch());
+    return cudaGetLastError();
 }
 
-// CTAs per cluster of the J v product (B slices multicast across row tiles).
-constexpr int kJvCluster = 2;
+cudaError_t sm_count(int *sms) {
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    return e == cudaSuccess ? cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev) : e;
+}
 
 // The largest K whose FP32 levels stay exact with 11-bit digits (K 2047 < 2^24).
 constexpr int kH3MaxK = 8192;
@@ -1337,14 +1283,12 @@ cudaError_t jvp4(const void *A, int64_t rows, int64_t ldA, const void *Bsl, cons
     const int n_nt = (int)((cols + kBN - 1) / kBN);
     const int64_t n_mt = (rows + kBM - 1) / kBM;
     const int kchunks = (int)((K + kBK - 1) / kBK);
-    for (int C = n_mt >= 2 * kJvCluster ? kJvCluster : 1;; C = 1) {
-        const int n_mg = (int)((n_mt + C - 1) / C);
-        Tc4Args a{rows, cols, kchunks, kchunks, 1, n_nt, n_mg, C, (int64_t)n_mg * n_nt, expB,
-                  reinterpret_cast<const float4 *>(Thl), P, 0, 0, err, skip};
-        const cudaError_t e = launch_tc4<kTcRowDot>(ma, mb, a, st);
-        if (e == cudaErrorInvalidConfiguration && C > 1) continue;  // no cluster fits: single CTAs
-        return e;
-    }
+    int sms = 0;
+    const cudaError_t e = sm_count(&sms);
+    if (e != cudaSuccess) return e;
+    Tc4Args a{rows, cols, kchunks, kchunks, 1, n_nt, (int)n_mt, n_mt * n_nt, expB,
+              reinterpret_cast<const float4 *>(Thl), P, 0, 0, err, skip};
+    return launch_tc4<kTcRowDot>(ma, mb, a, sms, st);
 }
 
 // P^T [ks][cols][ldp] (column-major split-K partial products) = A B^T by
@@ -1360,38 +1304,31 @@ cudaError_t vjp4(const void *A, int64_t rows, int64_t ldA, const void *Bsl, cons
     if (!make_rows_map(&ma, static_cast<const __nv_bfloat16 *>(A), rows, K, ldA, kBM) ||
         !make_sliced_map(&mb, static_cast<const __nv_bfloat16 *>(Bsl), cols, K, ldB, kJvSB, kBN))
         return cudaErrorInvalidValue;
-    int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    int sms = 0;
+    const cudaError_t e = sm_count(&sms);
     if (e != cudaSuccess) return e;
     const int n_nt = (int)((cols + kBN - 1) / kBN);
     const int n_mt = (int)((rows + kBM - 1) / kBM);
     const int kchunks = (int)((K + kBK - 1) / kBK);
     const int ks_min = (kchunks + kH3MaxK / kBK - 1) / (kH3MaxK / kBK);
     if (ks_min > max_ks) return cudaErrorInvalidValue;
-    // All row tiles of a unit in one cluster when there are 2 to 8 of them
-    // (N + 1 <= 1024): each tile of digits is then read from L2 once and
-    // multicast to every row tile (on the 24 x 24 workload, 5 row tiles:
-    // 100.5 against 102.4 ms of products a step).  Single CTAs otherwise, or
-    // where no cluster of that size fits.
-    for (int C = n_mt >= 2 && n_mt <= 8 ? n_mt : 1;; C = 1) {
-        const int n_mg = (n_mt + C - 1) / C, slots = sms / C;
-        int ks = ks_min;
-        double best = -1.0;
-        for (int k = ks_min; k <= max_ks; ++k) {
-            const int64_t units = (int64_t)n_mg * n_nt * k, rounds = (units + slots - 1) / slots;
-            const double score = (double)units / (double)(rounds * slots) - 0.01 * (k - ks_min);
-            if (score > best + 1e-12) best = score, ks = k;
-        }
-        const int kc_split = (kchunks + ks - 1) / ks;
-        ks = (kchunks + kc_split - 1) / kc_split;
-        *ks_out = ks;
-        Tc4Args a{rows, cols, kchunks, kc_split, ks, n_nt, n_mg, C, (int64_t)n_mg * n_nt * ks, expB, nullptr, P,
-                  ldp, split_stride, err, skip};
-        e = launch_tc4<kTcStoreT>(ma, mb, a, st);
-        if (e == cudaErrorInvalidConfiguration && C > 1) continue;
-        return e;
+    // Up to 8 row tiles (N + 1 <= 1024) run side by side, on a multiple of that many
+    // CTAs: each tile of digits is then in L2 for all of them, and a CTA keeps its rows
+    // of configurations.  The splits are counted in rounds of such groups.
+    const int side = n_mt <= 8 ? n_mt : 1, n_mg = (n_mt + side - 1) / side, slots = sms / side;
+    int ks = ks_min;
+    double best = -1.0;
+    for (int k = ks_min; k <= max_ks; ++k) {
+        const int64_t groups = (int64_t)n_mg * n_nt * k, rounds = (groups + slots - 1) / slots;
+        const double score = (double)groups / (double)(rounds * slots) - 0.01 * (k - ks_min);
+        if (score > best + 1e-12) best = score, ks = k;
     }
+    const int kc_split = (kchunks + ks - 1) / ks;
+    ks = (kchunks + kc_split - 1) / kc_split;
+    *ks_out = ks;
+    Tc4Args a{rows, cols, kchunks, kc_split, ks, n_nt, n_mt, (int64_t)n_mt * n_nt * ks, expB, nullptr, P,
+              ldp, split_stride, err, skip};
+    return launch_tc4<kTcStoreT>(ma, mb, a, slots * side, st);
 }
 
 double sgemm_flops(int64_t rows, int64_t cols, int64_t K, int SB) {

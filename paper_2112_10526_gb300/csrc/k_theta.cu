@@ -8,12 +8,10 @@
 // 128 x 32 tile.  (The 7 BF16 slices of 8 bits of the other products hold 56
 // bits in 7/5 of the tensor work and operand bytes.)
 //
-// A persistent kernel: each cluster of C CTAs (C row tiles of 128
-// configurations) walks a contiguous range of (row tile group, unit tile)
-// pairs, units fastest.  Up to 9 chunks of K (N <= 576) a CTA keeps its
-// configurations in shared memory for all its unit tiles and only the slices
-// stream through a TMA ring, each read once per cluster and multicast to it;
-// beyond, configurations stream along.  Warp 0 loads, warp 1 issues the MMAs into
+// A persistent kernel: each CTA walks a contiguous range of (row tile of 128
+// configurations, unit tile) pairs, units fastest.  Up to 9 chunks of K (N <= 576)
+// it keeps its configurations in shared memory for all its unit tiles and only the
+// slices stream through a TMA ring; beyond, configurations stream along.  Warp 0 loads, warp 1 issues the MMAs into
 // one of two accumulator sets, sixteen warps turn the other set into FP64 and
 // store it by rows.
 // What bounds it: the slices in flight (20 KB a chunk, three to six stages,
@@ -56,10 +54,10 @@ constexpr size_t kHSmem = 227 * 1024;
 struct ThetaArgs {
     int64_t rows;
     int units, N;
-    int kchunks, resident, nstages, C;
+    int kchunks, resident, nstages;
     int n_nt;            // unit tiles
-    int64_t tiles;       // row tile groups x n_nt
-    int64_t per;         // tiles per cluster
+    int64_t tiles;       // row tiles x n_nt
+    int64_t per;         // tiles per CTA
     int bits, drop;      // V 2^(expW - bits), its lowest `drop` bits left out
     const int *expW;     // [units]
     const double *bias;  // [units]
@@ -95,7 +93,7 @@ __global__ void __launch_bounds__(kHThreads, 1)
     extern __shared__ unsigned char smem_raw[];
     const uint32_t base = smem_u32(smem_raw);
     unsigned char *ops = smem_raw + ((1024 - (base & 1023)) & 1023);
-    const int NS = a.nstages, C = a.C;
+    const int NS = a.nstages;
     const int stage_bytes = kHS * kHB + (a.resident ? 0 : kHA);
     unsigned char *sA = ops;  // resident: [kchunks][128][64]
     unsigned char *sS = ops + (a.resident ? (size_t)a.kchunks * kHA : 0);
@@ -106,15 +104,13 @@ __global__ void __launch_bounds__(kHThreads, 1)
     uint32_t *tslot = reinterpret_cast<uint32_t *>(acc_empty + 2);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tslot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t rank = C > 1 ? cluster_rank() : 0u;
-    const uint16_t mask = (uint16_t)((1u << C) - 1u);
-    const int64_t cl = blockIdx.x / C, t0 = cl * a.per;
+    const int64_t t0 = blockIdx.x * a.per;
     const int64_t t1 = t0 + a.per < a.tiles ? t0 + a.per : a.tiles;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < NS; ++s) {
             mbar_init(&full[s], 1);
-            mbar_init(&empty[s], (uint32_t)C);  // one commit from every CTA of the cluster
+            mbar_init(&empty[s], 1);
         }
         mbar_init(a_full, 1);
         mbar_init(a_empty, 1);
@@ -127,10 +123,7 @@ __global__ void __launch_bounds__(kHThreads, 1)
     }
     if (warp == 0) tmem_alloc(tslot, 512);
     tc_fence_before();
-    if (C > 1)
-        cluster_sync_all();  // the peers' barriers exist before any multicast reaches them
-    else
-        __syncthreads();
+    __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tslot;
     auto fail = [&](int code) {
@@ -140,12 +133,11 @@ __global__ void __launch_bounds__(kHThreads, 1)
 
     if (warp == 0 && lane == 0) {
         // ---------------------------------------------------------- producer
-        const int q0 = (int)rank * kHS / C, q1 = ((int)rank + 1) * kHS / C;  // own slices, to every CTA
-        int64_t g = 0, row_loads = 0, mg_held = -1;
+        int64_t g = 0, row_loads = 0, mt_held = -1;
         for (int64_t t = t0; t < t1 && !*abort_flag; ++t) {
-            const int64_t mg = t / a.n_nt;
-            const int m0 = (int)((mg * C + rank) * kHM), n0 = (int)(t % a.n_nt) * kHN;
-            if (a.resident && mg != mg_held) {
+            const int64_t mt = t / a.n_nt;
+            const int m0 = (int)(mt * kHM), n0 = (int)(t % a.n_nt) * kHN;
+            if (a.resident && mt != mt_held) {
                 if (row_loads > 0 &&
                     !mbar_wait_or_abort_sleep(a_empty, (uint32_t)((row_loads - 1) & 1), abort_flag)) {
                     fail(3);
@@ -153,7 +145,7 @@ __global__ void __launch_bounds__(kHThreads, 1)
                 }
                 mbar_expect_tx(a_full, (uint32_t)(a.kchunks * kHA));
                 for (int kc = 0; kc < a.kchunks; ++kc) tma_load_2d(sA + (size_t)kc * kHA, &mapA, a_full, kc * kHK, m0);
-                mg_held = mg;
+                mt_held = mt;
                 ++row_loads;
             }
             for (int kc = 0; kc < a.kchunks; ++kc, ++g) {
@@ -164,12 +156,7 @@ __global__ void __launch_bounds__(kHThreads, 1)
                 }
                 unsigned char *sp = sS + (size_t)s * stage_bytes;
                 mbar_expect_tx(&full[s], (uint32_t)stage_bytes);
-                for (int q = q0; q < q1; ++q) {
-                    if (C > 1)
-                        tma_load_3d_mc(sp + q * kHB, &mapB, &full[s], kc * kHK, n0, q, mask);
-                    else
-                        tma_load_3d(sp + q * kHB, &mapB, &full[s], kc * kHK, n0, q);
-                }
+                for (int q = 0; q < kHS; ++q) tma_load_3d(sp + q * kHB, &mapB, &full[s], kc * kHK, n0, q);
                 if (!a.resident) tma_load_2d(sp + kHS * kHB, &mapA, &full[s], kc * kHK, m0);
             }
         }
@@ -181,21 +168,21 @@ __global__ void __launch_bounds__(kHThreads, 1)
     } else if (warp == 1 && lane == 0) {
         // ------------------------------------------------------- MMA issuer
         const uint32_t idesc = idesc_f16(kHM, kHN * kHS);
-        int64_t g = 0, rows_used = 0, mg_held = -1, committed = -1;
+        int64_t g = 0, rows_used = 0, mt_held = -1, committed = -1;
         for (int64_t t = t0; t < t1 && !*abort_flag; ++t) {
-            const int64_t li = t - t0, mg = t / a.n_nt;
+            const int64_t li = t - t0, mt = t / a.n_nt;
             const int b = (int)(li & 1);
             const uint32_t use = (uint32_t)(li >> 1);
             if (use > 0 && !mbar_wait_or_abort_sleep(&acc_empty[b], (use - 1) & 1, abort_flag)) {
                 fail(4);
                 break;
             }
-            if (a.resident && mg != mg_held) {
+            if (a.resident && mt != mt_held) {
                 if (!mbar_wait_or_abort_sleep(a_full, (uint32_t)(rows_used & 1), abort_flag)) {
                     fail(4);
                     break;
                 }
-                mg_held = mg;
+                mt_held = mt;
                 ++rows_used;
             }
             bool ok = true;
@@ -213,13 +200,9 @@ __global__ void __launch_bounds__(kHThreads, 1)
                 for (int kk = 0; kk < kHK / 16; ++kk)
                     umma_bf16(tmem + (uint32_t)b * kHAcc, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc,
                               (kc > 0 || kk > 0) ? 1u : 0u);
-                // the stage is free once every CTA of the cluster has read it
-                if (C > 1)
-                    umma_commit_mc(&empty[s], mask);
-                else
-                    umma_commit(&empty[s]);
+                umma_commit(&empty[s]);
             }
-            if (a.resident && (t + 1 == t1 || (t + 1) / a.n_nt != mg)) umma_commit(a_empty);
+            if (a.resident && (t + 1 == t1 || (t + 1) / a.n_nt != mt)) umma_commit(a_empty);
             umma_commit(&acc_full[b]);
             committed = li;
             if (!ok) {
@@ -240,7 +223,7 @@ __global__ void __launch_bounds__(kHThreads, 1)
         const int rr = lane >> 2, cc = lane & 3;
         for (int64_t t = t0; t < t1; ++t) {
             const int64_t li = t - t0;
-            const int64_t m0 = (t / a.n_nt * C + rank) * kHM + q * 32;
+            const int64_t m0 = t / a.n_nt * kHM + q * 32;
             const int n0 = (int)(t % a.n_nt) * kHN + c0;
             const int b = (int)(li & 1);
             int e_lane = 0;
@@ -301,13 +284,11 @@ __global__ void __launch_bounds__(kHThreads, 1)
                 if (kPairs) {
                     // 64-unit tiles of 32 column pairs x 128 rows
                     const int u0 = n0 + 4 * h;
-                    const int64_t mt = t / a.n_nt * C + rank;
-                    if (mt * kHM < a.rows) {
-                        float4 *dst = a.pairs + ((size_t)(mt * (a.n_nt / 2) + (u0 >> 6)) * 32 + ((u0 & 63) >> 1)) * kHM +
-                                      q * 32 + lane;
-                        __stcs(dst, make_float4(pr[0].x, pr[0].y, pr[1].x, pr[1].y));
-                        __stcs(dst + kHM, make_float4(pr[2].x, pr[2].y, pr[3].x, pr[3].y));
-                    }
+                    const int64_t mt = t / a.n_nt;
+                    float4 *dst = a.pairs + ((size_t)(mt * (a.n_nt / 2) + (u0 >> 6)) * 32 + ((u0 & 63) >> 1)) * kHM +
+                                  q * 32 + lane;
+                    __stcs(dst, make_float4(pr[0].x, pr[0].y, pr[1].x, pr[1].y));
+                    __stcs(dst + kHM, make_float4(pr[2].x, pr[2].y, pr[3].x, pr[3].y));
                     continue;
                 }
                 __syncwarp();
@@ -325,12 +306,7 @@ __global__ void __launch_bounds__(kHThreads, 1)
         }
     }
     tc_fence_before();
-    // no peer multicasts into this CTA's shared memory or arrives on its
-    // barriers after the cluster barrier; then the TMEM goes back
-    if (C > 1)
-        cluster_sync_all();
-    else
-        __syncthreads();
+    __syncthreads();
     if (warp == 0) {
         tc_fence_after();
         tmem_dealloc(tmem, 512);
@@ -396,40 +372,15 @@ cudaError_t launch_theta_product(const __half *A, int64_t rows, int64_t ldA, con
     if (a.nstages > kHMaxStages) a.nstages = kHMaxStages;
     const size_t smem = fixed + a.nstages * stage;
     const int64_t n_mt = (rows + kHM - 1) / kHM;
-    // clusters of two row tiles once there is more than one tile an SM (each
-    // slice is then read from L2 once for both)
-    for (int C = n_mt >= 2 && n_mt * a.n_nt > sms ? 2 : 1;; C = 1) {
-        a.C = C;
-        a.tiles = (n_mt + C - 1) / C * a.n_nt;
-        cudaLaunchConfig_t cfg = {};
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = (unsigned)C;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.blockDim = dim3(kHThreads);
-        cfg.dynamicSmemBytes = smem;
-        cfg.stream = st;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        int64_t ncl = sms / C;
-        if (C > 1) {
-            int fit = 0;
-            cfg.gridDim = dim3((unsigned)(ncl * C));
-            e = cudaOccupancyMaxActiveClusters(&fit, kern, &cfg);
-            if (e != cudaSuccess) return e;
-            if (fit < 1) continue;  // no cluster fits: single CTAs
-            if (fit < ncl) ncl = fit;
-        }
-        if (ncl > a.tiles) ncl = a.tiles;
-        a.per = (a.tiles + ncl - 1) / ncl;
-        ncl = (a.tiles + a.per - 1) / a.per;
-        cfg.gridDim = dim3((unsigned)(ncl * C));
-        e = pairs ? cudaLaunchKernelEx(&cfg, k_theta<true>, ma, mb, a)
-                  : cudaLaunchKernelEx(&cfg, k_theta<false>, ma, mb, a);
-        nk::note_launch();
-        return e != cudaSuccess ? e : cudaGetLastError();
-    }
+    a.tiles = n_mt * a.n_nt;
+    const int64_t ctas = sms < a.tiles ? sms : a.tiles;
+    a.per = (a.tiles + ctas - 1) / ctas;
+    const unsigned grid = (unsigned)((a.tiles + a.per - 1) / a.per);
+    if (pairs)
+        (k_theta<true><<<grid, kHThreads, smem, st>>>(ma, mb, a), nk::note_launch());
+    else
+        (k_theta<false><<<grid, kHThreads, smem, st>>>(ma, mb, a), nk::note_launch());
+    return cudaGetLastError();
 }
 
 }  // namespace nk
