@@ -309,45 +309,62 @@ __device__ __forceinline__ unsigned long long fixed_factor(long long t, long lon
     const long long p = __mul64hi(t, tau) * 4;  // 2^62 t tau
     return (1ULL << 62) - (unsigned long long)(up ? p : -p);  // 2^62 (1 - s t tau), in [0, 2^63]
 }
-// a times f 2^-point; kSmall: f may be small or 0.
-template <bool kSmall>
 __device__ __forceinline__ void fixed_mul(FixProd &a, unsigned long long f, int point) {
     const unsigned long long r = __umul64hi(a.m, f);  // 2^(point - 1) of the product
-    const int z = kSmall ? min(__clzll((long long)r), 63) : __clz((int)(r >> 32));
+    const int z = __clz((int)(r >> 32));
     a.m = r << z;
     a.e += 64 - point - z;
 }
-// Two factors f0, f1 (2^62 each) at once; one after the other where their product
-// is below 2^-8 and its high half would lose digits that they have (a pair of 2^-20
-// kept 22 bits).
-__device__ __forceinline__ void fixed_mul2(FixProd &a, unsigned long long f0, unsigned long long f1) {
-    const unsigned long long p = __umul64hi(f0, f1);  // 2^60 of the product
-    if ((p >> 52) != 0) {
-        fixed_mul<false>(a, p, 60);
-    } else {
-        fixed_mul<true>(a, f0, 62);
-        fixed_mul<true>(a, f1, 62);
-    }
+__device__ __forceinline__ Prod<double> fixed_value(const FixProd &a) {
+    // m 2^-63 2^e, as a mantissa in [1/2, 1)
+    return Prod<double>{window_to_double((long long)(a.m >> 1), -63), a.e + 1};
 }
 
+// The product where a factor is small or 0: one at a time, normalised over all 64
+// bits.
+__device__ __noinline__ Prod<double> strided_product_small(const long long *__restrict__ t,
+                                                           const long long *__restrict__ tau, size_t tstride, bool up,
+                                                           int j0, int step, int M) {
+    FixProd a{1ULL << 63, 0};
+    for (int j = j0; j < M; j += step) {
+        const unsigned long long r = __umul64hi(a.m, fixed_factor(t[j], tau[(size_t)j * tstride], up));
+        const int z = min(__clzll((long long)r), 63);
+        a.m = r << z;
+        a.e += 2 - z;
+    }
+    return fixed_value(a);
+}
+
+// Two factors go into the product through the high half of theirs, which keeps 2^-60:
+// enough down to 2^-8, where FP64 itself has 2^-49 left of a factor.  The smallest is
+// noted, and the product done over one by one if it was below (a pair of 2^-20 would
+// keep 22 bits; |W| from 1 on, units that a flip turns over).
 __device__ __forceinline__ Prod<double> strided_product(const long long *__restrict__ t,
                                                         const long long *__restrict__ tau, size_t tstride, double si,
                                                         int j0, int step, int M) {
     const bool up = si > 0.0;
     FixProd a{1ULL << 63, 0}, b{1ULL << 63, 0};
+    unsigned least = 1u << 20;
     int j = j0;
     for (; j + 3 * step < M; j += 4 * step) {
         const unsigned long long f0 = fixed_factor(t[j], tau[(size_t)j * tstride], up);
         const unsigned long long f1 = fixed_factor(t[j + step], tau[(size_t)(j + step) * tstride], up);
         const unsigned long long f2 = fixed_factor(t[j + 2 * step], tau[(size_t)(j + 2 * step) * tstride], up);
         const unsigned long long f3 = fixed_factor(t[j + 3 * step], tau[(size_t)(j + 3 * step) * tstride], up);
-        fixed_mul2(a, f0, f1);
-        fixed_mul2(b, f2, f3);
+        const unsigned long long p0 = __umul64hi(f0, f1), p1 = __umul64hi(f2, f3);  // 2^60 of the products
+        least = min(least, min((unsigned)(p0 >> 32), (unsigned)(p1 >> 32)));
+        fixed_mul(a, p0, 60);
+        fixed_mul(b, p1, 60);
     }
-    for (; j < M; j += step) fixed_mul<true>(a, fixed_factor(t[j], tau[(size_t)j * tstride], up), 62);
-    fixed_mul<true>(a, b.m, 63);
-    // value = m 2^-63 2^(a.e + b.e), as a mantissa in [1/2, 1)
-    return Prod<double>{window_to_double((long long)(a.m >> 1), -63), a.e + b.e + 1};
+    for (; j < M; j += step) {
+        const unsigned long long f = fixed_factor(t[j], tau[(size_t)j * tstride], up);
+        least = min(least, (unsigned)(f >> 34));
+        fixed_mul(a, f, 62);
+    }
+    if (least < 1u << 20) return strided_product_small(t, tau, tstride, up, j0, step, M);
+    fixed_mul(a, b.m, 63);
+    a.e += b.e;
+    return fixed_value(a);
 }
 
 // Lanes over hidden units, four consecutive units per lane (16-byte loads of
