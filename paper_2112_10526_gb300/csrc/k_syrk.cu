@@ -3,25 +3,32 @@
 // 3.5), with the integer slices of k_tc.cu.
 //
 // Every column of X is scaled by one power of two (its largest entry over all
-// rows, so that the scale does not depend on k) and cut into 7 slices of
-// 8-bit integers, stored with k contiguous: [7][n][ldk] BF16.  A CTA owns one
-// 128 x 32 tile of the lower triangle and a range of k (a split), and walks it
-// in chunks of 64: the products of slices s + t = g land in one FP32 level g
-// in TMEM, exact over a chunk, and are added up over the chunks as integers in
-// registers (two 64-bit sums an entry), so C is touched once however long K
-// is.  (The 64-row passes of k_ozaki_gemm that this replaces read and wrote C
+// rows, so that the scale does not depend on k), rounded to 56 bits and cut into
+// 7 slices of 8-bit integers, stored with k contiguous: [7][n][ldk] BF16.  A CTA
+// owns one 128 x 32 tile of the lower triangle and a range of k (a split), and
+// walks it in chunks of 64: the products of slices s + t = g, g = 2 .. 9, land in
+// one FP32 level g in TMEM, exact over a chunk, and are added up over the chunks
+// as integers in registers (two 64-bit sums an entry), so C is touched once
+// however long K is.  (The 64-row passes of k_ozaki_gemm that this replaces read and wrote C
 // once a chunk and took a slicing and a product launch each: 2.68 ms for the
 // 405 x 405 x 8192 matrix of the symmetric RBM; FP64 on CUDA cores took 16.8
 // ms for 880 x 880 x 8192.)
+//
+// Accuracy: with r = max |x| / rms x of a column, the rounding and the products left
+// out (s + t >= 10) err by at most 2^-56 r_i + 2^-56 r_j + 2^-59 r_i r_j of
+// sqrt(S_ii S_jj).  Where the scale's square is over 256 mean squares (a spin that
+// flips in a few samples of a thousand), the column's products are done over in
+// FP64 (k_syrk_exact), so that S is as accurate as sums in FP64 for every column.
+// (Without level 9, and truncated, a column of 1 flip in 1000 lost 10 bits.)
 //
 // Roles: warp 0 (one thread) streams operands by TMA, the 7 B slices of a
 // chunk into one of two 28 KB buffers and the A slices one by one into a ring
 // of nine 16 KB slots, so that a chunk's 140 KB need not be there before its
 // MMAs start; warp 1 (one thread) issues, per A slice, 4 MMAs against B slices
-// 1 .. 8-s side by side (M = 128, N = 32 (8-s), K = 16) into one of two TMEM
+// 1 .. min(7, 9-s) side by side (M = 128, N up to 224, K = 16) into one of two TMEM
 // accumulator sets; warps 2 - 17 drain the other set.  What bounds it: the
-// drain (7 float-to-integer conversions an entry and chunk, 16 lanes a clock
-// and SM, about 1.1 us a chunk) and the 28 slice products (about as long).
+// drain (8 float-to-integer conversions an entry and chunk, 16 lanes a clock
+// and SM, about 1.2 us a chunk) and the 34 slice products (about as long).
 // Every wait is bounded; on a time-out the kernel records a code, lets its
 // copies and MMAs in flight finish, frees its TMEM and returns.
 
@@ -38,6 +45,7 @@ namespace nk {
 namespace {
 
 constexpr int kS = 7;                          // slices
+constexpr int kLevels = 8;                     // s + t = 2 .. 9 (slices from 1)
 constexpr int kYM = 128, kYN = 32, kYK = 64;   // tile and chunk
 constexpr int kYA = kYM * kYK * 2;             // one A slice of a chunk, bytes
 constexpr int kYB = kYN * kYK * 2;             // one B slice
@@ -84,17 +92,27 @@ __global__ void __launch_bounds__(256) k_col_exponents(const double *__restrict_
     }
 }
 
-__global__ void k_exponents_init(int64_t n, int *__restrict__ expo) {
+__global__ void k_exponents_init(int64_t n, int *__restrict__ expo, unsigned long long *__restrict__ sq) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) expo[i] = -100000;
+    if (i < n) {
+        expo[i] = -100000;
+        sq[i] = 0;
+    }
+}
+
+// Whether a column's entries are too uneven for its slices: 2^(2 e) above 256 mean
+// squares (sq: sum of the squares of floor(2^12 |x| 2^-e)), or not finite.
+__device__ __forceinline__ bool uneven(int64_t rows, int e, unsigned long long sq) {
+    return e != -100000 && (e == kBadExp || (sq >> 16) < (unsigned long long)rows);
 }
 
 // X [rows][n] -> slices out [7][n][ldk] (column p of X is row p; zero from
 // rows to ldk): 64 rows x 32 columns per block through shared memory, BF16
-// pairs along k.
+// pairs along k; the squares of the columns' leading 12 bits are added to sq.
 __global__ void __launch_bounds__(256) k_slice_cols_long(const double *__restrict__ X, int64_t rows, int64_t n,
                                                          int64_t ldk, const int *__restrict__ expo,
-                                                         __nv_bfloat162 *__restrict__ out) {
+                                                         __nv_bfloat162 *__restrict__ out,
+                                                         unsigned long long *__restrict__ sq) {
     __shared__ double tile[64][33];
     const int tid = threadIdx.x;
     const int64_t p0 = (int64_t)blockIdx.x * 32, r0 = (int64_t)blockIdx.y * 64;
@@ -116,8 +134,14 @@ __global__ void __launch_bounds__(256) k_slice_cols_long(const double *__restric
             unsigned long long m;
             split_bits(tile[2 * k2 + h][c], b, m, neg[h]);
             const int sh = b - 1075 + 8 * kS - e;
-            y[h] = !m || sh <= -64 ? 0ULL : (sh >= 0 ? (m << sh) : (m >> (-sh)));
+            // (only values below 2^(e - 3) are rounded: none reaches 2^e)
+            y[h] = !m || sh <= -64 || e == kBadExp
+                       ? 0ULL
+                       : (sh >= 0 ? (m << sh) : (m >> (-sh)) + ((m >> (-sh - 1)) & 1ULL));
         }
+        const unsigned q0 = (unsigned)(y[0] >> 44), q1 = (unsigned)(y[1] >> 44);
+        const unsigned qq = __reduce_add_sync(0xffffffffu, q0 * q0 + q1 * q1);
+        if (k2 == 0 && qq) atomicAdd(&sq[p0 + c], (unsigned long long)qq);
         __nv_bfloat162 *o = out + ((size_t)(p0 + c) * ldk + r0) / 2 + k2;
 #pragma unroll
         for (int q = 0; q < kS; ++q) {
@@ -264,11 +288,21 @@ __global__ void __launch_bounds__(kYThreads, 1)
                 }
                 tc_fence_after();
                 const uint64_t da = sw128_desc(sA + (size_t)slot * kYA);
-                const uint32_t idesc = idesc_bf16(kYM, kYN * (kS - s));
+                // levels s .. 7 (from 0): B slices 0 .. 7 - s, of which there are 7; slice
+                // 1 opens level 7 with its product by B slice 6
+                const uint32_t ds = d + (uint32_t)(s * kYN);
+                const uint32_t idesc = idesc_bf16(kYM, kYN * (s == 0 ? kS : kLevels - s));
+                const uint64_t db6 = sw128_desc(sB + (size_t)(b * kS + kS - 1) * kYB);
 #pragma unroll
-                for (int kk = 0; kk < kYK / 16; ++kk)
-                    umma_bf16(d + (uint32_t)(s * kYN), da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc,
-                              (kk > 0 || s > 0) ? 1u : 0u);
+                for (int kk = 0; kk < kYK / 16; ++kk) {
+                    const uint64_t dak = da + (uint64_t)(kk * 2), dbk = db + (uint64_t)(kk * 2);
+                    if (s == 1 && kk == 0) {
+                        umma_bf16(ds, dak, dbk, idesc_bf16(kYM, kYN * (kS - 1)), 1u);
+                        umma_bf16(d + (uint32_t)((kLevels - 1) * kYN), dak, db6, idesc_bf16(kYM, kYN), 0u);
+                    } else {
+                        umma_bf16(ds, dak, dbk, idesc, (kk > 0 || s > 0) ? 1u : 0u);
+                    }
+                }
                 umma_commit(&a_empty[slot]);
             }
             umma_commit(&b_empty[b]);
@@ -284,9 +318,9 @@ __global__ void __launch_bounds__(kYThreads, 1)
     } else if (warp >= 2) {
         // --------------------------------------------------------- epilogue
         // warp: tile rows 32q .. 32q + 31 (its TMEM lane quarter), 8 columns;
-        // an entry's levels D_2 .. D_8 as hi = sum D_2 2^16 + D_3 2^8 + D_4 and
-        // lo = sum D_5 2^24 + D_6 2^16 + D_7 2^8 + D_8 over the chunks: the
-        // product is (hi 2^32 + lo) 2^(e_i + e_j - 64)
+        // an entry's levels D_2 .. D_9 as hi = sum D_2 2^24 + D_3 2^16 + D_4 2^8 +
+        // D_5 and lo = sum D_6 2^24 + D_7 2^16 + D_8 2^8 + D_9 over the chunks (both
+        // below 2^49 a chunk): the product is (hi 2^32 + lo) 2^(e_i + e_j - 72)
         const int q = warp & 3, cw = ((warp - 2) >> 2) * kYCols;
         const uint32_t lane_base = (uint32_t)(q * 32) << 16;
         long long hi[kYCols], lo[kYCols];
@@ -306,18 +340,18 @@ __global__ void __launch_bounds__(kYThreads, 1)
             tc_fence_after();
 #pragma unroll
             for (int c4 = 0; c4 < kYCols; c4 += 4) {
-                uint32_t r[kS][4];
+                uint32_t r[kLevels][4];
 #pragma unroll
-                for (int g = 0; g < kS; ++g)
+                for (int g = 0; g < kLevels; ++g)
                     tmem_ld4(tmem + (uint32_t)b * kYAcc + lane_base + (uint32_t)(g * kYN + cw + c4), r[g]);
                 tmem_wait_ld();
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    int v[kS];
+                    int v[kLevels];
 #pragma unroll
-                    for (int g = 0; g < kS; ++g) v[g] = __float2int_rn(__uint_as_float(r[g][j]));
-                    hi[c4 + j] += (long long)v[0] * 65536 + (long long)v[1] * 256 + v[2];
-                    lo[c4 + j] += (long long)v[3] * 16777216 + (long long)v[4] * 65536 + (long long)v[5] * 256 + v[6];
+                    for (int g = 0; g < kLevels; ++g) v[g] = __float2int_rn(__uint_as_float(r[g][j]));
+                    hi[c4 + j] += (long long)v[0] * 16777216 + (long long)v[1] * 65536 + (long long)v[2] * 256 + v[3];
+                    lo[c4 + j] += (long long)v[4] * 16777216 + (long long)v[5] * 65536 + (long long)v[6] * 256 + v[7];
                 }
             }
             tc_fence_before();
@@ -334,10 +368,8 @@ __global__ void __launch_bounds__(kYThreads, 1)
                 if (col > row) continue;  // also the columns past n
                 const int ej = a.expo[col];
                 double v = 0.0;
-                if (ei == kBadExp || ej == kBadExp)
-                    v = __longlong_as_double(0x7FF8000000000000LL);
-                else if (ei != -100000 && ej != -100000)
-                    v = scale_pow2(fma((double)hi[j], 4294967296.0, (double)lo[j]), ei + ej - 64);
+                if (ei != -100000 && ej != -100000 && ei != kBadExp && ej != kBadExp)  // (bad: k_syrk_exact)
+                    v = scale_pow2(fma((double)hi[j], 4294967296.0, (double)lo[j]), ei + ej - 72);
                 if (a.splits == 1) v = v * a.scale + (col == row ? a.eps : 0.0);
                 dst[col] = v;
             }
@@ -361,6 +393,55 @@ __global__ void k_syrk_finish(int64_t n, int splits, const double *__restrict__ 
     C[(size_t)i * n + j] = v * scale + (i == j ? eps : 0.0);
 }
 
+// The entries of C in the rows and columns of uneven columns of X, in FP64: items
+// of one such column by 64 others, 4 threads a pair over the rows, 4 chains each.
+// All columns so take what the FP64 pipe takes for the whole product (16 ms for 880
+// x 880 x 8192); without any, 3 us for the look at sq.
+__global__ void __launch_bounds__(256) k_syrk_exact(const double *__restrict__ X, int64_t rows, int64_t n,
+                                                    const int *__restrict__ expo,
+                                                    const unsigned long long *__restrict__ sq, double scale, double eps,
+                                                    double *__restrict__ C) {
+    __shared__ int list[256], count[8];
+    __shared__ double part[4][64];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5, c = t & 63, y = t >> 6;
+    const int64_t tiles = (n + 63) / 64;
+    for (int64_t base = 0; base < n; base += 256) {
+        const bool f = base + t < n && uneven(rows, expo[base + t], sq[base + t]);
+        const unsigned mask = __ballot_sync(0xffffffffu, f);
+        if (lane == 0) count[warp] = __popc(mask);
+        if (!__syncthreads_or(f)) continue;
+        int before = 0, total = 0;
+        for (int w = 0; w < 8; ++w) {
+            if (w < warp) before += count[w];
+            total += count[w];
+        }
+        if (f) list[before + __popc(mask & ((1u << lane) - 1u))] = t;
+        __syncthreads();
+        for (int64_t it = blockIdx.x; it < total * tiles; it += gridDim.x) {
+            const int64_t i = base + list[it / tiles], j = it % tiles * 64 + c;
+            // a pair of uneven columns is the later one's
+            const bool on = j < n && !(j > i && uneven(rows, expo[j], sq[j]));
+            double q[4] = {0.0, 0.0, 0.0, 0.0};
+            if (on) {
+                int64_t r = y;
+                for (; r + 12 < rows; r += 16)
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        q[u] = fma(X[(size_t)(r + 4 * u) * n + i], X[(size_t)(r + 4 * u) * n + j], q[u]);
+                for (; r < rows; r += 4) q[0] = fma(X[(size_t)r * n + i], X[(size_t)r * n + j], q[0]);
+            }
+            part[y][c] = (q[0] + q[1]) + (q[2] + q[3]);
+            __syncthreads();
+            if (y == 0 && on) {
+                const double v = ((part[0][c] + part[1][c]) + (part[2][c] + part[3][c])) * scale;
+                C[(size_t)(i > j ? i : j) * n + (i > j ? j : i)] = v + (i == j ? eps : 0.0);
+            }
+            __syncthreads();
+        }
+        __syncthreads();
+    }
+}
+
 int64_t lower_tiles(int64_t n) {
     int64_t t = 0;
     for (int64_t m0 = 0; m0 < n; m0 += kYM) {
@@ -380,12 +461,14 @@ int syrk_splits(int64_t rows, int64_t n) {
     return z < 1 ? 1 : (int)z;
 }
 
+size_t round256(size_t b) { return (b + 255) / 256 * 256; }
+
 }  // namespace
 
 size_t tc_syrk_ws_bytes(int64_t rows, int64_t n) {
     const int64_t ldk = (rows + kYK - 1) / kYK * kYK;
-    const int z = syrk_splits(rows, n);
-    return ((size_t)kS * n * ldk * 2 + 255) / 256 * 256 + ((size_t)n * 4 + 255) / 256 * 256 +
+    const int z = syrk_splits(ldk, n);
+    return round256((size_t)kS * n * ldk * 2) + round256((size_t)n * 4) + round256((size_t)n * 8) +
            (z > 1 ? (size_t)z * n * n * 8 : 0) + 256;
 }
 
@@ -397,15 +480,15 @@ cudaError_t launch_syrk_tc(const double *X, int64_t rows, int64_t n, double scal
     if (n > 65535 || ldk / kYK > 65535 || tiles > (1LL << 31) - 1) return cudaErrorInvalidValue;
     char *p = static_cast<char *>(ws);
     auto *sl = reinterpret_cast<__nv_bfloat16 *>(p);
-    p += ((size_t)kS * n * ldk * 2 + 255) / 256 * 256;
+    p += round256((size_t)kS * n * ldk * 2);
     int *expo = reinterpret_cast<int *>(p);
-    p += ((size_t)n * 4 + 255) / 256 * 256;
+    p += round256((size_t)n * 4);
+    auto *sq = reinterpret_cast<unsigned long long *>(p);
+    p += round256((size_t)n * 8);
     double *partial = reinterpret_cast<double *>(p);
     const int slot = prof_begin(NK_PROF_GRAM, st);
-    (k_exponents_init<<<nblk(n, 256), 256, 0, st>>>(n, expo), nk::note_launch());
+    (k_exponents_init<<<nblk(n, 256), 256, 0, st>>>(n, expo, sq), nk::note_launch());
     (k_col_exponents<<<dim3(nblk(n, 32), nblk(rows, 256)), 256, 0, st>>>(X, rows, n, expo), nk::note_launch());
-    (k_slice_cols_long<<<dim3(nblk(n, 32), (unsigned)(ldk / 64)), 256, 0, st>>>(
-        X, rows, n, ldk, expo, reinterpret_cast<__nv_bfloat162 *>(sl)), nk::note_launch());
     EncodeTiledFn fn = encode_fn();
     if (!fn) return cudaErrorInvalidValue;
     CUtensorMap ma, mb;
@@ -422,16 +505,20 @@ cudaError_t launch_syrk_tc(const double *X, int64_t rows, int64_t n, double scal
     cudaError_t e = nk::allow_max_dynamic_smem((const void *)k_oz_syrk);
     if (e != cudaSuccess) return e;
     const int chunks = (int)(ldk / kYK);
+    (k_slice_cols_long<<<dim3(nblk(n, 32), (unsigned)chunks), 256, 0, st>>>(
+        X, rows, n, ldk, expo, reinterpret_cast<__nv_bfloat162 *>(sl), sq), nk::note_launch());
     int z = syrk_splits(rows, n);
     const int per = (chunks + z - 1) / z;
     z = (chunks + per - 1) / per;
     SyrkArgs a{n, chunks, per, expo, z > 1 ? partial : C, scale, eps, z, err};
-    (k_oz_syrk<<<dim3((unsigned)tiles, (unsigned)z), kYThreads, syrk_smem_bytes(), st>>>(ma, mb, a), nk::note_launch());
+    (k_oz_syrk<<<dim3((unsigned)tiles, (unsigned)z), kYThreads, syrk_smem_bytes(), st>>>(ma, mb, a),
+     nk::note_launch());
     if (z > 1)
         (k_syrk_finish<<<dim3(nblk(n, 256), (unsigned)n), 256, 0, st>>>(n, z, partial, scale, eps, C),
          nk::note_launch());
+    (k_syrk_exact<<<304, 256, 0, st>>>(X, rows, n, expo, sq, scale, eps, C), nk::note_launch());
     prof_end(slot, st, (double)rows * n * (double)(n + 1),
-             (double)tiles * chunks * 28.0 * 2.0 * kYM * kYN * kYK);
+             (double)tiles * (double)((rows + kYK - 1) / kYK) * 34.0 * 2.0 * kYM * kYN * kYK);
     return cudaGetLastError();
 }
 
