@@ -55,6 +55,10 @@ constexpr int kYThreads = 64 + 32 * kYEpiWarps;
 constexpr int kYCols = kYN / (kYEpiWarps / 4);  // tile columns per epilogue warp: 8
 constexpr uint32_t kYAcc = 256;                // TMEM columns per accumulator set
 constexpr int kBadExp = 100000;                // column exponent of an infinity or NaN
+// The slices of at most this many bytes are held at a time (and of at most 2^19
+// rows: the integer sums of an entry stay below 2^62).
+constexpr size_t kSliceBytes = (size_t)1 << 30;
+constexpr int64_t kSegRows = 1 << 19;
 
 inline unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
@@ -163,6 +167,7 @@ struct SyrkArgs {
     double *C;       // one split: the result (row stride n); else partials [split][n][n]
     double scale, eps;
     int splits;
+    int add;         // C += the product (a later segment of rows; eps is in already)
     int *err;
 };
 
@@ -370,7 +375,7 @@ __global__ void __launch_bounds__(kYThreads, 1)
                 double v = 0.0;
                 if (ei != -100000 && ej != -100000 && ei != kBadExp && ej != kBadExp)  // (bad: k_syrk_exact)
                     v = scale_pow2(fma((double)hi[j], 4294967296.0, (double)lo[j]), ei + ej - 72);
-                if (a.splits == 1) v = v * a.scale + (col == row ? a.eps : 0.0);
+                if (a.splits == 1) v = v * a.scale + (a.add ? dst[col] : (col == row ? a.eps : 0.0));
                 dst[col] = v;
             }
         }
@@ -383,14 +388,14 @@ __global__ void __launch_bounds__(kYThreads, 1)
     }
 }
 
-// C <- scale sum_z P[z] + eps I on the lower triangle, in split order.
-__global__ void k_syrk_finish(int64_t n, int splits, const double *__restrict__ P, double scale, double eps,
+// C <- scale sum_z P[z] + eps I (add: + C) on the lower triangle, in split order.
+__global__ void k_syrk_finish(int64_t n, int splits, const double *__restrict__ P, double scale, double eps, int add,
                               double *__restrict__ C) {
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, i = blockIdx.y;
     if (j > i || i >= n) return;
     double v = 0.0;
     for (int z = 0; z < splits; ++z) v += P[(size_t)z * n * n + (size_t)i * n + j];
-    C[(size_t)i * n + j] = v * scale + (i == j ? eps : 0.0);
+    C[(size_t)i * n + j] = v * scale + (add ? C[(size_t)i * n + j] : (i == j ? eps : 0.0));
 }
 
 // The entries of C in the rows and columns of uneven columns of X, in FP64: items
@@ -461,12 +466,21 @@ int syrk_splits(int64_t rows, int64_t n) {
     return z < 1 ? 1 : (int)z;
 }
 
+// Rows sliced at a time.
+int64_t seg_rows(int64_t rows, int64_t n) {
+    int64_t cap = (int64_t)(kSliceBytes / ((size_t)kS * 2 * n)) / kYK * kYK;
+    if (cap > kSegRows) cap = kSegRows;
+    if (cap < kYK) cap = kYK;
+    const int64_t all = (rows + kYK - 1) / kYK * kYK;
+    return all < cap ? all : cap;
+}
+
 size_t round256(size_t b) { return (b + 255) / 256 * 256; }
 
 }  // namespace
 
 size_t tc_syrk_ws_bytes(int64_t rows, int64_t n) {
-    const int64_t ldk = (rows + kYK - 1) / kYK * kYK;
+    const int64_t ldk = seg_rows(rows, n);
     const int z = syrk_splits(ldk, n);
     return round256((size_t)kS * n * ldk * 2) + round256((size_t)n * 4) + round256((size_t)n * 8) +
            (z > 1 ? (size_t)z * n * n * 8 : 0) + 256;
@@ -475,9 +489,9 @@ size_t tc_syrk_ws_bytes(int64_t rows, int64_t n) {
 cudaError_t launch_syrk_tc(const double *X, int64_t rows, int64_t n, double scale, double eps, double *C, int *err,
                            void *ws, cudaStream_t st) {
     if (rows <= 0 || n <= 0) return cudaSuccess;
-    const int64_t ldk = (rows + kYK - 1) / kYK * kYK;
+    const int64_t ldk = seg_rows(rows, n);
     const int64_t tiles = lower_tiles(n);
-    if (n > 65535 || ldk / kYK > 65535 || tiles > (1LL << 31) - 1) return cudaErrorInvalidValue;
+    if (tiles > (1LL << 31) - 1) return cudaErrorInvalidValue;
     char *p = static_cast<char *>(ws);
     auto *sl = reinterpret_cast<__nv_bfloat16 *>(p);
     p += round256((size_t)kS * n * ldk * 2);
@@ -488,7 +502,12 @@ cudaError_t launch_syrk_tc(const double *X, int64_t rows, int64_t n, double scal
     double *partial = reinterpret_cast<double *>(p);
     const int slot = prof_begin(NK_PROF_GRAM, st);
     (k_exponents_init<<<nblk(n, 256), 256, 0, st>>>(n, expo, sq), nk::note_launch());
-    (k_col_exponents<<<dim3(nblk(n, 32), nblk(rows, 256)), 256, 0, st>>>(X, rows, n, expo), nk::note_launch());
+    constexpr int64_t kExpRows = 65535LL * 256;
+    for (int64_t r0 = 0; r0 < rows; r0 += kExpRows) {
+        const int64_t nr = rows - r0 < kExpRows ? rows - r0 : kExpRows;
+        (k_col_exponents<<<dim3(nblk(n, 32), nblk(nr, 256)), 256, 0, st>>>(X + (size_t)r0 * n, nr, n, expo),
+         nk::note_launch());
+    }
     EncodeTiledFn fn = encode_fn();
     if (!fn) return cudaErrorInvalidValue;
     CUtensorMap ma, mb;
@@ -504,18 +523,21 @@ cudaError_t launch_syrk_tc(const double *X, int64_t rows, int64_t n, double scal
     }
     cudaError_t e = nk::allow_max_dynamic_smem((const void *)k_oz_syrk);
     if (e != cudaSuccess) return e;
-    const int chunks = (int)(ldk / kYK);
-    (k_slice_cols_long<<<dim3(nblk(n, 32), (unsigned)chunks), 256, 0, st>>>(
-        X, rows, n, ldk, expo, reinterpret_cast<__nv_bfloat162 *>(sl), sq), nk::note_launch());
-    int z = syrk_splits(rows, n);
-    const int per = (chunks + z - 1) / z;
-    z = (chunks + per - 1) / per;
-    SyrkArgs a{n, chunks, per, expo, z > 1 ? partial : C, scale, eps, z, err};
-    (k_oz_syrk<<<dim3((unsigned)tiles, (unsigned)z), kYThreads, syrk_smem_bytes(), st>>>(ma, mb, a),
-     nk::note_launch());
-    if (z > 1)
-        (k_syrk_finish<<<dim3(nblk(n, 256), (unsigned)n), 256, 0, st>>>(n, z, partial, scale, eps, C),
+    for (int64_t r0 = 0; r0 < rows; r0 += ldk) {
+        const int64_t nr = rows - r0 < ldk ? rows - r0 : ldk;
+        const int chunks = (int)((nr + kYK - 1) / kYK), add = r0 > 0 ? 1 : 0;
+        (k_slice_cols_long<<<dim3(nblk(n, 32), (unsigned)chunks), 256, 0, st>>>(
+            X + (size_t)r0 * n, nr, n, ldk, expo, reinterpret_cast<__nv_bfloat162 *>(sl), sq), nk::note_launch());
+        int z = syrk_splits(nr, n);
+        const int per = (chunks + z - 1) / z;
+        z = (chunks + per - 1) / per;
+        SyrkArgs a{n, chunks, per, expo, z > 1 ? partial : C, scale, eps, z, add, err};
+        (k_oz_syrk<<<dim3((unsigned)tiles, (unsigned)z), kYThreads, syrk_smem_bytes(), st>>>(ma, mb, a),
          nk::note_launch());
+        if (z > 1)  // (at most 76 tiles, so n fits the grid)
+            (k_syrk_finish<<<dim3(nblk(n, 256), (unsigned)n), 256, 0, st>>>(n, z, partial, scale, eps, add, C),
+             nk::note_launch());
+    }
     (k_syrk_exact<<<304, 256, 0, st>>>(X, rows, n, expo, sq, scale, eps, C), nk::note_launch());
     prof_end(slot, st, (double)rows * n * (double)(n + 1),
              (double)tiles * (double)((rows + kYK - 1) / kYK) * 34.0 * 2.0 * kYM * kYN * kYK);

@@ -1,5 +1,5 @@
 """S = scale X^T X + eps I on the tensor cores (launch_syrk_tc), entry by entry against
-sums in extended precision: edges of its tiles and chunks of rows, columns of
+sums in extended precision: edges of its tiles, chunks and segments of rows, columns of
 very different scales, of rare large entries, of zeros and with a NaN.
 
 Tolerance, relative to sqrt(S_ii S_jj): with r = (power of two of the largest entry) /
@@ -124,5 +124,11 @@ def program():
 
 @pytest.mark.parametrize("rows,n", [(1, 1), (64, 31), (65, 33), (1000, 127), (4096, 129), (4096, 300), (3001, 257)])
 def test_entries(program, rows, n):
+    r = subprocess.run([program, str(rows), str(n)], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stdout + r.stderr
+
+
+@pytest.mark.parametrize("rows,n", [((1 << 19) + 1, 3), (1200000, 4)])
+def test_segments_of_rows(program, rows, n):
     r = subprocess.run([program, str(rows), str(n)], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stdout + r.stderr
