@@ -394,20 +394,30 @@ nk_status jacobi_eigen(nk_ctx *ctx, double *K, double *V, int64_t n, void *eig_w
 // The pseudo-inverse solve of the SVD solvers where nothing is cut off: x =
 // S^-1 b, with *done = true.  The cutoff keeps every eigenvalue of the positive
 // semidefinite S exactly when lambda_min > rcond lambda_max, and the Cholesky
-// factorisation of S - tau I proves that: it runs to the end only if
-// lambda_min(S) > tau - (n + 1) u tr S (the backward error of a Cholesky
-// factor is at most (n + 1) u || |L| |L^T| ||_2 <= (n + 1) u ||L||_F^2 = (n +
-// 1) u tr S), and lambda_max <= tr S, so tau = (rcond + 4 (n + 1) u) tr S is
-// enough.  The pseudo-inverse is then the inverse, taken by a second Cholesky,
-// of S itself.  *done = false with S untouched where the proof does not go
+// factorisation of S - tau I proves that: it runs to the end only if lambda_min(S)
+// > tau - ||E||, L L^T = S - tau I + E, and lambda_max <= tr S, so tau = (rcond + 2
+// ||E|| / tr S) tr S is enough.  The pseudo-inverse is then the inverse, taken by a
+// second Cholesky, of S itself.  E, in units of u = 2^-53 and sqrt(s_ii s_jj), which
+// also bounds ||E|| in units of u tr S:
+//   - the trailing updates, per panel of 64 columns with m_i the row's largest entry
+//     in it: slices truncated at 2^-56 of at most 2 m_i, 64 (2^-55 + 2^-55) m_i m_j =
+//     32; slice products s + t >= 9 left out, at most 6.03 255^2 2^-72 4 m_i m_j a
+//     column, 192; the recombination, 2; and sum_p m_i m_j <= sqrt(s_ii s_jj);
+//   - the additions to C, 2 a panel: n / 32;
+//   - diagonal blocks (64 operations of 2^-59, or FP64) and substitution in FP64: 70.
+// *done = false with S untouched where the proof does not go
 // through (a rank-deficient or nearly singular S): the eigensolver decides
 // there.  Order 880 (t-VMC on 20 sites): two factors and a solve take 3 ms, the
 // Jacobi sweeps 331 ms.  scratch: n x n; trace: one double.
+constexpr double kPanelErr = 226.0;  // of a panel's update
+constexpr double kBlockErr = 70.0;
+
 nk_status full_rank_solve(nk_ctx *ctx, double *S, double *scratch, int64_t n, double rcond, const double *b,
                           double *x, void *tcws, double *trace, int *info, cudaStream_t st, bool *done) {
     const nk::CholStreams cs{ctx->side, ctx->aux, ctx->ev[0], ctx->ev[1], ctx->ev[2], ctx->ev[3]};
     *done = false;
-    const double coef = rcond + 4.0 * (double)(n + 1) * 0x1p-53;
+    // (and n u for the trace itself)
+    const double coef = rcond + (2.0 * (kPanelErr + kBlockErr + (double)n / 32.0) + (double)n) * 0x1p-53;
     NK_CU(nk::launch_shifted_copy(n, S, coef, trace, scratch, st), "full rank");
     NK_CU(nk::launch_cholesky_tc(scratch, n, info, info + 1, tcws, st, &cs, true), "full rank");
     NK_CU(cudaMemcpyAsync(ctx->host_flags + 2, info, 2 * sizeof(int), cudaMemcpyDeviceToHost, st), "full rank");
