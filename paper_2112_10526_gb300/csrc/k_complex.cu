@@ -303,6 +303,12 @@ __global__ void __launch_bounds__(128) k_crbm_sweep(CSweepArgs A) {
 // over the connected configurations, the tables are unit-major as W is, so the
 // lanes' loads coalesce and no reduction is needed per ratio.  20 sites, M =
 // 20, 4096 samples: 1.7 ms with the logarithms, 0.16 now.
+// The exponentials stay in range, and above the subnormal numbers, for |Re 2 W| <=
+// 170 and |Re theta| <= 300 (|d| <= 340, the running product within e^{+-166}).
+// Samples beyond, and those whose sum is not finite for another reason, take the
+// differences of ln cosh.
+constexpr double kMaxRe2W = 170.0, kMaxReTheta = 300.0;
+
 struct CElocArgs {
     int N, M, E, E2, kind, marshall;
     double J, J2, h;
@@ -322,7 +328,8 @@ __global__ void k_crbm_exp_tables(int64_t n, const double2 *__restrict__ W, doub
     if (i >= n) return;
     double sn, cs;
     sincos(2.0 * W[i].y, &sn, &cs);
-    const double a = exp(2.0 * W[i].x), b = exp(-2.0 * W[i].x);
+    double a = exp(2.0 * W[i].x), b = exp(-2.0 * W[i].x);
+    if (!(fabs(2.0 * W[i].x) <= kMaxRe2W)) a = b = __longlong_as_double(0x7FF8000000000000LL);
     ep[i] = make_double2(a * cs, a * sn);
     em[i] = make_double2(b * cs, -b * sn);
 }
@@ -340,6 +347,29 @@ __device__ __forceinline__ void logistic_pair(double2 z, double2 &p, double2 &q)
     q = neg ? a : b;
 }
 
+// The off-diagonal part by logarithms, one connected configuration after the other,
+// the lanes over the hidden units; th: room for theta.
+__device__ __noinline__ double2 log_offdiag(const CElocArgs &A, const CView &v, const int8_t *sv, double2 *th,
+                                            int lane) {
+    const int N = A.N, M = A.M, E1 = A.E - A.E2;
+    __syncwarp();
+    hidden(v, N, M, sv, th, lane);
+    __syncwarp();
+    double2 off = make_double2(0.0, 0.0);
+    if (A.kind == NK_TFIM) {
+        for (int i = 0; i < N; ++i)
+            off = cadd(off, cscale(cexp(clog_ratio(v, N, M, sv, th, &i, 1, lane)), -A.h));
+        return off;
+    }
+    for (int e = 0; e < A.E; ++e) {
+        const int pair[2] = {A.edges[2 * e], A.edges[2 * e + 1]};
+        if ((unsigned)pair[0] >= (unsigned)N || (unsigned)pair[1] >= (unsigned)N || sv[pair[0]] == sv[pair[1]]) continue;
+        const double el = e < E1 ? (A.marshall ? -2.0 * A.J : 2.0 * A.J) : 2.0 * A.J2;
+        off = cadd(off, cscale(cexp(clog_ratio(v, N, M, sv, th, pair, 2, lane)), el));
+    }
+    return off;
+}
+
 __global__ void __launch_bounds__(128) k_crbm_eloc(CElocArgs A) {
     extern __shared__ __align__(16) unsigned char sm[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -355,6 +385,8 @@ __global__ void __launch_bounds__(128) k_crbm_eloc(CElocArgs A) {
     const CView v = cview(A.p, N, M);
     hidden(v, N, M, sv, pq, lane);  // theta in pq[0 .. M - 1]
     __syncwarp();
+    bool beyond = false;  // (also for a NaN)
+    for (int j = lane; j < M; j += 32) beyond |= !(fabs(pq[j].x) <= kMaxReTheta);
     // (p, q) of the units from the last to the first block of 32: a block's
     // theta is read by its lanes before pairs are written over it
     for (int j0 = (M - 1) / 32 * 32; j0 >= 0; j0 -= 32) {
@@ -427,7 +459,13 @@ __global__ void __launch_bounds__(128) k_crbm_eloc(CElocArgs A) {
                 ex += eb;
             }
         }
-        // e^{-2 s_i (a_i - a_k)} 2^ex
+        // e^{-2 s_i (a_i - a_k)} 2^ex, the product brought to [1, 2) first
+        const int eb = max((__double2hiint(r.x) >> 20) & 0x7FF, (__double2hiint(r.y) >> 20) & 0x7FF) - 1023;
+        if (eb < 1024 && eb > -1023) {
+            r.x = ldexp(r.x, -eb);
+            r.y = ldexp(r.y, -eb);
+            ex += eb;
+        }
         double2 av = v.a[i];
         if (kk >= 0) av = csub(av, v.a[kk]);
         const double sg = up ? -2.0 : 2.0;
@@ -435,8 +473,10 @@ __global__ void __launch_bounds__(128) k_crbm_eloc(CElocArgs A) {
         z.x += (double)ex * 0.69314718055994530942;
         off = cadd(off, cscale(cmul(r, cexp(z)), el));
     }
+    beyond |= !isfinite(off.x) || !isfinite(off.y);
     off = warp_csum(off);
     diag = warp_sum(diag);
+    if (__any_sync(0xffffffffu, beyond)) off = log_offdiag(A, v, sv, pq, lane);
     if (lane == 0) reinterpret_cast<double2 *>(A.eloc)[k] = make_double2(diag + off.x, off.y);
 }
 
