@@ -313,7 +313,7 @@ struct CElocArgs {
     int N, M, E, E2, kind, marshall;
     double J, J2, h;
     const double *p;
-    const double2 *ep, *em;  // e^{2 W}, e^{-2 W}, [M][N]
+    const double2 *ep, *em;  // e^{2 W}, e^{-2 W}, [M][N]; null: by logarithms
     const int32_t *edges;
     const int8_t *s;
     int64_t Ns;
@@ -425,6 +425,10 @@ __global__ void __launch_bounds__(128) k_crbm_eloc(CElocArgs A) {
         __syncwarp();
     }
     double2 off = make_double2(0.0, 0.0);
+    if (!A.ep) {
+        beyond = true;
+        n = 0;
+    }
     for (int x = lane; x < n; x += 32) {
         int i = x, kk = -1;
         double el = -A.h;
@@ -667,9 +671,10 @@ cudaError_t launch_crbm_eloc(int N, int M, const double *p, const nk_ham *ham, c
                              double *eloc, void *ws, cudaStream_t st) {
     if (Ns <= 0) return cudaSuccess;
     const int64_t nw = (int64_t)N * M;
-    double2 *ep = static_cast<double2 *>(ws), *em = ep + nw;
-    (k_crbm_exp_tables<<<nblk(nw, 256), 256, 0, st>>>(nw, reinterpret_cast<const double2 *>(p) + N + M, ep, em),
-     nk::note_launch());
+    double2 *ep = static_cast<double2 *>(ws), *em = ep ? ep + nw : nullptr;
+    if (ep)
+        (k_crbm_exp_tables<<<nblk(nw, 256), 256, 0, st>>>(nw, reinterpret_cast<const double2 *>(p) + N + M, ep, em),
+         nk::note_launch());
     const bool pairs = ham->kind != NK_TFIM;
     const int pq = M * 2 * (int)sizeof(double2), sb = (N + 15) / 16 * 16;
     const size_t lb = ((size_t)ham->n_edges * 4 + 15) / 16 * 16;

@@ -838,6 +838,21 @@ nk_status nk_ctx_create(int32_t device, nk_ctx **out) {
     for (int i = 0; i < 4 && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&c->ev[i], cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaMalloc(&c->tc_err, 256);
     if (e == cudaSuccess) e = cudaMemset(c->tc_err, 0, 256);
+    if (e == cudaSuccess) {
+        // keeps up to 256 MiB between calls (the driver would give it back at every
+        // synchronisation); without it the calls that draw on it still run
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = device;
+        uint64_t keep = 256ULL << 20;
+        if (cudaMemPoolCreate(&c->pool, &props) != cudaSuccess ||
+            cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+            cudaGetLastError();
+            if (c->pool) cudaMemPoolDestroy(c->pool);
+            c->pool = nullptr;
+        }
+    }
     if (e != cudaSuccess) {
         if (c->host_flags) cudaFreeHost(c->host_flags);
         if (c->host_vals) cudaFreeHost(c->host_vals);
@@ -864,6 +879,7 @@ nk_status nk_ctx_destroy(nk_ctx *ctx) {
     for (int i = 0; i < 4; ++i)
         if (ctx->ev[i]) cudaEventDestroy(ctx->ev[i]);
     if (ctx->tc_err) cudaFree(ctx->tc_err);
+    if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
     delete ctx;
     return NK_OK;
 }
@@ -1656,13 +1672,21 @@ nk_status nk_crbm_local_energy(nk_ctx *ctx, const nk_crbm *rbm, const nk_ham *ha
     if (Ns == 0) return NK_OK;
     NK_DEV(s, "s");
     if ((st0 = check_complex_out(eloc_out, "eloc_out")) != NK_OK) return st0;
-    return with_workspace(ctx, [&](Carver &c, bool run) -> nk_status {
-        void *exps = c.take<char>(nk::crbm_eloc_ws_bytes(rbm->N, rbm->M));
-        if (!run) return NK_OK;
-        NK_CU(nk::launch_crbm_eloc(rbm->N, rbm->M, rbm->params, ham, s, Ns, eloc_out, exps, (cudaStream_t)stream),
-              "local energy");
-        return NK_OK;
-    });
+    if (g_plan_only) return NK_OK;
+    // The tables come from the context's pool in stream order, not from its workspace:
+    // the call synchronises nothing, can be captured and may run beside another call of
+    // the context.  Where there is no room for them it does without.
+    cudaStream_t st = (cudaStream_t)stream;
+    void *exps = nullptr;
+    if (!ctx->pool ||
+        cudaMallocFromPoolAsync(&exps, nk::crbm_eloc_ws_bytes(rbm->N, rbm->M), ctx->pool, st) != cudaSuccess) {
+        cudaGetLastError();
+        exps = nullptr;
+    }
+    const cudaError_t e = nk::launch_crbm_eloc(rbm->N, rbm->M, rbm->params, ham, s, Ns, eloc_out, exps, st);
+    if (exps) NK_CU(cudaFreeAsync(exps, st), "local energy");
+    NK_CU(e, "local energy");
+    return NK_OK;
 }
 
 nk_status nk_crbm_jacobian(nk_ctx *ctx, const nk_crbm *rbm, const int8_t *s, int64_t Ns, double *O_out,

@@ -23,6 +23,7 @@ struct nk_ctx {
     int *tc_err;        // device, 256 bytes: [0] sticky code of the first tensor-core
                         // time-out; [16] flag of the symmetric RBM's permutation check
     size_t plan_bytes;  // workspace counted by plan-only calls
+    cudaMemPool_t pool; // scratch of the calls that use no workspace, or null
 };
 
 namespace nk {
@@ -380,6 +381,7 @@ cudaError_t launch_crbm_sweep(int N, int M, const double *p, int rule, int E, co
                               int64_t sweep0, int n_discard, int n_samples, uint64_t seed, uint32_t stream_id,
                               int8_t *samples, unsigned long long *n_accepted, cudaStream_t st);
 size_t crbm_eloc_ws_bytes(int N, int M);  // the tables e^{+-2 W}
+// ws null: by logarithms, ten times slower.
 cudaError_t launch_crbm_eloc(int N, int M, const double *p, const nk_ham *ham, const int8_t *s, int64_t Ns,
                              double *eloc, void *ws, cudaStream_t st);
 cudaError_t launch_crbm_jacobian(int N, int M, const double *p, const int8_t *s, int64_t Ns, double *O,
