@@ -624,6 +624,13 @@ nk_status run_sweeps(nk_ctx *ctx, const nk::Tables<R> &t, const nk::SweepArgs &a
     return NK_OK;
 }
 
+// Samples whose theta nk_rbm_logpsi and nk_local_energy hold at a time: NK_F64, which
+// needs it for speed alone, keeps to 256 MiB (in 128-row tiles).
+int64_t theta_slab(int M, int64_t B, int precision) {
+    const int64_t rows = ((int64_t)1 << 25) / M / 128 * 128;
+    return precision == NK_F64 && rows < B ? rows : B;
+}
+
 // Where tanh(theta) feeds NK_MIXED conjugate gradients it is CUDA's tanh()
 // instead of the integer one (which is closer to the exact value and eight
 // times as fast).  Those iterations work on 33-bit products up to a tolerance
@@ -901,14 +908,19 @@ nk_status nk_rbm_logpsi(nk_ctx *ctx, const nk_rbm *rbm, int32_t precision, const
         nk::Tables<double> t{};
         carve_tables(c, t, rbm, 0, nullptr, false, false, false, false);
         const bool tcp = precision == NK_MIXED || nk::f64_on_tensor(N, M, B);
-        double *theta = tcp ? c.take<double>((size_t)B * M) : nullptr;
-        void *tcm = tcp ? c.take<char>(nk::tc_theta_ws_bytes(N, M, B)) : nullptr;
+        const int64_t slab = theta_slab(M, B, precision);
+        double *theta = tcp ? c.take<double>((size_t)slab * M) : nullptr;
+        void *tcm = tcp ? c.take<char>(nk::tc_theta_ws_bytes(N, M, slab)) : nullptr;
         if (!run) return NK_OK;
-        if (tcp) {
-            NK_CU(nk::launch_theta_tc(N, M, t.b, t.W, s, B, theta, ctx->tc_err, tcm, st, 0, precision == NK_F64), "theta");
-            NK_CU(nk::launch_logpsi_theta(N, M, t.a, theta, s, B, logpsi_out, st), "logpsi");
-            return NK_OK;
+        for (int64_t k = 0; tcp && k < B; k += slab) {
+            const int64_t n = B - k < slab ? B - k : slab;
+            const int8_t *sk = s + (size_t)k * N;
+            NK_CU(nk::launch_theta_tc(N, M, t.b, t.W, sk, n, theta, ctx->tc_err, tcm, st, 0, precision == NK_F64,
+                                      k > 0 && n == slab),
+                  "theta");
+            NK_CU(nk::launch_logpsi_theta(N, M, t.a, theta, sk, n, logpsi_out + k, st), "logpsi");
         }
+        if (tcp) return NK_OK;
         NK_CU(nk::launch_tables(t, false, false, st), "tables");
         NK_CU(nk::launch_logpsi(N, M, t.a, t.b, t.Wt, s, B, logpsi_out, st), "logpsi");
         return NK_OK;
@@ -1017,18 +1029,25 @@ nk_status nk_local_energy(nk_ctx *ctx, const nk_rbm *rbm, int32_t precision, con
         // (the theta of the tensor cores and of the kernel are the same to the
         // last bit in NK_F64)
         const bool tcp = precision == NK_MIXED || nk::f64_on_tensor(rbm->N, rbm->M, Ns);
-        double *theta = tcp ? c.take<double>((size_t)Ns * rbm->M) : nullptr;
-        void *tcm = tcp ? c.take<char>(nk::tc_theta_ws_bytes(rbm->N, rbm->M, Ns)) : nullptr;
+        const int64_t slab = tcp ? theta_slab(rbm->M, Ns, precision) : Ns;
+        double *theta = tcp ? c.take<double>((size_t)slab * rbm->M) : nullptr;
+        void *tcm = tcp ? c.take<char>(nk::tc_theta_ws_bytes(rbm->N, rbm->M, slab)) : nullptr;
         if (!run) return NK_OK;
         NK_CU(nk::launch_tables(t, site, edge, st), "tables");
-        nk::ElocArgs am = a;
-        if (tcp) {
-            NK_CU(nk::launch_theta_tc(rbm->N, rbm->M, t.b, t.W, s, Ns, theta, ctx->tc_err, tcm, st, 0,
-                                      precision == NK_F64),
-                  "theta");
-            am.theta_in = theta;
+        for (int64_t k = 0; k < Ns; k += slab) {
+            nk::ElocArgs am = a;
+            am.Ns = Ns - k < slab ? Ns - k : slab;
+            am.s = s + (size_t)k * rbm->N;
+            am.eloc = eloc_out + k;
+            am.t_out = t_out ? t_out + (size_t)k * rbm->M : nullptr;
+            if (tcp) {
+                NK_CU(nk::launch_theta_tc(rbm->N, rbm->M, t.b, t.W, am.s, am.Ns, theta, ctx->tc_err, tcm, st, 0,
+                                          precision == NK_F64, k > 0 && am.Ns == slab),
+                      "theta");
+                am.theta_in = theta;
+            }
+            NK_CU(nk::launch_eloc(t, am, st), "local energy");
         }
-        NK_CU(nk::launch_eloc(t, am, st), "local energy");
         return NK_OK;
     };
     if (precision == NK_F64)
