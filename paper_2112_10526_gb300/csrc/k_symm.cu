@@ -66,7 +66,8 @@ __global__ void k_symm_expand(int N, int alpha, int G, const int32_t *__restrict
 }
 
 // One row of the symmetric Jacobian in FP64, thread (f, j) summing its G terms
-// in group order: for configurations that are not +-1.
+// in group order: for configurations that are not +-1, more than 512 group elements
+// and activations near the lower end of the FP64 range.
 __device__ __noinline__ void symm_row_f64(int N, int alpha, int G, const int32_t *__restrict__ perms, const int8_t *__restrict__ sv,
                              const double *__restrict__ t, double *__restrict__ row) {
     if (threadIdx.x < 32) {
@@ -100,14 +101,15 @@ __device__ __noinline__ void symm_row_f64(int N, int alpha, int G, const int32_t
 // their largest, and thread (f, j) adds those whose spin is up, two predicated
 // integer adds a term where FP64 has 2 lanes a cycle on an SM; twice that less
 // the sum of all is the result (exact modulo 2^64, and |result| <= 2^62).  Each
-// term is rounded once, to G 2^-62 of the largest (relative error below 2^-52
-// up to G = 1024), and the sum not at all, where FP64 rounded every partial
-// sum.  K samples share the loads of the permutation, coalesced over j, and
-// one byte a site holds their spins; the values of a (f, g) are broadcast.
+// term is rounded once, to at most 2^-54 of the largest, and the sum not at all,
+// where FP64 rounds every partial sum.  From 513 elements on a term would keep
+// fewer than 53 bits of the largest: those sums stay in FP64 (f64).  K samples
+// share the loads of the permutation, coalesced over j, and one byte a site holds
+// their spins; the values of a (f, g) are broadcast.
 // 10 x 10 lattice, 4 features, 100 translations, 4096 samples: 1290 us as one
 // block per sample with FP64 sums, 129 us now.
 template <int K>
-__global__ void __launch_bounds__(512) k_symm_jacobian(int N, int alpha, int G, int lg,
+__global__ void __launch_bounds__(512) k_symm_jacobian(int N, int alpha, int G, int lg, bool f64,
                                                        const int32_t *__restrict__ perms,
                                                        const int8_t *__restrict__ s, const double *__restrict__ T,
                                                        int64_t Ns, double *__restrict__ O) {
@@ -133,12 +135,16 @@ __global__ void __launch_bounds__(512) k_symm_jacobian(int N, int alpha, int G, 
         }
         up[j] = (uint8_t)b;
     }
-    if (__syncthreads_or(odd)) {
+    auto rows_f64 = [&] {
         for (int q = 0; q < nq; ++q)
             symm_row_f64(N, alpha, G, perms, s + (size_t)(k0 + q) * N, T + (size_t)(k0 + q) * M,
                          O + (size_t)(k0 + q) * Np);
+    };
+    if (__syncthreads_or(odd || f64)) {
+        rows_f64();
         return;
     }
+    bool tiny = false;
     for (int r = warp; r < alpha * K; r += warps) {
         const int f = r / K, q = r % K;
         if (q >= nq) {
@@ -147,8 +153,13 @@ __global__ void __launch_bounds__(512) k_symm_jacobian(int N, int alpha, int G, 
         }
         const double *tf = T + (size_t)(k0 + q) * M + (size_t)f * G;
         unsigned e = 0;
-        for (int g = lane; g < G; g += 32) e = max(e, ((unsigned)__double2hiint(tf[g]) >> 20) & 0x7ffu);
+        bool some = false;
+        for (int g = lane; g < G; g += 32) {
+            e = max(e, ((unsigned)__double2hiint(tf[g]) >> 20) & 0x7ffu);
+            some |= tf[g] != 0.0;
+        }
         e = __reduce_max_sync(0xffffffffu, e);  // |t| < 2^(e - 1022)
+        tiny |= some && e < 84;                 // below 2^-938: the scale has no such exponent
         const int sh = min(62 - lg + 1022 - (int)e, 1000);
         const double scale = __hiloint2double((sh + 1023) << 20, 0);
         long long sum = 0;
@@ -174,7 +185,10 @@ __global__ void __launch_bounds__(512) k_symm_jacobian(int N, int alpha, int G, 
         n = __reduce_add_sync(0xffffffffu, n);
         if (lane == 0) O[(size_t)(k0 + q) * Np] = (double)(2 * n - N);
     }
-    __syncthreads();
+    if (__syncthreads_or(tiny)) {
+        rows_f64();
+        return;
+    }
     for (int64_t x = threadIdx.x; x < (int64_t)alpha * N; x += blockDim.x) {
         const int f = (int)(x / N), j = (int)(x % N);
         const long long *tf = ti + (size_t)f * G * K;
@@ -215,7 +229,7 @@ cudaError_t symm_jacobian_launch(int N, int alpha, int G, const int32_t *perms, 
     for (int64_t k0 = 0; k0 < Ns; k0 += 65535 * K) {
         const int64_t kb = Ns - k0 < 65535 * K ? Ns - k0 : 65535 * K;
         (k_symm_jacobian<K><<<(unsigned)((kb + K - 1) / K), threads, smem, st>>>(
-             N, alpha, G, lg, perms, s + (size_t)k0 * N, T + (size_t)k0 * alpha * G, kb, O + (size_t)k0 * Np),
+             N, alpha, G, lg, G > 512, perms, s + (size_t)k0 * N, T + (size_t)k0 * alpha * G, kb, O + (size_t)k0 * Np),
          nk::note_launch());
     }
     return cudaGetLastError();
@@ -253,7 +267,9 @@ cudaError_t launch_symm_jacobian(int N, int alpha, int G, const int32_t *perms, 
     if (symm_jacobian_smem(N, alpha, G) > 227 * 1024) return cudaErrorInvalidValue;
     // Four samples a block, or two, while three blocks fit an SM and there are two
     // blocks for each SM; one sample always fits (alpha G <= 8192: 201 KB).
-    const auto good = [&](int K) { return symm_staged_smem(N, alpha, G, K) <= 75 * 1024 && Ns >= 304 * K; };
+    const auto good = [&](int K) {
+        return G <= 512 && symm_staged_smem(N, alpha, G, K) <= 75 * 1024 && Ns >= 304 * K;
+    };
     if (good(4)) return symm_jacobian_launch<4>(N, alpha, G, perms, s, T, Ns, O, st);
     if (good(2)) return symm_jacobian_launch<2>(N, alpha, G, perms, s, T, Ns, O, st);
     return symm_jacobian_launch<1>(N, alpha, G, perms, s, T, Ns, O, st);
