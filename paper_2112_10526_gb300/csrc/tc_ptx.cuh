@@ -270,14 +270,14 @@ __host__ __device__ __forceinline__ long long sgemm_window10(const int (&d)[7]) 
     return w;
 }
 
-// floor(V / 2^drop) for the same V when a product sums K terms: |V| < K 2^56,
-// so drop = max(0, ceil(log2 K) - 6) bits keep the window below 2^62 and leave
-// out less than 2^(drop - 56) of the operand row's scale (window10 drops 2^10
-// units whatever K is: 25 times the rounding of FP64 at K = 4096).
+// V / 2^drop to nearest for the same V when a product sums K terms: |V| < K 2^56,
+// so drop = max(0, ceil(log2 K) - 6) bits keep the window below 2^62 and round at
+// 2^(drop - 57) of the operand row's scale (window10 drops 2^10 units whatever K is:
+// 25 times the rounding of FP64 at K = 4096).
 __host__ __device__ __forceinline__ long long sgemm_window(const int (&d)[7], int drop) {
     const long long hi = (long long)d[0] * 65536 + (long long)d[1] * 256 + d[2];
     const long long lo = (long long)d[3] * 16777216 + (long long)d[4] * 65536 + (long long)d[5] * 256 + d[6];
-    return (long long)((unsigned long long)hi << (32 - drop)) + (lo >> drop);
+    return (long long)((unsigned long long)hi << (32 - drop)) + ((lo + ((1LL << drop) >> 1)) >> drop);
 }
 
 // ceil(log2 K) - 6, at least 0 (K <= 65792: at most 11)
