@@ -196,7 +196,10 @@ __global__ void __launch_bounds__(kSgThreads, 2)
             const uint32_t lane_base = tmem + ((uint32_t)(warp * 32) << 16);
             const bool row_ok = row < a.rows;
             const double *trow = (a.mode == 3 && row_ok) ? a.T + (size_t)row * a.Mt : nullptr;
-            double racc = 0.0;
+            // the row product: one chain of additions, or four in NK_F64, whose sum errs
+            // by half as much
+            const bool wide = a.drop >= 0;
+            double racc[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll 1
             for (int c8 = 0; c8 < kBN; c8 += 8) {
                 // column exponents of this chunk (lane & 7) and, for the fused
@@ -229,13 +232,16 @@ __global__ void __launch_bounds__(kSgThreads, 2)
                         const int64_t k1 = (int64_t)kc1 * kBK;
                         v = raw_product(a.raw, row, n0 + c8 + j, (int64_t)kc0 * kBK, k1 < a.K ? k1 : a.K);
                     }
-                    if (a.mode == 3)
-                        racc = fma(v, tv[j], racc);
-                    else
+                    if (a.mode == 3) {
+                        if (wide)
+                            racc[j & 3] = fma(v, tv[j], racc[j & 3]);
+                        else
+                            racc[0] = fma(v, tv[j], racc[0]);
+                    } else
                         tile[rloc * kSgOutLd + c8 + j] = v;
                 }
             }
-            if (a.mode == 3 && row_ok) a.C[(size_t)row * a.ldc + blockIdx.x] = racc;
+            if (a.mode == 3 && row_ok) a.C[(size_t)row * a.ldc + blockIdx.x] = (racc[0] + racc[1]) + (racc[2] + racc[3]);
         }
     }
     __syncthreads();
