@@ -391,8 +391,8 @@ def e2e_steps(st, K, dev):
 # sha256 of the kernel's own source section so that a changed kernel reports
 # no stale figure.
 # k_ozaki_gemm: per 128 x 32 output tile with 7 slices (the 8064 x 8064
-# lower update of the 10 x 10 workload: 472.33 MB over 8064 tiles).
-OZAKI_TRAFFIC = {"bytes_per_tile": 58573.3, "source_sha256_prefix": "06f197620660557f"}
+# lower update of the 10 x 10 workload: 473.07 MB over 8064 tiles).
+OZAKI_TRAFFIC = {"bytes_per_tile": 58665.0, "source_sha256_prefix": "9086c14dd41721e6"}
 OZAKI_TILE_FLOPS = 28 * 4 * 2.0 * 128 * 32 * 16  # executed BF16 flops per tile (7 slices)
 # k_tc4 (the CG's J v and J^T g products): bytes per launch captured on the
 # 24 x 24 workload at 1024 chains (Ns = 8192): J v 331.97 MB read + 3.85 MB

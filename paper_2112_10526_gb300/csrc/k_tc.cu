@@ -54,11 +54,14 @@ constexpr int kABytes = kTileM * kTileK * 2;  // one slice of the A tile
 // and the row exponent e_r (max |a_rk| < 2^e_r).  The slices are the bytes,
 // from the top, of the fixed-point magnitude floor(|a| 2^(8S - e_r)), with the
 // sign of a: exactly the digits of repeated multiply-by-256-and-truncate,
-// taken from the FP64 bit pattern with integer shifts only.
+// taken from the FP64 bit pattern with integer shifts only.  round (NK_F64): the
+// magnitude to nearest instead (only entries below 2^(e_r - 3) have bits to lose, so
+// none reaches 2^e_r).
 // The warp's row r, with lane l holding columns l (x0) and l + 32 (x1), as S
 // slices out[q][r][0..63] (plane stride `rows` rows) and the row exponent.
 __device__ __forceinline__ void slice_row_warp(double x0, double x1, int lane, int64_t rows, int64_t r, int S,
-                                               __nv_bfloat16 *__restrict__ out, int *__restrict__ expo) {
+                                               bool round, __nv_bfloat16 *__restrict__ out,
+                                               int *__restrict__ expo) {
     int b0, b1;
     unsigned long long m0, m1;
     bool n0, n1;
@@ -77,7 +80,7 @@ __device__ __forceinline__ void slice_row_warp(double x0, double x1, int lane, i
         const int sh = biased - 1075 + 8 * S - e;
         if (sh >= 0) return mant << sh;  // sh <= 3 here
         if (sh <= -64) return 0ULL;
-        return mant >> (-sh);
+        return (mant >> (-sh)) + (round ? (mant >> (-sh - 1)) & 1ULL : 0ULL);
     };
     const unsigned long long y0 = fixp(b0, m0), y1 = fixp(b1, m1);
     for (int q = 0; q < S; ++q) {
@@ -90,14 +93,14 @@ __device__ __forceinline__ void slice_row_warp(double x0, double x1, int lane, i
     if (lane == 0) expo[r] = e;
 }
 
-__global__ void k_slice_rows(const double *__restrict__ A, int64_t lda, int64_t rows, int kcols, int S,
+__global__ void k_slice_rows(const double *__restrict__ A, int64_t lda, int64_t rows, int kcols, int S, bool round,
                              __nv_bfloat16 *__restrict__ out, int *__restrict__ expo) {
     const int lane = threadIdx.x & 31;
     const int64_t r = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (r >= rows) return;
     const double x0 = lane < kcols ? A[(size_t)r * lda + lane] : 0.0;
     const double x1 = lane + 32 < kcols ? A[(size_t)r * lda + lane + 32] : 0.0;
-    slice_row_warp(x0, x1, lane, rows, r, S, out, expo);
+    slice_row_warp(x0, x1, lane, rows, r, S, round, out, expo);
 }
 
 // ------------------------------------------------------------- the GEMM ---
@@ -125,6 +128,9 @@ __global__ void k_slice_rows(const double *__restrict__ A, int64_t lda, int64_t 
 // Cholesky look-ahead) get SMs as strips retire.  mbarriers hand buffers
 // between the roles; every wait is bounded by the global timer and gives up
 // when another role of the CTA has aborted.
+// kWide (NK_F64, on rounded slices): the products of slices s + t = 9 as well, and the
+// window of the levels to nearest: 2^-56 of the rows' largest entries an operand and
+// 2^-57 a product, where the 28 slice products leave out up to 2^-51.
 
 struct OzArgs {
     int64_t rows, cols;   // output rows (A rows) and columns (B rows)
@@ -168,8 +174,9 @@ __host__ __device__ inline int64_t oz_row_strips(int64_t n_nb, bool lower, int64
 // MMA of that width adds A slice s times all of them to the contiguous levels
 // s+1 .. S+1.  S MMAs per K-step (instead of S(S+1)/2 of width 32) read each
 // A slice once; the first one of a tile (s = 1, K-step 0) initialises every
-// level.  SS > 0 fixes S at compile time.
-template <int SS>
+// level.  SS > 0 fixes S at compile time.  kWide adds level S + 2, which A slices 2 ..
+// S reach with one B slice more; slice 2 initialises it by itself (B slice S).
+template <int SS, bool kWide>
 __device__ __forceinline__ void issue_tile(uint32_t dbase, uint64_t da, uint64_t db,
                                            const uint32_t (&idesc)[kMaxSlices], int S_rt) {
     const int S = SS > 0 ? SS : S_rt;
@@ -181,13 +188,19 @@ __device__ __forceinline__ void issue_tile(uint32_t dbase, uint64_t da, uint64_t
             if (sa > S) continue;
             const uint32_t acc = (kk > 0 || sa > 1) ? 1u : 0u;
             // A slice sa starts (sa - 1) kABytes after slice 1 (descriptor address field in 16-byte units)
-            umma_bf16(dbase + (uint32_t)((sa - 1) * kPN), da + (uint64_t)((sa - 1) * (kABytes >> 4) + kk * 2),
-                      db + (uint64_t)(kk * 2), idesc[sa - 1], acc);
+            const uint64_t das = da + (uint64_t)((sa - 1) * (kABytes >> 4) + kk * 2), dbk = db + (uint64_t)(kk * 2);
+            if (kWide && sa == 2 && kk == 0) {
+                umma_bf16(dbase + (uint32_t)kPN, das, dbk, idesc_bf16(kTileM, kPN * (kS - 1)), 1u);
+                umma_bf16(dbase + (uint32_t)(kS * kPN), das, dbk + (uint64_t)((kS - 1) * (kPBBytes >> 4)),
+                          idesc_bf16(kTileM, kPN), 0u);
+                continue;
+            }
+            umma_bf16(dbase + (uint32_t)((sa - 1) * kPN), das, dbk, idesc[sa - 1], acc);
         }
     }
 }
 
-template <int SS>
+template <int SS, bool kWide>
 __global__ void __launch_bounds__(kPThreads, 1)
     k_ozaki_gemm(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, OzArgs a) {
     extern __shared__ unsigned char smem_raw[];
@@ -202,6 +215,8 @@ __global__ void __launch_bounds__(kPThreads, 1)
     uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + 10);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tslot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    static_assert(!kWide || SS == kMaxSlices, "level 9 of 7 slices");
+    constexpr int kLevels = kMaxSlices + (kWide ? 1 : 0);
     const int S = SS > 0 ? SS : a.S;
     // strip -> tile row mb, first tile column nb0, tile count: every warp scans
     // the strips per tile row, 32 rows per round (inclusive prefix by
@@ -284,9 +299,10 @@ __global__ void __launch_bounds__(kPThreads, 1)
     } else if (warp == 1 && lane == 0) {
         // ------------------------------------------------------- MMA issuer
         int issued = 0;
-        uint32_t idesc[kMaxSlices];  // A slice s + 1 meets B slices 1 .. S - s: N = 32 (S - s)
+        uint32_t idesc[kMaxSlices];  // A slice s + 1 meets B slices 1 .. S - s: N = 32 (S - s); kWide: one more
 #pragma unroll
-        for (int s = 0; s < kMaxSlices; ++s) idesc[s] = idesc_bf16(kTileM, kPN * (S - s > 0 ? S - s : 1));
+        for (int s = 0; s < kMaxSlices; ++s)
+            idesc[s] = idesc_bf16(kTileM, kPN * (kWide && s > 0 ? S + 1 - s : (S - s > 0 ? S - s : 1)));
         const uint64_t da = sw128_desc(sA), db0 = sw128_desc(sB),
                        db1 = sw128_desc(sB + (size_t)kMaxSlices * kPBBytes);
         if (!mbar_wait_or_abort(a_full, 0, abort_flag)) fail(13);
@@ -303,9 +319,9 @@ __global__ void __launch_bounds__(kPThreads, 1)
             }
             tc_fence_after();
             if (b)
-                issue_tile<SS>(tmem + kPAccCols, da, db1, idesc, S);
+                issue_tile<SS, kWide>(tmem + kPAccCols, da, db1, idesc, S);
             else
-                issue_tile<SS>(tmem, da, db0, idesc, S);
+                issue_tile<SS, kWide>(tmem, da, db0, idesc, S);
             umma_commit(&acc_full[b]);
             umma_commit(&b_empty[b]);
             ++issued;
@@ -393,10 +409,10 @@ __global__ void __launch_bounds__(kPThreads, 1)
             tc_fence_after();
 #pragma unroll 1
             for (int c4 = 0; c4 < kPColsPerWarp; c4 += 2) {
-                uint32_t r[kMaxSlices][2];
+                uint32_t r[kLevels][2];
 #pragma unroll
-                for (int gi = 0; gi < kMaxSlices; ++gi)
-                    if (gi < S)
+                for (int gi = 0; gi < kLevels; ++gi)
+                    if (kWide || gi < S)
                         tmem_ld2(tmem + (uint32_t)b * kPAccCols + lane_base + (uint32_t)(gi * kPN + c0 + c4), r[gi]);
                 tmem_wait_ld();
                 double v[2];
@@ -406,6 +422,8 @@ __global__ void __launch_bounds__(kPThreads, 1)
 #pragma unroll
                     for (int gi = 0; gi < kMaxSlices; ++gi)
                         d[gi] = gi < S ? __float2int_rn(__uint_as_float(r[gi][j])) : 0;
+                    if constexpr (kWide)  // D_9 2^-8, and the window's last bit to nearest
+                        d[kMaxSlices - 1] += ((__float2int_rn(__uint_as_float(r[kMaxSlices][j])) + 128) >> 8) + 128;
                     // V 2^sc with V = sum_g D_g 2^(8 (8 - g)); C - R as C + (-R)
                     const int sc = ei + __shfl_sync(0xffffffffu, fj_lane, c4 + j) - 56;
                     const double x = window_to_double_seldom(ozaki_window8(d), sc);
@@ -751,7 +769,7 @@ __global__ void __launch_bounds__(32 * kTrtriWarps) k_trtri64(const double *__re
         }
         x0 = acc0;
         x1 = acc1;
-        slice_row_warp(x0, x1, lane, kb, i, S, out, expo);
+        slice_row_warp(x0, x1, lane, kb, i, S, false, out, expo);
     }
     Linv[(size_t)i * kNB + lane] = x0;
     Linv[(size_t)i * kNB + lane + 32] = x1;
@@ -773,7 +791,8 @@ __global__ void __launch_bounds__(32 * kTrtriWarps) k_trtri64(const double *__re
 constexpr int64_t kTrsmRows = 3072;
 
 __global__ void __launch_bounds__(256) k_trsm_rows(double *__restrict__ A, int64_t n, int64_t k, int64_t rows, int S,
-                                                   __nv_bfloat16 *__restrict__ out, int *__restrict__ expo) {
+                                                   bool round, __nv_bfloat16 *__restrict__ out,
+                                                   int *__restrict__ expo) {
     __shared__ double V[kNB * kLd];
     __shared__ double rd[kNB];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -799,7 +818,7 @@ __global__ void __launch_bounds__(256) k_trsm_rows(double *__restrict__ A, int64
         const double x0 = y0 * rd[lane], x1 = y1 * rd[lane + 32];
         row[lane] = x0;
         row[lane + 32] = x1;
-        slice_row_warp(x0, x1, lane, rows, r, S, out, expo);
+        slice_row_warp(x0, x1, lane, rows, r, S, round, out, expo);
     }
 }
 
@@ -1152,28 +1171,29 @@ inline unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 size_t slice_elems(int64_t rows, int S) { return (size_t)S * (size_t)rows * kTileK; }
 
 cudaError_t launch_slice_rows(const double *A, int64_t lda, int64_t rows, int kcols, int S,
-                              __nv_bfloat16 *out, int *expo, cudaStream_t st) {
+                              __nv_bfloat16 *out, int *expo, cudaStream_t st, bool round) {
     if (rows <= 0) return cudaSuccess;
     if (kcols < 1 || kcols > kTileK || S < 1 || S > kMaxSlices) return cudaErrorInvalidValue;
-    (k_slice_rows<<<nblk(rows, 8), 256, 0, st>>>(A, lda, rows, kcols, S, out, expo), nk::note_launch());
+    (k_slice_rows<<<nblk(rows, 8), 256, 0, st>>>(A, lda, rows, kcols, S, round, out, expo), nk::note_launch());
     return cudaGetLastError();
 }
 
 // R = A B^T (FP64-accurate to the slice count), applied to C by mode.
 // A and B are given by their slices (rows x 64, as written by
-// launch_slice_rows) and row exponents.
+// launch_slice_rows) and row exponents.  wide: 7 slices, level 9 kept (NK_F64).
 cudaError_t launch_ozaki_gemm_strided(const __nv_bfloat16 *Asl, const int *expA, int64_t rows, int64_t a_stride,
                                       const __nv_bfloat16 *Bsl, const int *expB, int64_t cols, int64_t b_stride,
                                       int S, double *C, int64_t ldc, int mode, bool lower, int *err,
-                                      cudaStream_t st) {
+                                      cudaStream_t st, bool wide) {
     if (rows <= 0 || cols <= 0) return cudaSuccess;
-    if (S < 1 || S > kMaxSlices) return cudaErrorInvalidValue;
+    if (S < 1 || S > kMaxSlices || (wide && S != kMaxSlices)) return cudaErrorInvalidValue;
     if (rows > (1LL << 31) - kTileM || cols > (1LL << 31) - kPN) return cudaErrorInvalidValue;
     CUtensorMap ma, mb;
     if (!make_slice_map(&ma, Asl, rows, S, kTileM, a_stride) || !make_slice_map(&mb, Bsl, cols, S, kPN, b_stride))
         return cudaErrorInvalidValue;
-    const void *kern = S == kMaxSlices ? (const void *)k_ozaki_gemm<kMaxSlices> : (const void *)k_ozaki_gemm<0>;
-    cudaError_t e = nk::allow_max_dynamic_smem(kern);
+    const auto kern = wide ? k_ozaki_gemm<kMaxSlices, true>
+                           : (S == kMaxSlices ? k_ozaki_gemm<kMaxSlices, false> : k_ozaki_gemm<0, false>);
+    cudaError_t e = nk::allow_max_dynamic_smem((const void *)kern);
     if (e != cudaSuccess) return e;
     OzArgs a{rows, cols, S, expA, expB, C, ldc, mode, lower ? 1 : 0, err, (cols + kPN - 1) / kPN, 1, 0,
              ldc % 2 == 0 && reinterpret_cast<uintptr_t>(C) % 16 == 0};
@@ -1195,27 +1215,24 @@ cudaError_t launch_ozaki_gemm_strided(const __nv_bfloat16 *Asl, const int *expA,
     int64_t strips = 0;
     for (int64_t m = 0; m < n_mb; ++m) strips += oz_row_strips(a.n_nb, lower, m, a.chunk_log2);
     if (strips > (1LL << 31) - 1) return cudaErrorInvalidValue;
-    if (S == kMaxSlices)
-        (k_ozaki_gemm<kMaxSlices><<<(unsigned)strips, kPThreads, ozaki_smem_bytes(), st>>>(ma, mb, a),
-         nk::note_launch());
-    else
-        (k_ozaki_gemm<0><<<(unsigned)strips, kPThreads, ozaki_smem_bytes(), st>>>(ma, mb, a), nk::note_launch());
+    (kern<<<(unsigned)strips, kPThreads, ozaki_smem_bytes(), st>>>(ma, mb, a), nk::note_launch());
     return cudaGetLastError();
 }
 
-// BF16 MMA flops a launch executes: active tiles x S(S+1)/2 slice products x
-// 2 x 128 x 32 x 64.
-double ozaki_mma_flops(int64_t rows, int64_t cols, int S, bool lower) {
+// BF16 MMA flops a launch executes: active tiles x S(S+1)/2 slice products (wide: S -
+// 1 more) x 2 x 128 x 32 x 64.
+double ozaki_mma_flops(int64_t rows, int64_t cols, int S, bool lower, bool wide = false) {
     const int64_t tm = (rows + kTileM - 1) / kTileM, tn = (cols + kPN - 1) / kPN;
     int64_t tiles = 0;
     for (int64_t i = 0; i < tm; ++i) tiles += oz_row_tiles(tn, lower, i);
-    return (double)tiles * (S * (S + 1) / 2) * 2.0 * kTileM * kPN * kTileK;
+    return (double)tiles * (S * (S + 1) / 2 + (wide ? S - 1 : 0)) * 2.0 * kTileM * kPN * kTileK;
 }
 
 cudaError_t launch_ozaki_gemm(const __nv_bfloat16 *Asl, const int *expA, int64_t rows,
                               const __nv_bfloat16 *Bsl, const int *expB, int64_t cols, int S, double *C,
-                              int64_t ldc, int mode, bool lower, int *err, cudaStream_t st) {
-    return launch_ozaki_gemm_strided(Asl, expA, rows, rows, Bsl, expB, cols, cols, S, C, ldc, mode, lower, err, st);
+                              int64_t ldc, int mode, bool lower, int *err, cudaStream_t st, bool wide) {
+    return launch_ozaki_gemm_strided(Asl, expA, rows, rows, Bsl, expB, cols, cols, S, C, ldc, mode, lower, err, st,
+                                     wide);
 }
 
 size_t tc_chol_ws_bytes(int64_t n) {
@@ -1295,7 +1312,7 @@ cudaError_t panel_step(double *A, int64_t n, int64_t k0, int *info, int *err, Tc
          nk::note_launch());
         if (rest > 0) {
             const unsigned grid = nblk(rest, 8) < 304 ? nblk(rest, 8) : 304;
-            (k_trsm_rows<<<grid, 256, 0, st>>>(A, n, k0, rest, S, Lsl, Lexp), nk::note_launch());
+            (k_trsm_rows<<<grid, 256, 0, st>>>(A, n, k0, rest, S, exact, Lsl, Lexp), nk::note_launch());
         }
         prof_end(slot, st, 2.0 * (double)kb * kb * kb / 3.0 + (double)rest * kb * kb);
         return cudaGetLastError();
@@ -1305,7 +1322,7 @@ cudaError_t panel_step(double *A, int64_t n, int64_t k0, int *info, int *err, Tc
         if (e == cudaSuccess) e = cudaStreamWaitEvent(cs->aux, cs->ev_fork, 0);
         if (e != cudaSuccess) return e;
         const int aslot = prof_begin(NK_PROF_CHOL_PANEL, cs->aux);
-        e = launch_slice_rows(panel, n, rest, kb, S, Lsl, Lexp, cs->aux);
+        e = launch_slice_rows(panel, n, rest, kb, S, Lsl, Lexp, cs->aux, false);
         prof_end(aslot, cs->aux, 0.0);
         if (e == cudaSuccess) e = cudaEventRecord(cs->ev_join, cs->aux);
         if (e != cudaSuccess) return e;
@@ -1318,15 +1335,15 @@ cudaError_t panel_step(double *A, int64_t n, int64_t k0, int *info, int *err, Tc
     // the inverse and its slices (the B operand of the panel solve)
     (k_trtri64<<<kNB / kTrtriWarps, 32 * kTrtriWarps, 0, st>>>(A, n, k0, kb, Linv, S, w.Bsl, w.expB),
      nk::note_launch());
-    e = aux ? cudaStreamWaitEvent(st, cs->ev_join, 0) : launch_slice_rows(panel, n, rest, kb, S, Lsl, Lexp, st);
+    e = aux ? cudaStreamWaitEvent(st, cs->ev_join, 0) : launch_slice_rows(panel, n, rest, kb, S, Lsl, Lexp, st, false);
     prof_end(slot, st, 2.0 * (double)kb * kb * kb / 3.0);
     if (e == cudaSuccess) {
         slot = prof_begin(NK_PROF_CHOL_UPDATE, st);
-        e = launch_ozaki_gemm(Lsl, Lexp, rest, w.Bsl, w.expB, kb, S, panel, n, 0, false, err, st);
+        e = launch_ozaki_gemm(Lsl, Lexp, rest, w.Bsl, w.expB, kb, S, panel, n, 0, false, err, st, false);
         // the triangular solve L21 = A21 L11^-T: rest kb^2 flops in FP64
         prof_end(slot, st, (double)rest * kb * kb, ozaki_mma_flops(rest, kb, S, false));
         slot = prof_begin(NK_PROF_CHOL_PANEL, st);
-        if (e == cudaSuccess) e = launch_slice_rows(panel, n, rest, kb, S, Lsl, Lexp, st);
+        if (e == cudaSuccess) e = launch_slice_rows(panel, n, rest, kb, S, Lsl, Lexp, st, false);
         prof_end(slot, st, 0.0);
     }
     return e != cudaSuccess ? e : cudaGetLastError();
@@ -1370,10 +1387,10 @@ cudaError_t launch_cholesky_tc(double *A, int64_t n, int *info, int *err, void *
         }
         // narrow: block column k + 1 (all rows below panel k)
         int slot = prof_begin(NK_PROF_CHOL_UPDATE, ps);
-        e = launch_ozaki_gemm_strided(Lk, Le, rest, rest, Lk, Le, kb1, rest, S, C1, n, 1, true, err, ps);
+        e = launch_ozaki_gemm_strided(Lk, Le, rest, rest, Lk, Le, kb1, rest, S, C1, n, 1, true, err, ps, exact);
         // FP64 flops of the lower part of the rest x kb1 block column, K = kNB
         prof_end(slot, ps, 2.0 * kNB * ((double)rest * kb1 - 0.5 * (double)kb1 * (kb1 - 1)),
-                 ozaki_mma_flops(rest, kb1, S, true));
+                 ozaki_mma_flops(rest, kb1, S, true, exact));
         if (e != cudaSuccess) return e;
         e = panel_step(A, n, k0 + kNB, info, err, w, buf[(k + 1) & 1], bexp[(k + 1) & 1], ps, cs, exact,
                        joined);
@@ -1387,9 +1404,11 @@ cudaError_t launch_cholesky_tc(double *A, int64_t n, int *info, int *err, void *
         if (rest2 > 0) {
             slot = prof_begin(NK_PROF_CHOL_UPDATE, st);
             e = launch_ozaki_gemm_strided(Lk + (size_t)kb1 * kTileK, Le + kb1, rest2, rest, Lk + (size_t)kb1 * kTileK,
-                                          Le + kb1, rest2, rest, S, C1 + (size_t)kb1 * n + kb1, n, 1, true, err, st);
+                                          Le + kb1, rest2, rest, S, C1 + (size_t)kb1 * n + kb1, n, 1, true, err, st,
+                                          exact);
             // FP64 flops of the lower rest2 x rest2 trailing update, K = kNB
-            prof_end(slot, st, (double)kNB * rest2 * (double)(rest2 + 1), ozaki_mma_flops(rest2, rest2, S, true));
+            prof_end(slot, st, (double)kNB * rest2 * (double)(rest2 + 1),
+                     ozaki_mma_flops(rest2, rest2, S, true, exact));
             if (e != cudaSuccess) return e;
         }
         if (two) {
@@ -1441,14 +1460,15 @@ cudaError_t launch_cholesky_solve_tc(const double *L, int64_t n, const void *ws,
 // chunk of T [Ns][M], then the Jacobian-row Gram s.s + t.t + (t.t)(s.s)
 // written to both triangles.
 cudaError_t launch_gram_tc(int N, int M, int64_t Ns, const int8_t *s, const double *T, int S, double *K,
-                           int *err, void *ws, cudaStream_t st) {
+                           int *err, void *ws, cudaStream_t st, bool wide) {
     TcWs w = carve_tc(ws, Ns);
     const int slot = prof_begin(NK_PROF_GRAM, st);
     for (int c = 0; c < M; c += kTileK) {
         const int kc = M - c < kTileK ? M - c : kTileK;
-        cudaError_t e = launch_slice_rows(T + c, M, Ns, kc, S, w.Asl, w.expA, st);
+        cudaError_t e = launch_slice_rows(T + c, M, Ns, kc, S, w.Asl, w.expA, st, wide);
         if (e == cudaSuccess)
-            e = launch_ozaki_gemm(w.Asl, w.expA, Ns, w.Asl, w.expA, Ns, S, K, Ns, c == 0 ? 0 : 2, true, err, st);
+            e = launch_ozaki_gemm(w.Asl, w.expA, Ns, w.Asl, w.expA, Ns, S, K, Ns, c == 0 ? 0 : 2, true, err, st,
+                                  wide);
         if (e != cudaSuccess) return e;
     }
     dim3 grid(nblk(Ns, 64), nblk(Ns, 64));
@@ -1456,7 +1476,7 @@ cudaError_t launch_gram_tc(int N, int M, int64_t Ns, const int8_t *s, const doub
     // the lower triangle of the Jacobian-row Gram through s.s + t.t + (t.t)(s.s):
     // (N + M) flops per entry, the count of the FP64 path
     prof_end(slot, st, (double)Ns * (Ns + 1) * (double)(N + M),
-             (double)((M + kTileK - 1) / kTileK) * ozaki_mma_flops(Ns, Ns, S, true));
+             (double)((M + kTileK - 1) / kTileK) * ozaki_mma_flops(Ns, Ns, S, true, wide));
     return cudaGetLastError();
 }
 

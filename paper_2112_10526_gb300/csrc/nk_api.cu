@@ -400,16 +400,16 @@ nk_status jacobi_eigen(nk_ctx *ctx, double *K, double *V, int64_t n, void *eig_w
 // second Cholesky, of S itself.  E, in units of u = 2^-53 and sqrt(s_ii s_jj), which
 // also bounds ||E|| in units of u tr S:
 //   - the trailing updates, per panel of 64 columns with m_i the row's largest entry
-//     in it: slices truncated at 2^-56 of at most 2 m_i, 64 (2^-55 + 2^-55) m_i m_j =
-//     32; slice products s + t >= 9 left out, at most 6.03 255^2 2^-72 4 m_i m_j a
-//     column, 192; the recombination, 2; and sum_p m_i m_j <= sqrt(s_ii s_jj);
+//     in it: entries rounded at 2^-57 of at most 2 m_i, 64 (2^-56 + 2^-56) m_i m_j =
+//     16; slice products s + t >= 10 left out, at most 5.02 255^2 2^-80 4 m_i m_j a
+//     column, 0.7; the window, 0.3; and sum_p m_i m_j <= sqrt(s_ii s_jj);
 //   - the additions to C, 2 a panel: n / 32;
 //   - diagonal blocks (64 operations of 2^-59, or FP64) and substitution in FP64: 70.
 // *done = false with S untouched where the proof does not go
 // through (a rank-deficient or nearly singular S): the eigensolver decides
 // there.  Order 880 (t-VMC on 20 sites): two factors and a solve take 3 ms, the
 // Jacobi sweeps 331 ms.  scratch: n x n; trace: one double.
-constexpr double kPanelErr = 226.0;  // of a panel's update
+constexpr double kPanelErr = 17.0;  // of a panel's update
 constexpr double kBlockErr = 70.0;
 
 nk_status full_rank_solve(nk_ctx *ctx, double *S, double *scratch, int64_t n, double rcond, const double *b,
@@ -515,7 +515,7 @@ nk_status run_solve(nk_ctx *ctx, int N, int M, int64_t Ns, const int8_t *s, cons
         if (ss) {
             // the centred sample-space Gram X X^T, X = dJ / sqrt(Ns), no shift
             if (nk::gram_on_tensor(precision, M, Ns)) {
-                NK_CU(nk::launch_gram_tc(N, M, Ns, s, T, 7, w.K, w.info + 1, w.tc, st), "svd gram");
+                NK_CU(nk::launch_gram_tc(N, M, Ns, s, T, 7, w.K, w.info + 1, w.tc, st, !tc), "svd gram");
                 NK_CU(nk::launch_center_gram(Ns, w.K, w.rowmean, 0.0, st), "svd gram");
             } else {
                 NK_CU(nk::launch_gram_samplespace(N, M, Ns, s, T, 0.0, w.K, w.rowmean, st), "svd gram");
@@ -581,7 +581,7 @@ nk_status run_solve(nk_ctx *ctx, int N, int M, int64_t Ns, const int8_t *s, cons
     const double isq = 1.0 / std::sqrt((double)Ns);
     NK_CU(cudaMemsetAsync(w.info, 0, 2 * sizeof(int), st), "ss");
     if (nk::gram_on_tensor(precision, M, Ns)) {
-        NK_CU(nk::launch_gram_tc(N, M, Ns, s, T, 7, w.K, w.info + 1, w.tc, st), "ss gram");
+        NK_CU(nk::launch_gram_tc(N, M, Ns, s, T, 7, w.K, w.info + 1, w.tc, st, !tc), "ss gram");
         NK_CU(nk::launch_center_gram(Ns, w.K, w.rowmean, eps, st), "ss gram");
     } else {
         NK_CU(nk::launch_gram_samplespace(N, M, Ns, s, T, eps, w.K, w.rowmean, st), "ss gram");

@@ -206,11 +206,11 @@ cudaError_t launch_center_gram(int64_t Ns, double *K, double *rowmean, double ep
 // FP64 rows -> S BF16 integer slices [S][rows][64] + row exponents.
 size_t slice_elems(int64_t rows, int S);
 cudaError_t launch_slice_rows(const double *A, int64_t lda, int64_t rows, int kcols, int S,
-                              __nv_bfloat16 *out, int *expo, cudaStream_t st);
+                              __nv_bfloat16 *out, int *expo, cudaStream_t st, bool round = false);
 // C (mode 0: =, 1: -=, 2: +=) A B^T from slices, 128 x 32 tiles, K <= 64.
 cudaError_t launch_ozaki_gemm(const __nv_bfloat16 *Asl, const int *expA, int64_t rows,
                               const __nv_bfloat16 *Bsl, const int *expB, int64_t cols, int S, double *C,
-                              int64_t ldc, int mode, bool lower, int *err, cudaStream_t st);
+                              int64_t ldc, int mode, bool lower, int *err, cudaStream_t st, bool wide = false);
 size_t tc_chol_ws_bytes(int64_t n);
 // Streams of the panel look-ahead: `side` carries the panel chain, `aux`
 // the slicing of a panel beside its diagonal block; the events join them.
@@ -229,7 +229,7 @@ cudaError_t launch_cholesky_tc(double *A, int64_t n, int *info, int *err, void *
 cudaError_t launch_cholesky_solve_tc(const double *L, int64_t n, const void *ws, double *b, int *err,
                                      cudaStream_t st, bool exact);
 cudaError_t launch_gram_tc(int N, int M, int64_t Ns, const int8_t *s, const double *T, int S, double *K,
-                           int *err, void *ws, cudaStream_t st);
+                           int *err, void *ws, cudaStream_t st, bool wide);
 // Lower triangle of C = scale X^T X + eps I (X [rows][n]) by 7-slice
 // tensor-core products of any length (k_syrk.cu); ws of tc_syrk_ws_bytes.
 size_t tc_syrk_ws_bytes(int64_t rows, int64_t n);

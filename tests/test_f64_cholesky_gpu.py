@@ -1,10 +1,15 @@
-"""The NK_F64 triangular solves (launch_cholesky_solve_tc, `exact`) on matrices whose
-roundings all go one way.
+"""The NK_F64 factorisation and its triangular solves (launch_cholesky_tc and
+launch_cholesky_solve_tc, `exact`) on matrices whose roundings all go one way.
 
 fwd, bwd: L = I and one row, or column, of a 1 and otherwise 0.9 2^-53, which a single
 chain of n / 32 or n / 8 additions drops term by term: the sum of n terms comes back to
 (terms of a group + groups + 40) 2^-53, the groups those of the kernels (16 terms and n /
-512, 32 and n / 256; 40 for the lanes, warps, the block's solve and the data)."""
+512, 32 and n / 256; 40 for the lanes, warps, the block's solve and the data).
+
+panel: rows of one large entry and 63 of 2^-8 of it, against rows of large ones, with
+digits of 255: the update's error in units of 2^-53 sqrt(a_ii a_jj) is at most 18 / 8
+(the bound of a panel, 17 m_i m_j, and its addition, on |l_i| |l_j| = 8 m_i m_j), the
+diagonal block's and the data's roundings 2 more."""
 import os
 import shutil
 import subprocess
@@ -51,6 +56,34 @@ static int solve(int64_t n, std::vector<double> &A, std::vector<double> &b) {
 
 int main(int argc, char **argv) {
     const double u = 0x1p-53, q = 0.9 * u;
+    if (!strcmp(argv[1], "panel")) {
+        const int64_t n = 128;
+        const double big = ldexp((double)((1LL << 52) + (1LL << 45) - 1), -53);
+        const double small = ldexp((double)((1LL << 53) - 17), -61);
+        std::vector<double> l(64 * 64), A(n * n, 0.0), b(n, 1.0);
+        for (int r = 0; r < 64; ++r)
+            for (int c = 0; c < 64; ++c) l[r * 64 + c] = r % 2 || c == r / 2 ? big : small;
+        for (int i = 0; i < 64; ++i) A[i * n + i] = 1.0;
+        for (int r = 0; r < 64; ++r) {
+            for (int c = 0; c < 64; ++c) A[(64 + r) * n + c] = l[r * 64 + c];
+            for (int s = 0; s <= r; ++s) {
+                long double v = 0.0L;
+                for (int c = 0; c < 64; ++c) v += (long double)l[r * 64 + c] * l[s * 64 + c];
+                A[(64 + r) * n + 64 + s] = (double)(r == s ? 1.25L * v : v);
+            }
+        }
+        std::vector<double> L = A;
+        if (int e = solve(n, L, b)) return e;
+        double worst = 0;
+        for (int i = 0; i < n; ++i)
+            for (int j = 0; j <= i; ++j) {
+                long double v = 0.0L;
+                for (int c = 0; c <= j; ++c) v += (long double)L[i * n + c] * L[j * n + c];
+                worst = fmax(worst, (double)(fabsl(v - A[i * n + j]) / sqrt(A[i * n + i] * A[j * n + j]) / u));
+            }
+        printf("worst %g u\n", worst);
+        return worst <= 18.0 / 8 + 2 ? 0 : 1;
+    }
     const int64_t n = 8192;
     std::vector<double> A(n * n, 0.0), b(n, 1.0);
     for (int64_t i = 0; i < n; ++i) A[i * n + i] = 1.0;
@@ -97,7 +130,7 @@ def program():
         yield exe
 
 
-@pytest.mark.parametrize("what", ["fwd", "bwd"])
+@pytest.mark.parametrize("what", ["fwd", "bwd", "panel"])
 def test_roundings_that_go_one_way(program, what):
     r = subprocess.run([program, what], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stdout + r.stderr
