@@ -386,6 +386,9 @@ typedef struct {
  *   stats_out: device nk_sr_stats or NULL.
  *   samples_out [C*n_samples, N], eloc_out [C*n_samples]: optional device
  *   outputs of this step's samples and local energies (NULL = internal).
+ * With NK_MIXED and NK_SOLVER_CG the step's tanh(theta) is CUDA's, whose last bit may
+ * differ from the library's own in nk_local_energy and nk_force: a step put together
+ * from the single calls then agrees within the tolerance of the CG, not bit for bit.
  */
 nk_status nk_sr_step(nk_ctx *ctx, nk_rbm *rbm, const nk_ham *ham, nk_chains *chains,
                      const nk_sr_cfg *cfg, nk_sr_stats *stats_out, int8_t *samples_out,

@@ -505,8 +505,9 @@ __device__ __forceinline__ void renorm_fast(Prod<float> &p) {
 }
 
 // tanh(theta) of a unit after a flip: (t - s tau) / (1 - s t tau), s = +1 (kPos) or
-// -1, as a product with the approximate reciprocal: the value of __fdividef here
-// (the denominator is 0 or at least 2^-48, and below 2) in four instructions.
+// -1, as a product with the approximate reciprocal, in four instructions: the value of
+// __fdividef here, whose div.approx.f32 the PTX ISA manual defines as a * (1 / b) for b
+// in [2^-126, 2^126] (the denominator is 0 or at least 2^-48, and below 2).
 __device__ __forceinline__ float rcp_approx(float x) {
     float y;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
