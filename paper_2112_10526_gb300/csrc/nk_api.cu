@@ -845,6 +845,21 @@ nk_status nk_ctx_create(int32_t device, nk_ctx **out) {
     for (int i = 0; i < 4 && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&c->ev[i], cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaMalloc(&c->tc_err, 256);
     if (e == cudaSuccess) e = cudaMemset(c->tc_err, 0, 256);
+    if (e == cudaSuccess) {
+        // keeps up to 256 MiB between calls (the driver would give it back at every
+        // synchronisation); without it the calls that draw on it still run
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = device;
+        uint64_t keep = 256ULL << 20;
+        if (cudaMemPoolCreate(&c->pool, &props) != cudaSuccess ||
+            cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+            cudaGetLastError();
+            if (c->pool) cudaMemPoolDestroy(c->pool);
+            c->pool = nullptr;
+        }
+    }
     if (e != cudaSuccess) {
         if (c->host_flags) cudaFreeHost(c->host_flags);
         if (c->host_vals) cudaFreeHost(c->host_vals);
@@ -1565,25 +1580,6 @@ nk_status check_complex_out(const double *p, const char *name) {
     return NK_OK;
 }
 
-// The context's pool, made by the first call that wants it (it is no stream operation,
-// so also under capture); null without one.  It keeps up to 256 MiB between calls,
-// which the driver would otherwise give back at every synchronisation.
-cudaMemPool_t ctx_pool(nk_ctx *ctx) {
-    if (ctx->pool) return ctx->pool;
-    cudaMemPoolProps props = {};
-    props.allocType = cudaMemAllocationTypePinned;
-    props.location.type = cudaMemLocationTypeDevice;
-    props.location.id = ctx->device;
-    uint64_t keep = 256ULL << 20;
-    cudaMemPool_t pool = nullptr;
-    if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
-    }
-    if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) cudaGetLastError();
-    return ctx->pool = pool;
-}
-
 // One slope of the t-VMC equation of motion at parameters p: sample, local
 // energies and their statistics, the realified centred Jacobian R, the force
 // R^T g = [Re f; Im f], the real embedding of G + eps I and its solve for
@@ -1701,8 +1697,8 @@ nk_status nk_crbm_local_energy(nk_ctx *ctx, const nk_crbm *rbm, const nk_ham *ha
     // the context.  Where there is no room for them it does without.
     cudaStream_t st = (cudaStream_t)stream;
     void *exps = nullptr;
-    cudaMemPool_t pool = ctx_pool(ctx);
-    if (!pool || cudaMallocFromPoolAsync(&exps, nk::crbm_eloc_ws_bytes(rbm->N, rbm->M), pool, st) != cudaSuccess) {
+    if (!ctx->pool ||
+        cudaMallocFromPoolAsync(&exps, nk::crbm_eloc_ws_bytes(rbm->N, rbm->M), ctx->pool, st) != cudaSuccess) {
         cudaGetLastError();
         exps = nullptr;
     }
