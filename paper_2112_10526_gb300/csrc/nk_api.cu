@@ -845,21 +845,6 @@ nk_status nk_ctx_create(int32_t device, nk_ctx **out) {
     for (int i = 0; i < 4 && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&c->ev[i], cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaMalloc(&c->tc_err, 256);
     if (e == cudaSuccess) e = cudaMemset(c->tc_err, 0, 256);
-    if (e == cudaSuccess) {
-        // keeps up to 256 MiB between calls (the driver would give it back at every
-        // synchronisation); without it the calls that draw on it still run
-        cudaMemPoolProps props = {};
-        props.allocType = cudaMemAllocationTypePinned;
-        props.location.type = cudaMemLocationTypeDevice;
-        props.location.id = device;
-        uint64_t keep = 256ULL << 20;
-        if (cudaMemPoolCreate(&c->pool, &props) != cudaSuccess ||
-            cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
-            cudaGetLastError();
-            if (c->pool) cudaMemPoolDestroy(c->pool);
-            c->pool = nullptr;
-        }
-    }
     if (e != cudaSuccess) {
         if (c->host_flags) cudaFreeHost(c->host_flags);
         if (c->host_vals) cudaFreeHost(c->host_vals);
@@ -1580,6 +1565,46 @@ nk_status check_complex_out(const double *p, const char *name) {
     return NK_OK;
 }
 
+// The context's pool, made by the first call that wants it; null without one.  It keeps
+// up to 256 MiB between calls, which the device's own pool gives back at every
+// synchronisation (180 us a call).  The thread's capture mode is relaxed meanwhile, so
+// that a capture elsewhere is not disturbed.
+cudaMemPool_t ctx_pool(nk_ctx *ctx) {
+    if (ctx->pool) return ctx->pool;
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = ctx->device;
+    uint64_t keep = 256ULL << 20;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaError_t e = cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e == cudaSuccess) {
+        e = cudaMemPoolCreate(&ctx->pool, &props);
+        if (e != cudaSuccess)
+            ctx->pool = nullptr;
+        else
+            e = cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep);
+        cudaThreadExchangeStreamCaptureMode(&mode);
+    }
+    if (e != cudaSuccess) cudaGetLastError();
+    return ctx->pool;
+}
+
+// Stream-ordered scratch for a call on st: from the context's pool, or as a node of the
+// graph that st is captured into.  Null where there is no room.
+void *stream_scratch(nk_ctx *ctx, size_t bytes, cudaStream_t st) {
+    void *p = nullptr;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(st, &cap);
+    if (e == cudaSuccess) {
+        cudaMemPool_t pool = cap == cudaStreamCaptureStatusNone ? ctx_pool(ctx) : nullptr;
+        e = pool ? cudaMallocFromPoolAsync(&p, bytes, pool, st) : cudaMallocAsync(&p, bytes, st);
+    }
+    if (e == cudaSuccess) return p;
+    cudaGetLastError();
+    return nullptr;
+}
+
 // One slope of the t-VMC equation of motion at parameters p: sample, local
 // energies and their statistics, the realified centred Jacobian R, the force
 // R^T g = [Re f; Im f], the real embedding of G + eps I and its solve for
@@ -1692,16 +1717,11 @@ nk_status nk_crbm_local_energy(nk_ctx *ctx, const nk_crbm *rbm, const nk_ham *ha
     NK_DEV(s, "s");
     if ((st0 = check_complex_out(eloc_out, "eloc_out")) != NK_OK) return st0;
     if (g_plan_only) return NK_OK;
-    // The tables come from the context's pool in stream order, not from its workspace:
-    // the call synchronises nothing, can be captured and may run beside another call of
-    // the context.  Where there is no room for them it does without.
+    // The tables are stream-ordered scratch, not the context's workspace: the call
+    // synchronises nothing, can be captured and may run beside another call of the
+    // context.  Where there is no room for them it does without.
     cudaStream_t st = (cudaStream_t)stream;
-    void *exps = nullptr;
-    if (!ctx->pool ||
-        cudaMallocFromPoolAsync(&exps, nk::crbm_eloc_ws_bytes(rbm->N, rbm->M), ctx->pool, st) != cudaSuccess) {
-        cudaGetLastError();
-        exps = nullptr;
-    }
+    void *exps = stream_scratch(ctx, nk::crbm_eloc_ws_bytes(rbm->N, rbm->M), st);
     const cudaError_t e = nk::launch_crbm_eloc(rbm->N, rbm->M, rbm->params, ham, s, Ns, eloc_out, exps, st);
     if (exps) NK_CU(cudaFreeAsync(exps, st), "local energy");
     NK_CU(e, "local energy");

@@ -23,7 +23,7 @@ struct nk_ctx {
     int *tc_err;        // device, 256 bytes: [0] sticky code of the first tensor-core
                         // time-out; [16] flag of the symmetric RBM's permutation check
     size_t plan_bytes;  // workspace counted by plan-only calls
-    cudaMemPool_t pool; // scratch of the calls that use no workspace, or null
+    cudaMemPool_t pool; // scratch of the calls that use no workspace (null before the first)
 };
 
 namespace nk {
