@@ -673,8 +673,8 @@ def run_tdvp(name, K, warmup, dev):
             "config": {"workload": name, "lattice": lattice_text(N), "hamiltonian": "tfim (h = 1 quench)",
                        "model": "complex RBM, alpha = 1", "N": N, "M": M, "Np_complex": N + M + M * N,
                        "chains": C, "samples_per_chain": w["per_chain"], "Ns": Ns, "integrator": w["integrator"],
-                       "dt": w["dt"], "time": "real", "solver": f"pseudo-inverse (rcond {w['rcond']:g}), "
-                       f"Jacobi on the {2 * (N + M + M * N)}-dim real embedding", "precision": "f64"}}
+                       "dt": w["dt"], "time": "real", "solver": f"pseudo-inverse (rcond {w['rcond']:g}) "
+                       f"of the {2 * (N + M + M * N)}-dim real embedding", "precision": "f64"}}
 
 
 # ---------------------------------------------------------------- serving ----

@@ -523,9 +523,10 @@ typedef struct {
  * eq:tvmc); then the explicit Runge-Kutta update of Eq. eq:rk-step.  The
  * Hermitian system is solved through its real embedding [[Re G, -Im G],
  * [Im G, Re G]] of order 2 Np, built as R^T R / Ns from the realified
- * centred Jacobian R (2 Ns x 2 Np): by the FP64 Cholesky, or by the cyclic
- * Jacobi eigensolver of the SVD solvers (2 Np <= 8192; synchronises the
- * stream once per sweep).
+ * centred Jacobian R (2 Ns x 2 Np): by Cholesky, or with NK_SOLVER_SVD (2 Np <=
+ * 8192) by Cholesky where a factor of S - tau I proves that no eigenvalue is cut
+ * off, else by the cyclic Jacobi eigensolver of the SVD solvers; synchronises the
+ * stream.
  *   rbm->params updated in place; chains advanced (sweeps_done on the host).
  *   stats_out: device nk_tdvp_stats or NULL; theta_dot_out: device [Np]
  *   complex, the first slope, or NULL.

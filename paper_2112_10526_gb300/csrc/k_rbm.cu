@@ -1380,7 +1380,7 @@ __global__ void __launch_bounds__(128) k_sweep_rows(SweepK<float> P) {
 // proposals that share a site with it: then the row is fetched on demand).
 // k_sweep had a warp per chain, t in shared memory (12 chains an SM at M = 4608)
 // and read the row twice from L2: 12 TB/s of it, and three warps a scheduler.
-// 24 x 24 lattice, M = 4608, 8192 chains: 7.3 ms a sweep there, 5.4 here.
+// 24 x 24 lattice, M = 4608, 8192 chains: 6.8 ms a sweep there, 5.3 here.
 template <int kU>
 __global__ void __launch_bounds__(64, kU <= 16 ? (kU <= 8 ? 16 : 12) : (kU <= 24 ? 9 : (kU <= 40 ? 6 : 4))) k_sweep_pair(SweepK<float> P) {
     extern __shared__ __align__(16) unsigned char sm[];
@@ -2088,8 +2088,8 @@ cudaError_t launch_sweep<float>(const Tables<float> &t, const SweepArgs &a, cuda
     if (regs && chunks <= 4)
         return chunks == 1 ? launch_sweep_rows<1>(P, st)
                            : (chunks == 2 ? launch_sweep_rows<2>(P, st) : launch_sweep_rows<4>(P, st));
-    // ... or two: from 25 chunks of 128 units (M = 4608, 8192 chains: 5.5 ms a sweep,
-    // 6.3 by k_sweep; 256 chains: 0.74 and 1.19), and below with at most eight chains
+    // ... or two: from 25 chunks of 128 units (M = 4608, 8192 chains: 5.3 ms a sweep,
+    // 6.8 by k_sweep; 256 chains: 0.74 and 1.19), and below with at most eight chains
     // an SM (M = 2000, 512 chains: 0.21 and 0.31 ms; M = 1600, 8192 chains: 3.7 and 3.0)
     if (regs && chunks <= 48 && (chunks > 24 || a.C <= 1216))
         return chunks <= 8    ? launch_sweep_pair<8>(P, st)

@@ -14,10 +14,12 @@
 // slices stream through a TMA ring; beyond, configurations stream along.  Warp 0 loads, warp 1 issues the MMAs into
 // one of two accumulator sets, sixteen warps turn the other set into FP64 and
 // store it by rows.
-// What bounds it: the slices in flight (20 KB a chunk, three to six stages,
-// against about 1 us of L2 latency).  The tile kernel this replaces (k_sgemm:
-// one 128 x 64 tile a CTA, nothing overlapping its drain) took 19 us for 1024 x
-// 200 x 100 and 4.70 ms for 65536 x 4608 x 576.
+// What bounds it: for theta the slices in flight (20 KB a chunk, three to six
+// stages, against about 1 us of L2 latency); with tanh and pairs the epilogue's
+// integer instructions (8192 x 4608: ALU pipe 60 %, issue 54 %, tensor pipe 12 %).
+// The tile kernel this replaces (k_sgemm: one 128 x 64 tile a CTA, nothing
+// overlapping its drain) took 19 us for 1024 x 200 x 100 and 4.70 ms for 65536 x
+// 4608 x 576.
 // The epilogue writes theta in FP64, or (for the products of NK_MIXED that read
 // tanh(theta) as FP32 pairs) t' = [tanh(theta), 1] straight into the tile order
 // of k_tc4, with the exponents of its columns: the 24 x 24 lattice's 302 M
